@@ -9,12 +9,14 @@
 // place, which the second part holds exactly.  Only elements below 2^-10 of the row's largest
 // fall under e4m3's smallest step (2^-9); their error is at most 2^-17 of that largest.
 //
-// The two parts are stacked along the MMA's M dimension: the operand slab of a K step holds the
-// first parts of all token rows and, below them, the second parts, and ONE MMA per K step computes
-// both products (products of e4m3 numbers are exact in fp32).  A token's logit is the sum of its two
-// accumulator rows; they sit in different lane quadrants of tensor memory, so the epilogue warp of the
-// second parts passes its columns through shared memory to the warp of the first parts, which adds
-// them, multiplies by r (per token row) and by the weight row's scale, and folds as the bf16 path does.
+// The two parts are stacked along the MMA's M dimension in alternating groups of eight rows (tc8_part_row), and ONE
+// MMA per K step computes both products (products of e4m3 numbers are exact in fp32).  A token's logit is the sum of
+// two accumulator rows eight lanes apart; the epilogue reads tensor memory in the 16 x 256-bit fragment layout, which
+// gives both to the same thread, so it adds them in registers, multiplies by r (per token row) and by the weight row's
+// scale, and folds.  (With all first parts above all second parts the two sums sat in different lane quadrants and
+// went through shared memory from one warp to another, one thread per row with half of the threads idle: what
+// followed a CTA's last MMA took 5.5 us, now 2.0; decode16 -- d = 896, V = 151936 -- 33.9 -> 30.6 us per step in a
+// graph, n = 32 37.5 -> 34.3, n = 64 39.9 -> 38.9.)
 // One MMA per K step at twice the bf16 rate leaves the tensor pipe half as busy as the bf16 path; the
 // bytes from HBM are half.
 //
@@ -39,8 +41,8 @@ h_split_kernel(const __nv_bfloat16* __restrict__ h, int n, int d, int part_rows,
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int row = blockIdx.x;
-  const size_t part_stride = static_cast<size_t>(part_rows) * d;
-  uint8_t* out = parts + static_cast<size_t>(row) * d;
+  const size_t part_stride = static_cast<size_t>(tc8_part_stride(part_rows)) * d;
+  uint8_t* out = parts + static_cast<size_t>(tc8_part_row(row, part_rows)) * d;
   if (row >= n) {
     for (int k = threadIdx.x * 2; k < d; k += 256) {
       *reinterpret_cast<uint16_t*>(out + k) = 0;
@@ -77,7 +79,7 @@ void tc8_configure(int n, int d, TcConfig* c) {
   const int a_stage = 2 * part_rows * kRowBytes;
   const int b_stage = kBlockN * kRowBytes;
   const int k_slabs = (d + kRowBytes - 1) / kRowBytes;
-  const int extra = tc8_extra_bytes(part_rows);
+  const int extra = kTc8ExtraBytes;
   const int budget = kSmemLimit - 1024 - kBarrierBytes - kScratchBytes - extra;
   // n <= 16 and all of h (two parts) small enough: the kernel splits h itself and keeps it resident, one
   // launch less.  TLR_TC8_INLINE=0 is a tuning switch that keeps the separate split kernel.

@@ -38,6 +38,14 @@ __device__ __forceinline__ float2 from_e4m3x2(uint16_t v) {   // .x = low byte, 
   return __half22float2(*reinterpret_cast<__half2*>(&h2));
 }
 
+// Where a token's two parts sit in the operand slab.  Up to 64 token rows they alternate in groups of eight -- rows
+// 16g .. 16g + 7 hold the first parts of tokens 8g .. 8g + 7, the next eight their second parts -- so that one thread
+// of the epilogue's fragment layout holds both sums of a token; above, the first parts of all rows come first.
+__host__ __device__ __forceinline__ int tc8_part_row(int row, int part_rows) {
+  return part_rows > 64 ? row : (row >> 3) * 16 + (row & 7);
+}
+__host__ __device__ __forceinline__ int tc8_part_stride(int part_rows) { return part_rows > 64 ? part_rows : 8; }
+
 // The power of two r that puts a row's largest magnitude amax into [128, 256) after division.
 __device__ __forceinline__ float split_scale(float amax) {
   float r = 1.0f;
@@ -59,8 +67,8 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint16_t& p1, uin
 
 // Splits the (at most 16) rows of h into resident operand slabs, done by 288 threads numbered t (the caller's
 // warps 2..10; they synchronise among themselves with named barrier 1).  Slab ks is 32 rows of 128 bytes
-// with the 128-byte swizzle TMA would have produced: rows 0..15 hold the first parts, rows 16..31 the
-// second parts; the 16-byte chunk c of row r sits at position c ^ (r & 7).  hs_s[r] receives row r's scale
+// with the 128-byte swizzle TMA would have produced, the two parts in alternating groups of eight rows
+// (tc8_part_row); the 16-byte chunk c of row r sits at position c ^ (r & 7).  hs_s[r] receives row r's scale
 // (hs_s[32 + r] is scratch).  One pass over h: 18 threads per row, each keeps its (at most kSplitChunks) chunks of
 // 16 elements in registers between the maximum and the conversion, so the row is read from memory once and all
 // loads are in flight together.
@@ -117,9 +125,9 @@ __device__ __forceinline__ void split_h_resident(const __nv_bfloat16* __restrict
       q1[j >> 1] |= static_cast<uint32_t>(p1) << (16 * (j & 1));
       q2[j >> 1] |= static_cast<uint32_t>(p2) << (16 * (j & 1));
     }
-    unsigned char* dst = slabs + ks * 4096 + r * 128 + ((c ^ (r & 7)) << 4);
+    unsigned char* dst = slabs + ks * 4096 + tc8_part_row(r, 16) * 128 + ((c ^ (r & 7)) << 4);
     *reinterpret_cast<uint4*>(dst) = make_uint4(q1[0], q1[1], q1[2], q1[3]);
-    *reinterpret_cast<uint4*>(dst + 2048) = make_uint4(q2[0], q2[1], q2[2], q2[3]);
+    *reinterpret_cast<uint4*>(dst + 1024) = make_uint4(q2[0], q2[1], q2[2], q2[3]);
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic stores -> the MMA's (async proxy) reads
 }

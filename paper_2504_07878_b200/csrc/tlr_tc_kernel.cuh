@@ -10,10 +10,10 @@
 //               tensor cores read both halves, so a W byte enters shared memory once
 //               per 256 token rows.                                       (n > 128)
 //   <1, true>   8-bit (e4m3) head for decode batches of at most 128 rows: h is the sum of two e4m3
-//               parts, stacked in one operand slab (rows 0.. = first parts, rows part_rows.. =
-//               second parts).  Up to 64 rows ONE kind::f8f6f4 MMA per K step covers both parts
-//               along its M, and the epilogue adds the two accumulator rows of a token before it
-//               folds them; above, two MMAs per K step (one per part) add into the same rows.
+//               parts, stacked in one operand slab.  Up to 64 rows ONE kind::f8f6f4 MMA per K step
+//               covers both parts along its M, and the epilogue adds the two accumulator rows of a
+//               token before it folds them; above, two MMAs per K step (one per part) add into the
+//               same rows.
 //
 // Decomposition.  The vocabulary is cut into `chunks` contiguous ranges of granules
 // (a multiple of 16 * kCta rows); the token rows into units of 128 * kCta.  A work unit is
@@ -79,14 +79,11 @@ constexpr int kBarrierBytes = 640;
 constexpr int kScratchBytes = kBlockM * 16;  // one Partial per row: hand-over between the epilogue groups
 constexpr int kSmemLimit = 232448;           // 227 KiB opt-in maximum per CTA
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
-// 8-bit head: weight scales of a tile for each of the four warps that fold, the rows' power-of-two scales,
-// and four hand-over buffers (32 columns x lanes floats) between the warps that hold a token's two parts
-// (with more than 64 rows nothing is handed over and the buffers' space holds the scales for all eight warps)
-constexpr int kScaleBytes = 4 * kBlockN * 4;
+// 8-bit head: the weight scales of every epilogue warp's share of a tile, and the rows' power-of-two scales
+constexpr int kScaleBytes = kEpiWarps * (kBlockN / 2) * 4;
 constexpr int kRowScaleBytes = 64 * 4;
-__host__ __device__ constexpr int tc8_extra_bytes(int part_rows) {
-  return kScaleBytes + kRowScaleBytes + 4 * 32 * 4 * (part_rows > 32 ? 32 : 16);
-}
+constexpr int kTc8ExtraBytes = kScaleBytes + kRowScaleBytes;
+constexpr float kNoLogit = -1.0e30f;         // stands for a column beyond V: finite, so that 0 * y stays 0 in the folds
 
 // The static schedule, identical in every role: worker w walks units w, w + workers, ...;
 // each unit is `tiles_per_unit` tiles (possibly empty ones when the chunk is short).
@@ -165,7 +162,7 @@ struct RowFold {
     if (valid < 32) {
 #pragma unroll
       for (int j = 0; j < 32; ++j)
-        if (j >= valid) z[j] = -1.0e30f;   // finite, so 0 * y stays 0 below
+        if (j >= valid) z[j] = kNoLogit;
     }
     float cm = fmaxf(z[0], z[1]);
 #pragma unroll
@@ -200,6 +197,56 @@ struct RowFold {
     float ls0, ls1, lt0, lt1;
     unpack2(ls2, ls0, ls1);
     unpack2(lt2, lt0, lt1);
+    {
+      const float a = (ls0 + ls1) - cS;
+      const float b = S + a;
+      cS = (b - S) - a;
+      S = b;
+    }
+    {
+      const float a = (lt0 + lt1) - cT;
+      const float b = Tq + a;
+      cT = (b - Tq) - a;
+      Tq = b;
+    }
+  }
+  // The same for 16 logits of one row held by a thread of the fragment layout (tmem_ld16x64): z[2b + j] is column
+  // col0 + 8b + j.  Written for latency -- no branch but the index search, short dependent chains -- because the
+  // last tile's fold is exposed at the end of every step.
+  __device__ __forceinline__ void fragment(const float (&z)[16], int col0) {
+    const float m0 = max3(max3(z[0], z[1], z[2]), z[3], max3(z[4], z[5], z[6]));
+    const float m1 = max3(max3(z[7], z[8], z[9]), z[10], max3(z[11], z[12], z[13]));
+    const float cm = max3(fmaxf(m0, m1), z[14], z[15]);
+    if (cm > m) {
+      uint32_t hit = 0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) hit |= (z[k] == cm) ? 1u << k : 0u;
+      const int k = __ffs(hit) - 1;
+      idx = col0 + 8 * (k >> 1) + (k & 1);
+    }
+    const float m_old = fmaxf(m, kNoLogit);         // (finite before the first group)
+    m = fmaxf(m_old, cm);
+    const float dl = (m - m_old) * kLog2e;          // >= 0
+    const float sc = ex2_approx(-dl);
+    const float neg_ml = -m * kLog2e;
+    const uint64_t log2e2 = pack2(kLog2e, kLog2e), neg_ml2 = pack2(neg_ml, neg_ml);
+    uint64_t ls2[2] = {0ull, 0ull}, lt2[2] = {0ull, 0ull};
+#pragma unroll
+    for (int j = 0; j < 16; j += 2) {
+      const uint64_t y2 = fma2(pack2(z[j], z[j + 1]), log2e2, neg_ml2);
+      float y0, y1;
+      unpack2(y2, y0, y1);
+      const uint64_t e2 = pack2(ex2_approx(y0), ex2_approx(y1));
+      ls2[(j >> 1) & 1] = add2(ls2[(j >> 1) & 1], e2);
+      lt2[(j >> 1) & 1] = fma2(e2, y2, lt2[(j >> 1) & 1]);
+    }
+    float ls0, ls1, lt0, lt1;
+    unpack2(add2(ls2[0], ls2[1]), ls0, ls1);
+    unpack2(add2(lt2[0], lt2[1]), lt0, lt1);
+    Tq = sc * (Tq - dl * S);
+    cT *= sc;
+    S *= sc;
+    cS *= sc;
     {
       const float a = (ls0 + ls1) - cS;
       const float b = S + a;
@@ -256,12 +303,8 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
   // xch_empty[q]: the first group has read it.
   auto xch_full = [&](int q) { return bar_base + 8u * (kFixed + 4 + q); };
   auto xch_empty = [&](int q) { return bar_base + 8u * (kFixed + 8 + q); };
-  // 8-bit head: hx_full[c] / hx_empty[c]: hand-over buffer c holds / has given up 32 columns of second-part sums;
-  // h_ready: h has been split in place (inline mode)
-  auto hx_full = [&](int c) { return bar_base + 8u * (kFixed + 12 + c); };
-  auto hx_empty = [&](int c) { return bar_base + 8u * (kFixed + 16 + c); };
-  const uint32_t h_ready = bar_base + 8u * (kFixed + 20);
-  constexpr int kNumBarriers = kFixed + 21;
+  const uint32_t h_ready = bar_base + 8u * (kFixed + 12);   // 8-bit head: h has been split in place (inline mode)
+  constexpr int kNumBarriers = kFixed + 13;
   static_assert(kNumBarriers * 8 + 16 <= kBarrierBytes, "barrier block too small");
   unsigned char* gen_base = smem_raw + (base - smem_u32(smem_raw));
   unsigned char* tail = gen_base + (bar_base - base);
@@ -270,7 +313,6 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
   Partial* scratch = reinterpret_cast<Partial*>(tail + kBarrierBytes);
   float* scale_area = reinterpret_cast<float*>(tail + kBarrierBytes + kScratchBytes);   // 8-bit head only
   float* hs_s = scale_area + kScaleBytes / 4;
-  float* hx_area = hs_s + kRowScaleBytes / 4;
   const bool inl = kFp8 && p.inline_split != 0;
 
   const int warp = threadIdx.x >> 5;
@@ -291,10 +333,6 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
     for (int q = 0; q < 4; ++q) {
       mbar_init(xch_full(q), 1);
       mbar_init(xch_empty(q), 1);
-      if (kFp8) {
-        mbar_init(hx_full(q), 1);
-        mbar_init(hx_empty(q), 1);
-      }
     }
     if (kFp8) mbar_init(h_ready, 9);
     *abort_flag = 0;
@@ -485,44 +523,41 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
     // ------------------------------------------------------------------ epilogue (warps 2-5, 7-10)
     const int grp = warp >= 7 ? 1 : 0;       // 0: lower half of a tile's columns, 1: upper half
     const int quad = warp & 3;               // TMEM lane quadrant this warp may read
-    // 8-bit head: a token's first part is accumulator row r and its second part row r + part_rows, which lie in
-    // different lane quadrants (quadrant q and q + shift), so different warps read them: the warp of the second
-    // part (the donor) passes its 32 columns through shared memory to the warp of the first part, which adds
-    // them, applies the scales and folds.
-    const int shift = (kFp8 && !wide) ? (p.part_rows == 16 ? 1 : 2) : 4;
-    const bool donor = kFp8 && !wide && quad >= shift && quad < 2 * shift;
-    const bool idle = kFp8 && !wide && quad >= 2 * shift;              // quadrants that hold no operand rows
-    const int cquad = donor ? quad - shift : quad;                     // quadrant of the rows this warp works for
-    const int row_in_cta = m64 ? cquad * 16 + (lane & 15) : cquad * 32 + lane;
-    const bool lane_has_row = !m64 || lane < 16;   // with M = 64 the upper half of a quadrant holds nothing
-    const int hx = grp * 2 + cquad;                // hand-over buffer / scale area of this warp pair
-    const int hx_lanes = m64 ? 16 : 32;
-    float* hx_buf = hx_area + hx * 32 * hx_lanes;
-    // (more than 64 rows: all eight warps fold and each stages the tile's scales for itself, in the area the
-    // hand-over buffers do not need then)
-    float* ws = wide ? hx_area + (grp * 4 + quad) * kBlockN : scale_area + hx * kBlockN;
-    uint32_t hx_n = 0;                       // hand-overs done so far by this warp
+    // 8-bit head up to 64 token rows: the accumulator is read in the fragment layout (tmem_ld16x64), 16 lanes at a
+    // time.  Of those, lanes 0..7 are the first parts of eight tokens and lanes 8..15 their second parts
+    // (tc8_part_row), so the thread that holds a token's first part holds its second part too and adds them; four
+    // threads share a token's columns, and all 32 work.  With M = 64 a quadrant has one such group of 16 lanes, with
+    // M = 128 two, and a thread then keeps two tokens, eight apart.
+    const bool frag = kFp8 && !wide;
+    constexpr int kFolds = kFp8 ? 2 : 1;           // tokens a thread may keep
+    const int quad_rows = frag ? (m64 ? 8 : 16) : (m64 ? 16 : 32);     // token rows per quadrant
+    const int quad_row0 = quad * quad_rows;
+    const int my_row = quad_row0 + (frag ? lane >> 2 : (m64 ? lane & 15 : lane));   // this thread's (first) token row
+    const bool writer = frag ? (lane & 3) == 0 : (!m64 || lane < 16);  // one thread per token row
+    float* ws = scale_area + (grp * 4 + quad) * (kBlockN / 2);         // weight scales of this warp's half of a tile
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
     uint32_t ord = 0;                        // ordinal of the unit among this worker's units
-    float hs = 1.0f;
-    if (kFp8 && !donor && !idle && lane_has_row && row_in_cta < p.n) {
-      if (inl) {
-        // the scales are written by the splitting warps before they arrive on h_ready
-        ok = mbar_wait(h_ready, 0, abort_flag, p.status, wait_ns);
-        hs = hs_s[row_in_cta];
-      } else {
-        hs = p.hscale[row_in_cta];
+    float hs[kFolds] = {};
+    if (kFp8) {
+      // (inline mode: the scales are written by the splitting warps before they arrive on h_ready)
+      if (inl) ok = mbar_wait(h_ready, 0, abort_flag, p.status, wait_ns);
+#pragma unroll
+      for (int i = 0; i < kFolds; ++i) {
+        const int r = my_row + 8 * i;
+        if (r < p.n && (i == 0 || (frag && !m64))) hs[i] = inl ? hs_s[r] : p.hscale[r];
       }
+      ok = __all_sync(0xffffffffu, ok);
     }
-    if (kFp8) ok = __all_sync(0xffffffffu, ok);
     for (int unit = worker; unit < units && ok; unit += workers, ++ord) {
       const Unit first = unit_of<kCta>(p, unit, cta_rank);
-      const bool warp_has_rows = !idle && (first.row0 + (m64 ? cquad * 16 : cquad * 32)) < p.n;   // warp-uniform
+      const bool warp_has_rows = first.row0 + quad_row0 < p.n;            // warp-uniform
+      const bool two_tokens = kFp8 && frag && !m64 && quad_row0 + 8 < p.n;   // warp-uniform
       const bool mlp_unit = !kFp8 && first.chunk < 0;
-      RowFold f;
-      f.reset();
+      RowFold f[kFolds];
+#pragma unroll
+      for (int i = 0; i < kFolds; ++i) f[i].reset();
       float mlp_sum = 0.f;
       // The walk over the unit's tiles, compiled twice: once for vocabulary units (the hot loop, free of any
       // learned-router code) and once for learned-router units.
@@ -533,16 +568,17 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
         if (tl.rows == 0) continue;
         const int v0 = tl.v0;
         const int cols = min(tl.rows, (kRouter ? p.mlp_hidden : p.V) - v0);   // valid columns of this tile
-        // this group's share of them: [0, half) or [half, cols), half a multiple of 32
-        const int half = min(cols, ((tl.rows / 2 + 31) / 32) * 32);
+        // this group's share of them: [0, half) or [half, cols), half a multiple of the columns of a load
+        const int step = frag ? 64 : 32;
+        const int half = min(cols, (tl.rows / 2 + step - 1) & ~(step - 1));
         const int c_begin = grp ? half : 0, c_end = grp ? cols : half;
-        if (kFp8 && !donor && !idle) {
-          // this tile's weight scales into the warp pair's area, before the accumulator is waited for
+        if (kFp8 && warp_has_rows) {
+          // the share's weight scales, before the accumulator is waited for
           __syncwarp();
 #pragma unroll
-          for (int j = 0; j < kBlockN / 32; ++j) {
-            const int c = lane + 32 * j;
-            ws[c] = (c < cols) ? __ldg(p.wscale + v0 + c) : 0.f;
+          for (int j = 0; j < kBlockN / 64; ++j) {
+            const int c = c_begin + lane + 32 * j;
+            ws[lane + 32 * j] = (c < c_end) ? __ldg(p.wscale + v0 + c) : 0.f;
           }
           __syncwarp();
         }
@@ -550,65 +586,65 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
         tc_fence_after();
         if (warp_has_rows) {
           const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + acc * kBlockN;
-          for (int c0 = c_begin; c0 < c_end; c0 += 32) {
-            float z[32];
-            __syncwarp();                           // the load below is warp-collective
-            tmem_ld32(taddr + c0, z);
-            tmem_ld_wait();
-            if (kFp8 && wide) {
+          if (frag) {
+            for (int c0 = c_begin; c0 < c_end; c0 += 64) {
+              float x[kFolds][32];
+              __syncwarp();                           // the loads below are warp-collective
+              tmem_ld16x64(taddr + c0, x[0]);
+              if (two_tokens) tmem_ld16x64(taddr + (16u << 16) + c0, x[kFolds - 1]);
+              tmem_ld_wait();
+              const int c_mine = c0 + 2 * (lane & 3);         // this thread's columns: c_mine + 0, 1, 8, 9, 16 ..
+              const int valid = c_end - c_mine;
+              if (valid <= 0) continue;
 #pragma unroll
-              for (int j = 0; j < 32; j += 4) {
-                const float4 w4 = *reinterpret_cast<const float4*>(ws + c0 + j);
-                z[j] = z[j] * hs * w4.x;
-                z[j + 1] = z[j + 1] * hs * w4.y;
-                z[j + 2] = z[j + 2] * hs * w4.z;
-                z[j + 3] = z[j + 3] * hs * w4.w;
-              }
-            } else if (kFp8) {
-              if (donor) {
-                // second parts: wait until the partner has taken the previous 32 columns, then hand these over
-                if (hx_n > 0 && !mbar_wait(hx_empty(hx), (hx_n - 1) & 1u, abort_flag, p.status, wait_ns)) { ok = false; break; }
-                if (lane_has_row) {
+              for (int i = 0; i < kFolds; ++i) {
+                if (i == 1 && !two_tokens) continue;
+                float z[16];
 #pragma unroll
-                  for (int j = 0; j < 32; ++j) hx_buf[j * hx_lanes + (lane & (hx_lanes - 1))] = z[j];
+                for (int b = 0; b < 8; ++b) {
+                  const float2 w2 = *reinterpret_cast<const float2*>(ws + (c_mine - c_begin) + 8 * b);
+                  z[2 * b] = (x[i][4 * b] + x[i][4 * b + 2]) * hs[i] * w2.x;
+                  z[2 * b + 1] = (x[i][4 * b + 1] + x[i][4 * b + 3]) * hs[i] * w2.y;
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(hx_full(hx));
-                ++hx_n;
-                continue;
-              }
-              if (!mbar_wait(hx_full(hx), hx_n & 1u, abort_flag, p.status, wait_ns)) { ok = false; break; }
+                if (valid < 58) {                     // (the last of the columns is c_mine + 57)
 #pragma unroll
-              for (int j = 0; j < 32; j += 4) {
-                const float4 w4 = *reinterpret_cast<const float4*>(ws + c0 + j);
-                const int l = lane & (hx_lanes - 1);
-                z[j] = (z[j] + hx_buf[j * hx_lanes + l]) * hs * w4.x;
-                z[j + 1] = (z[j + 1] + hx_buf[(j + 1) * hx_lanes + l]) * hs * w4.y;
-                z[j + 2] = (z[j + 2] + hx_buf[(j + 2) * hx_lanes + l]) * hs * w4.z;
-                z[j + 3] = (z[j + 3] + hx_buf[(j + 3) * hx_lanes + l]) * hs * w4.w;
+                  for (int k = 0; k < 16; ++k)
+                    if (8 * (k >> 1) + (k & 1) >= valid) z[k] = kNoLogit;
+                }
+                f[i].fragment(z, v0 + c_mine);
               }
-              __syncwarp();
-              if (lane == 0) mbar_arrive(hx_empty(hx));
-              ++hx_n;
             }
-            if constexpr (kRouter) {
-              // hidden units v0 + c0 .. of the learned router: bias, ReLU, output-layer weight, sum
+          } else {
+            for (int c0 = c_begin; c0 < c_end; c0 += 32) {
+              float z[32];
+              __syncwarp();                           // the load below is warp-collective
+              tmem_ld32(taddr + c0, z);
+              tmem_ld_wait();
+              if (kFp8) {
 #pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                const int u = v0 + c0 + j;
-                if (u < p.mlp_hidden) mlp_sum += __ldg(p.mlp_w2 + u) * fmaxf(z[j] + __ldg(p.mlp_b1 + u), 0.f);
+                for (int j = 0; j < 32; j += 4) {
+                  const float4 w4 = *reinterpret_cast<const float4*>(ws + (c0 - c_begin) + j);
+                  z[j] = z[j] * hs[0] * w4.x;
+                  z[j + 1] = z[j + 1] * hs[0] * w4.y;
+                  z[j + 2] = z[j + 2] * hs[0] * w4.z;
+                  z[j + 3] = z[j + 3] * hs[0] * w4.w;
+                }
               }
-            } else {
-              f.group(z, cols - c0, v0 + c0);
+              if constexpr (kRouter) {
+                // hidden units v0 + c0 .. of the learned router: bias, ReLU, output-layer weight, sum
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                  const int u = v0 + c0 + j;
+                  if (u < p.mlp_hidden) mlp_sum += __ldg(p.mlp_w2 + u) * fmaxf(z[j] + __ldg(p.mlp_b1 + u), 0.f);
+                }
+              } else {
+                f[0].group(z, cols - c0, v0 + c0);
+              }
             }
           }
         }
         tc_fence_before();
         __syncwarp();
-        if (kFp8) {                                 // a hand-over wait may have run out in some lanes
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-        }
         if (lane == 0) {
           if (kCta == 1) mbar_arrive(acc_empty(acc));
           else mbar_arrive_cluster(map_to_cta(acc_empty(acc), 0));   // the leader's barrier
@@ -618,30 +654,44 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
       };
       if (mlp_unit) walk_tiles(std::true_type{});
       else walk_tiles(std::false_type{});
-      if (donor || idle) continue;
-      Partial out = f.result();
-      if (mlp_unit) out.s = mlp_sum;
+      Partial out[kFolds];
+#pragma unroll
+      for (int i = 0; i < kFolds; ++i) out[i] = f[i].result();
+      if (frag) {                              // the four threads of a token merge their summaries
+#pragma unroll
+        for (int i = 0; i < kFolds; ++i) {
+          if (i == 1 && !two_tokens) continue;
+          out[i] = merge(out[i], shfl_xor(out[i], 1));
+          out[i] = merge(out[i], shfl_xor(out[i], 2));
+        }
+      }
+      if (mlp_unit) out[0].s = mlp_sum;
       // The second group hands its summary to the first through the scratch block (bounded
       // waits on both sides: a warp that gave up never leaves its partner waiting forever).
       if (grp == 1) {
         if (ok && ord > 0) ok = mbar_wait(xch_empty(quad), (ord - 1) & 1u, abort_flag, p.status, wait_ns);
         if (ok) {
-          if (lane_has_row) scratch[row_in_cta] = out;
+          if (writer) {
+            scratch[my_row] = out[0];
+            if (two_tokens) scratch[my_row + 8] = out[kFolds - 1];
+          }
           __syncwarp();
           if (lane == 0) mbar_arrive(xch_full(quad));
         }
       } else {
         if (ok) ok = mbar_wait(xch_full(quad), ord & 1u, abort_flag, p.status, wait_ns);
         if (ok) {
-          const Partial other = scratch[row_in_cta];
+          Partial other[kFolds];
+          other[0] = scratch[my_row];
+          if (two_tokens) other[kFolds - 1] = scratch[my_row + 8];
           __syncwarp();
           if (lane == 0) mbar_arrive(xch_empty(quad));
-          const bool mine = lane_has_row && first.row0 + row_in_cta < p.n;
-          if (mlp_unit) {
-            if (mine) p.mlp_out[first.row0 + row_in_cta] = out.s + other.s;   // lower columns first: a fixed order
-          } else {
-            out = merge(out, other);
-            if (mine) p.partials[static_cast<size_t>(first.row0 + row_in_cta) * p.chunks + first.chunk] = out;
+#pragma unroll
+          for (int i = 0; i < kFolds; ++i) {
+            const int row = first.row0 + my_row + 8 * i;
+            if (!writer || row >= p.n || (i == 1 && !two_tokens)) continue;
+            if (mlp_unit) p.mlp_out[row] = out[i].s + other[i].s;   // lower columns first: a fixed order
+            else p.partials[static_cast<size_t>(row) * p.chunks + first.chunk] = merge(out[i], other[i]);
           }
         }
       }

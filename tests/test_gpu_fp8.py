@@ -173,3 +173,19 @@ def test_fp8_argument_errors(pkg):
     with pytest.raises(pkg.TlrError):
         pkg.tlr_set_path(r.ctx, pkg.TLR_PATH_SIMT)
     r.close()
+
+
+# The epilogue's fragment layout: token rows at the edges of the groups of 8 and of 16 lanes and of the quadrants
+# (both operand heights: 32 and 64 rows of M = 64, 128 rows), vocabularies that end inside a thread's columns.
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 15, 16, 17, 24, 25, 31, 32, 33, 40, 41, 56, 57, 63, 64])
+@pytest.mark.parametrize("V", [1, 2, 15, 57, 58, 130, 2500])
+def test_fp8_fragment_edges(pkg, n, V):
+    d = 48
+    codes, scale = S.make_W8(d, V, seed=n + V, std=0.1)
+    W64 = O.dequantize_e4m3(codes.numpy(), scale.numpy())
+    h = planted_h(n, d, W64, seed=n + V)
+    ref = O.route_oracle(S.bf16_bits(h), None, 0.5, W64=W64)
+    gpu = run_fp8(pkg, codes, scale, h, 0.5)
+    assert gpu["status"] == 0
+    check_self_consistency(gpu, 0.5, V)
+    check_against_oracle(ref, gpu, O.bf16_bits_to_f64(S.bf16_bits(h)), W64)
