@@ -54,8 +54,8 @@ typedef enum {
 /* Which projection kernel a call of n rows uses. */
 typedef enum {
   TLR_PATH_AUTO = 0,   /* choose by shape (default) */
-  TLR_PATH_SIMT = 1,   /* CUDA-core kernel: any d, any V; the only path when d % 8 != 0 */
-  TLR_PATH_TC = 2      /* tcgen05 tensor-core kernel fed by TMA; needs d % 8 == 0 */
+  TLR_PATH_SIMT = 1,   /* CUDA-core kernel: any d, any V (diagnostics) */
+  TLR_PATH_TC = 2      /* tcgen05 tensor-core kernel fed by TMA; when d % 8 != 0 W is read by residue classes of its rows */
 } tlr_path;
 
 /* Launch plan of the projection kernel for a given n (for reports and tests). */

@@ -16,6 +16,8 @@ namespace tlr {
 
 constexpr int kMaxChunks = 192;       // upper bound on partials per row (sizes the workspace)
 constexpr int kMaxTimedLaunches = 4096;
+constexpr int kOddRows = 2048;        // d no multiple of 8: rows of h whose shifted copies exist at a time (at most 8
+                                      // copies); from 2048 rows on W streams far below the tensor pipe's time
 
 const Tuning& tuning() {
   static const Tuning t = [] {
@@ -43,25 +45,26 @@ const Tuning& tuning() {
 // largest chunk + a fixed cost per tile) -- so that workers finish together.  With a learned
 // router in the launch (mlp_hidden > 0) one more unit per row unit, over the rows of its first
 // layer, follows the vocabulary units in the same round-robin order and is counted in the loads.
-void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden, TcPlan* plan) {
-  int g = 16 * cta;
+// With residue classes (d no multiple of 8) every class gets the same number of chunks.
+void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan) {
+  int g = (classes > 1 ? kOddBoxRows : 16) * cta;
   {
     const int e = tuning().granule;   // tuning switch
     if (e >= g && e <= 256 && e % g == 0 && 256 % e == 0) g = e;
   }
   const int row_units = (n + 128 * cta - 1) / (128 * cta);
-  const int granules = (V + g - 1) / g;
+  const int granules = ((V + classes - 1) / classes + g - 1) / g;      // of the longest class
   const int mlp_rows = mlp_hidden > 0 ? ((mlp_hidden + 16 * cta - 1) / (16 * cta)) * (16 * cta) : 0;
   const long long mlp_tiles = (mlp_rows + 255) / 256;
   const long long mlp_cost = mlp_rows + 24 * mlp_tiles;
-  int hi = granules < max_chunks ? granules : max_chunks;
+  int hi = granules < max_chunks / classes ? granules : max_chunks / classes;     // chunks per class
   if (hi < 1) hi = 1;
   long long best_cost = -1, best_passes = 0;
   int best = 1, best_tiles = 1;
   for (int c = 1; c <= hi; ++c) {
     const long long gmax = (granules + c - 1) / c;
     const long long tiles = (gmax * g + 255) / 256;
-    const long long units = 1ll * row_units * c;
+    const long long units = 1ll * row_units * c * classes;
     const long long unit_cost = gmax * g + 24 * tiles;
     // Pair mode: a tile costs a pass over all of h whatever its width (the pair MMA takes as long with 32
     // columns as with 256), so the busiest worker's TILE count is compared first and the row-based cost only
@@ -94,7 +97,8 @@ void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden,
     }
   }
   plan->row_units = row_units;
-  plan->chunks = best;
+  plan->classes = classes;
+  plan->chunks = best * classes;
   plan->granule_rows = g;
   plan->granules = granules;
   plan->tiles_per_unit = best_tiles;
@@ -130,6 +134,11 @@ struct tlr_ctx {
   bool tc_ok = false;
   EncodeTiledFn encode = nullptr;
   CUtensorMap map_w128, map_w64, map_w16;
+  // d no multiple of 8 (OddMaps): the maps of the residue classes, and the shifted copies of up to odd_rows rows of h
+  int classes = 1;
+  CUtensorMap map_cls[tlr::kMaxClasses];
+  void* h_shift = nullptr;
+  int odd_rows = 0, odd_pitch = 0;
 
   Partial* partials = nullptr;
   unsigned int* ticket = nullptr;
@@ -184,6 +193,8 @@ struct tlr_ctx {
     tlr::TcConfig cfg;
     tlr::TcParams params;     // all but the per-call fields
     tlr::TcMaps maps;
+    tlr::OddMaps odd;         // d no multiple of 8: these instead
+    int odd_block = 0;        // rows of h per projection launch then
     const void* h_mapped = nullptr;   // the address maps.h was encoded for
     const void* h_other = nullptr;    // ... and the address before that, with its map (two staging buffers alternate)
     CUtensorMap h_other_map;
@@ -218,9 +229,10 @@ bool make_map8(tlr_ctx* c, CUtensorMap* map, const void* base, int rows, int col
   return r == CUDA_SUCCESS;
 }
 
-bool make_map(tlr_ctx* c, CUtensorMap* map, const void* base, int rows, int cols, int box_rows) {
+bool make_map(const tlr_ctx* c, CUtensorMap* map, const void* base, int rows, int cols, int box_rows,
+              long long pitch = 0) {     // elements from row to row, 0 = cols
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch != 0 ? pitch : cols) * 2};
   const cuuint32_t box[2] = {64u, static_cast<cuuint32_t>(box_rows)};
   const cuuint32_t elem[2] = {1u, 1u};
   const CUresult r = c->encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
@@ -229,9 +241,14 @@ bool make_map(tlr_ctx* c, CUtensorMap* map, const void* base, int rows, int cols
   return r == CUDA_SUCCESS;
 }
 
-tlr_path pick_path(const tlr_ctx* c) {
-  if (c->forced == TLR_PATH_SIMT) return TLR_PATH_SIMT;
-  return c->tc_ok ? TLR_PATH_TC : TLR_PATH_SIMT;
+// Tensor cores wherever their set-up succeeded.  The one exception: a small batch on a head of at most 128 KB whose d is
+// no multiple of 8.  The tensor-core path needs a third launch there, for the shifted copies of h, which costs the
+// host 2 us and buys next to nothing on the device: n = 20, d = 36, V = 1500 13.1 us on CUDA cores and 9.1 on tensor
+// cores, n = 1, d = 9, V = 700 10.4 and 7.9; on larger heads it buys everything (n = 64, d = 300, V = 33000 194 and 17).
+tlr_path pick_path(const tlr_ctx* c, int n) {
+  if (c->forced != TLR_PATH_AUTO) return c->forced;
+  const bool tiny = c->classes > 1 && n <= 32 && static_cast<long long>(c->V) * c->d <= 65536;
+  return c->tc_ok && !tiny ? TLR_PATH_TC : TLR_PATH_SIMT;
 }
 
 void forget_steps(tlr_ctx* c) {
@@ -240,7 +257,7 @@ void forget_steps(tlr_ctx* c) {
 
 // Plans a call of n rows (with or without the learned router inside the projection launch).
 void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
-  const tlr_path path = pick_path(c);
+  const tlr_path path = pick_path(c, n);
   tlr_plan* out = &st->plan;
   st->n = n;
   st->mlp = mlp;
@@ -259,12 +276,20 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     if (c->fp8) {
       tlr::tc8_configure(n <= tlr::tc8_max_rows() ? n : tlr::tc8_max_rows(), c->d, &cfg);
       workers_max = c->sm_count;
-      tlr::tc_plan(n <= 128 ? n : 128, c->V, 1, workers_max, tlr::kMaxChunks, 0, &tp);
+      tlr::tc_plan(n <= 128 ? n : 128, c->V, 1, workers_max, tlr::kMaxChunks, 0, 1, &tp);
       out->launches = n > 0 ? (cfg.inline_split ? 2 : 3) : 1;
     } else {
-      tlr::tc_configure(n, &cfg);
+      int rows = n;
+      if (c->classes > 1 && n > 0) {     // equal blocks of whole row units, each with its own copies of h
+        const int blocks = (n + c->odd_rows - 1) / c->odd_rows;
+        rows = (n + blocks - 1) / blocks;
+        if (blocks > 1) rows = (rows + 255) / 256 * 256;
+        st->odd_block = rows;
+        out->launches = 2 * ((n + rows - 1) / rows) + 1;
+      }
+      tlr::tc_configure(rows, &cfg);
       workers_max = c->sm_count / cfg.cta;
-      tlr::tc_plan(n, c->V, cfg.cta, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, &tp);
+      tlr::tc_plan(rows, c->V, cfg.cta, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, c->classes, &tp);
     }
     const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;
     st->workers = units < workers_max ? units : workers_max;
@@ -299,6 +324,15 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     p.wscale = c->wscale;
     p.partials = c->partials;
     p.status = c->status;
+    if (c->classes > 1) {
+      p.d = c->d + tlr::odd_max_shift(c->d);
+      p.classes = c->classes;
+      p.class_chunks = tp.chunks / c->classes;
+      p.h_class_rows = c->odd_rows;
+      for (int r = 0; r < c->classes; ++r) st->odd.w[r] = c->map_cls[r];
+      if (n > 0) make_map(c, &st->odd.h, c->h_shift, c->classes * c->odd_rows, c->odd_pitch, cfg.a_rows);
+      return;
+    }
     st->maps.w128 = c->map_w128;
     st->maps.w64 = c->map_w64;
     st->maps.w16 = c->map_w16;
@@ -339,6 +373,7 @@ void free_all(tlr_ctx* c) {
   }
   if (c->copy_stream != nullptr) cudaStreamDestroy(c->copy_stream);
   cudaFree(c->mlp_scores);
+  cudaFree(c->h_shift);
   cudaFree(c->h_parts);
   cudaFree(c->hscale);
   for (int q = 0; q < 2; ++q) {
@@ -431,6 +466,21 @@ tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ct
     }
     st->params.h = h_bf16_dev;
     e = tlr::launch_tc8_projection(st->maps, st->params, cfg, st->workers, stream);
+  } else if (st->plan.path == TLR_PATH_TC && ctx->classes > 1) {
+    const int units_max = ctx->sm_count / st->cfg.cta;
+    e = cudaSuccess;
+    for (int row0 = 0; row0 < n && e == cudaSuccess; row0 += st->odd_block) {
+      const int rows = n - row0 < st->odd_block ? n - row0 : st->odd_block;
+      e = tlr::launch_odd_shift(static_cast<const unsigned short*>(h_bf16_dev) + static_cast<size_t>(row0) * ctx->d, rows,
+                                ctx->d, ctx->odd_rows, ctx->odd_pitch, ctx->h_shift, stream);
+      if (e != cudaSuccess) break;
+      tlr::TcParams p = st->params;
+      p.n = rows;
+      p.row_units = (rows + 128 * st->cfg.cta - 1) / (128 * st->cfg.cta);
+      p.partials = ctx->partials + static_cast<size_t>(row0) * p.chunks;
+      const int units = p.chunks * p.row_units;
+      e = tlr::launch_odd_projection(st->odd, p, st->cfg, units < units_max ? units : units_max, stream);
+    }
   } else if (st->plan.path == TLR_PATH_TC) {
     if (st->h_mapped != h_bf16_dev) {
       // the map in use moves to the second place; if that one was made for this address, it comes back
@@ -505,10 +555,34 @@ tlr_status tlr_create(int32_t d, int32_t V, const void* W_bf16_dev, int32_t max_
         tlr::tc_prepare() == cudaSuccess)
       c->tc_ok = true;
     cudaGetLastError();
-    if (!c->tc_ok) {   // on an sm_100 device with d % 8 == 0 this must work; do not fall back silently
+  } else {
+    // rows of W are no multiples of 16 bytes: one map per residue class of rows, and room for the shifted copies of h
+    c->classes = tlr::odd_classes(d);
+    c->odd_rows = max_n < tlr::kOddRows ? max_n : tlr::kOddRows;
+    c->odd_pitch = (d + tlr::odd_max_shift(d) + 7) / 8 * 8;
+    if (cudaMalloc(&c->h_shift, static_cast<size_t>(c->classes) * c->odd_rows * c->odd_pitch * 2) != cudaSuccess) {
+      cudaGetLastError();
       free_all(c);
-      return TLR_ERR_CUDA;
+      return TLR_ERR_NOMEM;
     }
+    bool ok = c->encode != nullptr && tlr::odd_prepare() == cudaSuccess;
+    for (int r = 0; r < c->classes && ok; ++r) {
+      const int shift = tlr::odd_shift(d, r);
+      const int rows = (V - r + c->classes - 1) / c->classes;
+      if (rows <= 0) {       // a vocabulary of fewer rows than classes: no unit ever loads this class
+        c->map_cls[r] = c->map_cls[0];
+        continue;
+      }
+      ok = make_map(c, &c->map_cls[r],
+                    static_cast<const unsigned short*>(W_bf16_dev) + (static_cast<size_t>(r) * d - shift), rows, d + shift,
+                    tlr::kOddBoxRows, static_cast<long long>(c->classes) * d);
+    }
+    c->tc_ok = ok;
+    cudaGetLastError();
+  }
+  if (!c->tc_ok) {   // on an sm_100 device this must work; do not fall back silently
+    free_all(c);
+    return TLR_ERR_CUDA;
   }
   *out = c;
   return TLR_OK;
@@ -595,7 +669,7 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
   tlr::TcPlan tp;
   tlr::tc_configure(n, &cfg);
   const int workers_max = sm_count / cfg.cta;
-  tlr::tc_plan(n, V, cfg.cta, workers_max, tlr::kMaxChunks, mlp_hidden, &tp);
+  tlr::tc_plan(n, V, cfg.cta, workers_max, tlr::kMaxChunks, mlp_hidden, 1, &tp);
   const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;
   const int workers = units < workers_max ? units : workers_max;
   tlr::TcParams p = {};
@@ -687,7 +761,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
   // the learned router runs inside the projection launch wherever the tensor-core kernel of the bf16 head runs
-  const bool mlp_inside = want_mlp && ctx->mlp_fused && !ctx->fp8 && pick_path(ctx) == TLR_PATH_TC;
+  const bool mlp_inside = want_mlp && ctx->mlp_fused && !ctx->fp8 && pick_path(ctx, n) == TLR_PATH_TC;
   tlr_ctx::Step* st = step_for(ctx, n, mlp_inside);
   const tlr_plan& plan = st->plan;
 
@@ -734,6 +808,11 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   f.routed_count = routed_count_dev;
   f.ticket = ctx->ticket;
   f.status = ctx->status;
+  if (ctx->classes > 1 && plan.path == TLR_PATH_TC) {
+    f.tie_W = static_cast<const unsigned short*>(ctx->W);
+    f.tie_h = static_cast<const unsigned short*>(h_bf16_dev);
+    f.tie_d = ctx->d;
+  }
   f.status_copy = status_copy;
   if (tlr::launch_finish(f, stream) != cudaSuccess) return TLR_ERR_CUDA;
   return TLR_OK;

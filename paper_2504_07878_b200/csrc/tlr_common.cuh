@@ -117,6 +117,11 @@ struct FinishLaunch {
   int32_t* routed_count;
   unsigned int* ticket;     // zero before the launch; the kernel leaves it zero again
   uint32_t* status;
+  // d no multiple of 8 on the tensor cores: equal rows of W in different residue classes get logits that agree to
+  // rounding only, so near-ties between partials are settled by dot products of their own (null = not needed)
+  const unsigned short* tie_W;   // bf16 [V][tie_d]
+  const unsigned short* tie_h;   // bf16 [n][tie_d]
+  int tie_d;
   uint32_t* status_copy;    // optional: receives the status word once every row is scored (host-mapped memory)
 };
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream);

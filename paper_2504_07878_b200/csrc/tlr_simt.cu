@@ -1,6 +1,6 @@
 // CUDA-core projection kernel: logits + online-softmax partials with plain FMAs.
-// Serves the shapes the TMA-fed tensor-core kernel cannot address (hidden size not a
-// multiple of 8, so rows of W are not 16-byte multiples) and is selectable for
+// Serves tiny heads whose hidden size is not a multiple of 8 (pick_path), every such head of the entry point without
+// a context (tlr_static.cu, which has no room for the shifted copies of h the tensor-core path needs), and is selectable for
 // diagnostics.  One thread owns one vocabulary row of a 128-row tile and kRows token
 // rows at a time; the block walks its vocabulary chunk tile by tile, each thread
 // keeping the running (m, idx, s, t) of its own rows, and the block folds its 128
@@ -52,6 +52,11 @@ simt_projection_kernel(const SimtLaunch a) {
   const unsigned short* W = reinterpret_cast<const unsigned short*>(a.W);
   const unsigned short* h = reinterpret_cast<const unsigned short*>(a.h);
 
+  // Programmatic dependent launch on both sides: the merge kernel is scheduled early, and this kernel's launch
+  // overlaps the kernel before it, which may have written h or W.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
   // stage the kRows hidden-state rows (zeros past n)
   for (int i = threadIdx.x; i < kRows * d; i += kSimtThreads) {
     const int r = i / d, k = i - r * d;
@@ -92,6 +97,7 @@ simt_projection_kernel(const SimtLaunch a) {
         }
       }
     } else {
+#pragma unroll 4
       for (int k = 0; k < d; ++k) {
         const float w = bf16_bits_to_float(wrow[k]);
 #pragma unroll
@@ -136,21 +142,22 @@ cudaError_t launch_simt_projection(const SimtLaunch& a, cudaStream_t stream) {
   const int smem = kRows * a.d * 2;
   const dim3 grid(a.chunks, (a.n + kRows - 1) / kRows);
   const bool vec = (a.d % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.W) & 15) == 0);
-  cudaError_t e;
-  if (vec) {
-    if (smem > 48 * 1024) {
-      e = cudaFuncSetAttribute(simt_projection_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-    }
-    simt_projection_kernel<true><<<grid, kSimtThreads, smem, stream>>>(a);
-  } else {
-    if (smem > 48 * 1024) {
-      e = cudaFuncSetAttribute(simt_projection_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-    }
-    simt_projection_kernel<false><<<grid, kSimtThreads, smem, stream>>>(a);
+  const auto kernel = vec ? simt_projection_kernel<true> : simt_projection_kernel<false>;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kSimtThreads, 1, 1);
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 }  // namespace tlr

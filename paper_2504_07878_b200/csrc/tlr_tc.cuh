@@ -22,9 +22,10 @@ struct TcConfig {
 // Work decomposition for a given (n, V) on `workers` workers (see tc_plan).
 struct TcPlan {
   int row_units;       // ceil(n / (128 * cta))
-  int chunks;          // vocabulary chunks == partials per row
+  int classes;         // residue classes of the vocabulary (1 unless d is odd-sized, see OddMaps)
+  int chunks;          // vocabulary chunks == partials per row; a multiple of `classes`
   int granule_rows;    // a multiple of 16 * cta
-  int granules;        // ceil(V / granule_rows)
+  int granules;        // ceil(rows of a class / granule_rows)
   int tiles_per_unit;  // every unit is walked in this many tiles (<= 256 rows each)
   int full_tiles_first;  // 1: full 256-row tiles, then one remainder tile; 0: tiles of equal size
   int mlp_rows;        // learned-router units: hidden width rounded up to the granule (0 = none); one such unit
@@ -34,6 +35,8 @@ struct TcPlan {
 struct TcParams {
   int n, d, V;
   int row_units, chunks, granules, tiles_per_unit, full_tiles_first, granule_rows;
+  int classes, class_chunks;          // odd-sized d only: residue classes, chunks per class (chunks == classes * class_chunks)
+  int h_class_rows;                   // odd-sized d only: rows between the shifted copies of h
   int a_rows, part_rows, a_stages, b_stages;
   unsigned long long wait_limit_ns;   // 0 = the default limit of every barrier wait
   int debug_drop_w_copies;            // test hook: the W producer issues no copies
@@ -59,10 +62,30 @@ struct TcMaps {
   CUtensorMap h, w128, w64, w16, m128, m64, m16;
 };
 
+// Tensor maps when d is not a multiple of 8 ("odd-sized"): rows of W are then no multiple of 16 bytes apart, which TMA
+// cannot address.  But C = 8 / gcd(d, 8) consecutive rows are, so the rows v = C q + r of one residue class r form a
+// matrix with an addressable pitch.  Its first element lies s = (r d) mod 8 elements past a 16-byte boundary: the map
+// of class r starts at that boundary, s elements early, and the class is multiplied by a copy of h shifted by s
+// elements, whose first s are zero.  W stays where it is; only h is copied, C times (tlr_odd.cu).
+constexpr int kMaxClasses = 8;
+constexpr int kOddBoxRows = 32;      // rows of W per TMA box (the vocabulary granule is this many rows per CTA)
+struct OddMaps {
+  CUtensorMap h, w[kMaxClasses];
+};
+inline int odd_classes(int d) { return d % 8 == 0 ? 1 : (d % 4 == 0 ? 2 : (d % 2 == 0 ? 4 : 8)); }
+inline int odd_shift(int d, int cls) { return static_cast<int>((static_cast<long long>(cls) * d) % 8); }
+inline int odd_max_shift(int d) { return 8 - 8 / odd_classes(d); }   // the shifts are all multiples of gcd(d, 8)
+// h [n][d] -> shifted copies [classes][class_rows][pitch]
+cudaError_t launch_odd_shift(const void* h_bf16, int n, int d, int class_rows, int pitch, void* out,
+                             cudaStream_t stream);
+cudaError_t odd_prepare();
+cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const TcConfig& c, int workers,
+                                  cudaStream_t stream);
+
 int tc_threads();
 int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
 void tc_configure(int n, TcConfig* c);
-void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden, TcPlan* plan);
+void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan);
 cudaError_t tc_prepare();   // opt in to the kernels' dynamic shared memory size (once per device)
 cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const TcConfig& c, int workers,
                                  cudaStream_t stream);

@@ -3,7 +3,7 @@
 // online-softmax reduction (max / argmax / sum-exp / entropy numerator) fused into
 // the epilogue, so the n x V logits never leave the SM.
 //
-// One kernel body, three instantiations (two kernels at the end of this file):
+// One kernel body, four instantiations (kernels at the end of this file):
 //   <1, false>  bf16 head, one CTA per worker, MMA M = 128 token rows     (n <= 128; M = 64 when n <= 64)
 //   <2, false>  bf16 head, a cluster of two CTAs per worker, MMA M = 256 rows (cta_group::2): each
 //               CTA stages its own 128 rows of h and HALF of the W tile, and the pair's
@@ -14,6 +14,8 @@
 //               covers both parts along its M, and the epilogue adds the two accumulator rows of a
 //               token before it folds them; above, two MMAs per K step (one per part) add into the
 //               same rows.
+//   OddMaps     bf16 head whose hidden size is no multiple of 8: the vocabulary is walked by residue class
+//               (see OddMaps), otherwise like the bf16 head.
 //
 // Decomposition.  The vocabulary is cut into `chunks` contiguous ranges of granules
 // (a multiple of 16 * kCta rows); the token rows into units of 128 * kCta.  A work unit is
@@ -92,6 +94,8 @@ struct Unit {
   int chunk;   // vocabulary chunk; -1 for a learned-router unit
   int g0;      // first granule of the chunk
   int G;       // granules in the chunk
+  int cls;     // residue class of the chunk's vocabulary rows (0 unless d is odd-sized)
+  int rows;    // vocabulary rows of that class (V unless d is odd-sized)
 };
 struct Tile {
   int v0;      // first vocabulary row of the tile (first row of W1 in a learned-router unit)
@@ -100,9 +104,11 @@ struct Tile {
 
 // What is fixed for a whole unit (the divisions happen here, once per unit: the tile walk of the MMA-issuing
 // warp is on the tensor pipe's critical path and must stay cheap).
-template <int kCta>
+template <int kCta, bool kOdd = false>
 __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, int cta_rank) {
   Unit u;
+  u.cls = 0;
+  u.rows = p.V;
   const int vocab_units = p.chunks * p.row_units;
   if (unit >= vocab_units) {          // learned-router unit: all rows of W1 for one row unit
     u.chunk = -1;
@@ -114,8 +120,15 @@ __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, in
   u.chunk = unit / p.row_units;
   const int ru = unit - u.chunk * p.row_units;
   u.row0 = (ru * kCta + cta_rank) * kBlockM;
-  u.g0 = static_cast<int>((static_cast<long long>(p.granules) * u.chunk) / p.chunks);
-  const int g1 = static_cast<int>((static_cast<long long>(p.granules) * (u.chunk + 1)) / p.chunks);
+  int c = u.chunk, chunks = p.chunks;
+  if (kOdd) {                         // class by class: the chunks of a class share its rows out
+    chunks = p.class_chunks;
+    u.cls = c / chunks;
+    c -= u.cls * chunks;
+    u.rows = (p.V - u.cls + p.classes - 1) / p.classes;
+  }
+  u.g0 = static_cast<int>((static_cast<long long>(p.granules) * c) / chunks);
+  const int g1 = static_cast<int>((static_cast<long long>(p.granules) * (c + 1)) / chunks);
   u.G = g1 - u.g0;
   return u;
 }
@@ -274,8 +287,9 @@ struct RowFold {
 
 // The kernel body (maps and p are the kernel's own parameters, maps a __grid_constant__ one: TMA reads the
 // tensor maps from parameter space).
-template <int kCta, bool kFp8>
-__device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcParams& p) {
+template <int kCta, bool kFp8, class Maps>
+__device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcParams& p) {
+  constexpr bool kOdd = std::is_same<Maps, OddMaps>::value;   // d no multiple of 8: vocabulary rows by residue class
   static_assert(!(kFp8 && kCta != 1), "the 8-bit head runs with one CTA per worker");
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment: the swizzle pattern is a function of the shared-memory address.
@@ -387,16 +401,21 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
       int slab = 0;     // running slab number, the same in every role
       bool ok = true;
       for (int unit = worker; unit < units && ok; unit += workers) {
-        const Unit un = unit_of<kCta>(p, unit, cta_rank);
+        const Unit un = unit_of<kCta, kOdd>(p, unit, cta_rank);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
           const int my_rows = tl.rows / kCta;                 // this CTA's share of the tile
           const int my_v0 = tl.v0 + static_cast<int>(cta_rank) * my_rows;
           const bool mlp = !kFp8 && un.chunk < 0;
-          const CUtensorMap* m128 = mlp ? &maps.m128 : &maps.w128;
-          const CUtensorMap* m64p = mlp ? &maps.m64 : &maps.w64;
-          const CUtensorMap* m16 = mlp ? &maps.m16 : &maps.w16;
+          const CUtensorMap *m128, *m64p, *m16;
+          if constexpr (kOdd) {
+            m128 = m64p = m16 = &maps.w[un.cls];
+          } else {
+            m128 = mlp ? &maps.m128 : &maps.w128;
+            m64p = mlp ? &maps.m64 : &maps.w64;
+            m16 = mlp ? &maps.m16 : &maps.w16;
+          }
           for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
             if (slab >= SB) {     // the stage is free once slab - SB has been consumed
               const int j = slab - SB;
@@ -407,6 +426,9 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
             if (p.debug_drop_w_copies) continue;   // test hook: the copies are "lost", the consumer's wait runs out
             if (leader) mbar_expect_tx(b_full(stage), tl.rows * kRowBytes);   // both CTAs' bytes
             int r = 0;
+            if (kOdd)
+              for (; r < my_rows; r += kOddBoxRows)
+                tma_load_2d<kCta>(dst + r * kRowBytes, m128, bar, ks * kSlabElems, my_v0 + r);
             for (; my_rows - r >= 128; r += 128)
               tma_load_2d<kCta>(dst + r * kRowBytes, m128, bar, ks * kSlabElems, my_v0 + r);
             for (; my_rows - r >= 64; r += 64)
@@ -427,7 +449,7 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
       int slab = 0;
       bool ok = true;
       for (int unit = worker; unit < units && ok; unit += workers) {
-        const Unit un = unit_of<kCta>(p, unit, cta_rank);
+        const Unit un = unit_of<kCta, kOdd>(p, unit, cta_rank);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
@@ -439,7 +461,8 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
             const uint32_t dst = a_ring + stage * a_stage_bytes;
             const uint32_t bar = (kCta == 2) ? map_to_cta(a_full(stage), 0) : a_full(stage);
             if (leader) mbar_expect_tx(a_full(stage), a_stage_bytes * kCta);
-            tma_load_2d<kCta>(dst, &maps.h, bar, ks * kSlabElems, kFp8 ? 0 : un.row0);
+            tma_load_2d<kCta>(dst, &maps.h, bar, ks * kSlabElems,
+                              kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0));
             if (++stage == SA) stage = 0;
           }
         }
@@ -474,7 +497,7 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
       // issued, so the poll's latency overlaps the issue instead of adding to it.
       bool ra = inl || mbar_test_wait(a_full(0), 0), rb = mbar_test_wait(b_full(0), 0);
       for (int unit = worker; unit < units && ok; unit += workers) {
-        const Unit un = unit_of<kCta>(p, unit, 0);
+        const Unit un = unit_of<kCta, kOdd>(p, unit, 0);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
@@ -551,7 +574,7 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
       ok = __all_sync(0xffffffffu, ok);
     }
     for (int unit = worker; unit < units && ok; unit += workers, ++ord) {
-      const Unit first = unit_of<kCta>(p, unit, cta_rank);
+      const Unit first = unit_of<kCta, kOdd>(p, unit, cta_rank);
       const bool warp_has_rows = first.row0 + quad_row0 < p.n;            // warp-uniform
       const bool two_tokens = kFp8 && frag && !m64 && quad_row0 + 8 < p.n;   // warp-uniform
       const bool mlp_unit = !kFp8 && first.chunk < 0;
@@ -567,7 +590,7 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
         const Tile tl = tile_of(p, first, t);
         if (tl.rows == 0) continue;
         const int v0 = tl.v0;
-        const int cols = min(tl.rows, (kRouter ? p.mlp_hidden : p.V) - v0);   // valid columns of this tile
+        const int cols = min(tl.rows, (kRouter ? p.mlp_hidden : first.rows) - v0);   // valid columns of this tile
         // this group's share of them: [0, half) or [half, cols), half a multiple of the columns of a load
         const int step = frag ? 64 : 32;
         const int half = min(cols, (tl.rows / 2 + step - 1) & ~(step - 1));
@@ -652,11 +675,12 @@ __device__ __forceinline__ void tc_projection_body(const TcMaps& maps, const TcP
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
       };
-      if (mlp_unit) walk_tiles(std::true_type{});
+      if (!kOdd && mlp_unit) walk_tiles(std::integral_constant<bool, !kOdd>{});
       else walk_tiles(std::false_type{});
       Partial out[kFolds];
 #pragma unroll
       for (int i = 0; i < kFolds; ++i) out[i] = f[i].result();
+      if (kOdd && out[0].idx != kNoToken) out[0].idx = out[0].idx * p.classes + first.cls;   // row q of the class
       if (frag) {                              // the four threads of a token merge their summaries
 #pragma unroll
         for (int i = 0; i < kFolds; ++i) {
@@ -713,6 +737,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_projection_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
   tc_projection_body<kCta, false>(maps, p);
 }
+
+// d no multiple of 8 (defined in the one file that launches them).
+#ifdef TLR_DEFINE_ODD_KERNELS
+template <int kCta>
+__global__ void __launch_bounds__(kThreads, 1)
+odd_projection_kernel(const __grid_constant__ OddMaps maps, const TcParams p) {
+  tc_projection_body<kCta, false>(maps, p);
+}
+#endif
 
 // 8-bit head (defined in the one file that launches it).  At most 128 registers per thread, so that a block of
 // the merge kernel (512 threads) fits on the SM beside this CTA and is resident, waiting, before this kernel ends.

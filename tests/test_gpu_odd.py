@@ -1,0 +1,99 @@
+"""Hidden sizes that are no multiple of 8 on the tensor-core path, against the CPU fp64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import tlr_synth as S
+from oracle import route_oracle as O
+from tests.parity import check_against_oracle, check_self_consistency, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def check(pkg, W, h, tau):
+    ref = O.route_oracle(S.bf16_bits(h), S.bf16_bits(W), tau)
+    gpu = run_gpu(pkg, W.cuda(), h, tau, path=2)
+    assert gpu["status"] == 0 and gpu["plan"].path == 2
+    check_self_consistency(gpu, tau, W.shape[0])
+    check_against_oracle(ref, gpu, O.bf16_bits_to_f64(S.bf16_bits(h)), O.bf16_bits_to_f64(S.bf16_bits(W)))
+    return gpu
+
+
+# 2, 4 and 8 residue classes; slabs that the shift just fills or just overflows; fewer vocabulary rows than classes,
+# classes of different lengths, boxes and granules that end inside a class; either side of every switch of the kernel's
+# row handling
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 7, 12, 57, 58, 60, 61, 100, 130, 257, 300])
+@pytest.mark.parametrize("n,V", [(1, 1), (3, 7), (16, 9), (17, 260), (65, 2049), (129, 1025), (300, 5003)])
+def test_small_shapes(pkg, n, d, V):
+    W = S.make_W(d, V, seed=n + d + V, std=0.1)
+    hid = S.make_h(n, d, seed=n + d, W=W, planted_fraction=0.1 if n >= 16 else 0.0)
+    check(pkg, W, hid.h, 0.5)
+
+
+@pytest.mark.parametrize("n,d,V", [(1, 2047, 20001), (64, 300, 33000), (256, 999, 30000), (100, 1500, 40000)])
+def test_larger_shapes(pkg, n, d, V):
+    W = S.make_W(d, V, seed=d, std=0.05)
+    hid = S.make_h(n, d, seed=n, W=W, planted_fraction=0.1 if n >= 16 else 0.0)
+    check(pkg, W, hid.h, 0.5)
+
+
+@pytest.mark.parametrize("n,d", [(2048, 12), (2049, 12), (4500, 9)])
+def test_batches_in_several_blocks(pkg, n, d):
+    W = S.make_W(d, 700, seed=n, std=0.3)
+    hid = S.make_h(n, d, seed=d, W=W, planted_fraction=0.1)
+    check(pkg, W, hid.h, 0.5)
+
+
+@pytest.mark.parametrize("d", [63, 130, 300])
+@pytest.mark.parametrize("n", [40, 1100])
+def test_equal_rows_of_different_classes_tie_to_the_lowest_index(pkg, n, d):
+    V = 3001
+    W = S.make_W(d, V, seed=d, std=0.2)
+    hid = S.make_h(n, d, seed=n, W=W, planted_fraction=0.5)
+    first = O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W), 0.5)
+    winners = np.unique(first.token)
+    W2 = W.clone()
+    for k, v in enumerate(winners[:200].tolist()):         # copies of the winners, mostly in other classes, at both ends
+        W2[(5 * k) % 1000] = W[v]
+        W2[V - 1 - (7 * k) % 1000] = W[v]
+    ref = O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W2), 0.5)
+    exact = (O.bf16_bits_to_f64(S.bf16_bits(hid.h)) @ O.bf16_bits_to_f64(S.bf16_bits(W2)).T)
+    top = exact.max(axis=1, keepdims=True)
+    runner = np.where(exact >= top - 1e-9, -np.inf, exact).max(axis=1)     # the best row that is not an equal one
+    sure = top[:, 0] - runner > 1e-3
+    assert sure.sum() >= n // 2
+    gpu = run_gpu(pkg, W2.cuda(), hid.h, 0.5)
+    assert np.array_equal(gpu["token"][sure], ref.token[sure])
+
+
+def test_learned_router_and_host_buffers(pkg):
+    n, d, V, dh = 70, 100, 3000, 48
+    W = S.make_W(d, V, seed=1, std=0.1)
+    hid = S.make_h(n, d, seed=2)
+    g = torch.Generator().manual_seed(5)
+    W1 = (torch.randn(dh, d, generator=g) / d ** 0.5).to(torch.bfloat16)
+    b1, w2 = torch.randn(dh, generator=g) * 0.1, torch.randn(dh, generator=g) * 0.5
+    want = O.mlp_router_score(S.bf16_bits(hid.h), S.bf16_bits(W1), b1.numpy(), w2.numpy(), 0.1)
+    ref = O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W), 0.5)
+    r = pkg.Router(W.cuda(), max_n=n)
+    r.set_router_mlp(W1.cuda(), b1.cuda(), w2.cuda(), 0.1)
+    score = torch.full((n,), float("nan"), device="cuda")
+    r.route(hid.h.cuda(), 0.5, score_source=pkg.TLR_SCORE_MLP, mlp_score=score)
+    torch.cuda.synchronize()
+    assert np.max(np.abs(score.cpu().numpy() - want)) <= 1e-3
+    out = [torch.zeros(n, dtype=torch.int32), torch.zeros(n), torch.zeros(n), torch.zeros(n, dtype=torch.uint8),
+           torch.zeros(n, dtype=torch.int32), torch.zeros(1, dtype=torch.int32)]
+    pkg.tlr_route_host(r.ctx, hid.h.pin_memory(), n, 0.5, *out)
+    assert np.max(np.abs(out[1].numpy() - ref.conf) / ref.conf) <= 1e-3
+    assert np.array_equal(out[0].numpy()[ref.top2_gap >= 1e-3], ref.token[ref.top2_gap >= 1e-3])
+    r.close()
+
+
+def test_tiny_heads_keep_the_cuda_core_kernel(pkg):
+    for n, d, V, path in ((32, 36, 1820, 1), (33, 36, 1820, 2), (32, 36, 1821, 2), (32, 32, 500, 2)):
+        W = S.make_W(d, V, seed=n, std=0.2)
+        hid = S.make_h(n, d, seed=V)
+        ref = O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W), 0.01)
+        gpu = run_gpu(pkg, W.cuda(), hid.h, 0.01)
+        assert gpu["plan"].path == path and gpu["status"] == 0
+        check_against_oracle(ref, gpu)
