@@ -211,13 +211,18 @@ __device__ __forceinline__ void wait_for_peers(const FinishLaunch& a) {
 // row in two passes over its partials: maximum and index first, then the sums rescaled to
 // that maximum.  L is chosen on the host so that every row has its group: n * L <=
 // gridDim.x * 1024.
+// (kTies: with settle_ties; a kernel of its own, because the call would cost the other one registers -- 40 is the most
+// that lets a block of 512 threads stand beside a CTA of the 8-bit projection kernel.)
+template <bool kTies>
 __global__ void __launch_bounds__(kSmallThreads)
-finish_small_kernel(const FinishLaunch a, const int L) {
+finish_small_kernel(const FinishLaunch a, const int log2_L) {
   __shared__ int warp_count[kSmallThreads / 32];
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int group = (blockIdx.x * blockDim.x + threadIdx.x) / L;
+  const int L = 1 << log2_L;
+  const int group = (blockIdx.x * blockDim.x + threadIdx.x) >> log2_L;
   const int gl = threadIdx.x & (L - 1);
+  const bool one_pass = ((a.chunks + L - 1) >> log2_L) <= kPerLane;
   pdl_enter();
   wait_for_peers(a);
   __shared__ unsigned char flags[kSmallRows];
@@ -230,7 +235,7 @@ finish_small_kernel(const FinishLaunch a, const int L) {
     float m = -INFINITY;
     int idx = kNoToken;
     float s = 0.f, t = 0.f;
-    if ((a.chunks + L - 1) / L <= kPerLane) {
+    if (one_pass) {
       // few partials per lane: one pass, the partials stay in registers
       Partial q[kPerLane];
 #pragma unroll
@@ -303,7 +308,7 @@ finish_small_kernel(const FinishLaunch a, const int L) {
       s += __shfl_xor_sync(0xffffffffu, s, off);
       t += __shfl_xor_sync(0xffffffffu, t, off);
     }
-    if (a.tie_W != nullptr && valid)
+    if (kTies && valid)
       idx = settle_ties(a.tie_W, a.tie_h + static_cast<size_t>(row) * a.tie_d, a.tie_d, p, a.chunks, a.chunk_stride, m, idx,
                         gl, L);
     if (valid && gl == 0) {
@@ -339,23 +344,19 @@ finish_small_kernel(const FinishLaunch a, const int L) {
   int base_out = 0;
   for (int base = 0; base < a.n; base += blockDim.x) {       // one pass when the block has a thread per row
     const int i = base + threadIdx.x;
-    int flag = 0;
-    if (i < a.n) flag = static_cast<int>(flags[i]);
+    const int flag = i < a.n ? static_cast<int>(flags[i]) : 0;
     const unsigned int bal = __ballot_sync(0xffffffffu, flag != 0);
     if (lane == 0) warp_count[warp] = __popc(bal);
     __syncthreads();
-    int before = 0, total = 0;
-    for (int w = 0; w < warps; ++w) {
-      const int c = warp_count[w];
-      before += (w < warp) ? c : 0;
-      total += c;
-    }
+    // at most 32 warps: lane w holds warp w's count
+    const int c = lane < warps ? warp_count[lane] : 0;
+    const int before = __reduce_add_sync(0xffffffffu, lane < warp ? c : 0);
     if (flag) {
       a.routed_idx[base_out + before + __popc(bal & ((1u << lane) - 1u))] = i;
       first_routed_note(a, i);
     }
-    base_out += total;
-    __syncthreads();
+    base_out += __reduce_add_sync(0xffffffffu, c);
+    if (base + static_cast<int>(blockDim.x) < a.n) __syncthreads();
   }
   if (threadIdx.x == 0) {
     *a.routed_count = base_out;
@@ -435,7 +436,7 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
   cfg.numAttrs = 1;
   if (a.n <= kSmallRows) {
     int blocks = 1;
-    while (blocks < 8 && blocks * 32 < a.n) blocks <<= 1;       // 32 rows per block until 8 blocks
+    while (blocks < 8 && blocks * 16 < a.n) blocks <<= 1;       // 16 rows per block until 8 blocks
     // 512-thread blocks fit on an SM beside a CTA of the tensor-core projection kernel, so they
     // are resident (waiting) before it ends and do not keep the next call's CTAs off their SMs;
     // they are used whenever a lane group still owns few enough partials for the one-pass fold.
@@ -450,7 +451,8 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
       const int e = tuning().finish_threads;   // tuning switch (TLR_FINISH_THREADS)
       if (e == 256 || e == 512 || e == 1024) threads = e;
     }
-    const int L = lanes_for(threads);
+    int log2_L = 0;
+    while ((1 << log2_L) < lanes_for(threads)) ++log2_L;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = static_cast<unsigned>(blocks);
     attr[1].val.clusterDim.y = 1;
@@ -458,7 +460,7 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     cfg.numAttrs = 2;
     cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
     cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
-    return cudaLaunchKernelEx(&cfg, finish_small_kernel, a, L);
+    return cudaLaunchKernelEx(&cfg, a.tie_W != nullptr ? finish_small_kernel<true> : finish_small_kernel<false>, a, log2_L);
   }
   const int blocks = (a.n + kFinishWarps - 1) / kFinishWarps;
   cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
