@@ -47,6 +47,10 @@ shard_summary_kernel(const Partial* __restrict__ partials, int n, int chunks, in
                      Partial* __restrict__ summary) {
   const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  // A programmatic dependent launch like the kernels around it: its blocks (512 small ones at most fit beside the
+  // projection's CTAs) wait for the projection where they stand, and a merge kernel behind it may be scheduled now.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row >= n) return;
   const Partial acc = row_summary(partials, row, chunks, v_offset, lane);
   if (lane == 0) summary[row] = acc;
@@ -106,8 +110,16 @@ rows_merge_kernel(const int32_t* __restrict__ gathered_idx, const int32_t* __res
 cudaError_t launch_shard_summary(const Partial* partials, int n, int chunks, int v_offset, Partial* summary,
                                  cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
-  shard_summary_kernel<<<(n + kWarps - 1) / kWarps, kWarps * 32, 0, stream>>>(partials, n, chunks, v_offset, summary);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>((n + kWarps - 1) / kWarps), 1, 1);
+  cfg.blockDim = dim3(kWarps * 32, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, shard_summary_kernel, partials, n, chunks, v_offset, summary);
 }
 
 cudaError_t launch_shard_push(const ShardPush& a, cudaStream_t stream) {
