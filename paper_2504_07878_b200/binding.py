@@ -112,20 +112,28 @@ def _check(code: int, where: str):
         raise TlrError(code, where)
 
 
-def _ptr(t) -> c_void_p:
-    if t is None:
-        return c_void_p(0)
-    if isinstance(t, int):
-        return c_void_p(t)
-    return c_void_p(t.data_ptr())
+def _ptr(t):
+    """The address a pointer argument stands for: a tensor's, an int's own value, None for null.  (Plain ints: the
+    argument types turn them into pointers, and a c_void_p object per argument costs as much as the call.)"""
+    if t is None or isinstance(t, int):
+        return t
+    return t.data_ptr()
 
 
-def _stream_handle(stream) -> c_void_p:
+# torch.cuda.current_stream() builds a Stream object per call (about 2 us, a third of what a call of this library costs
+# the host); this asks for the handle alone.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _stream_handle(stream):
     if stream is None:
+        if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         stream = torch.cuda.current_stream()
     if isinstance(stream, int):
-        return c_void_p(stream)
-    return c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def tlr_create(d: int, V: int, W, max_n: int) -> c_void_p:
@@ -326,6 +334,16 @@ class Router:
             self.route_mask = torch.empty(max_n, dtype=torch.uint8, device=dev)
             self.routed_idx = torch.empty(max_n, dtype=torch.int32, device=dev)
             self.routed_count = torch.zeros(1, dtype=torch.int32, device=dev)
+        self._views = {}                # n -> views of the output tensors for n rows (making four costs 6 us)
+
+    def _outputs(self, n: int):
+        views = self._views.get(n)
+        if views is None:
+            if len(self._views) >= 16:
+                self._views.clear()
+            views = self._views[n] = (self.token[:n], self.conf[:n], self.entropy[:n], self.route_mask[:n],
+                                      self.routed_idx, self.routed_count)
+        return views
 
     def set_router_mlp(self, W1: torch.Tensor, b1: torch.Tensor, w2: torch.Tensor, b2: float):
         """Attach a learned router; the tensors are kept alive by this object."""
@@ -347,8 +365,7 @@ class Router:
                          self.routed_count, stream, tau_per_row=tau_per_row, route_above=route_above,
                          seq_len=seq_len, first_routed=first_routed, score_source=score_source,
                          mlp_score=mlp_score)
-        return (self.token[:n], self.conf[:n], self.entropy[:n], self.route_mask[:n], self.routed_idx,
-                self.routed_count)
+        return self._outputs(n)
 
     def prepared(self, h: torch.Tensor, tau: float, stream=None):
         """The same step as route(h, tau, stream) as a callable with its arguments marshalled once: for a decode
