@@ -52,8 +52,11 @@ void tc_configure(int n, TcConfig* c) {
   const int a_stage = a_rows * kRowBytes;
   const int b_stage = (kBlockN / cta) * kRowBytes;
   // h slabs come from L2 (about a microsecond away under load) and one is consumed per W
-  // slab, so the h ring needs about half the depth of the W ring to keep up.
-  int sa = cta == 2 ? 4 : (a_rows <= 32 ? 6 : 4);
+  // slab, so the h ring needs about half the depth of the W ring to keep up.  In pair mode five
+  // stages: short units live on what the W ring holds when h arrives, and then h is what they wait for
+  // (n = 256, d = 896, V = 18976: 4 / 5 / 6 / 8 stages 19.66 / 19.15 / 19.35 / 20.07 us per step;
+  // n = 1024, d = 512, V = 32000: 39.2 / 38.5 / 38.6 / 39.4; no difference where W streams for long).
+  int sa = cta == 2 ? 5 : (a_rows <= 32 ? 6 : 4);
   const int budget = kSmemLimit - 1024 - kBarrierBytes - kScratchBytes;
   int sb = (budget - sa * a_stage) / b_stage;
   if (sb > kMaxBStages) sb = kMaxBStages;
