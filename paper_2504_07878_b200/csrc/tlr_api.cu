@@ -781,7 +781,9 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
     m.d = ctx->d;
     m.d_hidden = ctx->mlp_hidden;
     m.partial = ctx->mlp_scores;
-    if (tlr::launch_mlp_score(m, stream) != cudaSuccess) return TLR_ERR_CUDA;
+    const bool beside = ctx->fp8 && (reinterpret_cast<uintptr_t>(m.W1) & 15u) == 0;
+    if ((beside ? tlr::launch_mlp_beside(m, stream) : tlr::launch_mlp_score(m, stream)) != cudaSuccess)
+      return TLR_ERR_CUDA;
   }
 
   tlr::FinishLaunch f = {};

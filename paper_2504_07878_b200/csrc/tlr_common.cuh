@@ -162,5 +162,7 @@ struct MlpLaunch {
 };
 int mlp_hidden_blocks(int d_hidden);
 cudaError_t launch_mlp_score(const MlpLaunch& a, cudaStream_t stream);
+// directly behind a projection launch of tlr_tc_kernel.cuh and beside it; d % 8 == 0, W1 and h 16-byte aligned
+cudaError_t launch_mlp_beside(const MlpLaunch& a, cudaStream_t stream);
 
 }  // namespace tlr

@@ -4,8 +4,9 @@
 // the shape here (one hidden layer, ReLU, sigmoid output) is this library's assumption and
 // the weights are the caller's.  Where the tensor-core projection kernel runs, the first layer is
 // part of that launch (tlr_tc_kernel.cuh); this CUDA-core kernel serves the shapes it cannot take
-// (d % 8 != 0, an unaligned W1, the 8-bit head): a block stages kMlpRows hidden-state rows in shared
-// memory and covers kMlpUnits hidden units, eight threads per unit.
+// (d % 8 != 0, an unaligned W1): a block stages kMlpRows hidden-state rows in shared
+// memory and covers kMlpUnits hidden units, eight threads per unit.  The 8-bit head has a tensor-core kernel of its own
+// (mlp_mma_kernel) that runs beside the projection.
 #include "tlr_common.cuh"
 
 namespace tlr {
@@ -111,6 +112,110 @@ mlp_partial_kernel(const MlpLaunch a) {
     for (int w = 0; w < kMlpThreads / 32; ++w) v += red[w][threadIdx.x];
     a.partial[static_cast<size_t>(row0 + threadIdx.x) * gridDim.y + blockIdx.y] = v;
   }
+}
+
+// 8-bit head (d a multiple of 16, W1 and h 16-byte aligned): the same partial sums with mma.sync, beside the projection.
+// The projection kernel of the 8-bit head multiplies e4m3 only, so W1 cannot be units of that launch; what W1 needs is
+// small (100 rows, 256 units, d = 2048: 0.1 GFLOP, 1.5 MB) and hides behind the stream of W if it does not wait for it.
+// So this kernel reads h without waiting for the projection in front of it: that kernel lets its dependents be scheduled
+// only after its own wait, when h is complete.  One block waits for the projection at the END, so that this grid is not
+// complete before it and the merge kernel behind, which waits for this grid, finds both.  Four warps per block, each
+// a quarter of K, and 2 KB of shared memory: such blocks fit beside the projection's CTAs whatever their rings take.
+// As the CUDA-core kernel between projection and merge: 34 of 111 us per step at that size (V = 128256); now 4 of 79.
+constexpr int kMmaRows = 16;
+constexpr int kMmaWarps = 4;
+constexpr int kMmaBatch = 4;         // steps of 32 k values whose loads a warp has in flight together
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__global__ void __launch_bounds__(32 * kMmaWarps)
+mlp_mma_kernel(const MlpLaunch a) {
+  __shared__ float sums[16][32];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, t = lane & 3;          // row / column of the fragments, and which eight of 32 k values
+  const int row0 = blockIdx.x * kMmaRows + g, row1 = row0 + 8, unit0 = blockIdx.y * kMlpUnits;
+  const unsigned short* h = static_cast<const unsigned short*>(a.h);
+  const unsigned short* W1 = static_cast<const unsigned short*>(a.W1);
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  float acc[4][4] = {};
+  // A thread's 16 bytes are eight consecutive k values; which k an MMA calls which does not matter as long as both
+  // operands agree, so words 0, 1 go to one MMA (16 k values over the four threads) and words 2, 3 to the next.
+  const int steps = (a.d + 31) / 32, s0 = steps * warp / kMmaWarps, s1 = steps * (warp + 1) / kMmaWarps;
+  for (int sb = s0; sb < s1; sb += kMmaBatch) {
+    uint4 x[kMmaBatch], y[kMmaBatch], w[kMmaBatch][4];     // every load of a batch is in flight before its first MMA
+#pragma unroll
+    for (int i = 0; i < kMmaBatch; ++i) {
+      const int k = (sb + i) * 32 + t * 8;
+      const bool in = sb + i < s1 && k < a.d;
+      x[i] = in && row0 < a.n ? __ldcg(reinterpret_cast<const uint4*>(h + static_cast<size_t>(row0) * a.d + k)) : zero;
+      y[i] = in && row1 < a.n ? __ldcg(reinterpret_cast<const uint4*>(h + static_cast<size_t>(row1) * a.d + k)) : zero;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int u = unit0 + 8 * j + g;
+        w[i][j] = in && u < a.d_hidden ? __ldg(reinterpret_cast<const uint4*>(W1 + static_cast<size_t>(u) * a.d + k)) : zero;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kMmaBatch; ++i) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        mma_bf16(acc[j], x[i].x, y[i].x, x[i].y, y[i].y, w[i][j].x, w[i][j].y);
+        mma_bf16(acc[j], x[i].z, y[i].z, x[i].w, y[i].w, w[i][j].z, w[i][j].w);
+      }
+    }
+  }
+  // the warps' sums, added in a fixed order through one 2 KB buffer
+  for (int turn = kMmaWarps - 1; turn > 0; --turn) {
+    if (warp == turn) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) sums[i][lane] = acc[i >> 2][i & 3] + (turn == kMmaWarps - 1 ? 0.f : sums[i][lane]);
+    }
+    __syncthreads();
+  }
+  if (warp == 0) {
+    float v0 = 0.f, v1 = 0.f;                     // rows row0 and row1, units 2t and 2t + 1 of every eight
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int u = unit0 + 8 * j + 2 * t + i;
+        if (u >= a.d_hidden) continue;
+        const float b1 = __ldg(a.b1 + u), w2 = __ldg(a.w2 + u);
+        v0 += w2 * fmaxf(acc[j][i] + sums[4 * j + i][lane] + b1, 0.f);
+        v1 += w2 * fmaxf(acc[j][2 + i] + sums[4 * j + 2 + i][lane] + b1, 0.f);
+      }
+    }
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
+    v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
+    v1 += __shfl_xor_sync(0xffffffffu, v1, 2);
+    if (t == 0) {
+      if (row0 < a.n) a.partial[static_cast<size_t>(row0) * gridDim.y + blockIdx.y] = v0;
+      if (row1 < a.n) a.partial[static_cast<size_t>(row1) * gridDim.y + blockIdx.y] = v1;
+    }
+  }
+  if (blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+cudaError_t launch_mlp_beside(const MlpLaunch& a, cudaStream_t stream) {
+  if (a.n <= 0) return cudaSuccess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>((a.n + kMmaRows - 1) / kMmaRows),
+                     static_cast<unsigned>(mlp_hidden_blocks(a.d_hidden)), 1);
+  cfg.blockDim = dim3(32 * kMmaWarps, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, mlp_mma_kernel, a);
 }
 
 cudaError_t launch_mlp_score(const MlpLaunch& a, cudaStream_t stream) {

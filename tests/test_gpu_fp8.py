@@ -189,3 +189,32 @@ def test_fp8_fragment_edges(pkg, n, V):
     assert gpu["status"] == 0
     check_self_consistency(gpu, 0.5, V)
     check_against_oracle(ref, gpu, O.bf16_bits_to_f64(S.bf16_bits(h)), W64)
+
+
+# The learned router beside the 8-bit projection: rows at the edges of the 16-row fragments, hidden units at the edges of
+# the groups of 8 and 32, K that ends inside a 32-wide step; 20 steps in a row on changing h, so that a score taken from
+# the step before (or a step ahead) would show.
+@pytest.mark.parametrize("n,d,dh", [(1, 16, 1), (8, 48, 7), (9, 32, 8), (16, 64, 33), (17, 80, 31), (33, 144, 64),
+                                    (100, 2048, 256), (128, 896, 300)])
+def test_fp8_learned_router_beside_the_projection(pkg, n, d, dh):
+    V, steps = 3000, 20
+    codes, scale = S.make_W8(d, V, seed=3, std=0.1)
+    g = torch.Generator().manual_seed(dh + d)
+    W1 = (torch.randn(dh, d, generator=g) / d ** 0.5).to(torch.bfloat16)
+    b1, w2 = torch.randn(dh, generator=g) * 0.1, torch.randn(dh, generator=g) * 0.5
+    r = pkg.Router(codes.cuda(), max_n=n, wscale=scale.cuda())
+    r.set_router_mlp(W1.cuda(), b1.cuda(), w2.cuda(), -0.1)
+    hs = [S.make_h(n, d, seed=k).h for k in range(steps)]
+    dev = [h.cuda() for h in hs]
+    buf = torch.empty_like(dev[0])
+    scores = [torch.full((n,), float("nan"), device="cuda") for _ in range(steps)]
+    for k in range(steps):
+        buf.copy_(dev[k])
+        r.route(buf, 0.5, score_source=pkg.TLR_SCORE_MLP, mlp_score=scores[k])
+    torch.cuda.synchronize()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    for k in range(steps):
+        want = O.mlp_router_score(S.bf16_bits(hs[k]), S.bf16_bits(W1), b1.numpy(), w2.numpy(), -0.1)
+        # exact products, fp32 sums of d and dh terms: far below 1e-5 on scores in [0, 1]
+        assert np.max(np.abs(scores[k].cpu().numpy() - want)) <= 1e-5
+    r.close()
