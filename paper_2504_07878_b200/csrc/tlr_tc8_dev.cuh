@@ -65,6 +65,33 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint16_t& p1, uin
   p2 = to_e4m3x2(x1 - f1.y, x0 - f1.x);
 }
 
+__device__ __forceinline__ float abs_max8(const uint4& v) {     // of eight bf16
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  float m = 0.f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
+    m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
+  }
+  return m;
+}
+
+// Sixteen bf16 (lo, hi), times inv, as first parts q1 and second parts q2.
+__device__ __forceinline__ void split16(const uint4& lo, const uint4& hi, float inv, uint4& q1, uint4& q2) {
+  const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  uint32_t a[4] = {0u, 0u, 0u, 0u}, b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {                                // two elements per 32-bit word
+    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
+    uint16_t p1, p2;
+    split_pair(f.x * inv, f.y * inv, p1, p2);
+    a[j >> 1] |= static_cast<uint32_t>(p1) << (16 * (j & 1));
+    b[j >> 1] |= static_cast<uint32_t>(p2) << (16 * (j & 1));
+  }
+  q1 = make_uint4(a[0], a[1], a[2], a[3]);
+  q2 = make_uint4(b[0], b[1], b[2], b[3]);
+}
+
 // Splits the (at most 16) rows of h into resident operand slabs, done by 288 threads numbered t (the caller's
 // warps 2..10; they synchronise among themselves with named barrier 1).  Slab ks is 32 rows of 128 bytes
 // with the 128-byte swizzle TMA would have produced, the two parts in alternating groups of eight rows
@@ -93,14 +120,7 @@ __device__ __forceinline__ void split_h_resident(const __nv_bfloat16* __restrict
     }
   }
 #pragma unroll
-  for (int i = 0; i < kSplitChunks; ++i) {
-    const uint32_t w[8] = {va[i].x, va[i].y, va[i].z, va[i].w, vb[i].x, vb[i].y, vb[i].z, vb[i].w};
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-      amax = fmaxf(amax, fmaxf(fabsf(f.x), fabsf(f.y)));
-    }
-  }
+  for (int i = 0; i < kSplitChunks; ++i) amax = fmaxf(amax, fmaxf(abs_max8(va[i]), abs_max8(vb[i])));
   // the row's largest magnitude: non-negative floats order like their bit patterns
   unsigned int* amax_bits = reinterpret_cast<unsigned int*>(hs_s + 32);
   if (t < 16) amax_bits[t] = 0u;
@@ -115,19 +135,11 @@ __device__ __forceinline__ void split_h_resident(const __nv_bfloat16* __restrict
     const int cc = l + kSplitLanes * i;
     if (cc >= k_slabs * 8) continue;                             // (chunks between d and the slab's end are zeros)
     const int ks = cc >> 3, c = cc & 7;
-    const uint32_t w[8] = {va[i].x, va[i].y, va[i].z, va[i].w, vb[i].x, vb[i].y, vb[i].z, vb[i].w};
-    uint32_t q1[4] = {0u, 0u, 0u, 0u}, q2[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {                                // two elements per 32-bit word
-      const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-      uint16_t p1, p2;
-      split_pair(f.x * inv, f.y * inv, p1, p2);
-      q1[j >> 1] |= static_cast<uint32_t>(p1) << (16 * (j & 1));
-      q2[j >> 1] |= static_cast<uint32_t>(p2) << (16 * (j & 1));
-    }
+    uint4 q1, q2;
+    split16(va[i], vb[i], inv, q1, q2);
     unsigned char* dst = slabs + ks * 4096 + tc8_part_row(r, 16) * 128 + ((c ^ (r & 7)) << 4);
-    *reinterpret_cast<uint4*>(dst) = make_uint4(q1[0], q1[1], q1[2], q1[3]);
-    *reinterpret_cast<uint4*>(dst + 1024) = make_uint4(q2[0], q2[1], q2[2], q2[3]);
+    *reinterpret_cast<uint4*>(dst) = q1;
+    *reinterpret_cast<uint4*>(dst + 1024) = q2;
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic stores -> the MMA's (async proxy) reads
 }
