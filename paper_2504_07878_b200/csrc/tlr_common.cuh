@@ -76,6 +76,62 @@ __device__ __forceinline__ Partial warp_merge(Partial p) {
   return p;
 }
 
+constexpr int kPerLane = 6;            // ceil(192 / 32): the most partials a lane can own
+
+// Folds one row's partials.  Every lane returns the same result.
+__device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int chunks, int chunk_stride, int lane) {
+  Partial q[kPerLane];
+  float m = -INFINITY;
+  int idx = kNoToken;
+#pragma unroll
+  for (int k = 0; k < kPerLane; ++k) {
+    const int j = lane + 32 * k;
+    if (j < chunks) {
+      const float4 raw = __ldcg(reinterpret_cast<const float4*>(p + static_cast<size_t>(j) * chunk_stride));
+      q[k].m = raw.x;
+      q[k].idx = __float_as_int(raw.y);
+      q[k].s = raw.z;
+      q[k].t = raw.w;
+    } else {
+      q[k] = empty_partial();
+    }
+    if (q[k].m > m || (q[k].m == m && q[k].idx < idx)) {
+      m = q[k].m;
+      idx = q[k].idx;
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const float om = __shfl_xor_sync(0xffffffffu, m, off);
+    const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
+    if (om > m || (om == m && oi < idx)) {
+      m = om;
+      idx = oi;
+    }
+  }
+  float s = 0.f, t = 0.f;
+#pragma unroll
+  for (int k = 0; k < kPerLane; ++k) {
+    if (!(q[k].s == 0.f)) {           // an empty range contributes nothing; a NaN sum goes through
+      const float dm = q[k].m - m;    // <= 0
+      const float e = exp2f(dm * kLog2e);
+      s += q[k].s * e;
+      t += e * (q[k].t + dm * q[k].s);
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, off);
+    t += __shfl_xor_sync(0xffffffffu, t, off);
+  }
+  Partial r;
+  r.m = m;
+  r.idx = idx;
+  r.s = s;
+  r.t = t;
+  return r;
+}
+
 // Host-side launchers (one per .cu file).  All enqueue on `stream` and return the
 // launch error, if any.
 struct SimtLaunch {

@@ -27,7 +27,6 @@ constexpr int kFinishWarps = 8;
 constexpr int kFinishThreads = kFinishWarps * 32;
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallRows = 1024;
-constexpr int kPerLane = 6;            // ceil(192 / 32): the most partials a lane can own
 
 // The token of a row whose maximum m (at idx) may be tied with another partial's, see FinishLaunch::tie_W: the
 // candidates within the rounding of m are compared by fp32 dot products that all sum in the same order, so equal rows
@@ -71,91 +70,47 @@ __device__ __noinline__ int settle_ties(const unsigned short* __restrict__ W, co
   return token;
 }
 
-// Folds one row's partials.  Every lane returns the same result.
-__device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int chunks, int chunk_stride, int lane) {
-  Partial q[kPerLane];
-  float m = -INFINITY;
-  int idx = kNoToken;
-#pragma unroll
-  for (int k = 0; k < kPerLane; ++k) {
-    const int j = lane + 32 * k;
-    if (j < chunks) {
-      const float4 raw = __ldcg(reinterpret_cast<const float4*>(p + static_cast<size_t>(j) * chunk_stride));
-      q[k].m = raw.x;
-      q[k].idx = __float_as_int(raw.y);
-      q[k].s = raw.z;
-      q[k].t = raw.w;
-    } else {
-      q[k] = empty_partial();
-    }
-    if (q[k].m > m || (q[k].m == m && q[k].idx < idx)) {
-      m = q[k].m;
-      idx = q[k].idx;
-    }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float om = __shfl_xor_sync(0xffffffffu, m, off);
-    const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
-    if (om > m || (om == m && oi < idx)) {
-      m = om;
-      idx = oi;
-    }
-  }
-  float s = 0.f, t = 0.f;
-#pragma unroll
-  for (int k = 0; k < kPerLane; ++k) {
-    if (!(q[k].s == 0.f)) {           // an empty range contributes nothing; a NaN sum goes through
-      const float dm = q[k].m - m;    // <= 0
-      const float e = exp2f(dm * kLog2e);
-      s += q[k].s * e;
-      t += e * (q[k].t + dm * q[k].s);
-    }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, off);
-    t += __shfl_xor_sync(0xffffffffu, t, off);
-  }
-  Partial r;
-  r.m = m;
-  r.idx = idx;
-  r.s = s;
-  r.t = t;
-  return r;
-}
-
-// Scores and decision of one row from its folded summary; returns the route flag.
-__device__ __forceinline__ int score_row(const Partial& acc, const FinishLaunch& a, int row) {
-  float conf = 1.0f / acc.s;
-  float ent = logf(acc.s) - acc.t / acc.s;
-  const bool finite = (conf == conf) && (ent == ent) && acc.s > 0.f && acc.s < INFINITY;
+// Scores and decision of one row from its folded summary.
+struct Scored {
+  int token, flag;
+  float conf, entropy, learned;
+};
+__device__ __forceinline__ Scored score_row(const Partial& acc, const FinishLaunch& a, int row) {
+  Scored r;
+  r.token = acc.idx;
+  r.conf = 1.0f / acc.s;
+  r.entropy = logf(acc.s) - acc.t / acc.s;
+  const bool finite = (r.conf == r.conf) && (r.entropy == r.entropy) && acc.s > 0.f && acc.s < INFINITY;
   if (finite) {
-    conf = fminf(conf, 1.0f);
-    ent = fmaxf(ent, 0.0f);
+    r.conf = fminf(r.conf, 1.0f);
+    r.entropy = fmaxf(r.entropy, 0.0f);
   } else {
-    conf = __int_as_float(0x7fc00000);   // NaN: fails "conf >= tau", so the row is routed
-    ent = conf;
+    r.conf = __int_as_float(0x7fc00000);   // NaN: fails "conf >= tau", so the row is routed
+    r.entropy = r.conf;
     atomicOr(a.status, TLR_DEV_NONFINITE);
   }
   // "not (conf >= tau)": equals conf < tau for numbers, and routes a NaN row; likewise
   // "not (conf <= tau)" for the opposite polarity.
   const float tau = a.tau_rows != nullptr ? a.tau_rows[row] : a.tau;
-  float score = conf;
+  float score = r.conf;
+  r.learned = 0.f;
   if (a.mlp_partial != nullptr) {
     // learned score: the output layer's partial sums in a fixed order, then the sigmoid
     float v = a.mlp_b2;
+#pragma unroll 8
     for (int b = 0; b < a.mlp_blocks; ++b) v += __ldcg(a.mlp_partial + static_cast<size_t>(row) * a.mlp_blocks + b);
-    const float learned = 1.0f / (1.0f + expf(-v));
-    if (a.mlp_score_out != nullptr) a.mlp_score_out[row] = learned;
-    if (a.decide_on_mlp) score = learned;
+    r.learned = 1.0f / (1.0f + expf(-v));
+    if (a.decide_on_mlp) score = r.learned;
   }
-  const int flag = a.route_above ? ((score <= tau) ? 0 : 1) : ((score >= tau) ? 0 : 1);
-  a.token[row] = acc.idx;
-  a.conf[row] = conf;
-  a.entropy[row] = ent;
-  a.route_mask[row] = static_cast<uint8_t>(flag);
-  return flag;
+  r.flag = a.route_above ? ((score <= tau) ? 0 : 1) : ((score >= tau) ? 0 : 1);
+  return r;
+}
+__device__ __forceinline__ void store_row(const Scored& r, const FinishLaunch& a, int row) {
+  a.token[row] = r.token;
+  a.conf[row] = r.conf;
+  a.entropy[row] = r.entropy;
+  a.route_mask[row] = static_cast<uint8_t>(r.flag);
+  if (a.mlp_partial != nullptr && a.mlp_score_out != nullptr) a.mlp_score_out[row] = r.learned;
 }
 
 // First routed position of every sequence: an atomic minimum per sequence over the
@@ -227,9 +182,10 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
   wait_for_peers(a);
   __shared__ unsigned char flags[kSmallRows];
   const bool single_block = gridDim.x == 1;
+  const int row = group;
+  const bool valid = row < a.n;
+  Scored out;
   {
-    const int row = group;
-    const bool valid = row < a.n;
     const Partial* p = a.partials + static_cast<size_t>(valid ? row : 0) * a.row_stride;
     const size_t cs = static_cast<size_t>(a.chunk_stride);
     float m = -INFINITY;
@@ -317,7 +273,8 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
       acc.idx = idx;
       acc.s = s;
       acc.t = t;
-      const int f = score_row(acc, a, row);
+      out = score_row(acc, a, row);
+      const int f = out.flag;
       if (single_block) {
         flags[row] = static_cast<unsigned char>(f);
       } else {
@@ -336,8 +293,11 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
     // The cluster barrier (release / acquire) makes every block's stores into block 0's shared memory
     // visible to block 0, and keeps block 0 (and its shared memory) there until they have been made.
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
+  // The outputs go out behind the arrival: stores to global memory in front of it would have to be acknowledged by L2
+  // before the release, half a microsecond on every block's way to the compaction.
+  if (valid && gl == 0) store_row(out, a, row);
+  if (!single_block) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (blockIdx.x != 0) return;
   first_routed_init(a);
   const int warps = blockDim.x >> 5;
@@ -378,7 +338,7 @@ finish_kernel(const FinishLaunch a) {
     if (a.tie_W != nullptr)
       acc.idx = settle_ties(a.tie_W, a.tie_h + static_cast<size_t>(row) * a.tie_d, a.tie_d, p, a.chunks, a.chunk_stride,
                             acc.m, acc.idx, lane, 32);
-    if (lane == 0) score_row(acc, a, row);
+    if (lane == 0) store_row(score_row(acc, a, row), a, row);
   }
 
   // ---- which block is last?

@@ -27,17 +27,7 @@ constexpr int kWarps = 8;
 // One warp folds one row's chunk partials; every lane ends with the result.
 __device__ __forceinline__ Partial row_summary(const Partial* __restrict__ partials, int row, int chunks, int v_offset,
                                                int lane) {
-  Partial acc = empty_partial();
-  for (int j = lane; j < chunks; j += 32) {
-    const float4 raw = __ldcg(reinterpret_cast<const float4*>(partials + static_cast<size_t>(row) * chunks + j));
-    Partial q;
-    q.m = raw.x;
-    q.idx = __float_as_int(raw.y);
-    q.s = raw.z;
-    q.t = raw.w;
-    acc = merge(acc, q);
-  }
-  acc = warp_merge(acc);
+  Partial acc = fold_row(partials + static_cast<size_t>(row) * chunks, chunks, 1, lane);
   if (acc.idx != kNoToken) acc.idx += v_offset;
   return acc;
 }
