@@ -387,6 +387,8 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   const int units = (p.chunks + (p.mlp_hidden > 0 ? 1 : 0)) * p.row_units;
   const int T = p.tiles_per_unit;
   const unsigned long long wait_ns = p.wait_limit_ns != 0 ? p.wait_limit_ns : kWaitLimitNs;
+  Partial last = {};               // pair mode: this thread's partial of the worker's last unit
+  Partial* last_dst = nullptr;
 
   if (inl && warp >= 2) {
     // ---- 8-bit head, n <= 16: the nine warps that have nothing to do yet split h into its two e4m3
@@ -718,7 +720,16 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
             const int row = first.row0 + my_row + 8 * i;
             if (!writer || row >= p.n || (i == 1 && !two_tokens)) continue;
             if (mlp_unit) p.mlp_out[row] = out[i].s + other[i].s;   // lower columns first: a fixed order
-            else p.partials[static_cast<size_t>(row) * p.chunks + first.chunk] = merge(out[i], other[i]);
+            else {
+              Partial* dst = p.partials + static_cast<size_t>(row) * p.chunks + first.chunk;
+              const Partial sum = merge(out[i], other[i]);
+              if (kCta == 2 && unit + workers >= units) {     // (stored behind the arrival at the cluster's barrier)
+                last = sum;
+                last_dst = dst;
+              } else {
+                *dst = sum;
+              }
+            }
           }
         }
       }
@@ -726,8 +737,16 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   }
 
   tc_fence_before();
-  __syncthreads();
-  if (kCta == 2) cluster_sync_all();   // neither CTA frees TMEM or exits while the peer still works
+  if (kCta == 2) {
+    // Neither CTA frees TMEM or exits while the peer still works.  The last partials go out behind the arrival: in front
+    // of it the release would wait until L2 has acknowledged them, 0.7 us at the end of every launch.
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (last_dst != nullptr) *last_dst = last;
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc<kCta>(tmem_base, kTmemCols);
