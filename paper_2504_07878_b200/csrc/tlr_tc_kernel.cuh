@@ -737,15 +737,13 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   }
 
   tc_fence_before();
+  __syncthreads();      // (here also for the warps with nothing to do: waiting at the cluster's barrier takes issue slots)
   if (kCta == 2) {
     // Neither CTA frees TMEM or exits while the peer still works.  The last partials go out behind the arrival: in front
     // of it the release would wait until L2 has acknowledged them, 0.7 us at the end of every launch.
-    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     if (last_dst != nullptr) *last_dst = last;
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  } else {
-    __syncthreads();
   }
   if (warp == 1) {
     tc_fence_after();
