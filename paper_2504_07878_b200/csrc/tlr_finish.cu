@@ -9,9 +9,8 @@
 //
 // Compaction (ballot / popcount / prefix sum, ascending order):
 //   n <= 1024  a thread-block cluster of up to 8 blocks folds the rows (a group of L lanes
-//              per row, all rows at once) and store the route flags into block 0's shared memory;
-//              after a cluster barrier block 0 compacts them.  No ticket, no second launch, one L2
-//              round trip for the partials.  The blocks
+//              per row, all rows at once) and sends the route flags to block 0, which compacts
+//              them.  No ticket, no second launch, one L2 round trip for the partials.  The blocks
 //              have 512 threads where a lane group still owns at most 6 partials (else 1024):
 //              that size fits on an SM beside a CTA of the tensor-core projection kernel, so
 //              the blocks are resident and waiting before that kernel ends, and the next
@@ -88,6 +87,7 @@ __device__ __forceinline__ Scored score_row(const Partial& acc, const FinishLaun
     r.conf = __int_as_float(0x7fc00000);   // NaN: fails "conf >= tau", so the row is routed
     r.entropy = r.conf;
     atomicOr(a.status, TLR_DEV_NONFINITE);
+    __threadfence();                       // before this row's flag reaches the block that copies the status word
   }
   // "not (conf >= tau)": equals conf < tau for numbers, and routes a NaN row; likewise
   // "not (conf <= tau)" for the opposite polarity.
@@ -162,6 +162,29 @@ __device__ __forceinline__ void wait_for_peers(const FinishLaunch& a) {
   __syncthreads();
 }
 
+// Block 0 of the cluster waits until every warp's word has arrived (bounded like every wait; after a time-out the status
+// word says that the index list is not to be trusted).
+__device__ __forceinline__ void wait_for_words(uint32_t bar, uint32_t* status) {
+  unsigned long long t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar) : "memory");
+    if (ok) return;
+    if ((it & 63u) == 63u) {
+      unsigned long long t;
+      asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+      if (t0 == 0) t0 = t;
+      if (t - t0 > 2000000000ull) {
+        atomicOr(status, TLR_DEV_WAIT_TIMEOUT);
+        return;
+      }
+    }
+  }
+}
+
 // Cluster of gridDim.x blocks, n <= 1024.  A group of L lanes (L a power of two) folds one
 // row in two passes over its partials: maximum and index first, then the sums rescaled to
 // that maximum.  L is chosen on the host so that every row has its group: n * L <=
@@ -178,10 +201,25 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
   const int group = (blockIdx.x * blockDim.x + threadIdx.x) >> log2_L;
   const int gl = threadIdx.x & (L - 1);
   const bool one_pass = ((a.chunks + L - 1) >> log2_L) <= kPerLane;
+  // Every warp of the cluster sends the flags of its 32 / L rows -- bit r * L for its row r -- as one word to block 0,
+  // which waits for all words on a barrier of its own.  (st.async delivers the word and its arrival in one trip: n = 64, d = 512, V = 32000 11.90 us per step; flag
+  // bytes in distributed shared memory with a cluster barrier behind them 12.96; n = 256 14.61 and 15.55.)
+  __shared__ uint32_t flag_words[kSmallRows / 4];     // at most 8 blocks x 32 warps
+  __shared__ __align__(8) unsigned long long all_here;
+  const bool single_block = gridDim.x == 1;
+  const int warps = blockDim.x >> 5;
+  const uint32_t bar = static_cast<uint32_t>(__cvta_generic_to_shared(&all_here));
+  if (!single_block) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(gridDim.x * warps * 4u) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
   pdl_enter();
   wait_for_peers(a);
-  __shared__ unsigned char flags[kSmallRows];
-  const bool single_block = gridDim.x == 1;
   const int row = group;
   const bool valid = row < a.n;
   Scored out;
@@ -274,37 +312,31 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
       acc.s = s;
       acc.t = t;
       out = score_row(acc, a, row);
-      const int f = out.flag;
-      if (single_block) {
-        flags[row] = static_cast<unsigned char>(f);
-      } else {
-        // into block 0's shared memory (distributed shared memory of the cluster): block 0 then compacts
-        // without another trip to L2 for the flags
-        const uint32_t mine = static_cast<uint32_t>(__cvta_generic_to_shared(&flags[row]));
-        uint32_t remote;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(0));
-        asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(remote), "r"(f) : "memory");
-      }
     }
   }
-  if (single_block) {
-    __syncthreads();                    // the flags are in this block's shared memory
-  } else {
-    // The cluster barrier (release / acquire) makes every block's stores into block 0's shared memory
-    // visible to block 0, and keeps block 0 (and its shared memory) there until they have been made.
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  const uint32_t word = __ballot_sync(0xffffffffu, valid && gl == 0 && out.flag != 0);
+  if (lane == 0) {
+    if (single_block) {
+      flag_words[warp] = word;
+    } else {
+      const uint32_t mine = static_cast<uint32_t>(__cvta_generic_to_shared(&flag_words[blockIdx.x * warps + warp]));
+      uint32_t remote, remote_bar;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(0));
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote_bar) : "r"(bar), "r"(0));
+      asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                   ::"r"(remote), "r"(word), "r"(remote_bar) : "memory");
+    }
   }
-  // The outputs go out behind the arrival: stores to global memory in front of it would have to be acknowledged by L2
-  // before the release, half a microsecond on every block's way to the compaction.
   if (valid && gl == 0) store_row(out, a, row);
-  if (!single_block) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (blockIdx.x != 0) return;
+  if (single_block) __syncthreads();
+  else wait_for_words(bar, a.status);
   first_routed_init(a);
-  const int warps = blockDim.x >> 5;
+  const int log2_rpw = 5 - log2_L;          // rows per warp
   int base_out = 0;
   for (int base = 0; base < a.n; base += blockDim.x) {       // one pass when the block has a thread per row
     const int i = base + threadIdx.x;
-    const int flag = i < a.n ? static_cast<int>(flags[i]) : 0;
+    const int flag = i < a.n ? (flag_words[i >> log2_rpw] >> ((i & ((1 << log2_rpw) - 1)) << log2_L)) & 1u : 0;
     const unsigned int bal = __ballot_sync(0xffffffffu, flag != 0);
     if (lane == 0) warp_count[warp] = __popc(bal);
     __syncthreads();
