@@ -440,8 +440,10 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
   return TLR_OK;
 }
 
-// Enqueues the projection kernel of a call with n > 0 rows: chunk partials into ctx->partials.
-tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ctx::Step* st, cudaStream_t stream) {
+// Enqueues the projection kernel of a call with n > 0 rows: chunk partials into ctx->partials.  router_beside: the 8-bit
+// head's router kernel follows (launch_mlp_beside).
+tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ctx::Step* st, cudaStream_t stream,
+                             bool router_beside = false) {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   if (ctx->timing && ctx->timed < tlr::kMaxTimedLaunches) {
     const size_t need = 2 * static_cast<size_t>(ctx->timed + 1);
@@ -465,6 +467,7 @@ tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ct
       st->h_mapped = ctx->h_parts;
     }
     st->params.h = h_bf16_dev;
+    st->params.late_trigger = router_beside ? 1 : 0;
     e = tlr::launch_tc8_projection(st->maps, st->params, cfg, st->workers, stream);
   } else if (st->plan.path == TLR_PATH_TC && ctx->classes > 1) {
     const int units_max = ctx->sm_count / st->cfg.cta;
@@ -765,8 +768,9 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   tlr_ctx::Step* st = step_for(ctx, n, mlp_inside);
   const tlr_plan& plan = st->plan;
 
+  const bool router_beside = want_mlp && ctx->fp8 && (reinterpret_cast<uintptr_t>(ctx->mlp_W1) & 15u) == 0;
   if (n > 0) {
-    const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream);
+    const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, router_beside);
     if (ps != TLR_OK) return ps;
   }
 
@@ -781,8 +785,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
     m.d = ctx->d;
     m.d_hidden = ctx->mlp_hidden;
     m.partial = ctx->mlp_scores;
-    const bool beside = ctx->fp8 && (reinterpret_cast<uintptr_t>(m.W1) & 15u) == 0;
-    if ((beside ? tlr::launch_mlp_beside(m, stream) : tlr::launch_mlp_score(m, stream)) != cudaSuccess)
+    if ((router_beside ? tlr::launch_mlp_beside(m, stream) : tlr::launch_mlp_score(m, stream)) != cudaSuccess)
       return TLR_ERR_CUDA;
   }
 

@@ -42,6 +42,7 @@ struct TcParams {
   int debug_drop_w_copies;            // test hook: the W producer issues no copies
   int w_wait;                         // 1: W may have been written by the previous kernel in the stream, so the
                                       // W producer waits for it too (entry points that take W per call)
+  int late_trigger;                   // 1: the next kernel may be scheduled only behind this one's own wait
   // learned router inside the launch (bf16 head): one extra unit per row unit over the rows of W1
   int mlp_hidden;                     // hidden width, 0 = no learned router in this launch
   int mlp_rows;                       // hidden width rounded up to the granule
