@@ -370,8 +370,8 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   // that take W per call set w_wait).  It also lets the next kernel go ahead at once: done only behind
   // the wait, a step of n = 16, d = 896, V = 151936 takes 48.3 us in a stream instead of 47.1.  A kernel that reads
   // h without waiting for this one (mlp_mma_kernel) needs it behind the wait, though.
-  if (warp != 0 || p.w_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (warp != 0 || !p.late_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if ((warp != 0 && warp != 6) || inl || p.w_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if ((warp != 0 && warp != 6) || !p.late_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // With at most 64 operand rows (one CTA per worker) the MMAs run with M = 64: such an instruction takes
   // about two thirds of the time of an M = 128 one, and the padding rows were wasted work anyway.  Its
@@ -452,12 +452,20 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       int stage = 0;
       int slab = 0;
       bool ok = true;
+      bool h_there = false;
       for (int unit = worker; unit < units && ok; unit += workers) {
         const Unit un = unit_of<kCta, kOdd>(p, unit, cta_rank);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
           for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
+            if (!h_there) {
+              // here and not with the other warps above: the arithmetic of the first unit, two 64-bit divisions among it,
+              // would stand between the end of the wait and the first load of h, which the whole step waits for (n = 1,
+              // d = 256, V = 20000 9.43 -> 9.03 us per step in a stream, n = 256, d = 512, V = 32000 15.49 -> 14.86)
+              asm volatile("griddepcontrol.wait;" ::: "memory");
+              h_there = true;
+            }
             if (slab >= SA) {
               const int j = slab - SA;
               if (!mbar_wait(released(j & (kRelease - 1)), (j / kRelease) & 1, abort_flag, p.status, wait_ns)) { ok = false; break; }
