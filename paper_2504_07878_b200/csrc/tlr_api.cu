@@ -330,7 +330,7 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
       p.class_chunks = tp.chunks / c->classes;
       p.h_class_rows = c->odd_rows;
       for (int r = 0; r < c->classes; ++r) st->odd.w[r] = c->map_cls[r];
-      if (n > 0) make_map(c, &st->odd.h, c->h_shift, c->classes * c->odd_rows, c->odd_pitch, cfg.a_rows);
+      if (n > 0) make_map(c, &st->odd.h, c->h_shift, c->classes * c->odd_rows, c->odd_pitch, tlr::tc_h_box_rows(cfg));
       return;
     }
     st->maps.w128 = c->map_w128;
@@ -491,7 +491,7 @@ tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ct
       const CUtensorMap was_map = st->maps.h;
       if (st->h_other == h_bf16_dev && h_bf16_dev != nullptr) {
         st->maps.h = st->h_other_map;
-      } else if (!make_map(ctx, &st->maps.h, h_bf16_dev, n, ctx->d, st->cfg.a_rows)) {
+      } else if (!make_map(ctx, &st->maps.h, h_bf16_dev, n, ctx->d, tlr::tc_h_box_rows(st->cfg))) {
         st->h_mapped = nullptr;
         return TLR_ERR_CUDA;
       }

@@ -71,10 +71,12 @@ cudaError_t launch_odd_shift(const void* h_bf16, int n, int d, int class_rows, i
 }
 
 cudaError_t odd_prepare() {
-  const cudaError_t e = cudaFuncSetAttribute(odd_projection_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kSmemLimit);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(odd_projection_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+  for (const auto kernel :
+       {odd_projection_kernel<1, false>, odd_projection_kernel<1, true>, odd_projection_kernel<2, false>}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const TcConfig& c, int workers,
@@ -93,8 +95,9 @@ cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const 
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = c.cta == 1 ? 1 : 2;
-  return c.cta == 1 ? cudaLaunchKernelEx(&cfg, odd_projection_kernel<1>, maps, p)
-                    : cudaLaunchKernelEx(&cfg, odd_projection_kernel<2>, maps, p);
+  const auto kernel = c.cta == 2 ? odd_projection_kernel<2, false>
+                                 : (c.group8 ? odd_projection_kernel<1, true> : odd_projection_kernel<1, false>);
+  return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 
 }  // namespace tlr

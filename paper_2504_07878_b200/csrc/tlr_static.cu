@@ -139,7 +139,7 @@ extern "C" tlr_status tlr_route_static(int32_t d, int32_t V, const void* W_bf16_
     chunks = tp.chunks;
     const int units = tp.chunks * tp.row_units;
     workers = units < workers_max ? units : workers_max;
-    if (!encode_map(&maps.h, h_bf16_dev, n, d, cfg.a_rows) || !encode_map(&maps.w128, W_bf16_dev, V, d, 128) ||
+    if (!encode_map(&maps.h, h_bf16_dev, n, d, tlr::tc_h_box_rows(cfg)) || !encode_map(&maps.w128, W_bf16_dev, V, d, 128) ||
         !encode_map(&maps.w64, W_bf16_dev, V, d, 64) || !encode_map(&maps.w16, W_bf16_dev, V, d, 16))
       return TLR_ERR_CUDA;
     maps.m128 = maps.w128;
@@ -165,7 +165,7 @@ extern "C" tlr_status tlr_route_static(int32_t d, int32_t V, const void* W_bf16_
       p.full_tiles_first = tp.full_tiles_first;
       p.granule_rows = tp.granule_rows;
       p.a_rows = cfg.a_rows;
-      p.part_rows = cfg.part_rows;
+        p.part_rows = cfg.part_rows;
       p.a_stages = cfg.a_stages;
       p.b_stages = cfg.b_stages;
       // W is an argument of this call, so the kernel that precedes it in the stream may have written it:

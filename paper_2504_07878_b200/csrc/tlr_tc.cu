@@ -44,10 +44,18 @@ int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int ca
 void tc_configure(int n, TcConfig* c) {
   const int cta = n > kBlockM ? 2 : 1;
   int a_rows = kBlockM;
+  int group8 = 0;
   if (cta == 1) {
     a_rows = ((n + 15) / 16) * 16;
     if (a_rows < 16) a_rows = 16;
     if (a_rows > kBlockM) a_rows = kBlockM;
+    // Up to 16 token rows lie eight to every sixteen operand rows, so that two of the accumulator's lane quadrants have
+    // rows and the epilogue reads them with four threads to a row.  In a stream, one thread per row and this: d = 512,
+    // V = 32000 n = 1 11.26 and 10.55 us per step, n = 16 11.65 and 10.83; d = 2048, V = 128256 n = 16 88.7 and 86.
+    // With four such groups the loads of h, eight rows each, cost more than that: n = 32 11.70 and 11.74, 89.6 and
+    // 94.9; with two rows per thread n = 64 12.25 and 12.40.
+    group8 = n <= 16 ? 1 : 0;
+    if (group8) a_rows = n <= 8 ? 16 : 32;
   }
   const int a_stage = a_rows * kRowBytes;
   const int b_stage = (kBlockN / cta) * kRowBytes;
@@ -69,6 +77,7 @@ void tc_configure(int n, TcConfig* c) {
   }
   c->cta = cta;
   c->a_rows = a_rows;
+  c->group8 = group8;
   c->part_rows = a_rows;
   c->a_stages = sa;
   c->b_stages = sb;
@@ -77,10 +86,11 @@ void tc_configure(int n, TcConfig* c) {
 }
 
 cudaError_t tc_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(tc_projection_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSmemLimit);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(tc_projection_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+  for (const auto kernel : {tc_projection_kernel<1, false>, tc_projection_kernel<1, true>, tc_projection_kernel<2, false>}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const TcConfig& c, int workers,
@@ -98,12 +108,10 @@ cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const Tc
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  if (c.cta == 1) {
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tc_projection_kernel<1>, maps, p);
-  }
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, tc_projection_kernel<2>, maps, p);
+  cfg.numAttrs = c.cta == 1 ? 1 : 2;
+  const auto kernel = c.cta == 2 ? tc_projection_kernel<2, false>
+                                 : (c.group8 ? tc_projection_kernel<1, true> : tc_projection_kernel<1, false>);
+  return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 
 }  // namespace tlr

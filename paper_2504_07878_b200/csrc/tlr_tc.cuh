@@ -11,6 +11,7 @@ namespace tlr {
 struct TcConfig {
   int cta;          // 1: one CTA per worker (n <= 128); 2: a pair of CTAs per worker
   int a_rows;       // rows of an h slab held in shared memory (16..128); on the 8-bit head both parts of h stacked
+  int group8;       // 1: up to 16 token rows of a bf16 head, eight in every sixteen operand rows (the others unused)
   int part_rows;    // 8-bit head: rows of one part (a_rows / 2); otherwise a_rows
   int a_stages;     // depth of the h ring
   int b_stages;     // depth of the W ring
@@ -83,6 +84,7 @@ cudaError_t odd_prepare();
 cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const TcConfig& c, int workers,
                                   cudaStream_t stream);
 
+inline int tc_h_box_rows(const TcConfig& c) { return c.group8 ? 8 : c.a_rows; }   // rows of h per TMA box
 int tc_threads();
 int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
 void tc_configure(int n, TcConfig* c);

@@ -115,6 +115,7 @@ void tc8_configure(int n, int d, TcConfig* c) {
   if (sb > kMaxBStages) sb = kMaxBStages;
   c->cta = 1;
   c->a_rows = 2 * part_rows;
+  c->group8 = 0;
   c->part_rows = part_rows;
   c->a_stages = sa;
   c->b_stages = sb;

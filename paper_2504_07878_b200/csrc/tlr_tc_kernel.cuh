@@ -307,10 +307,11 @@ __device__ __forceinline__ Partial quad_merge(const Partial& p) {
 
 // The kernel body (maps and p are the kernel's own parameters, maps a __grid_constant__ one: TMA reads the
 // tensor maps from parameter space).
-template <int kCta, bool kFp8, class Maps>
+template <int kCta, bool kFp8, bool kGroup8, class Maps>
 __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcParams& p) {
   constexpr bool kOdd = std::is_same<Maps, OddMaps>::value;   // d no multiple of 8: vocabulary rows by residue class
   static_assert(!(kFp8 && kCta != 1), "the 8-bit head runs with one CTA per worker");
+  static_assert(!(kGroup8 && (kFp8 || kCta != 1)), "kGroup8 is the bf16 head's mode for up to 16 rows");
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment: the swizzle pattern is a function of the shared-memory address.
   // (The dynamic shared memory of both CTAs of a pair starts at the same offset, so the
@@ -397,7 +398,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   // about two thirds of the time of an M = 128 one, and the padding rows were wasted work anyway.  Its
   // accumulator row r lives in TMEM lane 32 * (r / 16) + r % 16, i.e. in lanes 0..15 of each 32-lane
   // quadrant (checked on the device), so an epilogue warp then holds 16 rows instead of 32.
-  const bool m64 = kCta == 1 && p.a_rows <= 64;
+  const bool m64 = kCta == 1 && (kGroup8 || p.a_rows <= 64);
   // 8-bit head with more than 64 token rows: the two parts of h no longer fit one MMA's M (128 at most with one
   // CTA), so every K step issues two MMAs -- first parts, then second parts, into the same accumulator rows --
   // and the epilogue reads finished logits as on the bf16 head (no hand-over between warps).
@@ -492,9 +493,15 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
             }
             const uint32_t dst = a_ring + stage * a_stage_bytes;
             const uint32_t bar = (kCta == 2) ? map_to_cta(a_full(stage), 0) : a_full(stage);
-            if (leader) mbar_expect_tx(a_full(stage), a_stage_bytes * kCta);
-            tma_load_2d<kCta>(dst, &maps.h, bar, ks * kSlabElems,
-                              kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0));
+            const int h_row = kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0);
+            if (kGroup8) {      // boxes of eight rows, sixteen operand rows apart
+              mbar_expect_tx(a_full(stage), a_stage_bytes >> 1);
+              for (int r = 0; r < p.a_rows; r += 16)
+                tma_load_2d<kCta>(dst + r * kRowBytes, &maps.h, bar, ks * kSlabElems, h_row + (r >> 1));
+            } else {
+              if (leader) mbar_expect_tx(a_full(stage), a_stage_bytes * kCta);
+              tma_load_2d<kCta>(dst, &maps.h, bar, ks * kSlabElems, h_row);
+            }
             if (++stage == SA) stage = 0;
           }
         }
@@ -578,12 +585,13 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
     // ------------------------------------------------------------------ epilogue (warps 2-5, 7-10)
     const int grp = warp >= 7 ? 1 : 0;       // 0: lower half of a tile's columns, 1: upper half
     const int quad = warp & 3;               // TMEM lane quadrant this warp may read
-    // 8-bit head up to 64 token rows: the accumulator is read in the fragment layout (tmem_ld16x64), 16 lanes at a
-    // time.  Of those, lanes 0..7 are the first parts of eight tokens and lanes 8..15 their second parts
-    // (tc8_part_row), so the thread that holds a token's first part holds its second part too and adds them; four
-    // threads share a token's columns, and all 32 work.  With M = 64 a quadrant has one such group of 16 lanes, with
-    // M = 128 two, and a thread then keeps two tokens, eight apart.
-    const bool frag = kFp8 && !wide;
+    // Fragment layout (tmem_ld16x64: 16 lanes at a time, four threads to a lane): the 8-bit head up to 64 token rows, the
+    // bf16 head up to 16.  Four threads share a token's columns, and all 32 work.
+    // 8-bit head: of the 16 lanes, 0..7 are the first parts of eight tokens and 8..15 their second parts
+    // (tc8_part_row), so the thread that holds a token's first part holds its second part too and adds them.  With
+    // M = 64 a quadrant has one such group of 16 lanes, with M = 128 two, and a thread then keeps two tokens, eight apart.
+    // bf16 head: lanes 0..7 are tokens, 8..15 unused (TcConfig::group8).
+    const bool frag = kFp8 ? !wide : kGroup8;
     constexpr int kFolds = kFp8 ? 2 : 1;           // tokens a thread may keep
     const int quad_rows = frag ? (m64 ? 8 : 16) : (m64 ? 16 : 32);     // token rows per quadrant
     const int quad_row0 = quad * quad_rows;
@@ -657,9 +665,21 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
                 float z[16];
 #pragma unroll
                 for (int b = 0; b < 8; ++b) {
-                  const float2 w2 = *reinterpret_cast<const float2*>(ws + (c_mine - c_begin) + 8 * b);
-                  z[2 * b] = (x[i][4 * b] + x[i][4 * b + 2]) * hs[i] * w2.x;
-                  z[2 * b + 1] = (x[i][4 * b + 1] + x[i][4 * b + 3]) * hs[i] * w2.y;
+                  z[2 * b] = x[i][4 * b];
+                  z[2 * b + 1] = x[i][4 * b + 1];
+                  if (kFp8) {
+                    const float2 w2 = *reinterpret_cast<const float2*>(ws + (c_mine - c_begin) + 8 * b);
+                    z[2 * b] = (z[2 * b] + x[i][4 * b + 2]) * hs[i] * w2.x;
+                    z[2 * b + 1] = (z[2 * b + 1] + x[i][4 * b + 3]) * hs[i] * w2.y;
+                  }
+                }
+                if constexpr (kRouter) {
+#pragma unroll
+                  for (int k = 0; k < 16; ++k) {
+                    const int o = 8 * (k >> 1) + (k & 1), u = v0 + c_mine + o;
+                    if (o < valid) mlp_sum += __ldg(p.mlp_w2 + u) * fmaxf(z[k] + __ldg(p.mlp_b1 + u), 0.f);
+                  }
+                  continue;
                 }
                 if (valid < 58) {                     // (the last of the columns is c_mine + 57)
 #pragma unroll
@@ -720,7 +740,13 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
           out[i] = quad_merge(out[i]);
         }
       }
-      if (mlp_unit) out[0].s = mlp_sum;
+      if (mlp_unit) {
+        if (frag) {
+          mlp_sum += __shfl_xor_sync(0xffffffffu, mlp_sum, 1);
+          mlp_sum += __shfl_xor_sync(0xffffffffu, mlp_sum, 2);
+        }
+        out[0].s = mlp_sum;
+      }
       // The second group hands its summary to the first through the scratch block (bounded
       // waits on both sides: a warp that gave up never leaves its partner waiting forever).
       if (grp == 1) {
@@ -778,18 +804,20 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
 }
 
 // bf16 head: one CTA per worker (kCta = 1) or a pair (kCta = 2).
-template <int kCta>
+// kGroup8: up to 16 rows (TcConfig::group8) -- a kernel of its own, because the other row counts lose 1.5 % to a switch at
+// run time (n = 24, d = 512, V = 32000 11.60 and 11.82 us).
+template <int kCta, bool kGroup8>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_projection_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
-  tc_projection_body<kCta, false>(maps, p);
+  tc_projection_body<kCta, false, kGroup8>(maps, p);
 }
 
 // d no multiple of 8 (defined in the one file that launches them).
 #ifdef TLR_DEFINE_ODD_KERNELS
-template <int kCta>
+template <int kCta, bool kGroup8>
 __global__ void __launch_bounds__(kThreads, 1)
 odd_projection_kernel(const __grid_constant__ OddMaps maps, const TcParams p) {
-  tc_projection_body<kCta, false>(maps, p);
+  tc_projection_body<kCta, false, kGroup8>(maps, p);
 }
 #endif
 
@@ -798,7 +826,7 @@ odd_projection_kernel(const __grid_constant__ OddMaps maps, const TcParams p) {
 #ifdef TLR_DEFINE_TC8_KERNEL
 __global__ void __maxnreg__(128)
 tc8_projection_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
-  tc_projection_body<1, true>(maps, p);
+  tc_projection_body<1, true, false>(maps, p);
 }
 #endif
 

@@ -314,3 +314,30 @@ def test_prepared_call_is_the_same_step(pkg):
     with pytest.raises(ValueError):
         r.prepared(h.float(), 0.4)
     r.close()
+
+
+# Small batches on the tensor cores: token rows at the edges of the groups of eight, vocabularies that end inside a
+# thread's columns or a group's half of a tile, with the learned router's units in the same launch.
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 15, 16, 17])
+@pytest.mark.parametrize("V", [1, 3, 57, 58, 130, 2500])
+def test_small_batches_at_the_edges_of_the_fragment_layout(pkg, n, V):
+    d, dh = 72, 37
+    W = S.make_W(d, V, seed=n + V, std=0.15)
+    hid = S.make_h(n, d, seed=V)
+    ref = O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W), 0.5)
+    gpu = run_gpu(pkg, W.cuda(), hid.h, 0.5)
+    assert gpu["status"] == 0 and gpu["plan"].path == 2
+    check_self_consistency(gpu, 0.5, V)
+    check_against_oracle(ref, gpu, O.bf16_bits_to_f64(S.bf16_bits(hid.h)), O.bf16_bits_to_f64(S.bf16_bits(W)))
+    g = torch.Generator().manual_seed(n)
+    W1 = (torch.randn(dh, d, generator=g) / d ** 0.5).to(torch.bfloat16)
+    b1, w2 = torch.randn(dh, generator=g) * 0.1, torch.randn(dh, generator=g) * 0.5
+    want = O.mlp_router_score(S.bf16_bits(hid.h), S.bf16_bits(W1), b1.numpy(), w2.numpy(), 0.2)
+    r = pkg.Router(W.cuda(), max_n=n)
+    r.set_router_mlp(W1.cuda(), b1.cuda(), w2.cuda(), 0.2)
+    score = torch.full((n,), float("nan"), device="cuda")
+    r.route(hid.h.cuda(), 0.5, mlp_score=score)
+    torch.cuda.synchronize()
+    assert np.max(np.abs(score.cpu().numpy() - want)) <= 1e-5     # fp32 sums of exact products
+    assert np.array_equal(r.token[:n].cpu().numpy(), gpu["token"])
+    r.close()
