@@ -44,7 +44,7 @@ int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int ca
 void tc_configure(int n, TcConfig* c) {
   const int cta = n > kBlockM ? 2 : 1;
   int a_rows = kBlockM;
-  int group8 = 0;
+  RowMode mode = RowMode::kM128;
   if (cta == 1) {
     a_rows = ((n + 15) / 16) * 16;
     if (a_rows < 16) a_rows = 16;
@@ -54,8 +54,11 @@ void tc_configure(int n, TcConfig* c) {
     // V = 32000 n = 1 11.26 and 10.55 us per step, n = 16 11.65 and 10.83; d = 2048, V = 128256 n = 16 88.7 and 86.
     // With four such groups the loads of h, eight rows each, cost more than that: n = 32 11.70 and 11.74, 89.6 and
     // 94.9; with two rows per thread n = 64 12.25 and 12.40.
-    group8 = n <= 16 ? 1 : 0;
-    if (group8) a_rows = n <= 8 ? 16 : 32;
+    if (a_rows <= 64) mode = RowMode::kM64;
+    if (n <= 16) {
+      mode = RowMode::kGroup8;
+      a_rows = n <= 8 ? 16 : 32;
+    }
   }
   const int a_stage = a_rows * kRowBytes;
   const int b_stage = (kBlockN / cta) * kRowBytes;
@@ -77,7 +80,7 @@ void tc_configure(int n, TcConfig* c) {
   }
   c->cta = cta;
   c->a_rows = a_rows;
-  c->group8 = group8;
+  c->mode = mode;
   c->part_rows = a_rows;
   c->a_stages = sa;
   c->b_stages = sb;
@@ -86,7 +89,8 @@ void tc_configure(int n, TcConfig* c) {
 }
 
 cudaError_t tc_prepare() {
-  for (const auto kernel : {tc_projection_kernel<1, false>, tc_projection_kernel<1, true>, tc_projection_kernel<2, false>}) {
+  for (const auto kernel : {tc_projection_kernel<1, RowMode::kM128>, tc_projection_kernel<1, RowMode::kM64>,
+                            tc_projection_kernel<1, RowMode::kGroup8>, tc_projection_kernel<2, RowMode::kM128>}) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
   }
@@ -109,8 +113,10 @@ cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const Tc
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = c.cta == 1 ? 1 : 2;
-  const auto kernel = c.cta == 2 ? tc_projection_kernel<2, false>
-                                 : (c.group8 ? tc_projection_kernel<1, true> : tc_projection_kernel<1, false>);
+  const auto kernel = c.cta == 2                    ? tc_projection_kernel<2, RowMode::kM128>
+                      : c.mode == RowMode::kGroup8 ? tc_projection_kernel<1, RowMode::kGroup8>
+                      : c.mode == RowMode::kM64    ? tc_projection_kernel<1, RowMode::kM64>
+                                                   : tc_projection_kernel<1, RowMode::kM128>;
   return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 

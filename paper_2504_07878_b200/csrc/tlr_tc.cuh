@@ -7,11 +7,21 @@
 
 namespace tlr {
 
+// How a projection kernel handles token rows.
+enum class RowMode : int {
+  kM128,      // bf16 head, more than 64 rows: MMA M = 128 (256 on a pair), one epilogue thread per row
+  kM64,       // bf16 head, 17..64 rows: M = 64, one thread per row
+  kGroup8,    // bf16 head, up to 16 rows: M = 64, eight rows in every sixteen operand rows, four threads per row
+  k8Small,    // 8-bit head, up to 32 rows: both parts through one MMA with M = 64, four threads per row
+  k8Half,     // 8-bit head, 33..64 rows: M = 128, four threads per two rows
+  k8Wide,     // 8-bit head, more than 64 rows: an MMA per part, M = 128, one thread per row
+};
+
 // Kernel shape for a given n (see tc_configure / tc8_configure).
 struct TcConfig {
   int cta;          // 1: one CTA per worker (n <= 128); 2: a pair of CTAs per worker
   int a_rows;       // rows of an h slab held in shared memory (16..128); on the 8-bit head both parts of h stacked
-  int group8;       // 1: up to 16 token rows of a bf16 head, eight in every sixteen operand rows (the others unused)
+  RowMode mode;
   int part_rows;    // 8-bit head: rows of one part (a_rows / 2); otherwise a_rows
   int a_stages;     // depth of the h ring
   int b_stages;     // depth of the W ring
@@ -84,7 +94,7 @@ cudaError_t odd_prepare();
 cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const TcConfig& c, int workers,
                                   cudaStream_t stream);
 
-inline int tc_h_box_rows(const TcConfig& c) { return c.group8 ? 8 : c.a_rows; }   // rows of h per TMA box
+inline int tc_h_box_rows(const TcConfig& c) { return c.mode == RowMode::kGroup8 ? 8 : c.a_rows; }   // rows of h per TMA box
 int tc_threads();
 int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
 void tc_configure(int n, TcConfig* c);

@@ -115,7 +115,7 @@ void tc8_configure(int n, int d, TcConfig* c) {
   if (sb > kMaxBStages) sb = kMaxBStages;
   c->cta = 1;
   c->a_rows = 2 * part_rows;
-  c->group8 = 0;
+  c->mode = part_rows <= 32 ? RowMode::k8Small : (part_rows <= 64 ? RowMode::k8Half : RowMode::k8Wide);
   c->part_rows = part_rows;
   c->a_stages = sa;
   c->b_stages = sb;
@@ -124,7 +124,12 @@ void tc8_configure(int n, int d, TcConfig* c) {
 }
 
 cudaError_t tc8_prepare() {
-  return cudaFuncSetAttribute(tc8_projection_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+  for (const auto kernel : {tc8_projection_kernel<RowMode::k8Small>, tc8_projection_kernel<RowMode::k8Half>,
+                            tc8_projection_kernel<RowMode::k8Wide>}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_h_split(const void* h_bf16, int n, int d, int part_rows, uint8_t* parts, float* hscale,
@@ -154,7 +159,10 @@ cudaError_t launch_tc8_projection(const TcMaps& maps, const TcParams& p, const T
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tc8_projection_kernel, maps, p);
+  const auto kernel = c.mode == RowMode::k8Small  ? tc8_projection_kernel<RowMode::k8Small>
+                      : c.mode == RowMode::k8Half ? tc8_projection_kernel<RowMode::k8Half>
+                                                  : tc8_projection_kernel<RowMode::k8Wide>;
+  return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 
 }  // namespace tlr

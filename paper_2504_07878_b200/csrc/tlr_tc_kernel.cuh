@@ -307,11 +307,11 @@ __device__ __forceinline__ Partial quad_merge(const Partial& p) {
 
 // The kernel body (maps and p are the kernel's own parameters, maps a __grid_constant__ one: TMA reads the
 // tensor maps from parameter space).
-template <int kCta, bool kFp8, bool kGroup8, class Maps>
+template <int kCta, RowMode kMode, class Maps>
 __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcParams& p) {
   constexpr bool kOdd = std::is_same<Maps, OddMaps>::value;   // d no multiple of 8: vocabulary rows by residue class
-  static_assert(!(kFp8 && kCta != 1), "the 8-bit head runs with one CTA per worker");
-  static_assert(!(kGroup8 && (kFp8 || kCta != 1)), "kGroup8 is the bf16 head's mode for up to 16 rows");
+  constexpr bool kFp8 = kMode >= RowMode::k8Small, kGroup8 = kMode == RowMode::kGroup8;
+  static_assert(kCta == 1 || kMode == RowMode::kM128, "a pair of CTAs runs the plain mode of the bf16 head");
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment: the swizzle pattern is a function of the shared-memory address.
   // (The dynamic shared memory of both CTAs of a pair starts at the same offset, so the
@@ -398,11 +398,11 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   // about two thirds of the time of an M = 128 one, and the padding rows were wasted work anyway.  Its
   // accumulator row r lives in TMEM lane 32 * (r / 16) + r % 16, i.e. in lanes 0..15 of each 32-lane
   // quadrant (checked on the device), so an epilogue warp then holds 16 rows instead of 32.
-  const bool m64 = kCta == 1 && (kGroup8 || p.a_rows <= 64);
+  constexpr bool m64 = kGroup8 || kMode == RowMode::kM64 || kMode == RowMode::k8Small;
   // 8-bit head with more than 64 token rows: the two parts of h no longer fit one MMA's M (128 at most with one
   // CTA), so every K step issues two MMAs -- first parts, then second parts, into the same accumulator rows --
   // and the epilogue reads finished logits as on the bf16 head (no hand-over between warps).
-  const bool wide = kFp8 && p.part_rows > 64;
+  constexpr bool wide = kMode == RowMode::k8Wide;
   const int k_slabs = (p.d + kSlabElems - 1) / kSlabElems;
   const int units = (p.chunks + (p.mlp_hidden > 0 ? 1 : 0)) * p.row_units;
   const int T = p.tiles_per_unit;
@@ -590,10 +590,10 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
     // 8-bit head: of the 16 lanes, 0..7 are the first parts of eight tokens and 8..15 their second parts
     // (tc8_part_row), so the thread that holds a token's first part holds its second part too and adds them.  With
     // M = 64 a quadrant has one such group of 16 lanes, with M = 128 two, and a thread then keeps two tokens, eight apart.
-    // bf16 head: lanes 0..7 are tokens, 8..15 unused (TcConfig::group8).
-    const bool frag = kFp8 ? !wide : kGroup8;
-    constexpr int kFolds = kFp8 ? 2 : 1;           // tokens a thread may keep
-    const int quad_rows = frag ? (m64 ? 8 : 16) : (m64 ? 16 : 32);     // token rows per quadrant
+    // bf16 head: lanes 0..7 are tokens, 8..15 unused (RowMode::kGroup8).
+    constexpr bool frag = kFp8 ? !wide : kGroup8;
+    constexpr int kFolds = kMode == RowMode::k8Half ? 2 : 1;           // tokens a thread may keep
+    constexpr int quad_rows = frag ? (m64 ? 8 : 16) : (m64 ? 16 : 32);     // token rows per quadrant
     const int quad_row0 = quad * quad_rows;
     const int my_row = quad_row0 + (frag ? lane >> 2 : (m64 ? lane & 15 : lane));   // this thread's (first) token row
     const bool writer = frag ? (lane & 3) == 0 : (!m64 || lane < 16);  // one thread per token row
@@ -609,14 +609,14 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
 #pragma unroll
       for (int i = 0; i < kFolds; ++i) {
         const int r = my_row + 8 * i;
-        if (r < p.n && (i == 0 || (frag && !m64))) hs[i] = inl ? hs_s[r] : p.hscale[r];
+        if (r < p.n) hs[i] = inl ? hs_s[r] : p.hscale[r];
       }
       ok = __all_sync(0xffffffffu, ok);
     }
     for (int unit = worker; unit < units && ok; unit += workers, ++ord) {
       const Unit first = unit_of<kCta, kOdd>(p, unit, cta_rank);
       const bool warp_has_rows = first.row0 + quad_row0 < p.n;            // warp-uniform
-      const bool two_tokens = kFp8 && frag && !m64 && quad_row0 + 8 < p.n;   // warp-uniform
+      const bool two_tokens = kFolds == 2 && quad_row0 + 8 < p.n;   // warp-uniform
       const bool mlp_unit = !kFp8 && first.chunk < 0;
       RowFold f[kFolds];
 #pragma unroll
@@ -804,29 +804,30 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
 }
 
 // bf16 head: one CTA per worker (kCta = 1) or a pair (kCta = 2).
-// kGroup8: up to 16 rows (TcConfig::group8) -- a kernel of its own, because the other row counts lose 1.5 % to a switch at
-// run time (n = 24, d = 512, V = 32000 11.60 and 11.82 us).
-template <int kCta, bool kGroup8>
+// Every way of handling token rows is a kernel of its own: switches at run time cost the others (one for kGroup8 1.5 %:
+// n = 24, d = 512, V = 32000 11.60 and 11.82 us).
+template <int kCta, RowMode kMode>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_projection_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
-  tc_projection_body<kCta, false, kGroup8>(maps, p);
+  tc_projection_body<kCta, kMode>(maps, p);
 }
 
 // d no multiple of 8 (defined in the one file that launches them).
 #ifdef TLR_DEFINE_ODD_KERNELS
-template <int kCta, bool kGroup8>
+template <int kCta, RowMode kMode>
 __global__ void __launch_bounds__(kThreads, 1)
 odd_projection_kernel(const __grid_constant__ OddMaps maps, const TcParams p) {
-  tc_projection_body<kCta, false, kGroup8>(maps, p);
+  tc_projection_body<kCta, kMode>(maps, p);
 }
 #endif
 
 // 8-bit head (defined in the one file that launches it).  At most 128 registers per thread, so that a block of
 // the merge kernel (512 threads) fits on the SM beside this CTA and is resident, waiting, before this kernel ends.
 #ifdef TLR_DEFINE_TC8_KERNEL
+template <RowMode kMode>
 __global__ void __maxnreg__(128)
 tc8_projection_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
-  tc_projection_body<1, true, false>(maps, p);
+  tc_projection_body<1, kMode>(maps, p);
 }
 #endif
 
