@@ -287,7 +287,7 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
         st->odd_block = rows;
         out->launches = 2 * ((n + rows - 1) / rows) + 1;
       }
-      tlr::tc_configure(rows, &cfg);
+      tlr::tc_configure(rows, c->d + (c->classes > 1 ? tlr::odd_max_shift(c->d) : 0), c->V, c->sm_count, &cfg);
       workers_max = c->sm_count / cfg.cta;
       tlr::tc_plan(rows, c->V, cfg.cta, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, c->classes, &tp);
     }
@@ -670,7 +670,7 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
     return TLR_ERR_ARG;
   tlr::TcConfig cfg;
   tlr::TcPlan tp;
-  tlr::tc_configure(n, &cfg);
+  tlr::tc_configure(n, 2048, V, sm_count, &cfg);
   const int workers_max = sm_count / cfg.cta;
   tlr::tc_plan(n, V, cfg.cta, workers_max, tlr::kMaxChunks, mlp_hidden, 1, &tp);
   const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;

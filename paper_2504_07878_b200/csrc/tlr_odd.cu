@@ -73,7 +73,8 @@ cudaError_t launch_odd_shift(const void* h_bf16, int n, int d, int class_rows, i
 cudaError_t odd_prepare() {
   for (const auto kernel :
        {odd_projection_kernel<1, RowMode::kM128>, odd_projection_kernel<1, RowMode::kM64>,
-        odd_projection_kernel<1, RowMode::kGroup8>, odd_projection_kernel<2, RowMode::kM128>}) {
+        odd_projection_kernel<1, RowMode::kGroup8>, odd_projection_kernel<2, RowMode::kM128>,
+        odd_projection_kernel<2, RowMode::kM128Keep>}) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
   }
@@ -96,7 +97,8 @@ cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const 
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = c.cta == 1 ? 1 : 2;
-  const auto kernel = c.cta == 2                    ? odd_projection_kernel<2, RowMode::kM128>
+  const auto kernel = c.mode == RowMode::kM128Keep ? odd_projection_kernel<2, RowMode::kM128Keep>
+                      : c.cta == 2                 ? odd_projection_kernel<2, RowMode::kM128>
                       : c.mode == RowMode::kGroup8 ? odd_projection_kernel<1, RowMode::kGroup8>
                       : c.mode == RowMode::kM64    ? odd_projection_kernel<1, RowMode::kM64>
                                                    : odd_projection_kernel<1, RowMode::kM128>;

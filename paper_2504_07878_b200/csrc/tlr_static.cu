@@ -133,7 +133,7 @@ extern "C" tlr_status tlr_route_static(int32_t d, int32_t V, const void* W_bf16_
   const bool tc = d % 8 == 0;
   if (n > 0 && tc) {
     if (!s->tc_ready) return TLR_ERR_CUDA;   // no silent change of kernel
-    tlr::tc_configure(n, &cfg);
+    tlr::tc_configure(n, d, V, s->sm_count, &cfg);
     const int workers_max = s->sm_count / cfg.cta;
     tlr::tc_plan(n, V, cfg.cta, workers_max, kStaticMaxChunks, 0, 1, &tp);
     chunks = tp.chunks;

@@ -41,7 +41,7 @@ int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int ca
 
 // Ring depths and shared-memory size for a given n.  The h ring is short (L2 latency),
 // the W ring takes everything that is left (HBM latency).
-void tc_configure(int n, TcConfig* c) {
+void tc_configure(int n, int d, int V, int sm_count, TcConfig* c) {
   const int cta = n > kBlockM ? 2 : 1;
   int a_rows = kBlockM;
   RowMode mode = RowMode::kM128;
@@ -71,9 +71,21 @@ void tc_configure(int n, TcConfig* c) {
   const int budget = kSmemLimit - 1024 - kBarrierBytes - kScratchBytes;
   int sb = (budget - sa * a_stage) / b_stage;
   if (sb > kMaxBStages) sb = kMaxBStages;
+  const int k_slabs = (d + kRowBytes / 2 - 1) / (kRowBytes / 2);
+  // Pair mode with all of a row unit's h beside at least four W stages (d = 193..576): h is loaded once per unit instead
+  // of once per tile.  Worth it from twelve tiles per worker on: V = 64000, streamed and kept, d = 256 n = 1024 44.9 and
+  // 43.8 us per step, n = 4096 156 and 151; d = 384 n = 4096 195 and 188; d = 512 n = 1024 69.7 and 67.5, n = 4096 246 and
+  // 237; but n = 256 (3.4 tiles), d = 512 23.7 and 24.4, and at eight (V = 151936) no difference.
+  const long long tiles = static_cast<long long>((n + 255) / 256) * ((V + kBlockN - 1) / kBlockN);
+  if (cta == 2 && k_slabs >= 4 && k_slabs * a_stage + 4 * b_stage <= budget && tiles >= 12ll * (sm_count / 2)) {
+    mode = RowMode::kM128Keep;
+    sa = k_slabs;
+    sb = (budget - sa * a_stage) / b_stage;
+    if (sb > kMaxBStages) sb = kMaxBStages;
+  }
   // Tuning override: TLR_TC_RINGS="<h stages>,<W stages>" (ignored if it does not fit).
   const Tuning& tn = tuning();
-  if (tn.ring_a >= 1 && tn.ring_a <= kRelease && tn.ring_b >= 1 && tn.ring_b <= kMaxBStages &&
+  if (mode != RowMode::kM128Keep && tn.ring_a >= 1 && tn.ring_a <= kRelease && tn.ring_b >= 1 && tn.ring_b <= kMaxBStages &&
       tn.ring_a * a_stage + tn.ring_b * b_stage <= budget) {
     sa = tn.ring_a;
     sb = tn.ring_b;
@@ -90,7 +102,8 @@ void tc_configure(int n, TcConfig* c) {
 
 cudaError_t tc_prepare() {
   for (const auto kernel : {tc_projection_kernel<1, RowMode::kM128>, tc_projection_kernel<1, RowMode::kM64>,
-                            tc_projection_kernel<1, RowMode::kGroup8>, tc_projection_kernel<2, RowMode::kM128>}) {
+                            tc_projection_kernel<1, RowMode::kGroup8>, tc_projection_kernel<2, RowMode::kM128>,
+                            tc_projection_kernel<2, RowMode::kM128Keep>}) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
   }
@@ -113,7 +126,8 @@ cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const Tc
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = c.cta == 1 ? 1 : 2;
-  const auto kernel = c.cta == 2                    ? tc_projection_kernel<2, RowMode::kM128>
+  const auto kernel = c.mode == RowMode::kM128Keep ? tc_projection_kernel<2, RowMode::kM128Keep>
+                      : c.cta == 2                 ? tc_projection_kernel<2, RowMode::kM128>
                       : c.mode == RowMode::kGroup8 ? tc_projection_kernel<1, RowMode::kGroup8>
                       : c.mode == RowMode::kM64    ? tc_projection_kernel<1, RowMode::kM64>
                                                    : tc_projection_kernel<1, RowMode::kM128>;

@@ -10,6 +10,7 @@ namespace tlr {
 // How a projection kernel handles token rows.
 enum class RowMode : int {
   kM128,      // bf16 head, more than 64 rows: MMA M = 128 (256 on a pair), one epilogue thread per row
+  kM128Keep,  // the same on a pair, where all of a row unit's h fits beside the W ring: it is loaded once per unit
   kM64,       // bf16 head, 17..64 rows: M = 64, one thread per row
   kGroup8,    // bf16 head, up to 16 rows: M = 64, eight rows in every sixteen operand rows, four threads per row
   k8Small,    // 8-bit head, up to 32 rows: both parts through one MMA with M = 64, four threads per row
@@ -97,7 +98,7 @@ cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const 
 inline int tc_h_box_rows(const TcConfig& c) { return c.mode == RowMode::kGroup8 ? 8 : c.a_rows; }   // rows of h per TMA box
 int tc_threads();
 int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
-void tc_configure(int n, TcConfig* c);
+void tc_configure(int n, int d, int V, int sm_count, TcConfig* c);
 void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan);
 cudaError_t tc_prepare();   // opt in to the kernels' dynamic shared memory size (once per device)
 cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const TcConfig& c, int workers,

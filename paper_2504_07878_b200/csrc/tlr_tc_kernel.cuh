@@ -311,7 +311,8 @@ template <int kCta, RowMode kMode, class Maps>
 __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcParams& p) {
   constexpr bool kOdd = std::is_same<Maps, OddMaps>::value;   // d no multiple of 8: vocabulary rows by residue class
   constexpr bool kFp8 = kMode >= RowMode::k8Small, kGroup8 = kMode == RowMode::kGroup8;
-  static_assert(kCta == 1 || kMode == RowMode::kM128, "a pair of CTAs runs the plain mode of the bf16 head");
+  constexpr bool kKeep = kMode == RowMode::kM128Keep;      // the stage of a K slab is its number, filled once per unit
+  static_assert(kCta == 1 || kMode == RowMode::kM128 || kKeep, "modes of a pair of CTAs");
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment: the swizzle pattern is a function of the shared-memory address.
   // (The dynamic shared memory of both CTAs of a pair starts at the same offset, so the
@@ -339,7 +340,9 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   auto xch_full = [&](int q) { return bar_base + 8u * (kFixed + 4 + q); };
   auto xch_empty = [&](int q) { return bar_base + 8u * (kFixed + 8 + q); };
   const uint32_t h_ready = bar_base + 8u * (kFixed + 12);   // 8-bit head: h has been split in place (inline mode)
-  constexpr int kNumBarriers = kFixed + 13;
+  // kept h: the MMAs of the unit's last tile have read K slab s
+  auto h_free = [&](int s) { return bar_base + 8u * (kFixed + 13 + s); };
+  constexpr int kNumBarriers = kFixed + 13 + kMaxAStages;
   static_assert(kNumBarriers * 8 + 16 <= kBarrierBytes, "barrier block too small");
   unsigned char* gen_base = smem_raw + (base - smem_u32(smem_raw));
   unsigned char* tail = gen_base + (bar_base - base);
@@ -359,6 +362,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
 
   if (threadIdx.x == 0) {
     if (!inl) for (int s = 0; s < SA; ++s) mbar_init(a_full(s), 1);   // (inline mode: SA = K slabs, nothing streams)
+    if (kKeep) for (int s = 0; s < SA; ++s) mbar_init(h_free(s), 1);
     for (int s = 0; s < SB; ++s) mbar_init(b_full(s), 1);
     for (int j = 0; j < kRelease; ++j) mbar_init(released(j), 1);
     for (int b = 0; b < 2; ++b) {
@@ -474,12 +478,15 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       int slab = 0;
       bool ok = true;
       bool h_there = false;
-      for (int unit = worker; unit < units && ok; unit += workers) {
+      uint32_t ord = 0;
+      for (int unit = worker; unit < units && ok; unit += workers, ++ord) {
         const Unit un = unit_of<kCta, kOdd>(p, unit, cta_rank);
+        const int h_row = kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
           for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
+            if (kKeep && t > 0) continue;      // (the first tile of a unit is never empty)
             if (!h_there) {
               // here and not with the other warps above: the arithmetic of the first unit, two 64-bit divisions among it,
               // would stand between the end of the wait and the first load of h, which the whole step waits for (n = 1,
@@ -487,13 +494,14 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
               asm volatile("griddepcontrol.wait;" ::: "memory");
               h_there = true;
             }
-            if (slab >= SA) {
+            if (kKeep) {
+              if (ord > 0 && !mbar_wait(h_free(ks), (ord - 1) & 1u, abort_flag, p.status, wait_ns)) { ok = false; break; }
+            } else if (slab >= SA) {
               const int j = slab - SA;
               if (!mbar_wait(released(j & (kRelease - 1)), (j / kRelease) & 1, abort_flag, p.status, wait_ns)) { ok = false; break; }
             }
             const uint32_t dst = a_ring + stage * a_stage_bytes;
             const uint32_t bar = (kCta == 2) ? map_to_cta(a_full(stage), 0) : a_full(stage);
-            const int h_row = kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0);
             if (kGroup8) {      // boxes of eight rows, sixteen operand rows apart
               mbar_expect_tx(a_full(stage), a_stage_bytes >> 1);
               for (int r = 0; r < p.a_rows; r += 16)
@@ -540,14 +548,16 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
+          const bool last_tile = kKeep && (t + 1 == T || tile_of(p, un, t + 1).rows == 0);
           const uint32_t idesc = kFp8 ? instr_desc_e4m3(mma_m, tl.rows) : instr_desc(mma_m, tl.rows);
           ok = __all_sync(0xffffffffu, mbar_wait(acc_empty(acc), acc_phase ^ 1u, abort_flag, p.status, wait_ns));
           if (!ok) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + acc * kBlockN;
           for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
+            if (kKeep && t > 0) ra = true;
             if (!__all_sync(0xffffffffu, ra && rb)) {
-              const bool got = (inl || mbar_wait(a_full(sa), pa, abort_flag, p.status, wait_ns)) &&
+              const bool got = (inl || (kKeep && t > 0) || mbar_wait(a_full(sa), pa, abort_flag, p.status, wait_ns)) &&
                                mbar_wait(b_full(sb), pb, abort_flag, p.status, wait_ns);
               ok = __all_sync(0xffffffffu, got);
               if (!ok) break;
@@ -555,7 +565,10 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
             tc_fence_after();
             const uint32_t a_lo = a_lo0 + sa * a_step;
             const uint32_t b_lo = b_lo0 + sb * b_step;
-            if (++sa == SA) { sa = 0; pa ^= 1u; }
+            if (++sa == SA) {
+              sa = 0;
+              if (!kKeep || t == 0) pa ^= 1u;
+            }
             if (++sb == SB) { sb = 0; pb ^= 1u; }
             ra = inl || mbar_test_wait(a_full(sa), pa);     // (inline mode: stage sa is slab sa, always there)
             rb = mbar_test_wait(b_full(sb), pb);
@@ -571,6 +584,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
                                   (ks | k) != 0 ? 1u : 0u);
               }
               umma_commit<kCta>(released(slab & (kRelease - 1)));   // both slabs are free once these MMAs are done
+              if (last_tile) umma_commit<kCta>(h_free(ks));
             }
             __syncwarp();
           }

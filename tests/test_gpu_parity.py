@@ -341,3 +341,18 @@ def test_small_batches_at_the_edges_of_the_fragment_layout(pkg, n, V):
     assert np.max(np.abs(score.cpu().numpy() - want)) <= 1e-5     # fp32 sums of exact products
     assert np.array_equal(r.token[:n].cpu().numpy(), gpu["token"])
     r.close()
+
+
+# Pair mode with h kept in shared memory for a whole unit (enough tiles per worker, d = 193..576): four to nine K slabs,
+# several units per worker and several row units, the last of them ragged; also without d % 8 == 0.
+@pytest.mark.parametrize("n,d,V", [(1100, 200, 47000), (2049, 320, 26000), (1025, 576, 46500), (4100, 256, 14000), (1100, 257, 47000)])
+def test_pair_mode_keeps_h_for_a_unit(pkg, n, d, V):
+    W = S.make_W(d, V, seed=n, std=0.08)
+    hid = S.make_h(n, d, seed=d, W=W, planted_fraction=0.1)
+    rows = np.unique(np.concatenate([np.arange(0, n, 7), np.arange(n - 140, n)]))
+    ref = O.route_oracle(S.bf16_bits(hid.h)[rows], S.bf16_bits(W), 0.5)
+    full = run_gpu(pkg, W.cuda(), hid.h, 0.5)
+    assert full["status"] == 0 and full["plan"].path == 2
+    check_self_consistency(full, 0.5, V)
+    gpu = {k: full[k][rows] for k in ("token", "conf", "entropy", "route_mask")}
+    check_against_oracle(ref, gpu)
