@@ -140,6 +140,8 @@ struct tlr_ctx {
   void* h_shift = nullptr;
   int odd_rows = 0, odd_pitch = 0;
 
+  unsigned char* workspace = nullptr;     // one device allocation: the partials, the ticket and status words, the staging
+                                          // buffers (ten allocations took most of the time of tlr_create)
   Partial* partials = nullptr;
   unsigned int* ticket = nullptr;
   uint32_t* status = nullptr;
@@ -361,13 +363,9 @@ tlr_ctx::Step* step_for(tlr_ctx* c, int n, bool mlp) {
 }
 
 void free_all(tlr_ctx* c) {
-  cudaFree(c->partials);
-  cudaFree(c->ticket);
-  cudaFree(c->status);
+  cudaFree(c->workspace);
+  cudaFreeHost(c->out_pinned[0]);
   for (int q = 0; q < 2; ++q) {
-    cudaFree(c->h_stage[q]);
-    cudaFree(c->out_stage[q]);
-    cudaFreeHost(c->out_pinned[q]);
     if (c->slot_done[q] != nullptr) cudaEventDestroy(c->slot_done[q]);
     if (c->copy_done[q] != nullptr) cudaEventDestroy(c->copy_done[q]);
   }
@@ -390,26 +388,40 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
   if (static_cast<long long>(V) + 256 > 0x7fffffffll) return TLR_ERR_UNSUPPORTED;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return TLR_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return TLR_ERR_CUDA;
-  if (prop.major != 10) return TLR_ERR_UNSUPPORTED;   // the kernels are built for sm_100a only
+  int major = 0, sm_count = 0;
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return TLR_ERR_CUDA;
+  if (major != 10) return TLR_ERR_UNSUPPORTED;   // the kernels are built for sm_100a only
   tlr_ctx* c = new (std::nothrow) tlr_ctx();
   if (c == nullptr) return TLR_ERR_NOMEM;
   c->device = dev;
-  c->sm_count = prop.multiProcessorCount;
+  c->sm_count = sm_count;
   c->d = d;
   c->V = V;
   c->max_n = max_n;
   c->W = W_dev;
   const size_t np = static_cast<size_t>(max_n);
-  bool ok = true;
-  ok = ok && cudaMalloc(&c->partials, np * tlr::kMaxChunks * sizeof(Partial)) == cudaSuccess;
-  ok = ok && cudaMalloc(&c->ticket, sizeof(unsigned int)) == cudaSuccess;
-  ok = ok && cudaMalloc(&c->status, sizeof(uint32_t)) == cudaSuccess;
+  auto padded = [](size_t bytes) { return (bytes + 255) & ~static_cast<size_t>(255); };
+  const size_t partial_bytes = padded(np * tlr::kMaxChunks * sizeof(Partial));
+  const size_t h_bytes = padded(np * d * 2), out_bytes = padded(np * 17 + 8), pinned_bytes = padded(np * 17 + 8 + 8);
+  bool ok = cudaMalloc(&c->workspace, 256 + partial_bytes + 2 * (h_bytes + out_bytes)) == cudaSuccess;
+  ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->out_pinned[0]), 2 * pinned_bytes, cudaHostAllocMapped) == cudaSuccess;
+  if (ok) {
+    unsigned char* at = c->workspace;
+    c->ticket = reinterpret_cast<unsigned int*>(at);
+    c->status = reinterpret_cast<uint32_t*>(at + 128);
+    at += 256;
+    c->partials = reinterpret_cast<Partial*>(at);
+    at += partial_bytes;
+    for (int q = 0; q < 2; ++q) {
+      c->h_stage[q] = at;
+      c->out_stage[q] = at + h_bytes;
+      at += h_bytes + out_bytes;
+    }
+    c->out_pinned[1] = c->out_pinned[0] + pinned_bytes;
+  }
   for (int q = 0; q < 2; ++q) {
-    ok = ok && cudaMalloc(&c->h_stage[q], np * d * 2) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->out_stage[q], np * 17 + 8) == cudaSuccess;
-    ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->out_pinned[q]), np * 17 + 8 + 8, cudaHostAllocMapped) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->slot_done[q], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->copy_done[q], cudaEventDisableTiming) == cudaSuccess;
   }
@@ -425,8 +437,7 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
       c->out_mapped[q] = nullptr;   // tlr_route_host then stages the outputs in device memory and copies them
     }
   }
-  if (cudaMemset(c->ticket, 0, sizeof(unsigned int)) != cudaSuccess ||
-      cudaMemset(c->status, 0, sizeof(uint32_t)) != cudaSuccess) {
+  if (cudaMemset(c->workspace, 0, 256) != cudaSuccess) {      // the ticket and the status word
     free_all(c);
     return TLR_ERR_CUDA;
   }
