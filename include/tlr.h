@@ -167,7 +167,7 @@ typedef struct {
  * and entropy are produced as always.  Where the tensor-core projection kernel runs (bf16 head, d % 8 == 0, W1
  * 16-byte aligned) the rows of W1 are walked by that same launch as one more work unit per 128 or 256 token rows --
  * same staged hidden states, same MMAs, an epilogue that applies b1, ReLU and w2 and sums -- so the step keeps its
- * two launches; otherwise one extra small kernel computes the score on CUDA cores.
+ * two launches; otherwise one extra small kernel computes the score (8-bit head: on tensor cores, beside the projection).
  * Errors: TLR_ERR_ARG, TLR_ERR_NOMEM.  tlr_route_ex returns TLR_ERR_ARG when the learned score is
  * requested but no router is attached.
  */

@@ -246,7 +246,7 @@ bool make_map(const tlr_ctx* c, CUtensorMap* map, const void* base, int rows, in
 // Tensor cores wherever their set-up succeeded.  The one exception: a small batch on a head of at most 128 KB whose d is
 // no multiple of 8.  The tensor-core path needs a third launch there, for the shifted copies of h, which costs the
 // host 2 us and buys next to nothing on the device: n = 20, d = 36, V = 1500 13.1 us on CUDA cores and 9.1 on tensor
-// cores, n = 1, d = 9, V = 700 10.4 and 7.9; on larger heads it buys everything (n = 64, d = 300, V = 33000 194 and 17).
+// cores, n = 1, d = 9, V = 700 10.4 and 7.9; on larger heads it buys everything (n = 64, d = 300, V = 33000 194 and 14).
 tlr_path pick_path(const tlr_ctx* c, int n) {
   if (c->forced != TLR_PATH_AUTO) return c->forced;
   const bool tiny = c->classes > 1 && n <= 32 && static_cast<long long>(c->V) * c->d <= 65536;

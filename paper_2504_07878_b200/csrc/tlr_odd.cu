@@ -4,7 +4,7 @@
 // Before, every such shape ran on the CUDA-core kernel (tlr_simt.cu), which is bound by its FMAs and by one thread
 // reading one row of W.  The projection here does the work of the bf16 head plus at most one more K slab and is bound by
 // what bounds that one; the copies of h cost a launch and C * n * d * 2 bytes, small beside W.  Per step in a graph,
-// before and after: n = 64, d = 300, V = 33000 194 -> 17 us; n = 1, d = 999, V = 60000 624 -> 29 (120 MB of W: 18);
+// before and after: n = 64, d = 300, V = 33000 194 -> 14 us; n = 1, d = 999, V = 60000 624 -> 29 (120 MB of W: 18);
 // n = 256, d = 999, V = 60000 3987 -> 48; n = 200, d = 101, V = 33000 160 -> 17.
 #include <cuda.h>
 #include <cuda_bf16.h>

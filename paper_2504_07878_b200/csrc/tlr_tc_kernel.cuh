@@ -3,18 +3,18 @@
 // online-softmax reduction (max / argmax / sum-exp / entropy numerator) fused into
 // the epilogue, so the n x V logits never leave the SM.
 //
-// One kernel body, four instantiations (kernels at the end of this file):
-//   <1, false>  bf16 head, one CTA per worker, MMA M = 128 token rows     (n <= 128; M = 64 when n <= 64)
-//   <2, false>  bf16 head, a cluster of two CTAs per worker, MMA M = 256 rows (cta_group::2): each
+// One kernel body; a kernel per way of handling token rows (RowMode) and per kind of head (kernels at the end of this file):
+//   bf16 head, one CTA per worker, MMA M = 64 or 128 token rows              (n <= 128)
+//   bf16 head, a cluster of two CTAs per worker, MMA M = 256 rows (cta_group::2): each
 //               CTA stages its own 128 rows of h and HALF of the W tile, and the pair's
 //               tensor cores read both halves, so a W byte enters shared memory once
-//               per 256 token rows.                                       (n > 128)
-//   <1, true>   8-bit (e4m3) head for decode batches of at most 128 rows: h is the sum of two e4m3
+//               per 256 token rows.                                          (n > 128)
+//   8-bit (e4m3) head for decode batches of at most 128 rows: h is the sum of two e4m3
 //               parts, stacked in one operand slab.  Up to 64 rows ONE kind::f8f6f4 MMA per K step
 //               covers both parts along its M, and the epilogue adds the two accumulator rows of a
 //               token before it folds them; above, two MMAs per K step (one per part) add into the
 //               same rows.
-//   OddMaps     bf16 head whose hidden size is no multiple of 8: the vocabulary is walked by residue class
+//   bf16 head whose hidden size is no multiple of 8: the vocabulary is walked by residue class
 //               (see OddMaps), otherwise like the bf16 head.
 //
 // Decomposition.  The vocabulary is cut into `chunks` contiguous ranges of granules
