@@ -65,9 +65,10 @@ void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden,
     const long long gmax = (granules + c - 1) / c;
     const long long tiles = (gmax * g + 255) / 256;
     const long long units = 1ll * row_units * c * classes;
-    const long long unit_cost = gmax * g + 24 * tiles;
-    // Pair mode: a tile costs a pass over all of h whatever its width (the pair MMA takes as long with 32
-    // columns as with 256), so the busiest worker's TILE count is compared first and the row-based cost only
+    // A pair's change of unit costs 1340 cycles against 1025 between two tiles, so that of two plans with the same passes the
+    // one with fewer units is taken (n = 1024, d = 256, V = 64000, with the walk free of divisions: 42.6 -> 40.0 us).
+    const long long unit_cost = gmax * g + 24 * tiles + (cta == 2 ? 100 : 0);
+    // Pair mode: a tile costs a pass over all of h whatever its width, so the busiest worker's TILE count is compared first and the row-based cost only
     // decides between plans with the same count.
     const bool by_passes = cta == 2 && !tuning().even_tiles && !tuning().row_cost;
     long long cost, passes = 0;
@@ -303,12 +304,7 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     p.n = n;
     p.d = c->d;
     p.V = c->V;
-    p.row_units = tp.row_units;
-    p.chunks = tp.chunks;
-    p.granules = tp.granules;
-    p.tiles_per_unit = tp.tiles_per_unit;
-    p.full_tiles_first = tp.full_tiles_first;
-    p.granule_rows = tp.granule_rows;
+    tlr::tc_set_schedule(tp, &p);
     p.a_rows = cfg.a_rows;
     p.part_rows = cfg.part_rows;
     p.a_stages = cfg.a_stages;
@@ -317,7 +313,6 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     p.debug_drop_w_copies = c->debug_kind == 1 ? 1 : 0;
     p.w_wait = 0;
     p.mlp_hidden = tp.mlp_rows > 0 ? c->mlp_hidden : 0;
-    p.mlp_rows = tp.mlp_rows;
     p.mlp_b1 = c->mlp_b1;
     p.mlp_w2 = c->mlp_w2;
     p.mlp_out = c->mlp_scores;
@@ -328,8 +323,6 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     p.status = c->status;
     if (c->classes > 1) {
       p.d = c->d + tlr::odd_max_shift(c->d);
-      p.classes = c->classes;
-      p.class_chunks = tp.chunks / c->classes;
       p.h_class_rows = c->odd_rows;
       for (int r = 0; r < c->classes; ++r) st->odd.w[r] = c->map_cls[r];
       if (n > 0) make_map(c, &st->odd.h, c->h_shift, c->classes * c->odd_rows, c->odd_pitch, tlr::tc_h_box_rows(cfg));
@@ -689,14 +682,8 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
   tlr::TcParams p = {};
   p.n = n;
   p.V = V;
-  p.row_units = tp.row_units;
-  p.chunks = tp.chunks;
-  p.granules = tp.granules;
-  p.tiles_per_unit = tp.tiles_per_unit;
-  p.full_tiles_first = tp.full_tiles_first;
-  p.granule_rows = tp.granule_rows;
+  tlr::tc_set_schedule(tp, &p);
   p.mlp_hidden = tp.mlp_rows > 0 ? mlp_hidden : 0;
-  p.mlp_rows = tp.mlp_rows;
   *count = tlr::tc_enumerate_tiles(p, cfg.cta, workers, out, capacity);
   if (plan_out != nullptr) {
     plan_out->path = TLR_PATH_TC;

@@ -158,12 +158,7 @@ extern "C" tlr_status tlr_route_static(int32_t d, int32_t V, const void* W_bf16_
       p.n = n;
       p.d = d;
       p.V = V;
-      p.row_units = tp.row_units;
-      p.chunks = tp.chunks;
-      p.granules = tp.granules;
-      p.tiles_per_unit = tp.tiles_per_unit;
-      p.full_tiles_first = tp.full_tiles_first;
-      p.granule_rows = tp.granule_rows;
+      tlr::tc_set_schedule(tp, &p);
       p.a_rows = cfg.a_rows;
         p.part_rows = cfg.part_rows;
       p.a_stages = cfg.a_stages;

@@ -47,6 +47,9 @@ struct TcPlan {
 struct TcParams {
   int n, d, V;
   int row_units, chunks, granules, tiles_per_unit, full_tiles_first, granule_rows;
+  int chunk_q, chunk_r;               // granules of a chunk: chunk_q, and one more in chunk_r of them (of a class)
+  uint32_t chunk_mul;                 // ceil(2^32 / chunks of a class), 0 for one chunk
+  int full_granules;                  // granules of a full tile
   int classes, class_chunks;          // odd-sized d only: residue classes, chunks per class (chunks == classes * class_chunks)
   int h_class_rows;                   // odd-sized d only: rows between the shifted copies of h
   int a_rows, part_rows, a_stages, b_stages;
@@ -96,6 +99,22 @@ cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const 
                                   cudaStream_t stream);
 
 inline int tc_h_box_rows(const TcConfig& c) { return c.mode == RowMode::kGroup8 ? 8 : c.a_rows; }   // rows of h per TMA box
+// The fields of a launch's parameters that describe its work decomposition.
+inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
+  p->row_units = plan.row_units;
+  p->chunks = plan.chunks;
+  p->granules = plan.granules;
+  p->tiles_per_unit = plan.tiles_per_unit;
+  p->full_tiles_first = plan.full_tiles_first;
+  p->granule_rows = plan.granule_rows;
+  p->mlp_rows = plan.mlp_rows;
+  p->classes = plan.classes;
+  p->class_chunks = plan.chunks / plan.classes;
+  p->chunk_q = plan.granules / p->class_chunks;
+  p->chunk_r = plan.granules % p->class_chunks;
+  p->chunk_mul = p->class_chunks > 1 ? static_cast<uint32_t>(((1ull << 32) + p->class_chunks - 1) / p->class_chunks) : 0u;
+  p->full_granules = 256 / plan.granule_rows;
+}
 int tc_threads();
 int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
 void tc_configure(int n, int d, int V, int sm_count, TcConfig* c);

@@ -94,6 +94,7 @@ struct Unit {
   int chunk;   // vocabulary chunk; -1 for a learned-router unit
   int g0;      // first granule of the chunk
   int G;       // granules in the chunk
+  int tile_q, tile_r;   // tiles of equal size: each has tile_q granules, the first tile_r one more
   int cls;     // residue class of the chunk's vocabulary rows (0 unless d is odd-sized)
   int rows;    // vocabulary rows of that class (V unless d is odd-sized)
 };
@@ -102,8 +103,10 @@ struct Tile {
   int rows;    // vocabulary rows in the tile (multiple of 16 * kCta); 0 = empty tile
 };
 
-// What is fixed for a whole unit (the divisions happen here, once per unit: the tile walk of the MMA-issuing
-// warp is on the tensor pipe's critical path and must stay cheap).
+// What is fixed for a whole unit.  The walk of the MMA-issuing warp is on the tensor pipe's critical path and must stay
+// cheap: no division per tile, two 32-bit ones per unit.  With 64-bit ones here and one per tile this function took 720
+// cycles of the 2020 between a unit's last slab and the next one's first (now 260 of 1340), a tile 1150 (now 1025):
+// prefill at n = 8192, d = 896 1743 -> 1713 us, n = 2000, d = 1024, V = 100000 341 -> 329, n = 1, d = 256 8.64 -> 8.45.
 template <int kCta, bool kOdd = false>
 __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, int cta_rank) {
   Unit u;
@@ -115,21 +118,29 @@ __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, in
     u.row0 = ((unit - vocab_units) * kCta + cta_rank) * kBlockM;
     u.g0 = 0;
     u.G = 0;
+    u.tile_q = u.tile_r = 0;
     return u;
   }
-  u.chunk = unit / p.row_units;
+  u.chunk = static_cast<int>(static_cast<uint32_t>(unit) / static_cast<uint32_t>(p.row_units));
   const int ru = unit - u.chunk * p.row_units;
   u.row0 = (ru * kCta + cta_rank) * kBlockM;
-  int c = u.chunk, chunks = p.chunks;
+  int c = u.chunk;
   if (kOdd) {                         // class by class: the chunks of a class share its rows out
-    chunks = p.class_chunks;
-    u.cls = c / chunks;
-    c -= u.cls * chunks;
-    u.rows = (p.V - u.cls + p.classes - 1) / p.classes;
+    u.cls = static_cast<int>(static_cast<uint32_t>(c) / static_cast<uint32_t>(p.class_chunks));
+    c -= u.cls * p.class_chunks;
+    u.rows = static_cast<int>(static_cast<uint32_t>(p.V - u.cls + p.classes - 1) / static_cast<uint32_t>(p.classes));
   }
-  u.g0 = static_cast<int>((static_cast<long long>(p.granules) * c) / chunks);
-  const int g1 = static_cast<int>((static_cast<long long>(p.granules) * (c + 1)) / chunks);
-  u.G = g1 - u.g0;
+  // chunk_r of the chunks have a granule more than the others, evenly spread: floor(chunk_r * c / chunks) of those before
+  // chunk c, by a multiplication (chunk_mul = ceil(2^32 / chunks) is exact here: chunk_r * c < 2^16, chunks <= 192)
+  const int e0 = static_cast<int>((static_cast<uint64_t>(p.chunk_r * c) * p.chunk_mul) >> 32);
+  const int e1 = static_cast<int>((static_cast<uint64_t>(p.chunk_r * (c + 1)) * p.chunk_mul) >> 32);
+  u.g0 = p.chunk_q * c + e0;
+  u.G = p.chunk_q + e1 - e0;
+  u.tile_q = u.tile_r = 0;
+  if (!p.full_tiles_first) {
+    u.tile_q = static_cast<int>(static_cast<uint32_t>(u.G) / static_cast<uint32_t>(p.tiles_per_unit));
+    u.tile_r = u.G - u.tile_q * p.tiles_per_unit;
+  }
   return u;
 }
 
@@ -145,12 +156,11 @@ __host__ __device__ __forceinline__ Tile tile_of(const TcParams& p, const Unit& 
   if (p.full_tiles_first) {
     // as many full 256-row tiles as fit, then one remainder tile: a tile costs a pass over all
     // of h whatever its width, so the fewest, widest tiles are the cheapest
-    const int full = kBlockN / p.granule_rows;
-    ga = full * t < u.G ? full * t : u.G;
-    gb = full * (t + 1) < u.G ? full * (t + 1) : u.G;
+    ga = p.full_granules * t < u.G ? p.full_granules * t : u.G;
+    gb = p.full_granules * (t + 1) < u.G ? p.full_granules * (t + 1) : u.G;
   } else {
-    ga = (u.G * t) / p.tiles_per_unit;
-    gb = (u.G * (t + 1)) / p.tiles_per_unit;
+    ga = u.tile_q * t + (t < u.tile_r ? t : u.tile_r);
+    gb = ga + u.tile_q + (t < u.tile_r ? 1 : 0);
   }
   r.v0 = (u.g0 + ga) * p.granule_rows;
   r.rows = (gb - ga) * p.granule_rows;
