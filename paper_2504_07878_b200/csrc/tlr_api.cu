@@ -1,4 +1,5 @@
 // C-ABI of the routing library: context, argument checks, launch planning, dispatch.
+#include <algorithm>
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -77,16 +78,19 @@ void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden,
       cost = waves * unit_cost;
       passes = waves * tiles;
     } else {
-      // worker w takes units w, w + workers, ...: vocabulary units first, then the row_units router units
+      // Worker w takes units w, w + workers, ...: vocabulary units first, then the row_units router units, dealt out from
+      // worker `rem` on.  The busiest is the first of those with `full` vocabulary units (worker rem) or the first of those
+      // with one more (worker 0): no other has more of either kind than one of these two.  (Asking every worker made the
+      // first call with a new n 80 us longer: n = 777, V = 151936, width 256.)
       const long long full = units / workers, rem = units % workers;
-      cost = 0;
-      for (int w = 0; w < workers; ++w) {
-        const long long nv = full + (w < rem ? 1 : 0);
-        const long long j0 = ((w - rem) % workers + workers) % workers;   // first router unit of this worker
-        const long long nm = j0 < row_units ? 1 + (row_units - 1 - j0) / workers : 0;
-        const long long load = nv * unit_cost + nm * mlp_cost;
-        if (load > cost) cost = load;
-        if (nv * tiles + nm * mlp_tiles > passes) passes = nv * tiles + nm * mlp_tiles;
+      const auto router_units = [&](long long j0) { return j0 < row_units ? 1 + (row_units - 1 - j0) / workers : 0; };
+      const long long nm0 = router_units(0);
+      cost = full * unit_cost + nm0 * mlp_cost;
+      passes = full * tiles + nm0 * mlp_tiles;
+      if (rem > 0) {
+        const long long nm1 = router_units(workers - rem);
+        cost = std::max(cost, (full + 1) * unit_cost + nm1 * mlp_cost);
+        passes = std::max(passes, (full + 1) * tiles + nm1 * mlp_tiles);
       }
     }
     if (!by_passes) passes = 0;

@@ -93,6 +93,33 @@ def test_learned_router_units_follow_the_vocabulary_units(n, V, hidden):
     assert plan.grid <= 148
 
 
+@pytest.mark.parametrize("n,V,hidden", [(1, 40, 16), (64, 2000, 256), (128, 151936, 512), (129, 5000, 40), (777, 151936, 256),
+                                        (4096, 300, 1024), (20000, 9000, 64)])
+@pytest.mark.parametrize("sms", [148, 10])
+def test_router_plan_is_the_best_over_all_workers(n, V, hidden, sms):
+    """The plan's number of chunks is the one whose busiest worker (every worker asked) is the least busy."""
+    _, plan = P.tlr_debug_plan_tiles(n, V, sms, hidden)
+    g, cta = plan.reserved, 2 if n > 128 else 1
+    workers, granules = sms // cta, -(-V // g)
+    padded = -(-hidden // (16 * cta)) * (16 * cta)
+    router_tiles = -(-padded // 256)
+    best = None
+    for c in range(1, min(granules, 192) + 1):
+        rows = -(-granules // c) * g
+        tiles = -(-rows // 256)
+        units = c * plan.row_units
+        passes = cost = 0
+        for w in range(min(workers, units + plan.row_units)):
+            nv = len(range(w, units, workers))
+            nm = len(range(w, units + plan.row_units, workers)) - nv
+            passes = max(passes, nv * tiles + nm * router_tiles)
+            cost = max(cost, nv * (rows + 24 * tiles + 100 * (cta - 1)) + nm * (padded + 24 * router_tiles))
+        key = (passes if cta == 2 else 0, cost)
+        if best is None or key < best[0]:
+            best = (key, c)
+    assert plan.vocab_chunks == best[1]
+
+
 def test_learned_router_costs_the_decode_plans_little():
     """The busiest worker of the decode plans carries at most 3 % more rows with a 256-wide router inside."""
     for n in (16, 256):
