@@ -36,8 +36,8 @@ RIDGE_ROWS_HBM = 256            # at or below this many rows the step is reporte
 # hash of that source is recorded here and traffic is reported as null when the source differs.
 NCU_TRAFFIC = {
     "kernel_sources": ["paper_2504_07878_b200/csrc/tlr_tc_kernel.cuh", "paper_2504_07878_b200/csrc/tlr_tc_ptx.cuh"],
-    "sha256": "818527e254f2ea237e319a293919ec7c3cd8c4fd7ff944e3d3c69e3e511d24f3",
-    "bytes_per_launch": {"decode256": 274.47e6, "decode16": 274.49e6, "sweep512": 529.31e6},
+    "sha256": "027cc4016f5fbd41125d70d0caeb6b54c54f34db1733dcdabb76f3ed464625c3",
+    "bytes_per_launch": {"decode256": 274.48e6, "decode16": 273.99e6, "sweep512": 529.40e6},
 }
 
 
