@@ -448,6 +448,12 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
   return TLR_OK;
 }
 
+// What settles near-ties between rows of W in different residue classes (nothing where d is a multiple of 8).
+tlr::Ties ties_of(const tlr_ctx* c, const void* h_bf16_dev) {
+  if (c->classes == 1) return {nullptr, nullptr, 0};
+  return {static_cast<const unsigned short*>(c->W), static_cast<const unsigned short*>(h_bf16_dev), c->d};
+}
+
 // Enqueues the projection kernel of a call with n > 0 rows: chunk partials into ctx->partials.  router_beside: the 8-bit
 // head's router kernel follows (launch_mlp_beside).
 tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ctx::Step* st, cudaStream_t stream,
@@ -815,11 +821,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   f.routed_count = routed_count_dev;
   f.ticket = ctx->ticket;
   f.status = ctx->status;
-  if (ctx->classes > 1 && plan.path == TLR_PATH_TC) {
-    f.tie_W = static_cast<const unsigned short*>(ctx->W);
-    f.tie_h = static_cast<const unsigned short*>(h_bf16_dev);
-    f.tie_d = ctx->d;
-  }
+  if (plan.path == TLR_PATH_TC) f.ties = ties_of(ctx, h_bf16_dev);
   f.status_copy = status_copy;
   if (tlr::launch_finish(f, stream) != cudaSuccess) return TLR_ERR_CUDA;
   return TLR_OK;
@@ -842,8 +844,8 @@ tlr_status tlr_shard_summary(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, in
   const tlr_plan& plan = st->plan;
   const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream);
   if (ps != TLR_OK) return ps;
-  if (tlr::launch_shard_summary(ctx->partials, n, plan.vocab_chunks, v_offset, static_cast<Partial*>(summary_dev),
-                                stream) != cudaSuccess)
+  if (tlr::launch_shard_summary(ctx->partials, n, plan.vocab_chunks, v_offset, ties_of(ctx, h_bf16_dev),
+                                static_cast<Partial*>(summary_dev), stream) != cudaSuccess)
     return TLR_ERR_CUDA;
   return TLR_OK;
 }
@@ -966,6 +968,7 @@ tlr_status tlr_shard_push(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, int32
   a.n = n;
   a.chunks = chunks;
   a.v_offset = v_offset;
+  a.ties = ties_of(ctx, h_bf16_dev);
   a.shards = ctx->shard_count;
   a.peer_slot = ctx->peer_slot[q];
   a.peer_flag = ctx->peer_flag[q];

@@ -132,6 +132,63 @@ __device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int c
   return r;
 }
 
+// Hidden sizes that are no multiple of 8 on the tensor cores: equal rows of W in different residue classes get logits that
+// agree to rounding only, so near-ties are settled by dot products of their own.
+struct Ties {
+  const unsigned short* W;   // bf16 [V][d]; null = not needed
+  const unsigned short* h;   // bf16 [n][d]
+  int d;
+};
+
+// The logit of token v in the row h by the L lanes of a row (lane gl of them, mask `group`), summed in fp32 in one fixed
+// order: equal rows of W give equal bits, whatever kernel, shard or GPU asks with the same L.
+__device__ __forceinline__ float row_logit(const unsigned short* __restrict__ W, const unsigned short* __restrict__ h, int d,
+                                           int v, int gl, int L, unsigned int group) {
+  const unsigned short* w = W + static_cast<size_t>(v) * d;
+  float z = 0.f;
+  for (int k = gl; k < d; k += L)
+    z = fmaf(__uint_as_float(static_cast<uint32_t>(h[k]) << 16), __uint_as_float(static_cast<uint32_t>(w[k]) << 16), z);
+  for (int off = L >> 1; off > 0; off >>= 1) z += __shfl_xor_sync(group, z, off);
+  return z;
+}
+
+// The token of a row whose maximum m (at idx) may be tied with another partial's: the candidates within the rounding of m
+// are compared by row_logit, so equal rows of W tie exactly and the lowest index wins.  Called by the L lanes of a row (lane
+// gl of them); rarely more than a look at the maxima.
+static __device__ __noinline__ int settle_ties(const Ties ties, int row, const Partial* __restrict__ p, int chunks,
+                                               int chunk_stride, float m, int idx, int gl, int L) {
+  const unsigned short* h = ties.h + static_cast<size_t>(row) * ties.d;
+  const unsigned int lane = threadIdx.x & 31;
+  const unsigned int group = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (lane - gl);
+  const float least = m - (1e-3f + 1e-5f * fabsf(m));
+  int near = 0;
+  for (int j = gl; j < chunks; j += L) near += __ldcg(&p[static_cast<size_t>(j) * chunk_stride].m) >= least ? 1 : 0;
+  for (int off = L >> 1; off > 0; off >>= 1) near += __shfl_xor_sync(group, near, off);
+  if (near < 2) return idx;
+  float best = -INFINITY;
+  int token = idx;
+  for (int j0 = 0; j0 < chunks; j0 += L) {
+    const int j = j0 + gl;
+    int mine = kNoToken;
+    if (j < chunks) {
+      const Partial* q = p + static_cast<size_t>(j) * chunk_stride;
+      if (__ldcg(&q->m) >= least) mine = __ldcg(&q->idx);
+    }
+    unsigned int todo = __ballot_sync(group, mine != kNoToken) & group;
+    while (todo != 0u) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int v = __shfl_sync(group, mine, src);
+      const float z = row_logit(ties.W, h, ties.d, v, gl, L, group);
+      if (z > best || (z == best && v < token)) {
+        best = z;
+        token = v;
+      }
+    }
+  }
+  return token;
+}
+
 // Host-side launchers (one per .cu file).  All enqueue on `stream` and return the
 // launch error, if any.
 struct SimtLaunch {
@@ -173,24 +230,21 @@ struct FinishLaunch {
   int32_t* routed_count;
   unsigned int* ticket;     // zero before the launch; the kernel leaves it zero again
   uint32_t* status;
-  // d no multiple of 8 on the tensor cores: equal rows of W in different residue classes get logits that agree to
-  // rounding only, so near-ties between partials are settled by dot products of their own (null = not needed)
-  const unsigned short* tie_W;   // bf16 [V][tie_d]
-  const unsigned short* tie_h;   // bf16 [n][tie_d]
-  int tie_d;
+  Ties ties;
   uint32_t* status_copy;    // optional: receives the status word once every row is scored (host-mapped memory)
 };
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream);
 
 // Vocabulary-sharded decode (tlr_shard.cu): one summary per row from a shard's chunk partials,
 // and the gathered summaries [shards][n] laid out as partials [n][shards].
-cudaError_t launch_shard_summary(const Partial* partials, int n, int chunks, int v_offset, Partial* summary,
-                                 cudaStream_t stream);
+cudaError_t launch_shard_summary(const Partial* partials, int n, int chunks, int v_offset, const Ties& ties,
+                                 Partial* summary, cudaStream_t stream);
 // Fused exchange: the summaries are stored straight into slot `rank` of every peer's exchange block and, once all
 // rows are out, this rank's flag in every peer's flag array is set to `epoch` (peer stores only).
 struct ShardPush {
   const Partial* partials;   // this shard's chunk partials [n][chunks]
   int n, chunks, v_offset;
+  Ties ties;
   int shards;                // peers, this rank included
   Partial* const* peer_slot; // device array [shards]: where this rank's n summaries go on peer g
   uint32_t* const* peer_flag;  // device array [shards]: this rank's flag on peer g

@@ -27,48 +27,6 @@ constexpr int kFinishThreads = kFinishWarps * 32;
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallRows = 1024;
 
-// The token of a row whose maximum m (at idx) may be tied with another partial's, see FinishLaunch::tie_W: the
-// candidates within the rounding of m are compared by fp32 dot products that all sum in the same order, so equal rows
-// of W tie exactly and the lowest index wins.  Called by the L lanes of a row (lane gl of them); rarely more than a
-// look at the maxima.
-__device__ __noinline__ int settle_ties(const unsigned short* __restrict__ W, const unsigned short* __restrict__ h, int d,
-                                        const Partial* __restrict__ p, int chunks, int chunk_stride, float m, int idx,
-                                        int gl, int L) {
-  const unsigned int lane = threadIdx.x & 31;
-  const unsigned int group = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (lane - gl);
-  const float least = m - (1e-3f + 1e-5f * fabsf(m));
-  int near = 0;
-  for (int j = gl; j < chunks; j += L) near += __ldcg(&p[static_cast<size_t>(j) * chunk_stride].m) >= least ? 1 : 0;
-  for (int off = L >> 1; off > 0; off >>= 1) near += __shfl_xor_sync(group, near, off);
-  if (near < 2) return idx;
-  float best = -INFINITY;
-  int token = idx;
-  for (int j0 = 0; j0 < chunks; j0 += L) {
-    const int j = j0 + gl;
-    int mine = kNoToken;
-    if (j < chunks) {
-      const Partial* q = p + static_cast<size_t>(j) * chunk_stride;
-      if (__ldcg(&q->m) >= least) mine = __ldcg(&q->idx);
-    }
-    unsigned int todo = __ballot_sync(group, mine != kNoToken) & group;
-    while (todo != 0u) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int v = __shfl_sync(group, mine, src);
-      const unsigned short* w = W + static_cast<size_t>(v) * d;
-      float z = 0.f;
-      for (int k = gl; k < d; k += L)
-        z = fmaf(__uint_as_float(static_cast<uint32_t>(h[k]) << 16), __uint_as_float(static_cast<uint32_t>(w[k]) << 16), z);
-      for (int off = L >> 1; off > 0; off >>= 1) z += __shfl_xor_sync(group, z, off);
-      if (z > best || (z == best && v < token)) {
-        best = z;
-        token = v;
-      }
-    }
-  }
-  return token;
-}
-
 // Scores and decision of one row from its folded summary.
 struct Scored {
   int token, flag;
@@ -303,8 +261,7 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
       t += __shfl_xor_sync(0xffffffffu, t, off);
     }
     if (kTies && valid)
-      idx = settle_ties(a.tie_W, a.tie_h + static_cast<size_t>(row) * a.tie_d, a.tie_d, p, a.chunks, a.chunk_stride, m, idx,
-                        gl, L);
+      idx = settle_ties(a.ties, row, p, a.chunks, a.chunk_stride, m, idx, gl, L);
     if (valid && gl == 0) {
       Partial acc;
       acc.m = m;
@@ -367,9 +324,7 @@ finish_kernel(const FinishLaunch a) {
   if (row < a.n) {
     const Partial* p = a.partials + static_cast<size_t>(row) * a.row_stride;
     Partial acc = fold_row(p, a.chunks, a.chunk_stride, lane);
-    if (a.tie_W != nullptr)
-      acc.idx = settle_ties(a.tie_W, a.tie_h + static_cast<size_t>(row) * a.tie_d, a.tie_d, p, a.chunks, a.chunk_stride,
-                            acc.m, acc.idx, lane, 32);
+    if (a.ties.W != nullptr) acc.idx = settle_ties(a.ties, row, p, a.chunks, a.chunk_stride, acc.m, acc.idx, lane, 32);
     if (lane == 0) store_row(score_row(acc, a, row), a, row);
   }
 
@@ -452,7 +407,7 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     cfg.numAttrs = 2;
     cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
     cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
-    return cudaLaunchKernelEx(&cfg, a.tie_W != nullptr ? finish_small_kernel<true> : finish_small_kernel<false>, a, log2_L);
+    return cudaLaunchKernelEx(&cfg, a.ties.W != nullptr ? finish_small_kernel<true> : finish_small_kernel<false>, a, log2_L);
   }
   const int blocks = (a.n + kFinishWarps - 1) / kFinishWarps;
   cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);

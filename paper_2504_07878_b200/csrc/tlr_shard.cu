@@ -25,15 +25,27 @@ namespace {
 constexpr int kWarps = 8;
 
 // One warp folds one row's chunk partials; every lane ends with the result.
+// kTies (d no multiple of 8): the shard's winner is settled among the residue classes, and m becomes its row_logit, so that
+// equal rows of W in different shards tie exactly in the merge behind -- also where one shard ran on CUDA cores and another
+// on tensor cores.  s and t stay as they are: all logits of the shard move with m, by no more than its rounding, and the
+// winner's own term stays exactly 1.
+template <bool kTies>
 __device__ __forceinline__ Partial row_summary(const Partial* __restrict__ partials, int row, int chunks, int v_offset,
-                                               int lane) {
-  Partial acc = fold_row(partials + static_cast<size_t>(row) * chunks, chunks, 1, lane);
+                                               const Ties& ties, int lane) {
+  const Partial* p = partials + static_cast<size_t>(row) * chunks;
+  Partial acc = fold_row(p, chunks, 1, lane);
+  if (kTies && acc.idx != kNoToken) {
+    acc.idx = settle_ties(ties, row, p, chunks, 1, acc.m, acc.idx, lane, 32);
+    const float z = row_logit(ties.W, ties.h + static_cast<size_t>(row) * ties.d, ties.d, acc.idx, lane, 32, 0xffffffffu);
+    if (fabsf(z) < INFINITY) acc.m = z;      // (a row that is not finite is left as the projection found it)
+  }
   if (acc.idx != kNoToken) acc.idx += v_offset;
   return acc;
 }
 
+template <bool kTies>
 __global__ void __launch_bounds__(kWarps * 32)
-shard_summary_kernel(const Partial* __restrict__ partials, int n, int chunks, int v_offset,
+shard_summary_kernel(const Partial* __restrict__ partials, int n, int chunks, int v_offset, const Ties ties,
                      Partial* __restrict__ summary) {
   const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -42,10 +54,11 @@ shard_summary_kernel(const Partial* __restrict__ partials, int n, int chunks, in
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row >= n) return;
-  const Partial acc = row_summary(partials, row, chunks, v_offset, lane);
+  const Partial acc = row_summary<kTies>(partials, row, chunks, v_offset, ties, lane);
   if (lane == 0) summary[row] = acc;
 }
 
+template <bool kTies>
 __global__ void __launch_bounds__(kWarps * 32)
 shard_push_kernel(const ShardPush a) {
   const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
@@ -55,7 +68,7 @@ shard_push_kernel(const ShardPush a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row < a.n) {
-    const Partial acc = row_summary(a.partials, row, a.chunks, a.v_offset, lane);
+    const Partial acc = row_summary<kTies>(a.partials, row, a.chunks, a.v_offset, a.ties, lane);
     for (int g = lane; g < a.shards; g += 32) a.peer_slot[g][row] = acc;     // lane g stores to peer g
   }
   // every summary of this block is on its way; the last block to get here publishes the flags
@@ -97,8 +110,8 @@ rows_merge_kernel(const int32_t* __restrict__ gathered_idx, const int32_t* __res
 
 }  // namespace
 
-cudaError_t launch_shard_summary(const Partial* partials, int n, int chunks, int v_offset, Partial* summary,
-                                 cudaStream_t stream) {
+cudaError_t launch_shard_summary(const Partial* partials, int n, int chunks, int v_offset, const Ties& ties,
+                                 Partial* summary, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>((n + kWarps - 1) / kWarps), 1, 1);
@@ -109,7 +122,8 @@ cudaError_t launch_shard_summary(const Partial* partials, int n, int chunks, int
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, shard_summary_kernel, partials, n, chunks, v_offset, summary);
+  const auto kernel = ties.W != nullptr ? shard_summary_kernel<true> : shard_summary_kernel<false>;
+  return cudaLaunchKernelEx(&cfg, kernel, partials, n, chunks, v_offset, ties, summary);
 }
 
 cudaError_t launch_shard_push(const ShardPush& a, cudaStream_t stream) {
@@ -123,7 +137,7 @@ cudaError_t launch_shard_push(const ShardPush& a, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, shard_push_kernel, a);
+  return cudaLaunchKernelEx(&cfg, a.ties.W != nullptr ? shard_push_kernel<true> : shard_push_kernel<false>, a);
 }
 
 cudaError_t launch_rows_merge(const int32_t* gathered_idx, const int32_t* counts, const int32_t* row_offsets,

@@ -16,6 +16,9 @@ from __future__ import annotations
 import numpy as np
 import torch
 
+import tlr_synth as S
+from oracle import route_oracle as O
+
 ABS_TOL = 1e-3
 REL_TOL = 1e-3
 GAP_TOL = 1e-3
@@ -96,3 +99,23 @@ def run_gpu(P, W_dev, h_cpu, tau, path=None, max_n=None, poison=True):
            "plan": P.tlr_plan_query(router.ctx, n)}
     router.close()
     return out
+
+
+def head_with_equal_rows(n, d, V):
+    """A head whose winning rows have copies at both ends of the vocabulary (in other residue classes and shards), hidden
+    states, the oracle's tokens, and the rows on which these are sure: the best row that is no copy of the winner is more
+    than 1e-3 behind."""
+    W = S.make_W(d, V, seed=d, std=0.2)
+    hid = S.make_h(n, d, seed=n, W=W, planted_fraction=0.5)
+    winners = np.unique(O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W), 0.5).token)
+    W2 = W.clone()
+    for k, v in enumerate(winners[:200].tolist()):
+        W2[(5 * k) % (V // 3)] = W[v]
+        W2[V - 1 - (7 * k) % (V // 3)] = W[v]
+    token = O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W2), 0.5).token
+    exact = O.bf16_bits_to_f64(S.bf16_bits(hid.h)) @ O.bf16_bits_to_f64(S.bf16_bits(W2)).T
+    top = exact.max(axis=1, keepdims=True)
+    runner = np.where(exact >= top - 1e-9, -np.inf, exact).max(axis=1)
+    sure = top[:, 0] - runner > 1e-3
+    assert sure.sum() >= n // 2
+    return W2, hid.h, token, sure

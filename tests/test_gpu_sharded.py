@@ -8,12 +8,12 @@ import torch
 
 import tlr_synth as S
 from oracle import route_oracle as O
-from tests.parity import check_against_oracle, check_self_consistency, run_gpu, to_np
+from tests.parity import check_against_oracle, check_self_consistency, head_with_equal_rows, run_gpu, to_np
 
 pytestmark = pytest.mark.gpu
 
 
-def run_sharded(P, W, h_cpu, tau, shards):
+def run_sharded(P, W, h_cpu, tau, shards, cuda_core_shard=None):
     n, V = h_cpu.shape[0], W.shape[0]
     h = h_cpu.cuda()
     Wd = W.cuda()
@@ -21,6 +21,8 @@ def run_sharded(P, W, h_cpu, tau, shards):
     for g in range(shards):
         v0, v1 = P.shard_bounds(V, shards, g)
         r = P.VocabShardedRouter(Wd[v0:v1], v0, max_n=n, world=shards)
+        if g == cuda_core_shard:
+            P.tlr_set_path(r.ctx, P.TLR_PATH_SIMT)
         parts.append(r.summarize(h).clone())
         routers.append(r)
     gathered = torch.stack(parts).contiguous()            # [shards, n, 4], rank-major like the all-gather
@@ -91,6 +93,20 @@ def test_tie_across_shards_goes_to_the_lower_index(pkg):
     h = W[100:101].clone().repeat(5, 1)
     gpu = run_sharded(pkg, W, h, 0.5, 4)
     assert np.all(gpu["token"] == 100)
+
+
+# d no multiple of 8: equal rows lie in different residue classes and in different shards, and one shard may run on CUDA
+# cores; 2, 4 and 8 classes, fewer and more rows than the merge kernel's small form takes
+@pytest.mark.parametrize("n,d,shards,cuda_core_shard", [(40, 63, 3, None), (40, 130, 4, None), (40, 300, 2, None),
+                                                        (40, 65, 3, 1), (1100, 63, 3, None)])
+def test_equal_rows_of_odd_sized_heads_tie_to_the_lowest_global_index(pkg, n, d, shards, cuda_core_shard):
+    W, h, token, sure = head_with_equal_rows(n, d, 3001)
+    gpu = run_sharded(pkg, W, h, 0.5, shards, cuda_core_shard)
+    assert gpu["status"] == 0
+    assert np.array_equal(gpu["token"][sure], token[sure])
+    ref = O.route_oracle(S.bf16_bits(h), S.bf16_bits(W), 0.5)
+    check_self_consistency(gpu, 0.5, W.shape[0])
+    check_against_oracle(ref, gpu, O.bf16_bits_to_f64(S.bf16_bits(h)), O.bf16_bits_to_f64(S.bf16_bits(W)))
 
 
 def test_shard_argument_errors(pkg):

@@ -12,7 +12,7 @@ import torch
 
 import tlr_synth as S
 from oracle import route_oracle as O
-from tests.parity import check_against_oracle, check_self_consistency, to_np
+from tests.parity import check_against_oracle, check_self_consistency, head_with_equal_rows, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -83,6 +83,24 @@ def test_fused_exchange_matches_oracle_for_two_calls_in_a_row(pkg, n, d, V, shar
         assert np.array_equal(gpu["routed_idx"][:gpu["routed_count"]], want["routed_idx"][:gpu["routed_count"]])
     for r in ranks:
         r.close()
+
+
+@pytest.mark.parametrize("n,d,shards", [(40, 63, 3), (40, 130, 4), (1100, 300, 2)])
+def test_equal_rows_of_odd_sized_heads_tie_to_the_lowest_global_index(pkg, n, d, shards):
+    W, h, token, sure = head_with_equal_rows(n, d, 3001)
+    ranks, block = make_ranks(pkg, W.cuda(), n, shards)
+    hd = h.cuda()
+    for r in ranks:
+        r.push(hd)
+    poison(ranks[0])
+    ranks[0].finish(n, 0.5)
+    torch.cuda.synchronize()
+    gpu = outputs(ranks[0], n)
+    for r in ranks:
+        assert pkg.tlr_last_device_status(r.ctx) == 0
+        r.close()
+    assert np.array_equal(gpu["token"][sure], token[sure])
+    check_self_consistency(gpu, 0.5, W.shape[0])
 
 
 def test_a_flag_that_is_never_set_runs_the_wait_out_and_the_context_survives(pkg):
