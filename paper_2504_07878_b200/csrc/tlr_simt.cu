@@ -14,10 +14,6 @@ namespace tlr {
 constexpr int kSimtThreads = 128;
 constexpr int kRows = 8;
 
-__device__ __forceinline__ float bf16_bits_to_float(unsigned short b) {
-  return __uint_as_float(((unsigned int)b) << 16);
-}
-
 // Fold one logit into a running summary (z is visited in ascending vocabulary order
 // per thread, so a strict comparison keeps the lowest index on ties).
 __device__ __forceinline__ void fold(Partial& p, float z, int v) {
@@ -99,9 +95,9 @@ simt_projection_kernel(const SimtLaunch a) {
     } else {
 #pragma unroll 4
       for (int k = 0; k < d; ++k) {
-        const float w = bf16_bits_to_float(wrow[k]);
+        const float w = bf16_value(wrow[k]);
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) acc[r] = fmaf(bf16_bits_to_float(hs[r * d + k]), w, acc[r]);
+        for (int r = 0; r < kRows; ++r) acc[r] = fmaf(bf16_value(hs[r * d + k]), w, acc[r]);
       }
     }
 #pragma unroll

@@ -66,6 +66,51 @@ def test_equal_rows_of_different_classes_tie_to_the_lowest_index(pkg, n, d):
     assert np.array_equal(gpu["token"][sure], ref.token[sure])
 
 
+# Rows of (nearly) equal logits, as padding leaves them: every partial is a candidate for the maximum.
+@pytest.mark.parametrize("n,d,V", [(3, 63, 3001), (40, 130, 3001), (300, 7, 9000), (1100, 300, 3001)])
+def test_rows_of_equal_logits(pkg, n, d, V):
+    W = S.make_W(d, V, seed=d, std=0.2)
+    h = S.make_h(n, d, seed=n).h
+    h[n // 2] = 0                                          # every logit is zero
+    h[n - 1] = (h[n - 1].float() * 1e-5).to(h.dtype)       # every logit within 1e-3 of the others
+    gpu = check(pkg, W, h, 0.5)
+    assert gpu["token"][n // 2] == 0 and abs(gpu["conf"][n // 2] * V - 1) <= 1e-5
+    z = O.bf16_bits_to_f64(S.bf16_bits(h[n - 1:]))[0] @ O.bf16_bits_to_f64(S.bf16_bits(W)).T
+    assert z.max() - z[gpu["token"][n - 1]] <= 1e-6 * np.abs(z).max()     # fp32 sums of exact products settle it
+
+
+@pytest.mark.parametrize("scale", [0.0, 1e-5])
+def test_a_row_of_equal_logits_does_not_hold_up_the_step(pkg, scale):
+    n, d, V, calls = 16, 300, 33000, 20
+    W, h = S.make_W(d, V, seed=1, std=0.06).cuda(), S.make_h(n, d, seed=2).h.cuda()
+    padded = h.clone()
+    padded[5] = padded[5].float() * scale
+    r = pkg.Router(W, max_n=n)
+    stream = torch.cuda.Stream()
+    times = []
+    with torch.cuda.stream(stream):
+        for x in (h, padded):
+            r.route(x, 0.5)
+            stream.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                for _ in range(calls):
+                    r.route(x, 0.5)
+            took = []
+            for _ in range(7):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                graph.replay()
+                b.record()
+                stream.synchronize()
+                took.append(a.elapsed_time(b))
+            times.append(sorted(took)[3])
+            del graph
+    r.close()
+    # with every partial a candidate it was 27 times as long
+    assert times[1] <= 3 * times[0], times
+
+
 def test_learned_router_and_host_buffers(pkg):
     n, d, V, dh = 70, 100, 3000, 48
     W = S.make_W(d, V, seed=1, std=0.1)
