@@ -271,7 +271,8 @@ def tlr_last_device_status(ctx) -> int:
 
 
 def tlr_debug_inject(ctx, kind: int, wait_limit_ms: int = 0):
-    """Test hook: kind=1 drops the W copies of the next calls so a bounded wait runs out; kind=0 restores."""
+    """Test hook: kind=1 drops the W copies of the next calls so a bounded wait runs out; kind=2 makes the
+    encoding of tensor maps fail; kind=0 restores."""
     _check(load_library().tlr_debug_inject(ctx, kind, wait_limit_ms), "tlr_debug_inject")
 
 

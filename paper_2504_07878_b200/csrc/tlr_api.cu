@@ -201,6 +201,7 @@ struct tlr_ctx {
     tlr::TcParams params;     // all but the per-call fields
     tlr::TcMaps maps;
     tlr::OddMaps odd;         // d no multiple of 8: these instead
+    bool odd_encoded = false;
     int odd_block = 0;        // rows of h per projection launch then
     const void* h_mapped = nullptr;   // the address maps.h was encoded for
     const void* h_other = nullptr;    // ... and the address before that, with its map (two staging buffers alternate)
@@ -226,6 +227,7 @@ namespace {
 
 // Rows of `cols` e4m3 bytes, boxes of 128 bytes x box_rows, 128-byte swizzle.
 bool make_map8(tlr_ctx* c, CUtensorMap* map, const void* base, int rows, int cols, int box_rows) {
+  if (c->debug_kind == 2) return false;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols)};
   const cuuint32_t box[2] = {128u, static_cast<cuuint32_t>(box_rows)};
@@ -238,6 +240,7 @@ bool make_map8(tlr_ctx* c, CUtensorMap* map, const void* base, int rows, int col
 
 bool make_map(const tlr_ctx* c, CUtensorMap* map, const void* base, int rows, int cols, int box_rows,
               long long pitch = 0) {     // elements from row to row, 0 = cols
+  if (c->debug_kind == 2) return false;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch != 0 ? pitch : cols) * 2};
   const cuuint32_t box[2] = {64u, static_cast<cuuint32_t>(box_rows)};
@@ -329,7 +332,8 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
       p.d = c->d + tlr::odd_max_shift(c->d);
       p.h_class_rows = c->odd_rows;
       for (int r = 0; r < c->classes; ++r) st->odd.w[r] = c->map_cls[r];
-      if (n > 0) make_map(c, &st->odd.h, c->h_shift, c->classes * c->odd_rows, c->odd_pitch, tlr::tc_h_box_rows(cfg));
+      st->odd_encoded = n > 0 && make_map(c, &st->odd.h, c->h_shift, c->classes * c->odd_rows, c->odd_pitch,
+                                          tlr::tc_h_box_rows(cfg));
       return;
     }
     st->maps.w128 = c->map_w128;
@@ -484,6 +488,10 @@ tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ct
     st->params.late_trigger = router_beside ? 1 : 0;
     e = tlr::launch_tc8_projection(st->maps, st->params, cfg, st->workers, stream);
   } else if (st->plan.path == TLR_PATH_TC && ctx->classes > 1) {
+    if (!st->odd_encoded) {
+      st->n = -1;          // planned again by the next call
+      return TLR_ERR_CUDA;
+    }
     const int units_max = ctx->sm_count / st->cfg.cta;
     e = cudaSuccess;
     for (int row0 = 0; row0 < n && e == cudaSuccess; row0 += st->odd_block) {
@@ -709,7 +717,7 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
 }
 
 tlr_status tlr_debug_inject(tlr_ctx* ctx, int32_t kind, uint32_t wait_limit_ms) {
-  if (ctx == nullptr || (kind != 0 && kind != 1)) return TLR_ERR_ARG;
+  if (ctx == nullptr || kind < 0 || kind > 2) return TLR_ERR_ARG;
   ctx->debug_kind = kind;
   ctx->debug_wait_ns = static_cast<unsigned long long>(wait_limit_ms) * 1000000ull;
   forget_steps(ctx);

@@ -76,3 +76,28 @@ def test_wait_runs_out_on_the_8bit_head(pkg):
     assert pkg.tlr_last_device_status(r.ctx) == 0
     assert np.array_equal(good[0], again[0]) and np.array_equal(good[1], again[1]) and good[2] == again[2]
     r.close()
+
+
+# d a multiple of 8, no multiple of 8 (one CTA per worker / a pair), the 8-bit head
+@pytest.mark.parametrize("n,d,fp8", [(48, 128, False), (48, 100, False), (300, 101, False), (48, 128, True)])
+def test_a_tensor_map_that_cannot_be_encoded_is_an_error(pkg, n, d, fp8):
+    V = 4000
+    W, scale = S.make_W8(d, V, seed=2, std=0.1) if fp8 else (S.make_W(d, V, seed=2, std=0.1), None)
+    h = S.make_h(n, d, seed=3).h.cuda()
+    r = pkg.Router(W.cuda(), max_n=n, wscale=None if scale is None else scale.cuda())
+    r.route(h, 0.5)
+    torch.cuda.synchronize()
+    good = to_np(r.token[:n]).copy()
+    pkg.tlr_debug_inject(r.ctx, 2)
+    for _ in range(2):
+        with pytest.raises(pkg.TlrError) as e:
+            r.route(h, 0.5)
+        assert e.value.code == 4
+    torch.cuda.synchronize()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    pkg.tlr_debug_inject(r.ctx, 0)
+    r.token.fill_(-1)
+    r.route(h, 0.5)
+    torch.cuda.synchronize()
+    assert np.array_equal(to_np(r.token[:n]), good)
+    r.close()
