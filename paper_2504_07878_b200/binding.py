@@ -335,16 +335,22 @@ class Router:
             self.route_mask = torch.empty(max_n, dtype=torch.uint8, device=dev)
             self.routed_idx = torch.empty(max_n, dtype=torch.int32, device=dev)
             self.routed_count = torch.zeros(1, dtype=torch.int32, device=dev)
-        self._views = {}                # n -> views of the output tensors for n rows (making four costs 6 us)
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        if name in ("token", "conf", "entropy", "route_mask"):
+            object.__setattr__(self, "_views", {})        # batch size -> views of these four tensors
 
     def _outputs(self, n: int):
-        views = self._views.get(n)
-        if views is None:
+        """Views of the output tensors for n rows, new objects on every call.  (`.data` of a view that is kept makes one
+        in a quarter of the time that a slice takes: n = 1, d = 256, V = 20000 8.6 us per call against 13.3.)"""
+        kept = self._views.get(n)
+        if kept is None:
             if len(self._views) >= 16:
                 self._views.clear()
-            views = self._views[n] = (self.token[:n], self.conf[:n], self.entropy[:n], self.route_mask[:n],
-                                      self.routed_idx, self.routed_count)
-        return views
+            kept = self._views[n] = (self.token[:n], self.conf[:n], self.entropy[:n], self.route_mask[:n])
+        token, conf, entropy, route_mask = kept
+        return token.data, conf.data, entropy.data, route_mask.data, self.routed_idx, self.routed_count
 
     def set_router_mlp(self, W1: torch.Tensor, b1: torch.Tensor, w2: torch.Tensor, b2: float):
         """Attach a learned router; the tensors are kept alive by this object."""
