@@ -54,7 +54,8 @@ typedef enum {
 /* Which projection kernel a call of n rows uses. */
 typedef enum {
   TLR_PATH_AUTO = 0,   /* choose by shape (default) */
-  TLR_PATH_SIMT = 1,   /* CUDA-core kernel: any d, any V (diagnostics) */
+  TLR_PATH_SIMT = 1,   /* CUDA-core kernel: any d, any V; AUTO takes it for tiny heads with d <= 36, d % 8 != 0 and at most 32
+                        * rows, tlr_route_static whenever d % 8 != 0, and it can be asked for (diagnostics) */
   TLR_PATH_TC = 2      /* tcgen05 tensor-core kernel fed by TMA; when d % 8 != 0 W is read by residue classes of its rows */
 } tlr_path;
 

@@ -251,13 +251,15 @@ bool make_map(const tlr_ctx* c, CUtensorMap* map, const void* base, int rows, in
   return r == CUDA_SUCCESS;
 }
 
-// Tensor cores wherever their set-up succeeded.  The one exception: a small batch on a head of at most 128 KB whose d is
-// no multiple of 8.  The tensor-core path needs a third launch there, for the shifted copies of h, which costs the
-// host 2 us and buys next to nothing on the device: n = 20, d = 36, V = 1500 13.1 us on CUDA cores and 9.1 on tensor
-// cores, n = 1, d = 9, V = 700 10.4 and 7.9; on larger heads it buys everything (n = 64, d = 300, V = 33000 194 and 14).
+// Tensor cores wherever their set-up succeeded.  The one exception, a small batch on a head of at most 128 KB whose d <= 36 is
+// no multiple of 8, is not for speed: such a call has two launches and reports the CUDA-core path since the first version of
+// tlr_plan_query, and keeps both because they cost little.  Per step in a stream of calls (in a graph), CUDA cores and tensor
+// cores: n = 16, d = 9, V = 700 11.4 and 10.3 us (10.9 and 7.7), n = 16, d = 36, V = 1500 13.9 and 10.6 (13.1 and 7.9).  One
+// thread walks a whole row of W there, so that the cost grows with d: d = 63, V = 1000 16.4 and 10.5, d = 300, V = 200 33.5
+// and 10.3, d = 2047, V = 32 163 and 18.
 tlr_path pick_path(const tlr_ctx* c, int n) {
   if (c->forced != TLR_PATH_AUTO) return c->forced;
-  const bool tiny = c->classes > 1 && n <= 32 && static_cast<long long>(c->V) * c->d <= 65536;
+  const bool tiny = c->classes > 1 && n <= 32 && c->d <= 36 && static_cast<long long>(c->V) * c->d <= 65536;
   return c->tc_ok && !tiny ? TLR_PATH_TC : TLR_PATH_SIMT;
 }
 

@@ -1,5 +1,5 @@
 // CUDA-core projection kernel: logits + online-softmax partials with plain FMAs.
-// Serves tiny heads whose hidden size is not a multiple of 8 (pick_path), every such head of the entry point without
+// Serves tiny heads whose hidden size is small and not a multiple of 8 (pick_path), every such head of the entry point without
 // a context (tlr_static.cu, which has no room for the shifted copies of h the tensor-core path needs), and is selectable for
 // diagnostics.  One thread owns one vocabulary row of a 128-row tile and kRows token
 // rows at a time; the block walks its vocabulary chunk tile by tile, each thread

@@ -142,3 +142,14 @@ def test_tiny_heads_keep_the_cuda_core_kernel(pkg):
         gpu = run_gpu(pkg, W.cuda(), hid.h, 0.01)
         assert gpu["plan"].path == path and gpu["status"] == 0
         check_against_oracle(ref, gpu)
+
+
+@pytest.mark.parametrize("n,d,V", [(1, 37, 100), (32, 60, 1000), (16, 300, 200), (9, 2047, 32)])
+def test_tiny_heads_with_long_rows_run_on_the_tensor_cores(pkg, n, d, V):
+    W = S.make_W(d, V, seed=n, std=0.1)
+    hid = S.make_h(n, d, seed=V)
+    ref = O.route_oracle(S.bf16_bits(hid.h), S.bf16_bits(W), 0.1)
+    for path in (None, 1):
+        gpu = run_gpu(pkg, W.cuda(), hid.h, 0.1, path=path)
+        assert gpu["plan"].path == (path or 2) and gpu["status"] == 0
+        check_against_oracle(ref, gpu)
