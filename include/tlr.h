@@ -68,7 +68,7 @@ typedef struct {
   int32_t vocab_chunks;  /* partial results per row that the merge step folds */
   int32_t smem_bytes;    /* dynamic shared memory per CTA */
   int32_t launches;      /* kernels launched per tlr_route call */
-  int32_t reserved;
+  int32_t reserved;      /* tlr_plan_query: 1 where a CTA pair keeps a row unit's h in shared memory for the whole unit */
 } tlr_plan;
 
 /* Bits of the device status word (tlr_last_device_status). */
@@ -85,7 +85,8 @@ typedef struct {
  *   max_n       largest n any later call will pass (>= 1).  Sizes the workspace.
  *   out         receives the context.
  * The only call that allocates device memory: the per-row partial-result workspace,
- * a status word, and two sets of staging buffers (device and pinned host) for tlr_route_host.  Uses the current CUDA device;
+ * a status word, two sets of staging buffers (device and pinned host) for tlr_route_host and, when d % 8 != 0,
+ * room for up to eight shifted copies of up to 2048 rows of h.  Uses the current CUDA device;
  * every later call on the context must be made with that device current.
  * Errors: TLR_ERR_ARG, TLR_ERR_ALIGN, TLR_ERR_UNSUPPORTED (not an sm_100 device),
  * TLR_ERR_NOMEM, TLR_ERR_CUDA.  On error *out is NULL and nothing is leaked.

@@ -310,6 +310,7 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     out->grid = st->workers * cfg.cta;
     out->block = tlr::tc_threads();
     out->smem_bytes = cfg.smem_bytes;
+    out->reserved = cfg.mode == tlr::RowMode::kM128Keep ? 1 : 0;
     p.n = n;
     p.d = c->d;
     p.V = c->V;

@@ -352,7 +352,33 @@ def test_pair_mode_keeps_h_for_a_unit(pkg, n, d, V):
     rows = np.unique(np.concatenate([np.arange(0, n, 7), np.arange(n - 140, n)]))
     ref = O.route_oracle(S.bf16_bits(hid.h)[rows], S.bf16_bits(W), 0.5)
     full = run_gpu(pkg, W.cuda(), hid.h, 0.5)
-    assert full["status"] == 0 and full["plan"].path == 2
+    assert full["status"] == 0 and full["plan"].path == 2 and full["plan"].reserved == 1      # h is kept
     check_self_consistency(full, 0.5, V)
     gpu = {k: full[k][rows] for k in ("token", "conf", "entropy", "route_mask")}
     check_against_oracle(ref, gpu)
+
+
+# The same with a learned router's units, whose number of tiles is their own, after the vocabulary's: one tile and several,
+# fewer and more than the vocabulary units have; several units per worker.
+@pytest.mark.parametrize("n,d,V,dh", [(1100, 200, 64000, 40), (1100, 256, 64000, 700), (4100, 576, 20000, 256),
+                                      (2049, 384, 34000, 1100)])
+def test_pair_mode_keeps_h_for_a_learned_routers_units(pkg, n, d, V, dh):
+    W = S.make_W(d, V, seed=n, std=0.08)
+    hid = S.make_h(n, d, seed=d, W=W, planted_fraction=0.1)
+    g = torch.Generator().manual_seed(dh)
+    W1 = (torch.randn(dh, d, generator=g) / d ** 0.5).to(torch.bfloat16)
+    b1, w2 = torch.randn(dh, generator=g) * 0.1, torch.randn(dh, generator=g) * 0.2
+    want = O.mlp_router_score(S.bf16_bits(hid.h), S.bf16_bits(W1), b1.numpy(), w2.numpy(), 0.2)
+    rows = np.unique(np.concatenate([np.arange(0, n, 13), np.arange(n - 140, n)]))
+    ref = O.route_oracle(S.bf16_bits(hid.h)[rows], S.bf16_bits(W), 0.5)
+    r = pkg.Router(W.cuda(), max_n=n)
+    r.set_router_mlp(W1.cuda(), b1.cuda(), w2.cuda(), 0.2)
+    assert pkg.tlr_plan_query(r.ctx, n).reserved == 1
+    score = torch.full((n,), float("nan"), device="cuda")
+    r.route(hid.h.cuda(), 0.5, mlp_score=score)
+    torch.cuda.synchronize()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    assert np.max(np.abs(score.cpu().numpy() - want)) <= 1e-5     # fp32 sums of exact products
+    gpu = {k: getattr(r, k).cpu().numpy()[rows] for k in ("token", "conf", "entropy", "route_mask")}
+    check_against_oracle(ref, gpu)
+    r.close()
