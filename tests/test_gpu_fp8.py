@@ -192,8 +192,8 @@ def test_fp8_fragment_edges(pkg, n, V):
 
 
 # The learned router beside the 8-bit projection: rows at the edges of the 16-row fragments, hidden units at the edges of
-# the groups of 8 and 32, K that ends inside a 32-wide step; 20 steps in a row on changing h, so that a score taken from
-# the step before (or a step ahead) would show.
+# the groups of 8 and 32, K that ends inside a 32-wide step; 20 steps in a row on one buffer whose contents change, so that
+# a score of a buffer's old contents would show.
 @pytest.mark.parametrize("n,d,dh", [(1, 16, 1), (8, 48, 7), (9, 32, 8), (16, 64, 33), (17, 80, 31), (33, 144, 64),
                                     (100, 2048, 256), (128, 896, 300)])
 def test_fp8_learned_router_beside_the_projection(pkg, n, d, dh):
@@ -217,4 +217,46 @@ def test_fp8_learned_router_beside_the_projection(pkg, n, d, dh):
         want = O.mlp_router_score(S.bf16_bits(hs[k]), S.bf16_bits(W1), b1.numpy(), w2.numpy(), -0.1)
         # exact products, fp32 sums of d and dh terms: far below 1e-5 on scores in [0, 1]
         assert np.max(np.abs(scores[k].cpu().numpy() - want)) <= 1e-5
+    r.close()
+
+
+# The router kernel writes its scores without waiting for the projection in front of it, which must not let it go ahead of
+# the step before: steps back to back with nothing between them, in a stream and in a graph, on a head so small that they
+# overlap (h split by the projection and by a kernel of its own; one MMA and two MMAs per K step).
+@pytest.mark.parametrize("n,d,dh", [(1, 64, 33), (16, 512, 256), (20, 512, 256), (100, 2048, 256), (128, 256, 512)])
+@pytest.mark.parametrize("graph", [False, True])
+def test_fp8_learned_router_steps_do_not_mix(pkg, n, d, dh, graph):
+    V, steps = 600, 60
+    codes, scale = S.make_W8(d, V, seed=3, std=0.1)
+    g = torch.Generator().manual_seed(dh + d)
+    W1 = (torch.randn(dh, d, generator=g) / d ** 0.5).to(torch.bfloat16)
+    b1, w2 = torch.randn(dh, generator=g) * 0.1, torch.randn(dh, generator=g) * 0.5
+    r = pkg.Router(codes.cuda(), max_n=n, wscale=scale.cuda())
+    r.set_router_mlp(W1.cuda(), b1.cuda(), w2.cuda(), -0.1)
+    hs = [S.make_h(n, d, seed=k).h for k in range(3)]
+    dev = [h.cuda() for h in hs]
+    scores = [torch.full((n,), float("nan"), device="cuda") for _ in range(steps)]
+
+    def run():
+        for k in range(steps):
+            r.route(dev[k % 3], 0.5, score_source=pkg.TLR_SCORE_MLP, mlp_score=scores[k])
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        run()
+        if graph:
+            stream.synchronize()
+            for s in scores:
+                s.fill_(float("nan"))
+            captured = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(captured, stream=stream):
+                run()
+            captured.replay()
+        stream.synchronize()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    for i, h in enumerate(hs):
+        want = O.mlp_router_score(S.bf16_bits(h), S.bf16_bits(W1), b1.numpy(), w2.numpy(), -0.1)
+        for k in range(i, steps, 3):
+            # exact products, fp32 sums of d and dh terms: far below 1e-5 on scores in [0, 1]
+            assert np.max(np.abs(scores[k].cpu().numpy() - want)) <= 1e-5
     r.close()
