@@ -46,7 +46,7 @@ struct TcPlan {
 
 struct TcParams {
   int n, d, V;
-  int row_units, chunks, granules, tiles_per_unit, full_tiles_first, granule_rows;
+  int row_units, chunks, tiles_per_unit, full_tiles_first, granule_rows;
   int chunk_q, chunk_r;               // granules of a chunk: chunk_q, and one more in chunk_r of them (of a class)
   uint32_t chunk_mul;                 // ceil(2^32 / chunks of a class), 0 for one chunk
   int full_granules;                  // granules of a full tile
@@ -103,7 +103,6 @@ inline int tc_h_box_rows(const TcConfig& c) { return c.mode == RowMode::kGroup8 
 inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
   p->row_units = plan.row_units;
   p->chunks = plan.chunks;
-  p->granules = plan.granules;
   p->tiles_per_unit = plan.tiles_per_unit;
   p->full_tiles_first = plan.full_tiles_first;
   p->granule_rows = plan.granule_rows;
