@@ -597,7 +597,7 @@ tlr_status tlr_create(int32_t d, int32_t V, const void* W_bf16_dev, int32_t max_
     for (int r = 0; r < c->classes && ok; ++r) {
       const int shift = tlr::odd_shift(d, r);
       const int rows = (V - r + c->classes - 1) / c->classes;
-      if (rows <= 0) {       // a vocabulary of fewer rows than classes: no unit ever loads this class
+      if (rows <= 0) {       // fewer rows than classes: this class's units load a stand-in and fold none of its columns
         c->map_cls[r] = c->map_cls[0];
         continue;
       }

@@ -160,7 +160,7 @@ extern "C" tlr_status tlr_route_static(int32_t d, int32_t V, const void* W_bf16_
       p.V = V;
       tlr::tc_set_schedule(tp, &p);
       p.a_rows = cfg.a_rows;
-        p.part_rows = cfg.part_rows;
+      p.part_rows = cfg.part_rows;
       p.a_stages = cfg.a_stages;
       p.b_stages = cfg.b_stages;
       // W is an argument of this call, so the kernel that precedes it in the stream may have written it:

@@ -21,8 +21,8 @@
 // bytes from HBM are half.
 //
 // This file holds what only the 8-bit head has: the split kernel, the shape of the launch and the
-// launch of tc8_projection_kernel (the <1, true> instantiation of the projection kernel's body in
-// tlr_tc_kernel.cuh; device helpers in tlr_tc8_dev.cuh).
+// launch of tc8_projection_kernel (the projection kernel's body in tlr_tc_kernel.cuh in the row modes
+// k8Small, k8Half and k8Wide; device helpers in tlr_tc8_dev.cuh).
 #include <cuda.h>
 #include <cuda_bf16.h>
 

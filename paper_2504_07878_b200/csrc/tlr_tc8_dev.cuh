@@ -101,7 +101,7 @@ __device__ __forceinline__ void split16(const uint4& lo, const uint4& hi, float 
 // loads are in flight together.
 constexpr int kSplitThreads = 288;
 constexpr int kSplitLanes = kSplitThreads / 16;       // threads per row
-constexpr int kSplitChunks = 6;                       // chunks of 16 elements per thread: d <= 16 * 18 * 6 = 1728
+constexpr int kSplitChunks = 6;                       // chunks of 16 elements per thread: 108 per row, 13 whole slabs of 8, d <= 1664
 __device__ __forceinline__ void split_h_resident(const __nv_bfloat16* __restrict__ hb, int n, int d, int k_slabs,
                                                  unsigned char* slabs, float* hs_s, int t) {
   const int r = t / kSplitLanes, l = t - r * kSplitLanes;

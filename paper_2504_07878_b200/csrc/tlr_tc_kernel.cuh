@@ -498,9 +498,9 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
           for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
             if (kKeep && t > 0) continue;      // (the first tile of a unit is never empty)
             if (!h_there) {
-              // here and not with the other warps above: the arithmetic of the first unit, two 64-bit divisions among it,
-              // would stand between the end of the wait and the first load of h, which the whole step waits for (n = 1,
-              // d = 256, V = 20000 9.43 -> 9.03 us per step in a stream, n = 256, d = 512, V = 32000 15.49 -> 14.86)
+              // here and not with the other warps above: the arithmetic of the first unit would stand between the end of the
+              // wait and the first load of h, which the whole step waits for (n = 1, d = 256, V = 20000 8.60 -> 8.18 us per
+              // step in a stream, n = 16, d = 512, V = 32000 10.53 -> 9.98, n = 256 there 14.76 -> 14.39)
               asm volatile("griddepcontrol.wait;" ::: "memory");
               h_there = true;
             }
