@@ -21,9 +21,10 @@ namespace {
 constexpr int kShiftThreads = 256;
 
 // Copy r of h has its rows `pitch` elements apart (a multiple of 8), each beginning with the class's shift in zeros.
-// One thread writes 16 bytes; the reads of h are 2 bytes wide (its rows have no alignment) and hit L1.
+// One thread writes 16 bytes; the reads of h are 2 bytes wide (its rows have no alignment) and hit L1.  (h is not
+// __restrict__: a copy kernel in front may still be writing it when this kernel starts, so it is not read-only data.)
 __global__ void __launch_bounds__(kShiftThreads)
-odd_shift_kernel(const unsigned short* __restrict__ h, int n, int d, int classes, int class_rows, int pitch,
+odd_shift_kernel(const unsigned short* h, int n, int d, int classes, int class_rows, int pitch,
                  unsigned short* __restrict__ out) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

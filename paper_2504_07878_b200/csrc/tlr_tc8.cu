@@ -36,7 +36,7 @@ namespace tlr {
 // One block per row of the padded batch (rows >= n are written as zeros): the row's power-of-two
 // scale r (largest |h| / r in [128, 256)), and h / r as the sum of two e4m3 arrays, [2][part_rows][d].
 __global__ void __launch_bounds__(128)
-h_split_kernel(const __nv_bfloat16* __restrict__ h, int n, int d, int part_rows, uint8_t* __restrict__ parts,
+h_split_kernel(const __nv_bfloat16* h, int n, int d, int part_rows, uint8_t* __restrict__ parts,
                float* __restrict__ hscale) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

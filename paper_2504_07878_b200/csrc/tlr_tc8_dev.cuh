@@ -115,8 +115,8 @@ __device__ __forceinline__ void split_h_resident(const __nv_bfloat16* __restrict
     vb[i] = va[i];
     if (r < n && c < valid_chunks) {
       const uint4* src = reinterpret_cast<const uint4*>(hb + static_cast<size_t>(r) * d + c * 16);
-      va[i] = __ldg(src);
-      vb[i] = __ldg(src + 1);
+      va[i] = __ldcg(src);        // (not the read-only path: h may still have been on its way when this kernel started)
+      vb[i] = __ldcg(src + 1);
     }
   }
 #pragma unroll

@@ -7,7 +7,7 @@ import torch
 
 import tlr_synth as S
 from oracle import route_oracle as O
-from tests.parity import check_against_oracle, check_self_consistency, run_gpu
+from tests.parity import check_against_oracle, check_self_consistency, run_gpu, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -248,6 +248,32 @@ def test_two_host_calls_in_flight(pkg):
     check(2, o)
     assert pkg.tlr_last_device_status(ctx) == 0
     pkg.tlr_destroy(ctx)
+
+
+# Heads whose first kernel rewrites h (shifted copies, two e4m3 parts in the projection or in a kernel of its own): two host
+# calls in flight on four batches in turn, every result bit for bit what the device-buffer call gives.
+@pytest.mark.parametrize("n,d,fp8", [(64, 300, False), (200, 100, False), (16, 896, True), (48, 512, True)])
+def test_host_calls_in_flight_on_odd_and_8bit_heads(pkg, n, d, fp8):
+    V, calls = 5000, 60
+    W, scale = S.make_W8(d, V, seed=3, std=0.1) if fp8 else (S.make_W(d, V, seed=3, std=0.1), None)
+    r = pkg.Router(W.cuda(), max_n=n, wscale=None if scale is None else scale.cuda())
+    hosts = [S.make_h(n, d, seed=k).h.pin_memory() for k in range(4)]
+    want = []
+    for h in hosts:
+        r.route(h.cuda(), 0.01)
+        torch.cuda.synchronize()
+        want.append([to_np(t).copy() for t in (r.token, r.conf, r.entropy, r.route_mask, r.routed_count)])
+    got = [torch.empty(n, dtype=torch.int32), torch.empty(n), torch.empty(n), torch.empty(n, dtype=torch.uint8),
+           torch.empty(n, dtype=torch.int32), torch.empty(1, dtype=torch.int32)]
+    pkg.tlr_route_host_submit(r.ctx, hosts[0], n, 0.01)
+    for i in range(1, calls + 1):
+        if i < calls:
+            pkg.tlr_route_host_submit(r.ctx, hosts[i % 4], n, 0.01)
+        pkg.tlr_route_host_collect(r.ctx, *got)
+        for a, b in zip(got[:4] + got[5:], want[(i - 1) % 4]):
+            assert np.array_equal(to_np(a), b)
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    r.close()
 
 
 def test_argument_errors(pkg):
