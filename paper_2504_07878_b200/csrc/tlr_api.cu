@@ -457,8 +457,8 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
 
 // What settles near-ties between rows of W in different residue classes (nothing where d is a multiple of 8).
 tlr::Ties ties_of(const tlr_ctx* c, const void* h_bf16_dev) {
-  if (c->classes == 1) return {nullptr, nullptr, 0};
-  return {static_cast<const unsigned short*>(c->W), static_cast<const unsigned short*>(h_bf16_dev), c->d};
+  if (c->classes == 1) return {nullptr, nullptr, 0, 0};
+  return {static_cast<const unsigned short*>(c->W), static_cast<const unsigned short*>(h_bf16_dev), c->d, c->V};
 }
 
 // Enqueues the projection kernel of a call with n > 0 rows: chunk partials into ctx->partials.  router_beside: the 8-bit

@@ -137,7 +137,7 @@ __device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int c
 struct Ties {
   const unsigned short* W;   // bf16 [V][d]; null = not needed
   const unsigned short* h;   // bf16 [n][d]
-  int d;
+  int d, V;
 };
 
 __device__ __forceinline__ float bf16_value(unsigned short bits) { return __uint_as_float(static_cast<uint32_t>(bits) << 16); }
@@ -162,7 +162,8 @@ __device__ __forceinline__ float row_logit(const unsigned short* __restrict__ W,
 // are compared by row_logit, so equal rows of W tie exactly and the lowest index wins.  Called by the L lanes of a row (lane
 // gl of them); rarely more than a look at the maxima, because a candidate costs an L2 trip.  Candidates are few: maxima that
 // agree to the bit need none (the merge has taken the lowest index), and the others are held against what rounding can do,
-// 2^-21 of the products' magnitudes per accumulation of 16 products and 8 more, twice.  With every maximum within 1e-3 a
+// 2^-21 of the products' magnitudes per accumulation of 16 products and 8 more, twice.  (An index can lie beyond V: the column
+// that stands for one there is -1e30, and wins where every logit is below that.)  With every maximum within 1e-3 a
 // candidate, a hidden state of zeros (padding) in the batch made a step of n = 16, d = 300, V = 33000 322 us long instead of
 // 11.9; now 11.9 (every hidden state scaled by 1e-5: 17.0).
 static __device__ __noinline__ int settle_ties(const Ties ties, int row, const Partial* __restrict__ p, int chunks,
@@ -177,7 +178,7 @@ static __device__ __noinline__ int settle_ties(const Ties ties, int row, const P
     near += other >= least && other != m ? 1 : 0;
   }
   for (int off = L >> 1; off > 0; off >>= 1) near += __shfl_xor_sync(group, near, off);
-  if (near == 0) return idx;
+  if (near == 0 || idx >= ties.V) return idx;
   least = m - (ties.d / 16 + 9) * 0x1p-20f * row_logit<true>(ties.W, h, ties.d, idx, gl, L, group);
   float best = -INFINITY;
   int token = idx;
@@ -188,7 +189,7 @@ static __device__ __noinline__ int settle_ties(const Ties ties, int row, const P
       const Partial* q = p + static_cast<size_t>(j) * chunk_stride;
       if (__ldcg(&q->m) >= least) mine = __ldcg(&q->idx);
     }
-    unsigned int todo = __ballot_sync(group, mine != kNoToken) & group;
+    unsigned int todo = __ballot_sync(group, mine < ties.V) & group;
     while (todo != 0u) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;

@@ -34,7 +34,7 @@ __device__ __forceinline__ Partial row_summary(const Partial* __restrict__ parti
                                                const Ties& ties, int lane) {
   const Partial* p = partials + static_cast<size_t>(row) * chunks;
   Partial acc = fold_row(p, chunks, 1, lane);
-  if (kTies && acc.idx != kNoToken) {
+  if (kTies && acc.idx < ties.V) {
     acc.idx = settle_ties(ties, row, p, chunks, 1, acc.m, acc.idx, lane, 32);
     const float z = row_logit(ties.W, ties.h + static_cast<size_t>(row) * ties.d, ties.d, acc.idx, lane, 32, 0xffffffffu);
     if (fabsf(z) < INFINITY) acc.m = z;      // (a row that is not finite is left as the projection found it)

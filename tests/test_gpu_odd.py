@@ -66,6 +66,40 @@ def test_equal_rows_of_different_classes_tie_to_the_lowest_index(pkg, n, d):
     assert np.array_equal(gpu["token"][sure], ref.token[sure])
 
 
+# One row whose logits all lie below -1e30: what it gives is not specified, but nothing is read beyond W for it and the other
+# rows are untouched (one thread per row and four, a pair of CTAs; the call, the gathered and the pushed summaries).
+@pytest.mark.parametrize("n,d", [(9, 63), (40, 100), (200, 63), (1100, 130)])
+def test_a_row_of_huge_negative_logits_leaves_the_others_alone(pkg, n, d):
+    V = 3001
+    W = S.make_W(d, V, seed=d, std=0.2)
+    W[:, :8] = -1.0
+    h = S.make_h(n, d, seed=n).h
+    h[:, :8] = 0
+    bad = h.clone()
+    bad[3, :8] = 1e30
+    rows = np.arange(n) != 3
+    Wd = W.cuda()
+    for cls in (pkg.Router, pkg.VocabShardedRouter, pkg.FusedVocabShardedRouter):
+        got = []
+        for x in (h, bad):
+            if cls is pkg.Router:
+                r = cls(Wd, max_n=n)
+                r.route(x.cuda(), 0.5)
+            elif cls is pkg.VocabShardedRouter:
+                r = cls(Wd, 0, max_n=n, world=1)
+                r.finish(r.summarize(x.cuda()).unsqueeze(0).contiguous(), n, 0.5)
+            else:
+                block = torch.zeros(pkg.tlr_shard_block_bytes(n, 1), dtype=torch.uint8, device="cuda")
+                r = cls(Wd, 0, n, 0, 1, [block], keep=block)
+                r.push(x.cuda())
+                r.finish(n, 0.5)
+            torch.cuda.synchronize()
+            got.append([t[:n].cpu().numpy()[rows] for t in (r.token, r.conf, r.entropy, r.route_mask)])
+            r.close()
+        for a, b in zip(*got):
+            assert np.array_equal(a, b)
+
+
 # Rows of (nearly) equal logits, as padding leaves them: every partial is a candidate for the maximum.
 @pytest.mark.parametrize("n,d,V", [(3, 63, 3001), (40, 130, 3001), (300, 7, 9000), (1100, 300, 3001)])
 def test_rows_of_equal_logits(pkg, n, d, V):
