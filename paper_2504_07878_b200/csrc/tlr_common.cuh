@@ -78,8 +78,10 @@ __device__ __forceinline__ Partial warp_merge(Partial p) {
 
 constexpr int kPerLane = 6;            // ceil(192 / 32): the most partials a lane can own
 
-// Folds one row's partials.  Every lane returns the same result.
-__device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int chunks, int chunk_stride, int lane) {
+// Folds one row's partials.  Every lane returns the same result.  `second` (optional): the largest of the partials' maxima
+// below the row's.
+__device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int chunks, int chunk_stride, int lane,
+                                            float* second = nullptr) {
   Partial q[kPerLane];
   float m = -INFINITY;
   int idx = kNoToken;
@@ -124,6 +126,14 @@ __device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int c
     s += __shfl_xor_sync(0xffffffffu, s, off);
     t += __shfl_xor_sync(0xffffffffu, t, off);
   }
+  if (second != nullptr) {
+    float below = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kPerLane; ++k) below = q[k].m < m ? fmaxf(below, q[k].m) : below;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) below = fmaxf(below, __shfl_xor_sync(0xffffffffu, below, off));
+    *second = below;
+  }
   Partial r;
   r.m = m;
   r.idx = idx;
@@ -132,8 +142,7 @@ __device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int c
   return r;
 }
 
-// Hidden sizes that are no multiple of 8 on the tensor cores: equal rows of W in different residue classes get logits that
-// agree to rounding only, so near-ties are settled by dot products of their own.
+// Hidden sizes that are no multiple of 8 on the tensor cores: what settles a row's winner and its logit (settle_row).
 struct Ties {
   const unsigned short* W;   // bf16 [V][d]; null = not needed
   const unsigned short* h;   // bf16 [n][d]
@@ -143,44 +152,62 @@ struct Ties {
 __device__ __forceinline__ float bf16_value(unsigned short bits) { return __uint_as_float(static_cast<uint32_t>(bits) << 16); }
 
 // The logit of token v in the row h by the L lanes of a row (lane gl of them, mask `group`), summed in fp32 in one fixed
-// order: equal rows of W give equal bits, whatever kernel, shard or GPU asks with the same L.  kSize: the sum of the products'
-// magnitudes instead.
-template <bool kSize = false>
-__device__ __forceinline__ float row_logit(const unsigned short* __restrict__ W, const unsigned short* __restrict__ h, int d,
-                                           int v, int gl, int L, unsigned int group) {
-  const unsigned short* w = W + static_cast<size_t>(v) * d;
-  float z = 0.f;
-  for (int k = gl; k < d; k += L) {
-    const float x = bf16_value(h[k]), y = bf16_value(w[k]);
-    z = kSize ? fmaf(fabsf(x), fabsf(y), z) : fmaf(x, y, z);
+// order: equal rows of W give equal bits, whatever kernel, shard or GPU asks with the same L.  `size` receives the sum of the
+// products' magnitudes.  Bound by the trips to memory and, a row's lanes being few, by instructions: every line of the row of W
+// is asked for before the first is used, a lane has six loads of either operand in flight, and they are two elements wide
+// where d is even (rows have no alignment beyond one element or two).
+template <bool kPairs>
+__device__ __forceinline__ float2 lane_logit(const unsigned short* w, const unsigned short* h, int d, int gl, int L) {
+  constexpr int kBatch = 6;
+  const int loads = kPairs ? d >> 1 : d;
+  float z = 0.f, size = 0.f;
+  for (int k0 = gl; k0 < loads; k0 += kBatch * L) {
+    uint32_t x[kBatch], y[kBatch];
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const int k = k0 + i * L;
+      x[i] = y[i] = 0u;
+      if (k < loads) {
+        x[i] = kPairs ? reinterpret_cast<const uint32_t*>(h)[k] : h[k];
+        y[i] = kPairs ? reinterpret_cast<const uint32_t*>(w)[k] : w[k];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const float a = __uint_as_float(x[i] << 16), b = __uint_as_float(y[i] << 16);
+      z = fmaf(a, b, z);
+      size = fmaf(fabsf(a), fabsf(b), size);
+      if (kPairs) {
+        const float c = __uint_as_float(x[i] & 0xffff0000u), e = __uint_as_float(y[i] & 0xffff0000u);
+        z = fmaf(c, e, z);
+        size = fmaf(fabsf(c), fabsf(e), size);
+      }
+    }
   }
-  for (int off = L >> 1; off > 0; off >>= 1) z += __shfl_xor_sync(group, z, off);
-  return z;
+  return make_float2(z, size);
+}
+__device__ __forceinline__ float row_logit(const unsigned short* W, const unsigned short* h, int d, int v, int gl, int L,
+                                           unsigned int group, float* size) {
+  const unsigned short* w = W + static_cast<size_t>(v) * d;
+  for (int k = gl * 64; k < d; k += L * 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(w + k));
+  float2 r = (d & 1) == 0 ? lane_logit<true>(w, h, d, gl, L) : lane_logit<false>(w, h, d, gl, L);
+  for (int off = L >> 1; off > 0; off >>= 1) {
+    r.x += __shfl_xor_sync(group, r.x, off);
+    r.y += __shfl_xor_sync(group, r.y, off);
+  }
+  *size = r.y;
+  return r.x;
 }
 
-// The token of a row whose maximum m (at idx) may be tied with another partial's: the candidates within the rounding of m
-// are compared by row_logit, so equal rows of W tie exactly and the lowest index wins.  Called by the L lanes of a row (lane
-// gl of them); rarely more than a look at the maxima, because a candidate costs an L2 trip.  Candidates are few: maxima that
-// agree to the bit need none (the merge has taken the lowest index), and the others are held against what rounding can do,
-// 2^-21 of the products' magnitudes per accumulation of 16 products and 8 more, twice.  (An index can lie beyond V: the column
-// that stands for one there is -1e30, and wins where every logit is below that.)  With every maximum within 1e-3 a
-// candidate, a hidden state of zeros (padding) in the batch made a step of n = 16, d = 300, V = 33000 322 us long instead of
-// 11.9; now 11.9 (every hidden state scaled by 1e-5: 17.0).
+// The winner among idx and the partials of a row whose maxima are at least `least`, by row_logit (*z, idx's at first): equal
+// rows of W tie exactly and the lowest index wins.  Rarely called; a candidate costs a trip to L2.
 static __device__ __noinline__ int settle_ties(const Ties ties, int row, const Partial* __restrict__ p, int chunks,
-                                               int chunk_stride, float m, int idx, int gl, int L) {
+                                               int chunk_stride, float least, int idx, float* z, int gl, int L) {
   const unsigned short* h = ties.h + static_cast<size_t>(row) * ties.d;
   const unsigned int lane = threadIdx.x & 31;
   const unsigned int group = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (lane - gl);
-  float least = m - (1e-3f + 1e-5f * fabsf(m));
-  int near = 0;
-  for (int j = gl; j < chunks; j += L) {
-    const float other = __ldcg(&p[static_cast<size_t>(j) * chunk_stride].m);
-    near += other >= least && other != m ? 1 : 0;
-  }
-  for (int off = L >> 1; off > 0; off >>= 1) near += __shfl_xor_sync(group, near, off);
-  if (near == 0 || idx >= ties.V) return idx;
-  least = m - (ties.d / 16 + 9) * 0x1p-20f * row_logit<true>(ties.W, h, ties.d, idx, gl, L, group);
-  float best = -INFINITY;
+  float size;
+  float best = *z;
   int token = idx;
   for (int j0 = 0; j0 < chunks; j0 += L) {
     const int j = j0 + gl;
@@ -189,19 +216,52 @@ static __device__ __noinline__ int settle_ties(const Ties ties, int row, const P
       const Partial* q = p + static_cast<size_t>(j) * chunk_stride;
       if (__ldcg(&q->m) >= least) mine = __ldcg(&q->idx);
     }
-    unsigned int todo = __ballot_sync(group, mine < ties.V) & group;
+    unsigned int todo = __ballot_sync(group, mine < ties.V && mine != idx) & group;
     while (todo != 0u) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
       const int v = __shfl_sync(group, mine, src);
-      const float z = row_logit(ties.W, h, ties.d, v, gl, L, group);
-      if (z > best || (z == best && v < token)) {
-        best = z;
+      const float zv = row_logit(ties.W, h, ties.d, v, gl, L, group, &size);
+      if (zv > best || (zv == best && v < token)) {
+        best = zv;
         token = v;
       }
     }
   }
+  *z = best;
   return token;
+}
+
+// The row's summary (m, idx, s, t) with its winner settled among the residue classes and the winner's logit replaced by its
+// row_logit; `second` is the largest of its partials' maxima below m.  Called by the L lanes of a row.
+//
+// Ties: equal rows of W in different classes get logits that agree to rounding only.  Candidates are the partials within what
+// rounding can do to sums of the winner's products: 2^-21 of their magnitudes for each accumulation of 16 and 8 more, twice.
+// Maxima that agree to the bit need no settling (the merge has taken the lowest index), so that a row of equal logits -- a
+// hidden state of zeros, as padding leaves it -- costs nothing; with every partial within 1e-3 a candidate, one such row in the
+// batch made a step of n = 16, d = 300, V = 33000 322 us long.
+// The logit: the tensor cores truncate where they add, by more the larger the sum, so that the largest logit comes out low
+// against the others; s counts the winner's own term as e^0 = 1 and everything else moves by m's error.  Confidences against
+// 64 bits (2-norm) as the projection leaves them, here, and on CUDA cores, where these heads ran before: d = 300 6.7e-7,
+// 1.7e-7, 3.2e-7; d = 999 2.3e-6, 1.7e-7, 8.7e-7.
+// A row that is not finite stays as it is; so does one whose index lies beyond V.
+__device__ __forceinline__ void settle_row(const Ties& ties, int row, const Partial* __restrict__ p, int chunks,
+                                           int chunk_stride, float second, float& m, int& idx, float& s, float& t, int gl,
+                                           int L) {
+  if (idx >= ties.V) return;
+  const unsigned int lane = threadIdx.x & 31;
+  const unsigned int group = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (lane - gl);
+  float size;
+  float z = row_logit(ties.W, ties.h + static_cast<size_t>(row) * ties.d, ties.d, idx, gl, L, group, &size);
+  const float least = m - (ties.d / 16 + 9) * 0x1p-20f * size;
+  if (second >= least) idx = settle_ties(ties, row, p, chunks, chunk_stride, least, idx, &z, gl, L);
+  if (!(fabsf(z) < INFINITY && fabsf(m) < INFINITY)) return;
+  const float dm = m - z;
+  m = z;
+  if (fabsf(dm) > 1.0f) return;     // logits so large that neighbouring numbers are further apart
+  const float e = exp2f(dm * kLog2e);
+  t = e * (t + dm * (s - 1.0f));
+  s = 1.0f + e * (s - 1.0f);
 }
 
 // Host-side launchers (one per .cu file).  All enqueue on `stream` and return the

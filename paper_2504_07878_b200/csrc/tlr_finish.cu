@@ -147,10 +147,10 @@ __device__ __forceinline__ void wait_for_words(uint32_t bar, uint32_t* status) {
 // row in two passes over its partials: maximum and index first, then the sums rescaled to
 // that maximum.  L is chosen on the host so that every row has its group: n * L <=
 // gridDim.x * 1024.
-// (kTies: with settle_ties; a kernel of its own, because the call would cost the other one registers -- 40 is the most
-// that lets a block of 512 threads stand beside a CTA of the 8-bit projection kernel.)
+// (kTies: with settle_row; a kernel of its own, because that would cost the other one registers -- 40 is the most
+// that lets a block of 512 threads stand beside a CTA of the 8-bit projection kernel or of one for d % 8 != 0.)
 template <bool kTies>
-__global__ void __launch_bounds__(kSmallThreads)
+__global__ void __maxnreg__(40)
 finish_small_kernel(const FinishLaunch a, const int log2_L) {
   __shared__ int warp_count[kSmallThreads / 32];
   const int warp = threadIdx.x >> 5;
@@ -186,7 +186,7 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
     const size_t cs = static_cast<size_t>(a.chunk_stride);
     float m = -INFINITY;
     int idx = kNoToken;
-    float s = 0.f, t = 0.f;
+    float s = 0.f, t = 0.f, second = -INFINITY;
     if (one_pass) {
       // few partials per lane: one pass, the partials stay in registers
       Partial q[kPerLane];
@@ -223,6 +223,7 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
           s += q[k].s * e;
           t += e * (q[k].t + dm * q[k].s);
         }
+        if (kTies && q[k].m < m) second = fmaxf(second, q[k].m);
       }
     } else {
       // many partials per lane: maximum and index first, then the rescaled sums
@@ -253,15 +254,16 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
             s += raw.z * e;
             t += e * (raw.w + dm * raw.z);
           }
+          if (kTies && raw.x < m) second = fmaxf(second, raw.x);
         }
       }
     }
     for (int off = L >> 1; off > 0; off >>= 1) {
       s += __shfl_xor_sync(0xffffffffu, s, off);
       t += __shfl_xor_sync(0xffffffffu, t, off);
+      if (kTies) second = fmaxf(second, __shfl_xor_sync(0xffffffffu, second, off));
     }
-    if (kTies && valid)
-      idx = settle_ties(a.ties, row, p, a.chunks, a.chunk_stride, m, idx, gl, L);
+    if (kTies && valid) settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, m, idx, s, t, gl, L);
     if (valid && gl == 0) {
       Partial acc;
       acc.m = m;
@@ -323,8 +325,10 @@ finish_kernel(const FinishLaunch a) {
 
   if (row < a.n) {
     const Partial* p = a.partials + static_cast<size_t>(row) * a.row_stride;
-    Partial acc = fold_row(p, a.chunks, a.chunk_stride, lane);
-    if (a.ties.W != nullptr) acc.idx = settle_ties(a.ties, row, p, a.chunks, a.chunk_stride, acc.m, acc.idx, lane, 32);
+    float second;
+    Partial acc = fold_row(p, a.chunks, a.chunk_stride, lane, &second);
+    if (a.ties.W != nullptr)
+      settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, acc.m, acc.idx, acc.s, acc.t, lane, 32);
     if (lane == 0) store_row(score_row(acc, a, row), a, row);
   }
 

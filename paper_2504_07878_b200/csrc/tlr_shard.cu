@@ -27,18 +27,14 @@ constexpr int kWarps = 8;
 // One warp folds one row's chunk partials; every lane ends with the result.
 // kTies (d no multiple of 8): the shard's winner is settled among the residue classes, and m becomes its row_logit, so that
 // equal rows of W in different shards tie exactly in the merge behind -- also where one shard ran on CUDA cores and another
-// on tensor cores.  s and t stay as they are: all logits of the shard move with m, by no more than its rounding, and the
-// winner's own term stays exactly 1.
+// on tensor cores.
 template <bool kTies>
 __device__ __forceinline__ Partial row_summary(const Partial* __restrict__ partials, int row, int chunks, int v_offset,
                                                const Ties& ties, int lane) {
   const Partial* p = partials + static_cast<size_t>(row) * chunks;
-  Partial acc = fold_row(p, chunks, 1, lane);
-  if (kTies && acc.idx < ties.V) {
-    acc.idx = settle_ties(ties, row, p, chunks, 1, acc.m, acc.idx, lane, 32);
-    const float z = row_logit(ties.W, ties.h + static_cast<size_t>(row) * ties.d, ties.d, acc.idx, lane, 32, 0xffffffffu);
-    if (fabsf(z) < INFINITY) acc.m = z;      // (a row that is not finite is left as the projection found it)
-  }
+  float second;
+  Partial acc = fold_row(p, chunks, 1, lane, kTies ? &second : nullptr);
+  if (kTies) settle_row(ties, row, p, chunks, 1, second, acc.m, acc.idx, acc.s, acc.t, lane, 32);
   if (acc.idx != kNoToken) acc.idx += v_offset;
   return acc;
 }

@@ -171,6 +171,10 @@ __host__ __device__ __forceinline__ Tile tile_of(const TcParams& p, const Unit& 
 // S = sum 2^y and T = sum 2^y * y with y = (z - m) * log2(e) <= 0; both are accumulated per
 // 32-column group first and then added with a compensated (Kahan) sum, so that one dominant term -- a
 // confident row has S ~ 1 with thousands of terms ~1e-8 after it -- does not swallow the rest.
+// kExact: z - m is rounded by itself, so that the largest logit's y is zero whatever its size; with one fma, against the
+// rounded m * log2(e), every y of a row is off by up to 2^-24 of that.  The heads whose hidden size is no multiple of 8 ran on
+// CUDA cores with the former before they ran here.  Their columns beyond V are left out of the maximum, too.
+template <bool kExact>
 struct RowFold {
   float m, S, cS, Tq, cT;
   int idx;
@@ -179,13 +183,21 @@ struct RowFold {
     S = cS = Tq = cT = 0.f;
     idx = kNoToken;
   }
+  // y of the logits z0 and z1; neg_m is -m (kExact) or -m * log2(e)
+  static __device__ __forceinline__ uint64_t exponents(float z0, float z1, float neg_m) {
+    const uint64_t log2e2 = pack2(kLog2e, kLog2e), neg2 = pack2(neg_m, neg_m);
+    if (kExact) return fma2(add2(pack2(z0, z1), neg2), log2e2, 0ull);
+    return fma2(pack2(z0, z1), log2e2, neg2);
+  }
+  // kExact: what stands for a column beyond V once the maximum is known: far enough below it for e^(z-m) = 0, and finite
+  __device__ __forceinline__ float far_below() const { return m - fmaxf(1000.f, fabsf(m) * 0.015625f); }
   // Folds 32 consecutive logits z[0..32) whose first has vocabulary index col0; only the first
   // `valid` of them exist (the rest lie beyond V).
   __device__ __forceinline__ void group(float (&z)[32], int valid, int col0) {
     if (valid < 32) {
 #pragma unroll
       for (int j = 0; j < 32; ++j)
-        if (j >= valid) z[j] = kNoLogit;
+        if (j >= valid) z[j] = kExact ? -INFINITY : kNoLogit;
     }
     float cm = fmaxf(z[0], z[1]);
 #pragma unroll
@@ -205,12 +217,16 @@ struct RowFold {
       for (int j = 30; j >= 0; --j) first_j = (z[j] == cm) ? j : first_j;
       idx = col0 + first_j;
     }
-    const float neg_ml = -m * kLog2e;
-    const uint64_t log2e2 = pack2(kLog2e, kLog2e), neg_ml2 = pack2(neg_ml, neg_ml);
+    if (kExact && valid < 32) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (j >= valid) z[j] = far_below();
+    }
+    const float neg_m = kExact ? -m : -m * kLog2e;
     uint64_t ls2 = pack2(0.f, 0.f), lt2 = pack2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < 32; j += 2) {
-      const uint64_t y2 = fma2(pack2(z[j], z[j + 1]), log2e2, neg_ml2);   // (z - m) * log2(e)
+      const uint64_t y2 = exponents(z[j], z[j + 1], neg_m);
       float y0, y1;
       unpack2(y2, y0, y1);
       const uint64_t e2 = pack2(ex2_approx(y0), ex2_approx(y1));
@@ -234,9 +250,14 @@ struct RowFold {
     }
   }
   // The same for 16 logits of one row held by a thread of the fragment layout (tmem_ld16x64): z[2b + j] is column
-  // col0 + 8b + j.  Written for latency -- no branch but the index search, short dependent chains -- because the
-  // last tile's fold is exposed at the end of every step.
-  __device__ __forceinline__ void fragment(const float (&z)[16], int col0) {
+  // col0 + 8b + j, and those from `valid` on do not exist.  Written for latency -- no branch but the index search, short
+  // dependent chains -- because the last tile's fold is exposed at the end of every step.
+  __device__ __forceinline__ void fragment(float (&z)[16], int valid, int col0) {
+    if (valid < 58) {                                  // (the last of the columns is col0 + 57)
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (8 * (k >> 1) + (k & 1) >= valid) z[k] = kExact ? -INFINITY : kNoLogit;
+    }
     const float m0 = max3(max3(z[0], z[1], z[2]), z[3], max3(z[4], z[5], z[6]));
     const float m1 = max3(max3(z[7], z[8], z[9]), z[10], max3(z[11], z[12], z[13]));
     const float cm = max3(fmaxf(m0, m1), z[14], z[15]);
@@ -247,16 +268,20 @@ struct RowFold {
       const int k = __ffs(hit) - 1;
       idx = col0 + 8 * (k >> 1) + (k & 1);
     }
-    const float m_old = fmaxf(m, kNoLogit);         // (finite before the first group)
+    const float m_old = kExact ? (m == -INFINITY ? cm : m) : fmaxf(m, kNoLogit);    // (finite before the first group)
     m = fmaxf(m_old, cm);
     const float dl = (m - m_old) * kLog2e;          // >= 0
     const float sc = ex2_approx(-dl);
-    const float neg_ml = -m * kLog2e;
-    const uint64_t log2e2 = pack2(kLog2e, kLog2e), neg_ml2 = pack2(neg_ml, neg_ml);
+    if (kExact && valid < 58) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (8 * (k >> 1) + (k & 1) >= valid) z[k] = far_below();
+    }
+    const float neg_m = kExact ? -m : -m * kLog2e;
     uint64_t ls2[2] = {0ull, 0ull}, lt2[2] = {0ull, 0ull};
 #pragma unroll
     for (int j = 0; j < 16; j += 2) {
-      const uint64_t y2 = fma2(pack2(z[j], z[j + 1]), log2e2, neg_ml2);
+      const uint64_t y2 = exponents(z[j], z[j + 1], neg_m);
       float y0, y1;
       unpack2(y2, y0, y1);
       const uint64_t e2 = pack2(ex2_approx(y0), ex2_approx(y1));
@@ -642,7 +667,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       const bool warp_has_rows = first.row0 + quad_row0 < p.n;            // warp-uniform
       const bool two_tokens = kFolds == 2 && quad_row0 + 8 < p.n;   // warp-uniform
       const bool mlp_unit = !kFp8 && first.chunk < 0;
-      RowFold f[kFolds];
+      RowFold<kOdd> f[kFolds];
 #pragma unroll
       for (int i = 0; i < kFolds; ++i) f[i].reset();
       float mlp_sum = 0.f;
@@ -705,12 +730,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
                   }
                   continue;
                 }
-                if (valid < 58) {                     // (the last of the columns is c_mine + 57)
-#pragma unroll
-                  for (int k = 0; k < 16; ++k)
-                    if (8 * (k >> 1) + (k & 1) >= valid) z[k] = kNoLogit;
-                }
-                f[i].fragment(z, v0 + c_mine);
+                f[i].fragment(z, valid, v0 + c_mine);
               }
             }
           } else {

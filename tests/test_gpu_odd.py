@@ -145,6 +145,27 @@ def test_a_row_of_equal_logits_does_not_hold_up_the_step(pkg, scale):
     assert times[1] <= 3 * times[0], times
 
 
+# The error against 64 bits: what fp32 results and the 2^-22 of ex2.approx leave, whatever d; and of large logits no more, up
+# to sizes whose neighbours are further apart than the logits' differences.
+@pytest.mark.parametrize("n,d,V", [(9, 255, 20000), (64, 300, 20000), (100, 999, 20000), (200, 101, 33000), (1100, 501, 9000)])
+def test_scores_are_as_exact_as_fp32_sums_of_exact_products(pkg, n, d, V):
+    W = S.make_W(d, V, seed=d, std=0.06)
+    h = S.make_h(n, d, seed=n, W=W, planted_fraction=0.5).h
+    gpu = check(pkg, W, h, 0.5)
+    ref = O.route_oracle(S.bf16_bits(h), S.bf16_bits(W), 0.5)
+    err = np.linalg.norm(gpu["conf"].astype(np.float64) - ref.conf) / np.linalg.norm(ref.conf)
+    assert err <= 4e-7, err
+    for scale in (100.0, 1e30):
+        big = (h[:8].float() * scale).to(h.dtype)
+        ref = O.route_oracle(S.bf16_bits(big), S.bf16_bits(W), 0.5)
+        clear = ref.top2_gap >= 0.05 * scale
+        assert clear.sum() >= 4
+        gpu = run_gpu(pkg, W.cuda(), torch.cat([big, h[8:]]), 0.5)
+        assert gpu["status"] == 0
+        assert np.array_equal(gpu["token"][:8][clear], ref.token[clear])
+        assert np.max(np.abs(gpu["conf"][:8][clear] - ref.conf[clear])) <= 1e-5
+
+
 def test_learned_router_and_host_buffers(pkg):
     n, d, V, dh = 70, 100, 3000, 48
     W = S.make_W(d, V, seed=1, std=0.1)
