@@ -147,11 +147,8 @@ __device__ __forceinline__ void wait_for_words(uint32_t bar, uint32_t* status) {
 // row in two passes over its partials: maximum and index first, then the sums rescaled to
 // that maximum.  L is chosen on the host so that every row has its group: n * L <=
 // gridDim.x * 1024.
-// (kTies: with settle_row; a kernel of its own, because that would cost the other one registers -- 40 is the most
-// that lets a block of 512 threads stand beside a CTA of the 8-bit projection kernel or of one for d % 8 != 0.)
 template <bool kTies>
-__global__ void __maxnreg__(40)
-finish_small_kernel(const FinishLaunch a, const int log2_L) {
+__device__ __forceinline__ void finish_small(const FinishLaunch& a, const int log2_L) {
   __shared__ int warp_count[kSmallThreads / 32];
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -223,7 +220,7 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
           s += q[k].s * e;
           t += e * (q[k].t + dm * q[k].s);
         }
-        if (kTies && q[k].m < m) second = fmaxf(second, q[k].m);
+        if constexpr (kTies) second = q[k].m < m ? fmaxf(second, q[k].m) : second;
       }
     } else {
       // many partials per lane: maximum and index first, then the rescaled sums
@@ -254,16 +251,18 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
             s += raw.z * e;
             t += e * (raw.w + dm * raw.z);
           }
-          if (kTies && raw.x < m) second = fmaxf(second, raw.x);
+          if constexpr (kTies) second = raw.x < m ? fmaxf(second, raw.x) : second;
         }
       }
     }
     for (int off = L >> 1; off > 0; off >>= 1) {
       s += __shfl_xor_sync(0xffffffffu, s, off);
       t += __shfl_xor_sync(0xffffffffu, t, off);
-      if (kTies) second = fmaxf(second, __shfl_xor_sync(0xffffffffu, second, off));
+      if constexpr (kTies) second = fmaxf(second, __shfl_xor_sync(0xffffffffu, second, off));
     }
-    if (kTies && valid) settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, m, idx, s, t, gl, L);
+    if constexpr (kTies) {
+      if (valid) settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, m, idx, s, t, gl, L);
+    }
     if (valid && gl == 0) {
       Partial acc;
       acc.m = m;
@@ -315,6 +314,21 @@ finish_small_kernel(const FinishLaunch a, const int log2_L) {
   }
 }
 
+// 32 registers: with 38 a shard's step of n = 444, d = 752, 6766 rows of W takes 15.8 us instead of 14.1, and a spilled one
+// costs 2 to 4 % of most small steps.
+__global__ void __launch_bounds__(kSmallThreads)
+finish_small_kernel(const FinishLaunch a, const int log2_L) {
+  finish_small<false>(a, log2_L);
+}
+
+// With settle_row, which would cost the other one registers; 40 is the most that lets a block of 512 threads stand beside a
+// CTA of the projection kernel for d % 8 != 0.
+__global__ void __maxnreg__(40)
+finish_small_ties_kernel(const FinishLaunch a, const int log2_L) {
+  finish_small<true>(a, log2_L);
+}
+
+template <bool kTies>
 __global__ void __launch_bounds__(kFinishThreads)
 finish_kernel(const FinishLaunch a) {
   const int warp = threadIdx.x >> 5;
@@ -326,8 +340,8 @@ finish_kernel(const FinishLaunch a) {
   if (row < a.n) {
     const Partial* p = a.partials + static_cast<size_t>(row) * a.row_stride;
     float second;
-    Partial acc = fold_row(p, a.chunks, a.chunk_stride, lane, &second);
-    if (a.ties.W != nullptr)
+    Partial acc = fold_row(p, a.chunks, a.chunk_stride, lane, kTies ? &second : nullptr);
+    if constexpr (kTies)
       settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, acc.m, acc.idx, acc.s, acc.t, lane, 32);
     if (lane == 0) store_row(score_row(acc, a, row), a, row);
   }
@@ -411,12 +425,12 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     cfg.numAttrs = 2;
     cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
     cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
-    return cudaLaunchKernelEx(&cfg, a.ties.W != nullptr ? finish_small_kernel<true> : finish_small_kernel<false>, a, log2_L);
+    return cudaLaunchKernelEx(&cfg, a.ties.W != nullptr ? finish_small_ties_kernel : finish_small_kernel, a, log2_L);
   }
   const int blocks = (a.n + kFinishWarps - 1) / kFinishWarps;
   cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
   cfg.blockDim = dim3(kFinishThreads, 1, 1);
-  return cudaLaunchKernelEx(&cfg, finish_kernel, a);
+  return cudaLaunchKernelEx(&cfg, a.ties.W != nullptr ? finish_kernel<true> : finish_kernel<false>, a);
 }
 
 }  // namespace tlr
