@@ -126,9 +126,12 @@ _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 _current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
+_raw_handle = _raw_stream is not None and _current_device is not None
+
+
 def _stream_handle(stream):
     if stream is None:
-        if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+        if _raw_handle and torch.cuda.is_initialized():
             return _raw_stream(_current_device())
         stream = torch.cuda.current_stream()
     if isinstance(stream, int):
@@ -326,6 +329,7 @@ class Router:
         self.wscale = wscale
         self.V, self.d = W.shape
         self.max_n = max_n
+        self._tlr_route = load_library().tlr_route
         with torch.cuda.device(W.device):
             self.ctx = tlr_create_fp8(self.d, self.V, W, wscale, max_n) if fp8 else tlr_create(self.d, self.V, W, max_n)
             dev = W.device
@@ -343,7 +347,8 @@ class Router:
 
     def _outputs(self, n: int):
         """Views of the output tensors for n rows, new objects on every call.  (`.data` of a view that is kept makes one
-        in a quarter of the time that a slice takes: n = 1, d = 256, V = 20000 8.6 us per call against 13.3.)"""
+        in a quarter of the time that a slice takes: n = 1, d = 256, V = 20000 9.0 us per call, slices 13.3, the same four objects
+        every time 8.6.)"""
         kept = self._views.get(n)
         if kept is None:
             if len(self._views) >= 16:
@@ -365,8 +370,13 @@ class Router:
             raise ValueError("h must be a contiguous CUDA bf16 [n, d] tensor")
         n = h.shape[0]
         if tau_per_row is None and not route_above and seq_len == 0 and score_source == 0 and mlp_score is None:
-            tlr_route(self.ctx, h, n, tau, self.token, self.conf, self.entropy, self.route_mask, self.routed_idx,
-                      self.routed_count, stream)
+            # (tlr_route without its calls per argument: they cost about what the views do that are handed out)
+            handle = _raw_stream(_current_device()) if stream is None and _raw_handle else _stream_handle(stream)
+            code = self._tlr_route(self.ctx, h.data_ptr(), n, tau, self.token.data_ptr(), self.conf.data_ptr(),
+                                   self.entropy.data_ptr(), self.route_mask.data_ptr(), self.routed_idx.data_ptr(),
+                                   self.routed_count.data_ptr(), handle)
+            if code != TLR_OK:
+                raise TlrError(code, "tlr_route")
         else:
             tlr_route_ex(self.ctx, h, n, tau, self.token, self.conf, self.entropy, self.route_mask, self.routed_idx,
                          self.routed_count, stream, tau_per_row=tau_per_row, route_above=route_above,
