@@ -192,7 +192,8 @@ tlr_status tlr_route_ex(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, float t
  * 16-byte summary {float m; int32 idx; float s; float t} into summary_dev[n] (device, 16-byte
  * aligned, caller-owned): m = the largest logit in the shard, idx = the lowest GLOBAL vocabulary
  * index attaining it (v_offset already added), s = sum exp(z - m), t = sum exp(z - m)(z - m) over
- * the shard.  No decision is taken.  The caller then exchanges the summaries -- an all-gather of
+ * the shard.  (d % 8 != 0: m is the fp32 dot product of h with row idx in one summation order on every shard, so
+ * that equal rows of W in different shards tie exactly.)  No decision is taken.  The caller then exchanges the summaries -- an all-gather of
  * n x 16 bytes per GPU, NCCL in the Python helper -- into a block laid out [shards][n].
  *
  * tlr_shard_finish merges the `shards` summaries of every row (the same associative rule that merges
