@@ -810,6 +810,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
 
   tlr::FinishLaunch f = {};
   f.partials = ctx->partials;
+  f.small_blocks = ctx->fp8 || ctx->classes > 1;
   f.n = n;
   f.chunks = plan.vocab_chunks;
   f.row_stride = plan.vocab_chunks;

@@ -34,7 +34,14 @@ __device__ __forceinline__ Partial empty_partial() {
   return p;
 }
 
-// Associative and commutative merge; ties on m go to the lower vocabulary index.
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Associative and commutative merge; ties on m go to the lower vocabulary index.  (No branches, and ex2 without care for
+// results below 2^-126: this and the folds below stand between the last logit and the decision, and nothing overlaps them.)
 __device__ __forceinline__ Partial merge(const Partial& a, const Partial& b) {
   Partial r;
   const bool a_wins = (a.m > b.m) || (a.m == b.m && a.idx <= b.idx);
@@ -43,21 +50,11 @@ __device__ __forceinline__ Partial merge(const Partial& a, const Partial& b) {
   // Rescale each side to the new maximum.  A side with s == 0 (an empty range) contributes
   // nothing: its m is -inf, which must not reach the arithmetic below.  A NaN sum is not
   // "empty": it goes through and poisons the result, which the final step then flags.
-  float s = 0.f, t = 0.f;
-  if (!(a.s == 0.f)) {
-    const float da = a.m - r.m;  // <= 0
-    const float ea = exp2f(da * kLog2e);
-    s += a.s * ea;
-    t += ea * (a.t + da * a.s);
-  }
-  if (!(b.s == 0.f)) {
-    const float db = b.m - r.m;
-    const float eb = exp2f(db * kLog2e);
-    s += b.s * eb;
-    t += eb * (b.t + db * b.s);
-  }
-  r.s = s;
-  r.t = t;
+  const float da = a.s == 0.f ? 0.f : a.m - r.m;  // <= 0
+  const float db = b.s == 0.f ? 0.f : b.m - r.m;
+  const float ea = ex2_approx(da * kLog2e), eb = ex2_approx(db * kLog2e);
+  r.s = fmaf(b.s, eb, a.s * ea);
+  r.t = fmaf(eb, fmaf(db, b.s, b.t), ea * fmaf(da, a.s, a.t));
   return r;
 }
 
@@ -77,68 +74,108 @@ __device__ __forceinline__ Partial warp_merge(Partial p) {
 }
 
 constexpr int kPerLane = 6;            // ceil(192 / 32): the most partials a lane can own
+constexpr int kRowsPerLane = 5;        // ... in the kernels bound by latency (148 / 32): registers
 
-// Folds one row's partials.  Every lane returns the same result.  `second` (optional): the largest of the partials' maxima
-// below the row's.
-__device__ __forceinline__ Partial fold_row(const Partial* __restrict__ p, int chunks, int chunk_stride, int lane,
-                                            float* second = nullptr) {
-  Partial q[kPerLane];
-  float m = -INFINITY;
-  int idx = kNoToken;
+// A lane's share of a row's partials -- first, first + stride, ... below `count`: maxima and sums, and the largest maximum
+// with its lowest index.
+template <int kN>
+struct LaneFold {
+  float m[kN], s[kN], t[kN];
+  float best;
+  int idx;
+  __device__ __forceinline__ void clear() {
+    best = -INFINITY;
+    idx = kNoToken;
 #pragma unroll
-  for (int k = 0; k < kPerLane; ++k) {
-    const int j = lane + 32 * k;
-    if (j < chunks) {
-      const float4 raw = __ldcg(reinterpret_cast<const float4*>(p + static_cast<size_t>(j) * chunk_stride));
-      q[k].m = raw.x;
-      q[k].idx = __float_as_int(raw.y);
-      q[k].s = raw.z;
-      q[k].t = raw.w;
-    } else {
-      q[k] = empty_partial();
-    }
-    if (q[k].m > m || (q[k].m == m && q[k].idx < idx)) {
-      m = q[k].m;
-      idx = q[k].idx;
+    for (int k = 0; k < kN; ++k) {
+      m[k] = -INFINITY;
+      s[k] = t[k] = 0.f;
     }
   }
+  __device__ __forceinline__ void put(int k, const Partial& v) {
+    m[k] = v.m;
+    s[k] = v.s;
+    t[k] = v.t;
+    idx = v.m > best ? v.idx : (v.m == best ? min(v.idx, idx) : idx);
+    best = fmaxf(best, v.m);
+  }
+  __device__ __forceinline__ void load(const Partial* p, int first, int stride, int count, size_t chunk_stride) {
+    clear();
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
+    for (int k = 0; k < kN; ++k) {
+      const int j = first + stride * k;
+      Partial v = empty_partial();
+      if (j < count) {
+        const float4 raw = __ldcg(reinterpret_cast<const float4*>(p + j * chunk_stride));
+        v.m = raw.x;
+        v.idx = __float_as_int(raw.y);
+        v.s = raw.z;
+        v.t = raw.w;
+      }
+      put(k, v);
+    }
+  }
+  // The sums rescaled to the row's maximum.  An empty range contributes nothing; a NaN sum goes through.
+  __device__ __forceinline__ void sums(float row_m, float& sum_s, float& sum_t) const {
+    sum_s = sum_t = 0.f;
+#pragma unroll
+    for (int k = 0; k < kN; ++k) {
+      const float dm = s[k] == 0.f ? 0.f : m[k] - row_m;    // <= 0
+      const float e = ex2_approx(dm * kLog2e);
+      sum_s = fmaf(s[k], e, sum_s);
+      sum_t = fmaf(e, fmaf(dm, s[k], t[k]), sum_t);
+    }
+  }
+  // The largest of the maxima below the row's.
+  __device__ __forceinline__ float second(float row_m) const {
+    float below = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kN; ++k) below = m[k] < row_m ? fmaxf(below, m[k]) : below;
+    return below;
+  }
+};
+
+// The largest maximum of a group of L lanes (a power of two, aligned) and its lowest index; all of them get it.
+__device__ __forceinline__ void group_best(float& m, int& idx, int L) {
+  if (L == 32) {      // two warp reductions, the floats as integers of the same order
+    const int bits = __float_as_int(m);
+    const int top = __reduce_max_sync(0xffffffffu, bits ^ ((bits >> 31) & 0x7fffffff));
+    const float best = __int_as_float(top ^ ((top >> 31) & 0x7fffffff));
+    idx = __reduce_min_sync(0xffffffffu, m == best ? idx : kNoToken);      // (+0 and -0 are equal here, too)
+    m = best;
+    return;
+  }
+  for (int off = L >> 1; off > 0; off >>= 1) {
     const float om = __shfl_xor_sync(0xffffffffu, m, off);
     const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
-    if (om > m || (om == m && oi < idx)) {
-      m = om;
-      idx = oi;
-    }
+    idx = om > m ? oi : (om == m ? min(oi, idx) : idx);
+    m = fmaxf(m, om);
   }
-  float s = 0.f, t = 0.f;
-#pragma unroll
-  for (int k = 0; k < kPerLane; ++k) {
-    if (!(q[k].s == 0.f)) {           // an empty range contributes nothing; a NaN sum goes through
-      const float dm = q[k].m - m;    // <= 0
-      const float e = exp2f(dm * kLog2e);
-      s += q[k].s * e;
-      t += e * (q[k].t + dm * q[k].s);
-    }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
+}
+__device__ __forceinline__ void group_sum(float& s, float& t, int L) {
+  for (int off = L >> 1; off > 0; off >>= 1) {
     s += __shfl_xor_sync(0xffffffffu, s, off);
     t += __shfl_xor_sync(0xffffffffu, t, off);
   }
-  if (second != nullptr) {
-    float below = -INFINITY;
-#pragma unroll
-    for (int k = 0; k < kPerLane; ++k) below = q[k].m < m ? fmaxf(below, q[k].m) : below;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) below = fmaxf(below, __shfl_xor_sync(0xffffffffu, below, off));
-    *second = below;
-  }
+}
+__device__ __forceinline__ float group_max(float v, int L) {
+  for (int off = L >> 1; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+  return v;
+}
+
+// Folds one row's partials.  Every lane returns the same result.  `second` (optional): the largest of the partials' maxima
+// below the row's.
+__device__ __forceinline__ Partial fold_row(const Partial* p, int chunks, int chunk_stride, int lane,
+                                            float* second = nullptr) {
   Partial r;
-  r.m = m;
-  r.idx = idx;
-  r.s = s;
-  r.t = t;
+  LaneFold<kPerLane> f;
+  f.load(p, lane, 32, chunks, chunk_stride);
+  r.m = f.best;
+  r.idx = f.idx;
+  group_best(r.m, r.idx, 32);
+  f.sums(r.m, r.s, r.t);
+  group_sum(r.s, r.t, 32);
+  if (second != nullptr) *second = group_max(f.second(r.m), 32);
   return r;
 }
 
@@ -199,16 +236,20 @@ __device__ __forceinline__ float row_logit(const unsigned short* W, const unsign
   return r.x;
 }
 
-// The winner among idx and the partials of a row whose maxima are at least `least`, by row_logit (*z, idx's at first): equal
-// rows of W tie exactly and the lowest index wins.  Rarely called; a candidate costs a trip to L2.
-static __device__ __noinline__ int settle_ties(const Ties ties, int row, const Partial* __restrict__ p, int chunks,
-                                               int chunk_stride, float least, int idx, float* z, int gl, int L) {
+// The winner among idx and the partials of a row whose maxima are at least `least`, by row_logit (z, idx's): its index and its
+// logit.  Equal rows of W tie exactly and the lowest index wins.  Rarely called; a candidate costs a trip to L2.  (Not a function
+// of its own: around a call the loads of row_logit went out a few at a time, n = 200, d = 999, V = 60000 51.0 -> 55.5 us.)
+struct Winner {
+  int idx;
+  float z;
+};
+static __device__ __forceinline__ Winner settle_ties(const Ties ties, int row, const Partial* __restrict__ p, int chunks,
+                                               int chunk_stride, float least, int idx, float z, int gl, int L) {
   const unsigned short* h = ties.h + static_cast<size_t>(row) * ties.d;
   const unsigned int lane = threadIdx.x & 31;
   const unsigned int group = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (lane - gl);
   float size;
-  float best = *z;
-  int token = idx;
+  Winner win = {idx, z};
   for (int j0 = 0; j0 < chunks; j0 += L) {
     const int j = j0 + gl;
     int mine = kNoToken;
@@ -222,14 +263,13 @@ static __device__ __noinline__ int settle_ties(const Ties ties, int row, const P
       todo &= todo - 1;
       const int v = __shfl_sync(group, mine, src);
       const float zv = row_logit(ties.W, h, ties.d, v, gl, L, group, &size);
-      if (zv > best || (zv == best && v < token)) {
-        best = zv;
-        token = v;
+      if (zv > win.z || (zv == win.z && v < win.idx)) {
+        win.z = zv;
+        win.idx = v;
       }
     }
   }
-  *z = best;
-  return token;
+  return win;
 }
 
 // The row's summary (m, idx, s, t) with its winner settled among the residue classes and the winner's logit replaced by its
@@ -254,7 +294,11 @@ __device__ __forceinline__ void settle_row(const Ties& ties, int row, const Part
   float size;
   float z = row_logit(ties.W, ties.h + static_cast<size_t>(row) * ties.d, ties.d, idx, gl, L, group, &size);
   const float least = m - (ties.d / 16 + 9) * 0x1p-20f * size;
-  if (second >= least) idx = settle_ties(ties, row, p, chunks, chunk_stride, least, idx, &z, gl, L);
+  if (second >= least) {
+    const Winner win = settle_ties(ties, row, p, chunks, chunk_stride, least, idx, z, gl, L);
+    idx = win.idx;
+    z = win.z;
+  }
   if (!(fabsf(z) < INFINITY && fabsf(m) < INFINITY)) return;
   const float dm = m - z;
   m = z;
@@ -278,6 +322,7 @@ void simt_plan(int n, int d, int V, int sm_count, int* chunks, int* grid, int* b
 
 struct FinishLaunch {
   const Partial* partials;  // partial j of row i at partials[i * row_stride + j * chunk_stride]
+  bool small_blocks;        // the projection's CTAs leave room for small blocks only (and always with ties to settle)
   int n, chunks;
   int row_stride, chunk_stride;   // [n][chunks]: (chunks, 1); a block gathered shard-major [shards][rows]: (1, rows)
   // optional: before reading the partials, wait until wait_flags[0 .. wait_count) all hold wait_value (flags that

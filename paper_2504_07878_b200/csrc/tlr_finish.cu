@@ -10,9 +10,11 @@
 // Compaction (ballot / popcount / prefix sum, ascending order):
 //   n <= 1024  a thread-block cluster of up to 8 blocks folds the rows (a group of L lanes
 //              per row, all rows at once) and sends the route flags to block 0, which compacts
-//              them.  No ticket, no second launch, one L2 round trip for the partials.  The blocks
-//              have 512 threads where a lane group still owns at most 6 partials (else 1024):
-//              that size fits on an SM beside a CTA of the tensor-core projection kernel, so
+//              them.  No ticket, no second launch, one L2 round trip for the partials.
+//              finish_rows_kernel where a lane owns at most 5 partials: the compaction has a warp
+//              of its own.  Otherwise finish_small_kernel, 512 threads where a lane group still owns
+//              at most 6 partials (else 1024).  Blocks of 17 or 9 warps, and of 512 threads, fit on an
+//              SM beside a CTA of the tensor-core projection kernel, so
 //              the blocks are resident and waiting before that kernel ends, and the next
 //              call's CTAs do not have to wait for the merge to leave their SMs.
 //   larger n   many blocks of 8 warps; the block that finishes last (fence + ticket
@@ -26,30 +28,28 @@ constexpr int kFinishWarps = 8;
 constexpr int kFinishThreads = kFinishWarps * 32;
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallRows = 1024;
+constexpr int kMaxBlocks = 8;           // of a cluster
 
-// Scores and decision of one row from its folded summary.
+// Scores and decision of one row from its folded summary.  The flag, which the compaction waits for, needs no entropy.
 struct Scored {
-  int token, flag;
-  float conf, entropy, learned;
+  float conf, learned;
+  int flag;
+  bool finite;
 };
-__device__ __forceinline__ Scored score_row(const Partial& acc, const FinishLaunch& a, int row) {
+__device__ __forceinline__ Scored decide_row(float s, float t, const FinishLaunch& a, int row) {
   Scored r;
-  r.token = acc.idx;
-  r.conf = 1.0f / acc.s;
-  r.entropy = logf(acc.s) - acc.t / acc.s;
-  const bool finite = (r.conf == r.conf) && (r.entropy == r.entropy) && acc.s > 0.f && acc.s < INFINITY;
-  if (finite) {
+  r.conf = 1.0f / s;
+  r.finite = s > 0.f && s < INFINITY && t == t;        // (and so are both scores no NaN)
+  if (r.finite) {
     r.conf = fminf(r.conf, 1.0f);
-    r.entropy = fmaxf(r.entropy, 0.0f);
   } else {
     r.conf = __int_as_float(0x7fc00000);   // NaN: fails "conf >= tau", so the row is routed
-    r.entropy = r.conf;
     atomicOr(a.status, TLR_DEV_NONFINITE);
     __threadfence();                       // before this row's flag reaches the block that copies the status word
   }
   // "not (conf >= tau)": equals conf < tau for numbers, and routes a NaN row; likewise
   // "not (conf <= tau)" for the opposite polarity.
-  const float tau = a.tau_rows != nullptr ? a.tau_rows[row] : a.tau;
+  const float tau = a.tau_rows != nullptr ? __ldcg(a.tau_rows + row) : a.tau;
   float score = r.conf;
   r.learned = 0.f;
   if (a.mlp_partial != nullptr) {
@@ -63,10 +63,10 @@ __device__ __forceinline__ Scored score_row(const Partial& acc, const FinishLaun
   r.flag = a.route_above ? ((score <= tau) ? 0 : 1) : ((score >= tau) ? 0 : 1);
   return r;
 }
-__device__ __forceinline__ void store_row(const Scored& r, const FinishLaunch& a, int row) {
-  a.token[row] = r.token;
+__device__ __forceinline__ void store_row(const Scored& r, int token, float s, float t, const FinishLaunch& a, int row) {
+  a.token[row] = token;
   a.conf[row] = r.conf;
-  a.entropy[row] = r.entropy;
+  a.entropy[row] = r.finite ? fmaxf(logf(s) - t / s, 0.0f) : r.conf;
   a.route_mask[row] = static_cast<uint8_t>(r.flag);
   if (a.mlp_partial != nullptr && a.mlp_score_out != nullptr) a.mlp_score_out[row] = r.learned;
 }
@@ -120,6 +120,26 @@ __device__ __forceinline__ void wait_for_peers(const FinishLaunch& a) {
   __syncthreads();
 }
 
+// The barrier of block 0 that counts the bytes of `words` words, and a warp's word on its way there.
+__device__ __forceinline__ void expect_words(uint32_t bar, int words) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(words * 4) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void send_word(const uint32_t* slot, uint32_t bar, uint32_t word) {
+  const uint32_t at = static_cast<uint32_t>(__cvta_generic_to_shared(slot));
+  uint32_t remote, remote_bar;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(at), "r"(0));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote_bar) : "r"(bar), "r"(0));
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+               ::"r"(remote), "r"(word), "r"(remote_bar) : "memory");
+}
+// Row i's flag in the words of warps with L lanes to a row.
+__device__ __forceinline__ int flag_of(const uint32_t* words, int i, int log2_L) {
+  const int log2_rpw = 5 - log2_L;
+  return (words[i >> log2_rpw] >> ((i & ((1 << log2_rpw) - 1)) << log2_L)) & 1;
+}
+
 // Block 0 of the cluster waits until every warp's word has arrived (bounded like every wait; after a time-out the status
 // word says that the index list is not to be trusted).
 __device__ __forceinline__ void wait_for_words(uint32_t bar, uint32_t* status) {
@@ -165,11 +185,7 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
   const int warps = blockDim.x >> 5;
   const uint32_t bar = static_cast<uint32_t>(__cvta_generic_to_shared(&all_here));
   if (!single_block) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(gridDim.x * warps * 4u) : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) expect_words(bar, gridDim.x * warps);
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
@@ -177,7 +193,9 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
   wait_for_peers(a);
   const int row = group;
   const bool valid = row < a.n;
-  Scored out;
+  Scored out = {};
+  int out_token;
+  float out_s, out_t;
   {
     const Partial* p = a.partials + static_cast<size_t>(valid ? row : 0) * a.row_stride;
     const size_t cs = static_cast<size_t>(a.chunk_stride);
@@ -263,29 +281,17 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
     if constexpr (kTies) {
       if (valid) settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, m, idx, s, t, gl, L);
     }
-    if (valid && gl == 0) {
-      Partial acc;
-      acc.m = m;
-      acc.idx = idx;
-      acc.s = s;
-      acc.t = t;
-      out = score_row(acc, a, row);
-    }
+    if (valid && gl == 0) out = decide_row(s, t, a, row);
+    out_token = idx;
+    out_s = s;
+    out_t = t;
   }
   const uint32_t word = __ballot_sync(0xffffffffu, valid && gl == 0 && out.flag != 0);
   if (lane == 0) {
-    if (single_block) {
-      flag_words[warp] = word;
-    } else {
-      const uint32_t mine = static_cast<uint32_t>(__cvta_generic_to_shared(&flag_words[blockIdx.x * warps + warp]));
-      uint32_t remote, remote_bar;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(0));
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote_bar) : "r"(bar), "r"(0));
-      asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-                   ::"r"(remote), "r"(word), "r"(remote_bar) : "memory");
-    }
+    if (single_block) flag_words[warp] = word;
+    else send_word(&flag_words[blockIdx.x * warps + warp], bar, word);
   }
-  if (valid && gl == 0) store_row(out, a, row);
+  if (valid && gl == 0) store_row(out, out_token, out_s, out_t, a, row);
   if (blockIdx.x != 0) return;
   if (single_block) __syncthreads();
   else wait_for_words(bar, a.status);
@@ -311,6 +317,75 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
   if (threadIdx.x == 0) {
     *a.routed_count = base_out;
     if (a.status_copy != nullptr) *a.status_copy = atomicOr(a.status, 0u);   // every row has been scored by now
+  }
+}
+
+// The same for steps whose lanes own few partials (rows_shape), and then what stands between the last partial and the end of
+// the step is latency alone: the compaction has a warp of its own -- the last one of block 0 -- that waits for the words and
+// does it while the others still work out their entropies and store their rows.  Per step in a stream, with finish_small_kernel
+// and with this one (partials not tagged): n = 1, d = 256, V = 20000 8.36 and 7.30 us, n = 16, d = 896, V = 151936 45.73 and 44.26
+// (8-bit head 30.0 and 28.4), n = 64, d = 512, V = 32000 12.24 and 11.03, n = 128 there 13.26 and 12.13.
+// kRowWarps: 16, or 8 where a block of 17 warps would not stand beside a CTA of the projection.  No register may be spilled: a kernel that writes local memory ends a
+// microsecond later (four bytes of it, n = 1, d = 256, V = 20000: 6.2 and 7.6 us per step).
+template <bool kTies, int kRowWarps>
+__global__ void __maxnreg__(kTies ? 64 : 40)
+finish_rows_kernel(const FinishLaunch a, const int log2_L) {
+  constexpr int row_warps = kRowWarps;
+  __shared__ uint32_t flag_words[kMaxBlocks * kRowWarps];
+  __shared__ __align__(8) unsigned long long all_here;
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const uint32_t bar = static_cast<uint32_t>(__cvta_generic_to_shared(&all_here));
+  if (blockIdx.x == 0 && threadIdx.x == 0) expect_words(bar, gridDim.x * row_warps);
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  pdl_enter();
+  wait_for_peers(a);
+  if (warp < row_warps) {
+    const int L = 1 << log2_L;
+    const int row = (blockIdx.x * row_warps * 32 + threadIdx.x) >> log2_L;
+    const int gl = threadIdx.x & (L - 1);
+    const bool valid = row < a.n;
+    const int count = valid ? a.chunks : 0;
+    const Partial* p = a.partials + static_cast<size_t>(valid ? row : 0) * a.row_stride;
+    LaneFold<kRowsPerLane> f;
+    f.load(p, gl, L, count, static_cast<size_t>(a.chunk_stride));
+    float m = f.best, s, t;
+    int idx = f.idx;
+    group_best(m, idx, L);
+    f.sums(m, s, t);
+    group_sum(s, t, L);
+    if constexpr (kTies) {
+      const float second = group_max(f.second(m), L);
+      if (valid) settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, m, idx, s, t, gl, L);
+    }
+    const bool mine = valid && gl == 0;
+    Scored out = {};
+    if (mine) out = decide_row(s, t, a, row);
+    const uint32_t word = __ballot_sync(0xffffffffu, out.flag != 0);
+    if (lane == 0) send_word(&flag_words[blockIdx.x * row_warps + warp], bar, word);
+    if (mine) store_row(out, idx, s, t, a, row);
+  } else if (blockIdx.x == 0) {
+    wait_for_words(bar, a.status);
+    if (a.seq_len > 0) {
+      for (int b = lane; b < a.n / a.seq_len; b += 32) a.first_routed[b] = a.seq_len;
+      __syncwarp();
+    }
+    // (A scan over the words, every lane writing the rows of its own, took a microsecond at n = 1 and more than this loop's
+    // eight turns at n = 256.)
+    int total = 0;
+    for (int base = 0; base < a.n; base += 32) {
+      const int i = base + lane;
+      const int flag = i < a.n ? flag_of(flag_words, i, log2_L) : 0;
+      const unsigned int bal = __ballot_sync(0xffffffffu, flag != 0);
+      if (flag) {
+        a.routed_idx[total + __popc(bal & ((1u << lane) - 1u))] = i;
+        first_routed_note(a, i);
+      }
+      total += __popc(bal);
+    }
+    if (lane == 0) *a.routed_count = total;
+    if (lane == 0 && a.status_copy != nullptr) *a.status_copy = atomicOr(a.status, 0u);   // every row has been scored by now
   }
 }
 
@@ -343,7 +418,7 @@ finish_kernel(const FinishLaunch a) {
     Partial acc = fold_row(p, a.chunks, a.chunk_stride, lane, kTies ? &second : nullptr);
     if constexpr (kTies)
       settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, acc.m, acc.idx, acc.s, acc.t, lane, 32);
-    if (lane == 0) store_row(score_row(acc, a, row), a, row);
+    if (lane == 0) store_row(decide_row(acc.s, acc.t, a, row), acc.idx, acc.s, acc.t, a, row);
   }
 
   // ---- which block is last?
@@ -389,6 +464,49 @@ finish_kernel(const FinishLaunch a) {
   }
 }
 
+namespace {
+
+// The launch of the small merge kernel for n <= kSmallRows rows.
+struct SmallShape {
+  int blocks, threads, lanes;
+};
+SmallShape small_shape(int n, int chunks) {
+  SmallShape s;
+  s.blocks = 1;
+  while (s.blocks < 8 && s.blocks * 16 < n) s.blocks <<= 1;       // 16 rows per block until 8 blocks
+  // 512-thread blocks fit on an SM beside a CTA of the tensor-core projection kernel, so they
+  // are resident (waiting) before it ends and do not keep the next call's CTAs off their SMs;
+  // they are used whenever a lane group still owns few enough partials for the one-pass fold.
+  const auto lanes_for = [&](int threads) {
+    int l = 32;
+    while (l > 1 && n * l > s.blocks * threads) l >>= 1;
+    return l;
+  };
+  s.threads = kSmallThreads;
+  if ((chunks + lanes_for(512) - 1) / lanes_for(512) <= kPerLane) s.threads = 512;
+  const int e = tuning().finish_threads;   // tuning switch (TLR_FINISH_THREADS)
+  if (e == 256 || e == 512 || e == 1024) s.threads = e;
+  s.lanes = lanes_for(s.threads);
+  return s;
+}
+
+}  // namespace
+
+// finish_rows_kernel for n rows of `chunks` partials: row warps per block, blocks and lanes per row; false where a lane would own
+// more than kRowsPerLane partials.  small: blocks of 8 row warps.
+bool rows_shape(int n, int chunks, bool small, int* row_warps, int* blocks, int* lanes) {
+  if (n <= 0 || n > kSmallRows) return false;
+  // Eight row warps as long as eight blocks of them give every row a warp: 8 and 16 at n = 16, d = 512, V = 32000 9.5 and 9.9 us,
+  // n = 64 11.1 and 11.3; where only such blocks stand beside the projection's CTAs (64 rows of the 8-bit head, d = 896,
+  // V = 60000) 18.0 and 19.0.
+  *row_warps = small || n <= 8 * kMaxBlocks ? 8 : 16;
+  *blocks = 1;
+  while (*blocks < kMaxBlocks && *blocks * *row_warps < n) *blocks <<= 1;
+  *lanes = 32;
+  while (*lanes > 1 && n * *lanes > *blocks * *row_warps * 32) *lanes >>= 1;
+  return n * *lanes <= *blocks * *row_warps * 32 && (chunks + *lanes - 1) / *lanes <= kRowsPerLane;
+}
+
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
   if (a.chunks > 32 * kPerLane) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
@@ -400,24 +518,20 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (a.n <= kSmallRows) {
-    int blocks = 1;
-    while (blocks < 8 && blocks * 16 < a.n) blocks <<= 1;       // 16 rows per block until 8 blocks
-    // 512-thread blocks fit on an SM beside a CTA of the tensor-core projection kernel, so they
-    // are resident (waiting) before it ends and do not keep the next call's CTAs off their SMs;
-    // they are used whenever a lane group still owns few enough partials for the one-pass fold.
-    auto lanes_for = [&](int threads) {
-      int l = 32;
-      while (l > 1 && a.n * l > blocks * threads) l >>= 1;
-      return l;
-    };
-    int threads = kSmallThreads;
-    if ((a.chunks + lanes_for(512) - 1) / lanes_for(512) <= kPerLane) threads = 512;
-    {
-      const int e = tuning().finish_threads;   // tuning switch (TLR_FINISH_THREADS)
-      if (e == 256 || e == 512 || e == 1024) threads = e;
+    int blocks, threads, lanes, row_warps;
+    const bool ties = a.ties.W != nullptr;
+    auto kernel = ties ? finish_small_ties_kernel : finish_small_kernel;
+    if (rows_shape(a.n, a.chunks, a.small_blocks, &row_warps, &blocks, &lanes)) {
+      threads = (row_warps + 1) * 32;
+      kernel = ties ? finish_rows_kernel<true, 8> : (row_warps == 8 ? finish_rows_kernel<false, 8> : finish_rows_kernel<false, 16>);
+    } else {
+      const SmallShape s = small_shape(a.n, a.chunks);
+      blocks = s.blocks;
+      threads = s.threads;
+      lanes = s.lanes;
     }
     int log2_L = 0;
-    while ((1 << log2_L) < lanes_for(threads)) ++log2_L;
+    while ((1 << log2_L) < lanes) ++log2_L;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = static_cast<unsigned>(blocks);
     attr[1].val.clusterDim.y = 1;
@@ -425,7 +539,7 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     cfg.numAttrs = 2;
     cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
     cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
-    return cudaLaunchKernelEx(&cfg, a.ties.W != nullptr ? finish_small_ties_kernel : finish_small_kernel, a, log2_L);
+    return cudaLaunchKernelEx(&cfg, kernel, a, log2_L);
   }
   const int blocks = (a.n + kFinishWarps - 1) / kFinishWarps;
   cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);

@@ -101,9 +101,9 @@ void tc_configure(int n, int d, int V, int sm_count, TcConfig* c) {
 }
 
 cudaError_t tc_prepare() {
-  for (const auto kernel : {tc_projection_kernel<1, RowMode::kM128>, tc_projection_kernel<1, RowMode::kM64>,
-                            tc_projection_kernel<1, RowMode::kGroup8>, tc_projection_kernel<2, RowMode::kM128>,
-                            tc_projection_kernel<2, RowMode::kM128Keep>}) {
+  for (const auto kernel : {tc_projection_kernel<1, RowMode::kM128, true>, tc_projection_kernel<1, RowMode::kM64, true>,
+                            tc_projection_kernel<1, RowMode::kGroup8, true>, tc_projection_kernel<2, RowMode::kM128, true>,
+                            tc_projection_kernel<2, RowMode::kM128, false>, tc_projection_kernel<2, RowMode::kM128Keep, false>}) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
   }
@@ -126,11 +126,12 @@ cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const Tc
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = c.cta == 1 ? 1 : 2;
-  const auto kernel = c.mode == RowMode::kM128Keep ? tc_projection_kernel<2, RowMode::kM128Keep>
-                      : c.cta == 2                 ? tc_projection_kernel<2, RowMode::kM128>
-                      : c.mode == RowMode::kGroup8 ? tc_projection_kernel<1, RowMode::kGroup8>
-                      : c.mode == RowMode::kM64    ? tc_projection_kernel<1, RowMode::kM64>
-                                                   : tc_projection_kernel<1, RowMode::kM128>;
+  const auto kernel = c.mode == RowMode::kM128Keep ? tc_projection_kernel<2, RowMode::kM128Keep, false>
+                      : c.cta == 2 && p.n > 256    ? tc_projection_kernel<2, RowMode::kM128, false>
+                      : c.cta == 2                 ? tc_projection_kernel<2, RowMode::kM128, true>
+                      : c.mode == RowMode::kGroup8 ? tc_projection_kernel<1, RowMode::kGroup8, true>
+                      : c.mode == RowMode::kM64    ? tc_projection_kernel<1, RowMode::kM64, true>
+                                                   : tc_projection_kernel<1, RowMode::kM128, true>;
   return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 

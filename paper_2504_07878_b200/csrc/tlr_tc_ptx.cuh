@@ -252,12 +252,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes, laid out
 // by TMA with the 128-byte swizzle: 8-row groups 1024 bytes apart (stride offset 64 in
 // 16-byte units), leading offset unused (1), descriptor version 1, layout code 2.
