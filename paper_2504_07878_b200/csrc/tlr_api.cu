@@ -148,6 +148,9 @@ struct tlr_ctx {
   unsigned char* workspace = nullptr;     // one device allocation: the partials, the ticket and status words, the staging
                                           // buffers (ten allocations took most of the time of tlr_create)
   Partial* partials = nullptr;
+  Partial* tagged = nullptr;              // partials of tagged steps (tlr_common.cuh)
+  bool tagged_ok = true;                  // false once a reader's launch has failed: its slots were not left pending
+  uint32_t last_tag = 0;
   unsigned int* ticket = nullptr;
   uint32_t* status = nullptr;
 
@@ -329,7 +332,6 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     p.inline_split = cfg.inline_split;
     p.hscale = c->hscale;
     p.wscale = c->wscale;
-    p.partials = c->partials;
     p.status = c->status;
     if (c->classes > 1) {
       p.d = c->d + tlr::odd_max_shift(c->d);
@@ -408,8 +410,9 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
   const size_t np = static_cast<size_t>(max_n);
   auto padded = [](size_t bytes) { return (bytes + 255) & ~static_cast<size_t>(255); };
   const size_t partial_bytes = padded(np * tlr::kMaxChunks * sizeof(Partial));
+  const size_t tagged_bytes = padded(std::min<size_t>(np * 32 * tlr::kRowsPerLane, tlr::kTaggedPartials) * sizeof(Partial));
   const size_t h_bytes = padded(np * d * 2), out_bytes = padded(np * 17 + 8), pinned_bytes = padded(np * 17 + 8 + 8);
-  bool ok = cudaMalloc(&c->workspace, 256 + partial_bytes + 2 * (h_bytes + out_bytes)) == cudaSuccess;
+  bool ok = cudaMalloc(&c->workspace, 256 + partial_bytes + tagged_bytes + 2 * (h_bytes + out_bytes)) == cudaSuccess;
   ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->out_pinned[0]), 2 * pinned_bytes, cudaHostAllocMapped) == cudaSuccess;
   if (ok) {
     unsigned char* at = c->workspace;
@@ -418,6 +421,8 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
     at += 256;
     c->partials = reinterpret_cast<Partial*>(at);
     at += partial_bytes;
+    c->tagged = reinterpret_cast<Partial*>(at);
+    at += tagged_bytes;
     for (int q = 0; q < 2; ++q) {
       c->h_stage[q] = at;
       c->out_stage[q] = at + h_bytes;
@@ -441,7 +446,8 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
       c->out_mapped[q] = nullptr;   // tlr_route_host then stages the outputs in device memory and copies them
     }
   }
-  if (cudaMemset(c->workspace, 0, 256) != cudaSuccess) {      // the ticket and the status word
+  if (cudaMemset(c->workspace, 0, 256) != cudaSuccess ||      // the ticket and the status word
+      cudaMemset(c->tagged, 0xff, tagged_bytes) != cudaSuccess) {      // every slot pending
     free_all(c);
     return TLR_ERR_CUDA;
   }
@@ -461,10 +467,22 @@ tlr::Ties ties_of(const tlr_ctx* c, const void* h_bf16_dev) {
   return {static_cast<const unsigned short*>(c->W), static_cast<const unsigned short*>(h_bf16_dev), c->d, c->V};
 }
 
-// Enqueues the projection kernel of a call with n > 0 rows: chunk partials into ctx->partials.  router_beside: the 8-bit
-// head's router kernel follows (launch_mlp_beside).
+// The tag of the next call of n rows whose partials are read by the kernel right behind the projection; 0: no tag.
+uint32_t next_tag(tlr_ctx* c, const tlr_ctx::Step* st, int n) {
+  if (!c->tagged_ok || n <= 0 || st->plan.vocab_chunks > 32 * tlr::kRowsPerLane ||
+      static_cast<long long>(n) * st->plan.vocab_chunks > tlr::kTaggedPartials ||
+      st->plan.path != TLR_PATH_TC || c->V >= tlr::kTagIdxMask || (c->classes > 1 && st->odd_block < n))
+    return 0;
+  c->last_tag = c->last_tag % tlr::kMaxTag + 1;
+  return c->last_tag;
+}
+
+// Enqueues the projection kernel of a call with n > 0 rows: chunk partials into ctx->partials, or with a tag into
+// ctx->tagged.  router_beside: the 8-bit head's router kernel follows (launch_mlp_beside).
 tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ctx::Step* st, cudaStream_t stream,
-                             bool router_beside = false) {
+                             uint32_t tag, bool router_beside = false) {
+  st->params.tag = tag;
+  st->params.partials = tag != 0 ? ctx->tagged : ctx->partials;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   if (ctx->timing && ctx->timed < tlr::kMaxTimedLaunches) {
     const size_t need = 2 * static_cast<size_t>(ctx->timed + 1);
@@ -505,7 +523,7 @@ tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ct
       tlr::TcParams p = st->params;
       p.n = rows;
       p.row_units = (rows + 128 * st->cfg.cta - 1) / (128 * st->cfg.cta);
-      p.partials = ctx->partials + static_cast<size_t>(row0) * p.chunks;
+      p.partials += static_cast<size_t>(row0) * p.chunks;
       const int units = p.chunks * p.row_units;
       e = tlr::launch_odd_projection(st->odd, p, st->cfg, units < units_max ? units : units_max, stream);
     }
@@ -788,8 +806,10 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   const tlr_plan& plan = st->plan;
 
   const bool router_beside = want_mlp && ctx->fp8 && (reinterpret_cast<uintptr_t>(ctx->mlp_W1) & 15u) == 0;
+  const bool small_blocks = ctx->fp8 || ctx->classes > 1;
+  const uint32_t tag = !want_mlp && tlr::merges_tagged(n, plan.vocab_chunks, small_blocks) ? next_tag(ctx, st, n) : 0;
   if (n > 0) {
-    const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, router_beside);
+    const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, tag, router_beside);
     if (ps != TLR_OK) return ps;
   }
 
@@ -809,8 +829,9 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   }
 
   tlr::FinishLaunch f = {};
-  f.partials = ctx->partials;
-  f.small_blocks = ctx->fp8 || ctx->classes > 1;
+  f.partials = tag != 0 ? ctx->tagged : ctx->partials;
+  f.tag = tag;
+  f.small_blocks = small_blocks;
   f.n = n;
   f.chunks = plan.vocab_chunks;
   f.row_stride = plan.vocab_chunks;
@@ -835,7 +856,10 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   f.status = ctx->status;
   if (plan.path == TLR_PATH_TC) f.ties = ties_of(ctx, h_bf16_dev);
   f.status_copy = status_copy;
-  if (tlr::launch_finish(f, stream) != cudaSuccess) return TLR_ERR_CUDA;
+  if (tlr::launch_finish(f, stream) != cudaSuccess) {
+    if (tag != 0) ctx->tagged_ok = false;
+    return TLR_ERR_CUDA;
+  }
   return TLR_OK;
 }
 
@@ -854,11 +878,14 @@ tlr_status tlr_shard_summary(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, in
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   tlr_ctx::Step* st = step_for(ctx, n, false);
   const tlr_plan& plan = st->plan;
-  const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream);
+  const uint32_t tag = ctx->classes > 1 ? 0 : next_tag(ctx, st, n);    // (settling ties waits for the grid there)
+  const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, tag);
   if (ps != TLR_OK) return ps;
-  if (tlr::launch_shard_summary(ctx->partials, n, plan.vocab_chunks, v_offset, ties_of(ctx, h_bf16_dev),
-                                static_cast<Partial*>(summary_dev), stream) != cudaSuccess)
+  if (tlr::launch_shard_summary(st->params.partials, tag, n, plan.vocab_chunks, v_offset, ties_of(ctx, h_bf16_dev),
+                                static_cast<Partial*>(summary_dev), stream) != cudaSuccess) {
+    if (tag != 0) ctx->tagged_ok = false;
     return TLR_ERR_CUDA;
+  }
   return TLR_OK;
 }
 
@@ -876,7 +903,7 @@ tlr_status tlr_shard_finish(tlr_ctx* ctx, const void* summaries_dev, int32_t sha
   }
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   tlr::FinishLaunch f = {};
-  f.partials = static_cast<const Partial*>(summaries_dev);   // read in place: summary of shard g, row i at [g * n + i]
+  f.partials = static_cast<Partial*>(const_cast<void*>(summaries_dev));   // read in place: summary of shard g, row i at [g * n + i]
   f.n = n;
   f.chunks = shards;
   f.row_stride = 1;
@@ -966,17 +993,20 @@ tlr_status tlr_shard_push(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, int32
   if (ctx->fp8 && n > tlr::tc8_max_rows()) return TLR_ERR_UNSUPPORTED;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   int chunks = 1;
+  uint32_t tag = 0;
   if (n > 0) {
     tlr_ctx::Step* st = step_for(ctx, n, false);
     chunks = st->plan.vocab_chunks;
-    const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream);
+    tag = ctx->classes > 1 ? 0 : next_tag(ctx, st, n);
+    const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, tag);
     if (ps != TLR_OK) return ps;
   }
   ctx->shard_epoch += 1;
   if (ctx->shard_epoch == 0) ctx->shard_epoch = 2;    // (wrapped: keep the parity sequence, never publish 0)
   const int q = static_cast<int>(ctx->shard_epoch & 1u);
   tlr::ShardPush a;
-  a.partials = ctx->partials;
+  a.partials = tag != 0 ? ctx->tagged : ctx->partials;
+  a.tag = tag;
   a.n = n;
   a.chunks = chunks;
   a.v_offset = v_offset;
@@ -986,7 +1016,10 @@ tlr_status tlr_shard_push(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, int32
   a.peer_flag = ctx->peer_flag[q];
   a.epoch = ctx->shard_epoch;
   a.ticket = ctx->ticket;
-  if (tlr::launch_shard_push(a, stream) != cudaSuccess) return TLR_ERR_CUDA;
+  if (tlr::launch_shard_push(a, stream) != cudaSuccess) {
+    if (tag != 0) ctx->tagged_ok = false;
+    return TLR_ERR_CUDA;
+  }
   return TLR_OK;
 }
 
@@ -1004,7 +1037,7 @@ tlr_status tlr_shard_finish_fused(tlr_ctx* ctx, int32_t n, float tau, int32_t* t
   const int G = ctx->shard_count;
   const size_t np = static_cast<size_t>(ctx->max_n);
   tlr::FinishLaunch f = {};
-  f.partials = reinterpret_cast<const Partial*>(ctx->my_block + shard_header_bytes(G)) + static_cast<size_t>(q) * G * np;
+  f.partials = reinterpret_cast<Partial*>(ctx->my_block + shard_header_bytes(G)) + static_cast<size_t>(q) * G * np;
   f.n = n;
   f.chunks = G;
   f.row_stride = 1;

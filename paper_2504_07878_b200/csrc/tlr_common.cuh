@@ -34,6 +34,56 @@ __device__ __forceinline__ Partial empty_partial() {
   return p;
 }
 
+// Tagged partials.  A kernel that merges partials and stands behind the projection kernel as its programmatic dependent is
+// resident, waiting, long before that kernel ends.  Instead of waiting for the end of that grid and reading the partials
+// then -- about a microsecond for the grid to drain and the wait to be released, and a trip to L2 behind it -- it may look
+// at the partials themselves until they are there.  For that the projection kernel puts the call's tag (1..254) into the
+// index's top byte, and the reader leaves every slot it has read as kPendingIdx: a slot with the call's tag holds this
+// call's partial.  The tag keeps a reader from taking the partials of the call before, whose merge kernel may still be
+// running when this one looks; the reset makes a tag that comes back (after 254 calls, or in a replayed graph) as good as new.
+//   * 16 bytes are written and read by one 128-bit access, so that a partial is never seen in part.
+//   * The reader's grid starts when every CTA of the projection grid has started, so that looking never keeps a writer from
+//     running; and it looks for a bounded number of times only, then waits for the grid like an untagged reader.
+//   * A partial that is there says that its CTA has passed its own wait: whatever came before the projection in the stream
+//     is complete, and outputs may be written.
+//   * The reader waits for the projection grid before it ends, so that who waits for the reader's grid waits for both.
+// Tagged steps have partials of their own (no other path writes there).  Per step in a stream, untagged and tagged: n = 1,
+// d = 256, V = 20000 7.30 and 6.20 us, n = 16, d = 896, V = 151936 44.26 and 42.90 (8-bit head 28.4 and 27.1), n = 64, d = 300,
+// V = 33000 12.31 and 11.57, one of eight shards at n = 256 18.07 and 17.34; n = 256, d = 512, V = 32000 14.5 either way.
+constexpr int kTagShift = 24;
+constexpr int kTagIdxMask = (1 << kTagShift) - 1;      // an index; all ones stand for kNoToken
+constexpr int kPendingIdx = -1;
+constexpr int kMaxTag = 254;
+constexpr int kTaggedPartials = 8 * 16 * 32 * 5;        // of a step: what finish_rows_kernel's lanes can own (328 KB)
+constexpr int kMaxLooks = 1 << 14;                     // about 10 ms
+
+__device__ __forceinline__ void store_partial(Partial* dst, const Partial& p) {
+  asm volatile("{\n\t.reg .b128 v;\n\t.reg .b64 lo, hi;\n\t"
+               "mov.b64 lo, {%1, %2};\n\tmov.b64 hi, {%3, %4};\n\tmov.b128 v, {lo, hi};\n\t"
+               "st.relaxed.gpu.global.b128 [%0], v;\n\t}"
+               ::"l"(dst), "f"(p.m), "r"(p.idx), "f"(p.s), "f"(p.t) : "memory");
+}
+__device__ __forceinline__ Partial load_partial(const Partial* src) {
+  Partial p;
+  asm volatile("{\n\t.reg .b128 v;\n\t.reg .b64 lo, hi;\n\t"
+               "ld.relaxed.gpu.global.b128 v, [%4];\n\tmov.b128 {lo, hi}, v;\n\t"
+               "mov.b64 {%0, %1}, lo;\n\tmov.b64 {%2, %3}, hi;\n\t}"
+               : "=f"(p.m), "=r"(p.idx), "=f"(p.s), "=f"(p.t) : "l"(src) : "memory");
+  return p;
+}
+__device__ __forceinline__ int tagged_idx(int idx, uint32_t tag) {
+  return static_cast<int>((static_cast<uint32_t>(idx) & kTagIdxMask) | (tag << kTagShift));
+}
+__device__ __forceinline__ int untagged_idx(int idx) {
+  const int i = idx & kTagIdxMask;
+  return i == kTagIdxMask ? kNoToken : i;
+}
+
+// Leaves the slots of a lane pending.
+__device__ __forceinline__ void reset_tagged(Partial* p, int first, int stride, int count) {
+  for (int j = first; j < count; j += stride) p[j].idx = kPendingIdx;
+}
+
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -92,11 +142,11 @@ struct LaneFold {
       s[k] = t[k] = 0.f;
     }
   }
-  __device__ __forceinline__ void put(int k, const Partial& v) {
+  __device__ __forceinline__ void put(int k, const Partial& v, int v_idx) {
     m[k] = v.m;
     s[k] = v.s;
     t[k] = v.t;
-    idx = v.m > best ? v.idx : (v.m == best ? min(v.idx, idx) : idx);
+    idx = v.m > best ? v_idx : (v.m == best ? min(v_idx, idx) : idx);
     best = fmaxf(best, v.m);
   }
   __device__ __forceinline__ void load(const Partial* p, int first, int stride, int count, size_t chunk_stride) {
@@ -112,7 +162,40 @@ struct LaneFold {
         v.s = raw.z;
         v.t = raw.w;
       }
-      put(k, v);
+      put(k, v, v.idx);
+    }
+  }
+  // Tagged partials, chunk stride 1; called by whole warps.  hint: look at nothing but the row's last one until it is there.
+  // A look is one trip to L2: all of a lane's loads go out before the first is examined (one after the other they took
+  // 1.8 us a look).
+  __device__ __forceinline__ void take(const Partial* p, int first, int stride, int count, uint32_t tag, bool hint) {
+    const auto here = [&](int i) { return (static_cast<uint32_t>(i) >> kTagShift) == tag; };
+    Partial v[kN];
+    int looks = 0;
+    if (hint)
+      while (looks < kMaxLooks && !__all_sync(0xffffffffu, count == 0 || here(load_partial(p + count - 1).idx))) ++looks;
+    bool waited = false;
+    for (;;) {
+      bool all = true;
+#pragma unroll
+      for (int k = 0; k < kN; ++k)
+        if (first + stride * k < count) v[k] = load_partial(p + first + stride * k);
+#pragma unroll
+      for (int k = 0; k < kN; ++k)
+        if (first + stride * k < count) all = all && here(v[k].idx);
+      if (__all_sync(0xffffffffu, all) || waited) break;
+      if (++looks >= kMaxLooks) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        waited = true;
+      }
+    }
+    best = -INFINITY;
+    idx = kNoToken;
+#pragma unroll
+    for (int k = 0; k < kN; ++k) {
+      // (one that was never written -- the projection gave up -- counts as empty)
+      const bool there = first + stride * k < count && here(v[k].idx);
+      put(k, there ? v[k] : empty_partial(), there ? untagged_idx(v[k].idx) : kNoToken);
     }
   }
   // The sums rescaled to the row's maximum.  An empty range contributes nothing; a NaN sum goes through.
@@ -163,11 +246,21 @@ __device__ __forceinline__ float group_max(float v, int L) {
   return v;
 }
 
-// Folds one row's partials.  Every lane returns the same result.  `second` (optional): the largest of the partials' maxima
-// below the row's.
+// Folds one row's partials (tagged ones if tag is not 0; chunk_stride is 1 then).  Every lane returns the same result.
+// `second` (optional, untagged only): the largest of the partials' maxima below the row's.
 __device__ __forceinline__ Partial fold_row(const Partial* p, int chunks, int chunk_stride, int lane,
-                                            float* second = nullptr) {
+                                            float* second = nullptr, uint32_t tag = 0) {
   Partial r;
+  if (tag != 0) {
+    LaneFold<kRowsPerLane> f;
+    f.take(p, lane, 32, chunks, tag, true);
+    r.m = f.best;
+    r.idx = f.idx;
+    group_best(r.m, r.idx, 32);
+    f.sums(r.m, r.s, r.t);
+    group_sum(r.s, r.t, 32);
+    return r;
+  }
   LaneFold<kPerLane> f;
   f.load(p, lane, 32, chunks, chunk_stride);
   r.m = f.best;
@@ -193,7 +286,8 @@ __device__ __forceinline__ float bf16_value(unsigned short bits) { return __uint
 // products' magnitudes.  Bound by the trips to memory and, a row's lanes being few, by instructions: every line of the row of W
 // is asked for before the first is used, a lane has six loads of either operand in flight, and they are two elements wide
 // where d is even (rows have no alignment beyond one element or two).
-template <bool kPairs>
+// kFresh: h may have been written since this grid started and is read past L1 (which costs n = 200, d = 999, V = 60000 51.6 -> 56.6 us).
+template <bool kPairs, bool kFresh>
 __device__ __forceinline__ float2 lane_logit(const unsigned short* w, const unsigned short* h, int d, int gl, int L) {
   constexpr int kBatch = 6;
   const int loads = kPairs ? d >> 1 : d;
@@ -205,7 +299,8 @@ __device__ __forceinline__ float2 lane_logit(const unsigned short* w, const unsi
       const int k = k0 + i * L;
       x[i] = y[i] = 0u;
       if (k < loads) {
-        x[i] = kPairs ? reinterpret_cast<const uint32_t*>(h)[k] : h[k];
+        if (kFresh) x[i] = kPairs ? __ldcg(reinterpret_cast<const uint32_t*>(h) + k) : __ldcg(h + k);
+        else x[i] = kPairs ? reinterpret_cast<const uint32_t*>(h)[k] : h[k];
         y[i] = kPairs ? reinterpret_cast<const uint32_t*>(w)[k] : w[k];
       }
     }
@@ -223,11 +318,12 @@ __device__ __forceinline__ float2 lane_logit(const unsigned short* w, const unsi
   }
   return make_float2(z, size);
 }
+template <bool kFresh>
 __device__ __forceinline__ float row_logit(const unsigned short* W, const unsigned short* h, int d, int v, int gl, int L,
                                            unsigned int group, float* size) {
   const unsigned short* w = W + static_cast<size_t>(v) * d;
   for (int k = gl * 64; k < d; k += L * 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(w + k));
-  float2 r = (d & 1) == 0 ? lane_logit<true>(w, h, d, gl, L) : lane_logit<false>(w, h, d, gl, L);
+  float2 r = (d & 1) == 0 ? lane_logit<true, kFresh>(w, h, d, gl, L) : lane_logit<false, kFresh>(w, h, d, gl, L);
   for (int off = L >> 1; off > 0; off >>= 1) {
     r.x += __shfl_xor_sync(group, r.x, off);
     r.y += __shfl_xor_sync(group, r.y, off);
@@ -243,6 +339,7 @@ struct Winner {
   int idx;
   float z;
 };
+template <bool kTagged>
 static __device__ __forceinline__ Winner settle_ties(const Ties ties, int row, const Partial* __restrict__ p, int chunks,
                                                int chunk_stride, float least, int idx, float z, int gl, int L) {
   const unsigned short* h = ties.h + static_cast<size_t>(row) * ties.d;
@@ -255,14 +352,14 @@ static __device__ __forceinline__ Winner settle_ties(const Ties ties, int row, c
     int mine = kNoToken;
     if (j < chunks) {
       const Partial* q = p + static_cast<size_t>(j) * chunk_stride;
-      if (__ldcg(&q->m) >= least) mine = __ldcg(&q->idx);
+      if (__ldcg(&q->m) >= least) mine = kTagged ? untagged_idx(__ldcg(&q->idx)) : __ldcg(&q->idx);
     }
     unsigned int todo = __ballot_sync(group, mine < ties.V && mine != idx) & group;
     while (todo != 0u) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
       const int v = __shfl_sync(group, mine, src);
-      const float zv = row_logit(ties.W, h, ties.d, v, gl, L, group, &size);
+      const float zv = row_logit<kTagged>(ties.W, h, ties.d, v, gl, L, group, &size);
       if (zv > win.z || (zv == win.z && v < win.idx)) {
         win.z = zv;
         win.idx = v;
@@ -285,6 +382,7 @@ static __device__ __forceinline__ Winner settle_ties(const Ties ties, int row, c
 // 64 bits (2-norm) as the projection leaves them, here, and on CUDA cores, where these heads ran before: d = 300 6.7e-7,
 // 1.7e-7, 3.2e-7; d = 999 2.3e-6, 1.7e-7, 8.7e-7.
 // A row that is not finite stays as it is; so does one whose index lies beyond V.
+template <bool kTagged = false>
 __device__ __forceinline__ void settle_row(const Ties& ties, int row, const Partial* __restrict__ p, int chunks,
                                            int chunk_stride, float second, float& m, int& idx, float& s, float& t, int gl,
                                            int L) {
@@ -292,10 +390,10 @@ __device__ __forceinline__ void settle_row(const Ties& ties, int row, const Part
   const unsigned int lane = threadIdx.x & 31;
   const unsigned int group = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (lane - gl);
   float size;
-  float z = row_logit(ties.W, ties.h + static_cast<size_t>(row) * ties.d, ties.d, idx, gl, L, group, &size);
+  float z = row_logit<kTagged>(ties.W, ties.h + static_cast<size_t>(row) * ties.d, ties.d, idx, gl, L, group, &size);
   const float least = m - (ties.d / 16 + 9) * 0x1p-20f * size;
   if (second >= least) {
-    const Winner win = settle_ties(ties, row, p, chunks, chunk_stride, least, idx, z, gl, L);
+    const Winner win = settle_ties<kTagged>(ties, row, p, chunks, chunk_stride, least, idx, z, gl, L);
     idx = win.idx;
     z = win.z;
   }
@@ -321,7 +419,8 @@ cudaError_t launch_simt_projection(const SimtLaunch& a, cudaStream_t stream);
 void simt_plan(int n, int d, int V, int sm_count, int* chunks, int* grid, int* block, int* smem);
 
 struct FinishLaunch {
-  const Partial* partials;  // partial j of row i at partials[i * row_stride + j * chunk_stride]
+  Partial* partials;        // partial j of row i at partials[i * row_stride + j * chunk_stride]
+  uint32_t tag;             // not 0: tagged partials, chunk_stride 1 (only where merges_tagged())
   bool small_blocks;        // the projection's CTAs leave room for small blocks only (and always with ties to settle)
   int n, chunks;
   int row_stride, chunk_stride;   // [n][chunks]: (chunks, 1); a block gathered shard-major [shards][rows]: (1, rows)
@@ -354,15 +453,18 @@ struct FinishLaunch {
   uint32_t* status_copy;    // optional: receives the status word once every row is scored (host-mapped memory)
 };
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream);
+bool merges_tagged(int n, int chunks, bool small_blocks);    // whether launch_finish takes tagged partials for this size
 
 // Vocabulary-sharded decode (tlr_shard.cu): one summary per row from a shard's chunk partials,
 // and the gathered summaries [shards][n] laid out as partials [n][shards].
-cudaError_t launch_shard_summary(const Partial* partials, int n, int chunks, int v_offset, const Ties& ties,
+// (tag not 0: tagged partials)
+cudaError_t launch_shard_summary(Partial* partials, uint32_t tag, int n, int chunks, int v_offset, const Ties& ties,
                                  Partial* summary, cudaStream_t stream);
 // Fused exchange: the summaries are stored straight into slot `rank` of every peer's exchange block and, once all
 // rows are out, this rank's flag in every peer's flag array is set to `epoch` (peer stores only).
 struct ShardPush {
-  const Partial* partials;   // this shard's chunk partials [n][chunks]
+  Partial* partials;         // this shard's chunk partials [n][chunks]
+  uint32_t tag;              // not 0: tagged ones
   int n, chunks, v_offset;
   Ties ties;
   int shards;                // peers, this rank included

@@ -86,9 +86,11 @@ __device__ __forceinline__ void first_routed_note(const FinishLaunch& a, int row
 // Programmatic dependent launch: let the next kernel in the stream be scheduled now (it
 // waits for this grid to complete before touching memory), then wait for the projection
 // kernel's partials.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_trigger();
+  pdl_wait();
 }
 
 // Vocabulary-sharded step with the fused exchange: the other GPUs store their summaries into this GPU's
@@ -325,9 +327,10 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
 // does it while the others still work out their entropies and store their rows.  Per step in a stream, with finish_small_kernel
 // and with this one (partials not tagged): n = 1, d = 256, V = 20000 8.36 and 7.30 us, n = 16, d = 896, V = 151936 45.73 and 44.26
 // (8-bit head 30.0 and 28.4), n = 64, d = 512, V = 32000 12.24 and 11.03, n = 128 there 13.26 and 12.13.
+// kTagged: the partials are tagged ones (tlr_common.cuh), no peers and no learned router.
 // kRowWarps: 16, or 8 where a block of 17 warps would not stand beside a CTA of the projection.  No register may be spilled: a kernel that writes local memory ends a
 // microsecond later (four bytes of it, n = 1, d = 256, V = 20000: 6.2 and 7.6 us per step).
-template <bool kTies, int kRowWarps>
+template <bool kTies, bool kTagged, int kRowWarps>
 __global__ void __maxnreg__(kTies ? 64 : 40)
 finish_rows_kernel(const FinishLaunch a, const int log2_L) {
   constexpr int row_warps = kRowWarps;
@@ -339,17 +342,21 @@ finish_rows_kernel(const FinishLaunch a, const int log2_L) {
   if (blockIdx.x == 0 && threadIdx.x == 0) expect_words(bar, gridDim.x * row_warps);
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  pdl_enter();
-  wait_for_peers(a);
+  pdl_trigger();
+  if constexpr (!kTagged) {
+    pdl_wait();
+    wait_for_peers(a);
+  }
   if (warp < row_warps) {
     const int L = 1 << log2_L;
     const int row = (blockIdx.x * row_warps * 32 + threadIdx.x) >> log2_L;
     const int gl = threadIdx.x & (L - 1);
     const bool valid = row < a.n;
     const int count = valid ? a.chunks : 0;
-    const Partial* p = a.partials + static_cast<size_t>(valid ? row : 0) * a.row_stride;
+    Partial* p = a.partials + static_cast<size_t>(valid ? row : 0) * a.row_stride;
     LaneFold<kRowsPerLane> f;
-    f.load(p, gl, L, count, static_cast<size_t>(a.chunk_stride));
+    if constexpr (kTagged) f.take(p, gl, L, count, a.tag, gridDim.x > 1);
+    else f.load(p, gl, L, count, static_cast<size_t>(a.chunk_stride));
     float m = f.best, s, t;
     int idx = f.idx;
     group_best(m, idx, L);
@@ -357,7 +364,7 @@ finish_rows_kernel(const FinishLaunch a, const int log2_L) {
     group_sum(s, t, L);
     if constexpr (kTies) {
       const float second = group_max(f.second(m), L);
-      if (valid) settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, m, idx, s, t, gl, L);
+      if (valid) settle_row<kTagged>(a.ties, row, p, a.chunks, a.chunk_stride, second, m, idx, s, t, gl, L);
     }
     const bool mine = valid && gl == 0;
     Scored out = {};
@@ -365,6 +372,7 @@ finish_rows_kernel(const FinishLaunch a, const int log2_L) {
     const uint32_t word = __ballot_sync(0xffffffffu, out.flag != 0);
     if (lane == 0) send_word(&flag_words[blockIdx.x * row_warps + warp], bar, word);
     if (mine) store_row(out, idx, s, t, a, row);
+    if (kTagged && valid) reset_tagged(p, gl, L, a.chunks);
   } else if (blockIdx.x == 0) {
     wait_for_words(bar, a.status);
     if (a.seq_len > 0) {
@@ -385,6 +393,7 @@ finish_rows_kernel(const FinishLaunch a, const int log2_L) {
       total += __popc(bal);
     }
     if (lane == 0) *a.routed_count = total;
+    if (kTagged) pdl_wait();
     if (lane == 0 && a.status_copy != nullptr) *a.status_copy = atomicOr(a.status, 0u);   // every row has been scored by now
   }
 }
@@ -507,8 +516,13 @@ bool rows_shape(int n, int chunks, bool small, int* row_warps, int* blocks, int*
   return n * *lanes <= *blocks * *row_warps * 32 && (chunks + *lanes - 1) / *lanes <= kRowsPerLane;
 }
 
+bool merges_tagged(int n, int chunks, bool small) {
+  int row_warps, blocks, lanes;
+  return rows_shape(n, chunks, small, &row_warps, &blocks, &lanes);
+}
+
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
-  if (a.chunks > 32 * kPerLane) return cudaErrorInvalidValue;
+  if (a.chunks > 32 * kPerLane || (a.tag != 0 && !merges_tagged(a.n, a.chunks, a.small_blocks))) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.dynamicSmemBytes = 0;
   cfg.stream = stream;
@@ -523,7 +537,9 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     auto kernel = ties ? finish_small_ties_kernel : finish_small_kernel;
     if (rows_shape(a.n, a.chunks, a.small_blocks, &row_warps, &blocks, &lanes)) {
       threads = (row_warps + 1) * 32;
-      kernel = ties ? finish_rows_kernel<true, 8> : (row_warps == 8 ? finish_rows_kernel<false, 8> : finish_rows_kernel<false, 16>);
+      if (ties) kernel = a.tag != 0 ? finish_rows_kernel<true, true, 8> : finish_rows_kernel<true, false, 8>;
+      else if (row_warps == 8) kernel = a.tag != 0 ? finish_rows_kernel<false, true, 8> : finish_rows_kernel<false, false, 8>;
+      else kernel = a.tag != 0 ? finish_rows_kernel<false, true, 16> : finish_rows_kernel<false, false, 16>;
     } else {
       const SmallShape s = small_shape(a.n, a.chunks);
       blocks = s.blocks;

@@ -70,6 +70,7 @@ struct TcParams {
   const float* hscale;   // [n] power-of-two scale of every row of h (written by the split kernel)
   const float* wscale;   // [V] scale of every row of W
   Partial* partials;     // [n][chunks]
+  uint32_t tag;          // not 0: they are tagged (tlr_common.cuh)
   uint32_t* status;
 };
 

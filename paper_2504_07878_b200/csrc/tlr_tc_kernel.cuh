@@ -818,12 +818,13 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
             if (mlp_unit) p.mlp_out[row] = out[i].s + other[i].s;   // lower columns first: a fixed order
             else {
               Partial* dst = p.partials + static_cast<size_t>(row) * p.chunks + first.chunk;
-              const Partial sum = merge(out[i], other[i]);
+              Partial sum = merge(out[i], other[i]);
+              if (p.tag != 0) sum.idx = tagged_idx(sum.idx, p.tag);
               if (kCta == 2 && unit + workers >= units) {     // (stored behind the arrival at the cluster's barrier)
                 last = sum;
                 last_dst = dst;
               } else {
-                *dst = sum;
+                store_partial(dst, sum);
               }
             }
           }
@@ -838,7 +839,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
     // Neither CTA frees TMEM or exits while the peer still works.  The last partials go out behind the arrival: in front
     // of it the release would wait until L2 has acknowledged them, 0.7 us at the end of every launch.
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    if (last_dst != nullptr) *last_dst = last;
+    if (last_dst != nullptr) store_partial(last_dst, last);
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
   if (warp == 1) {

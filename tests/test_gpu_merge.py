@@ -48,3 +48,52 @@ def test_edges_of_the_merge_blocks(pkg, kind, n):
     assert got["routed_count"] == mask.sum() and np.array_equal(got["routed_idx"][:mask.sum()], np.flatnonzero(mask))
     assert np.array_equal(to_np(first), 1 - mask)         # sequences of one row: position 0 if routed, else 1
     r.close()
+
+
+def _expect(kind, r, h, n):
+    """What the router gives for a batch when nothing else is in flight."""
+    torch.cuda.synchronize()
+    r.route(h, 0.5)
+    torch.cuda.synchronize()
+    return [t.copy() for t in (to_np(r.token[:n]), to_np(r.conf[:n]), to_np(r.entropy[:n]), to_np(r.route_mask[:n]))]
+
+
+# Steps that nothing waits between, of different sizes and inputs: each merge may look for its partials while the one before is
+# still at work on its own, in the same memory.  More steps than there are tags (254); and replayed, when the tags come back.
+@pytest.mark.parametrize("kind", ["bf16", "8bit", "odd"])
+@pytest.mark.parametrize("graph", [False, True])
+def test_steps_back_to_back_keep_their_partials(pkg, kind, graph):
+    (W, scale), _, d = _head(kind)
+    sizes = [1, 16, 8, 64, 17, 128] + ([] if kind == "8bit" else [256, 200, 300])
+    r = pkg.Router(W, max_n=max(sizes), wscale=scale)
+    batches = [S.make_h(n, d, seed=100 + n).h.cuda() for n in sizes]
+    want = [_expect(kind, r, h, n) for h, n in zip(batches, sizes)]
+    steps = 600
+    kept = [[torch.empty_like(t[:n]) for t in (r.token, r.conf, r.entropy, r.route_mask)] for n in sizes]
+
+    def loop():
+        for i in range(steps):
+            k = (i * 7) % len(sizes)
+            r.route(batches[k], 0.5)
+            if i >= steps - 2 * len(sizes):               # the last rounds are looked at
+                for dst, src in zip(kept[k], (r.token, r.conf, r.entropy, r.route_mask)):
+                    dst.copy_(src[:sizes[k]])
+
+    if graph:
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            loop()
+        for _ in range(3):
+            g.replay()
+    else:
+        loop()
+    torch.cuda.synchronize()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    for got, ref in zip(kept, want):
+        for a, b in zip(got, ref):
+            assert np.array_equal(to_np(a), b)
+    if graph:
+        del g
+    r.close()
