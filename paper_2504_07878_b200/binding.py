@@ -43,6 +43,16 @@ class TlrError(RuntimeError):
 _lib = None
 
 
+def _native_route():
+    """tlr_torch.cpp's route, or a function that declines every call."""
+    try:
+        from . import _tlr_torch
+    except ImportError:
+        return lambda *args: None
+    _tlr_torch.bind(ctypes.cast(load_library().tlr_route, c_void_p).value)
+    return _tlr_torch.route
+
+
 def load_library() -> ctypes.CDLL:
     """Loads libtlr.so from the package directory; raises if it has not been built."""
     global _lib
@@ -330,6 +340,7 @@ class Router:
         self.V, self.d = W.shape
         self.max_n = max_n
         self._tlr_route = load_library().tlr_route
+        self._native = _native_route()
         with torch.cuda.device(W.device):
             self.ctx = tlr_create_fp8(self.d, self.V, W, wscale, max_n) if fp8 else tlr_create(self.d, self.V, W, max_n)
             dev = W.device
@@ -365,11 +376,19 @@ class Router:
     def route(self, h: torch.Tensor, tau: float, stream=None, tau_per_row=None, route_above=False, seq_len=0,
               first_routed=None, score_source=0, mlp_score=None):
         """Enqueues one routing step; returns views of the output tensors (valid after the stream syncs)."""
+        plain = tau_per_row is None and not route_above and seq_len == 0 and score_source == 0 and mlp_score is None
+        if plain and stream is None and _raw_handle and self.ctx is not None:
+            done = self._native(self.ctx.value, self.d, h, tau, self._views, self.routed_idx, self.routed_count,
+                                _raw_stream(_current_device()))
+            if done.__class__ is tuple:
+                return done
+            if done is not None:
+                raise TlrError(done, "tlr_route")
         if not (h.is_cuda and h.dtype == torch.bfloat16 and h.dim() == 2 and h.is_contiguous()
                 and h.shape[1] == self.d):
             raise ValueError("h must be a contiguous CUDA bf16 [n, d] tensor")
         n = h.shape[0]
-        if tau_per_row is None and not route_above and seq_len == 0 and score_source == 0 and mlp_score is None:
+        if plain:
             # (tlr_route without its calls per argument: they cost about what the views do that are handed out)
             handle = _raw_stream(_current_device()) if stream is None and _raw_handle else _stream_handle(stream)
             code = self._tlr_route(self.ctx, h.data_ptr(), n, tau, self.token.data_ptr(), self.conf.data_ptr(),

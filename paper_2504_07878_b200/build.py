@@ -1,4 +1,4 @@
-"""Builds libtlr.so (the C-ABI routing library) in-tree with nvcc for sm_100a.
+"""Builds libtlr.so (the C-ABI routing library) in-tree with nvcc for sm_100a, and _tlr_torch.so (Router.route's marshalling).
 
     python -m paper_2504_07878_b200.build [--force] [--verbose]
 """
@@ -14,6 +14,8 @@ PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libtlr.so")
+TORCH_PATH = os.path.join(PKG_DIR, "_tlr_torch.so")
+TORCH_SOURCE = os.path.join(CSRC, "tlr_torch.cpp")
 
 
 def sources():
@@ -31,7 +33,32 @@ def is_stale() -> bool:
     return any(os.path.getmtime(p) > built for p in _deps())
 
 
+def torch_is_stale() -> bool:
+    return not os.path.exists(TORCH_PATH) or os.path.getmtime(TORCH_PATH) < os.path.getmtime(TORCH_SOURCE)
+
+
+def build_torch() -> str:
+    """The extension module: host code only, against the headers of the torch that imports it."""
+    import sysconfig
+
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    libs = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi()),
+           "-I", os.path.join(ROOT, "include"), "-isystem", sysconfig.get_paths()["include"]]
+    for path in include_paths():
+        cmd += ["-isystem", path]
+    cmd += [TORCH_SOURCE, "-o", TORCH_PATH, "-L", libs, "-ltorch_python", "-ltorch_cpu", "-lc10"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
+    return TORCH_PATH
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    if force or torch_is_stale():
+        build_torch()
     if not force and not is_stale():
         return LIB_PATH
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"

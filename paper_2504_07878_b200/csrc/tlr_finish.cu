@@ -552,7 +552,7 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     attr[1].val.clusterDim.x = static_cast<unsigned>(blocks);
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 2;      // (a single block, too, is launched as a cluster: mapa and st.async are illegal without one)
     cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
     cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
     return cudaLaunchKernelEx(&cfg, kernel, a, log2_L);

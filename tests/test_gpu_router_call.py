@@ -1,0 +1,49 @@
+"""Router.route's native call against the same call through ctypes: outputs, views, errors."""
+import pytest
+import torch
+
+import tlr_synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [0, 1, 5])
+def test_native_call_hands_out_what_the_other_does(pkg, n):
+    from paper_2504_07878_b200 import binding, build
+    build.build()
+    r = pkg.Router(S.make_W(64, 3000, seed=1, std=0.2).cuda(), max_n=5)
+    assert "built-in" in repr(binding._native_route()) and "built-in" in repr(r._native)
+    h = S.make_h(max(n, 1), 64, seed=2).h[:n].cuda()
+    native, r._native = r._native, lambda *args: None
+    want = [t.clone() for t in r.route(h, 0.01)]                 # through ctypes; makes the views of this size
+    r._native = native
+    first, second = r.route(h, 0.01), r.route(h, 0.01)
+    torch.cuda.synchronize()
+    own = (r.token, r.conf, r.entropy, r.route_mask)
+    assert all(torch.equal(a, b) for a, b in zip(first[:4], want[:4])) and torch.equal(first[5], want[5])
+    assert all(a is not b for a, b in zip(first[:4], second[:4]))
+    assert all(a.shape == (n,) and (n == 0 or a.data_ptr() == t.data_ptr()) for a, t in zip(first, own))
+    assert first[4] is r.routed_idx and first[5] is r.routed_count
+    r.conf = torch.zeros_like(r.conf)                            # a replaced tensor is the one that is written
+    again = r.route(h, 0.01)
+    torch.cuda.synchronize()
+    assert torch.equal(again[1], want[1]) and (n == 0 or again[1].data_ptr() == r.conf.data_ptr())
+    r.close()
+
+
+def test_native_call_refuses_what_the_other_does(pkg):
+    r = pkg.Router(S.make_W(64, 3000, seed=1, std=0.2).cuda(), max_n=4)
+    h = S.make_h(4, 64, seed=2).h.cuda()
+    r.route(h, 0.5)
+    for bad in (h.float(), h.cpu(), h[:, :32], h.t(), h[0], torch.cat([h, h], 1)):
+        with pytest.raises(ValueError):
+            r.route(bad, 0.5)
+    shifted = torch.empty(4 * 64 + 1, dtype=torch.bfloat16, device="cuda")[1:].view(4, 64)      # 2 bytes past 16
+    with pytest.raises(pkg.TlrError) as e:
+        r.route(shifted, 0.5)
+    assert e.value.code == 2
+    with pytest.raises(pkg.TlrError) as e:
+        r.route(torch.cat([h, h]), 0.5)
+    assert e.value.code == 6
+    torch.cuda.synchronize()
+    r.close()
