@@ -59,7 +59,7 @@ h_split_kernel(const __nv_bfloat16* h, int n, int d, int part_rows, uint8_t* __r
   const uint4* src = reinterpret_cast<const uint4*>(h + static_cast<size_t>(row) * d);
   const int chunks = d >> 4;                                   // d is a multiple of 16
   uint4 v[kKeep][2];
-  float amax = 0.f;
+  uint32_t pair = 0u;
 #pragma unroll
   for (int i = 0; i < kKeep; ++i) {
     const int c = threadIdx.x + 128 * i;
@@ -68,9 +68,10 @@ h_split_kernel(const __nv_bfloat16* h, int n, int d, int part_rows, uint8_t* __r
     v[i][1] = in ? __ldcg(src + 2 * c + 1) : make_uint4(0u, 0u, 0u, 0u);
   }
 #pragma unroll
-  for (int i = 0; i < kKeep; ++i) amax = fmaxf(amax, fmaxf(abs_max8(v[i][0]), abs_max8(v[i][1])));
+  for (int i = 0; i < kKeep; ++i) pair = abs_max8(abs_max8(pair, v[i][0]), v[i][1]);
   for (int c = threadIdx.x + 128 * kKeep; c < chunks; c += 128)
-    amax = fmaxf(amax, fmaxf(abs_max8(src[2 * c]), abs_max8(src[2 * c + 1])));
+    pair = abs_max8(abs_max8(pair, src[2 * c]), src[2 * c + 1]);
+  float amax = larger_of(pair);
   __shared__ float red[4];
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));

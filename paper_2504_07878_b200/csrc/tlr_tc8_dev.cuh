@@ -26,16 +26,16 @@ __device__ __forceinline__ uint32_t instr_desc_e4m3(int m_rows, int n_cols) {
   return (1u << 4) | (static_cast<uint32_t>(n_cols >> 3) << 17) | (static_cast<uint32_t>(m_rows >> 4) << 24);
 }
 
-// Two floats -> two e4m3 (round to nearest even, saturating), and back.
-__device__ __forceinline__ uint16_t to_e4m3x2(float hi, float lo) {
+// Two halves -> two e4m3 (round to nearest even, saturating), and back.
+__device__ __forceinline__ uint16_t to_e4m3x2(uint32_t h2) {
   uint16_t r;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
+  asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(r) : "r"(h2));
   return r;
 }
-__device__ __forceinline__ float2 from_e4m3x2(uint16_t v) {   // .x = low byte, .y = high byte
+__device__ __forceinline__ uint32_t from_e4m3x2(uint16_t v) {
   uint32_t h2;
   asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"(v));
-  return __half22float2(*reinterpret_cast<__half2*>(&h2));
+  return h2;
 }
 
 // Where a token's two parts sit in the operand slab.  Up to 64 token rows they alternate in groups of eight -- rows
@@ -58,22 +58,30 @@ __device__ __forceinline__ float split_scale(float amax) {
   return r;
 }
 
-// x * inv as the sum of two e4m3 numbers: p1 = round(x), p2 = round(x - p1), two elements at a time.
+// x * inv as the sum of two e4m3 numbers: p1 = round(x), p2 = round(x - p1), two elements at a time and in halves: down to
+// 2^-17 a bf16 number below 256 is a half, and below that both parts are zero (e4m3's smallest step is 2^-9).
+// (In floats, with the magnitudes compared one by one: n = 16, d = 896, V = 151936 26.9 us per step, so 26.5; n = 32, d = 512,
+// V = 30000 9.36 and 9.19.)
 __device__ __forceinline__ void split_pair(float x0, float x1, uint16_t& p1, uint16_t& p2) {
-  p1 = to_e4m3x2(x1, x0);
-  const float2 f1 = from_e4m3x2(p1);
-  p2 = to_e4m3x2(x1 - f1.y, x0 - f1.x);
+  const __half2 x = __floats2half2_rn(x0, x1);
+  p1 = to_e4m3x2(*reinterpret_cast<const uint32_t*>(&x));
+  const uint32_t back = from_e4m3x2(p1);
+  const __half2 rest = __hsub2(x, *reinterpret_cast<const __half2*>(&back));
+  p2 = to_e4m3x2(*reinterpret_cast<const uint32_t*>(&rest));
 }
 
-__device__ __forceinline__ float abs_max8(const uint4& v) {     // of eight bf16
+// The larger magnitudes of the pair m and of eight bf16, pair by pair (NaNs are dropped), and the larger of a pair.
+__device__ __forceinline__ uint32_t abs_max8(uint32_t m, const uint4& v) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  float m = 0.f;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-    m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
+    const uint32_t a = w[j] & 0x7fff7fffu;
+    asm("max.bf16x2 %0, %0, %1;" : "+r"(m) : "r"(a));
   }
   return m;
+}
+__device__ __forceinline__ float larger_of(uint32_t pair) {
+  return fmaxf(__uint_as_float(pair << 16), __uint_as_float(pair & 0xffff0000u));
 }
 
 // Sixteen bf16 (lo, hi), times inv, as first parts q1 and second parts q2.
@@ -107,7 +115,7 @@ __device__ __forceinline__ void split_h_resident(const __nv_bfloat16* __restrict
   const int r = t / kSplitLanes, l = t - r * kSplitLanes;
   const int valid_chunks = d >> 4;                          // d is a multiple of 16
   uint4 va[kSplitChunks], vb[kSplitChunks];
-  float amax = 0.f;
+  uint32_t amax = 0u;
 #pragma unroll
   for (int i = 0; i < kSplitChunks; ++i) {
     const int c = l + kSplitLanes * i;
@@ -120,12 +128,12 @@ __device__ __forceinline__ void split_h_resident(const __nv_bfloat16* __restrict
     }
   }
 #pragma unroll
-  for (int i = 0; i < kSplitChunks; ++i) amax = fmaxf(amax, fmaxf(abs_max8(va[i]), abs_max8(vb[i])));
+  for (int i = 0; i < kSplitChunks; ++i) amax = abs_max8(abs_max8(amax, va[i]), vb[i]);
   // the row's largest magnitude: non-negative floats order like their bit patterns
   unsigned int* amax_bits = reinterpret_cast<unsigned int*>(hs_s + 32);
   if (t < 16) amax_bits[t] = 0u;
   asm volatile("bar.sync 1, %0;" ::"n"(kSplitThreads) : "memory");   // only the splitting warps; nothing asynchronous is waited for
-  atomicMax(amax_bits + r, __float_as_uint(amax));               // (fmaxf drops NaNs, so amax is a number >= 0)
+  atomicMax(amax_bits + r, __float_as_uint(larger_of(amax)));    // (NaNs are dropped: a number >= 0)
   asm volatile("bar.sync 1, %0;" ::"n"(kSplitThreads) : "memory");
   const float sc = split_scale(__uint_as_float(amax_bits[r]));
   if (l == 0) hs_s[r] = sc;
