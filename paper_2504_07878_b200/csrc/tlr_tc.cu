@@ -126,9 +126,13 @@ cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const Tc
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = c.cta == 1 ? 1 : 2;
+  // Pairs: short steps gain from a merge kernel that is resident before they end, others from registers (see the kernel).  At
+  // n = 256 with 104 registers and without the limit: V = 32000, d = 512 14.25 and 14.55 us, V = 40000, d = 1024 24.1 and 24.9;
+  // V = 64000, d = 512 22.9 and 22.6, d = 896 35.7 and 35.3.
+  const bool beside = p.n <= 256 && p.tiles_per_unit <= 3;
   const auto kernel = c.mode == RowMode::kM128Keep ? tc_projection_kernel<2, RowMode::kM128Keep, false>
-                      : c.cta == 2 && p.n > 256    ? tc_projection_kernel<2, RowMode::kM128, false>
-                      : c.cta == 2                 ? tc_projection_kernel<2, RowMode::kM128, true>
+                      : c.cta == 2 && beside       ? tc_projection_kernel<2, RowMode::kM128, true>
+                      : c.cta == 2                 ? tc_projection_kernel<2, RowMode::kM128, false>
                       : c.mode == RowMode::kGroup8 ? tc_projection_kernel<1, RowMode::kGroup8, true>
                       : c.mode == RowMode::kM64    ? tc_projection_kernel<1, RowMode::kM64, true>
                                                    : tc_projection_kernel<1, RowMode::kM128, true>;

@@ -852,7 +852,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
 // Every way of handling token rows is a kernel of its own: switches at run time cost the others (one for kGroup8 1.5 %:
 // n = 24, d = 512, V = 32000 11.60 and 11.82 us).
 // kBeside: so few registers that a block of 17 warps of the merge kernel (40 registers) stands beside a CTA and is resident,
-// waiting, before this kernel ends -- batches of up to 256 rows.  Larger ones are bound by the epilogue's and the MMAs' rate, and
+// waiting, before this kernel ends -- one CTA per worker, and pairs with short units.  Others are bound by the epilogue's and the MMAs' rate, and
 // that costs them (113 and 100 registers: n = 264, d = 696, V = 128256 75.8 and 80.4 us, n = 7969, d = 680, V = 25141 248 and 266).
 template <int kCta, RowMode kMode, bool kBeside>
 __global__ void __maxnreg__(kBeside ? 104 : 184)
