@@ -43,8 +43,18 @@ class TlrError(RuntimeError):
 _lib = None
 
 
+_native = None
+
+
 def _native_route():
     """tlr_torch.cpp's route, or a function that declines every call."""
+    global _native
+    if _native is None:
+        _native = _load_native_route()
+    return _native
+
+
+def _load_native_route():
     try:
         from . import _tlr_torch
     except ImportError:

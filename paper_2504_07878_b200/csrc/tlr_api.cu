@@ -419,10 +419,10 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
     c->ticket = reinterpret_cast<unsigned int*>(at);
     c->status = reinterpret_cast<uint32_t*>(at + 128);
     at += 256;
-    c->partials = reinterpret_cast<Partial*>(at);
-    at += partial_bytes;
     c->tagged = reinterpret_cast<Partial*>(at);
     at += tagged_bytes;
+    c->partials = reinterpret_cast<Partial*>(at);
+    at += partial_bytes;
     for (int q = 0; q < 2; ++q) {
       c->h_stage[q] = at;
       c->out_stage[q] = at + h_bytes;
@@ -446,8 +446,7 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
       c->out_mapped[q] = nullptr;   // tlr_route_host then stages the outputs in device memory and copies them
     }
   }
-  if (cudaMemset(c->workspace, 0, 256) != cudaSuccess ||      // the ticket and the status word
-      cudaMemset(c->tagged, 0xff, tagged_bytes) != cudaSuccess) {      // every slot pending
+  if (cudaMemset(c->workspace, 0, 256 + tagged_bytes) != cudaSuccess) {      // the ticket, the status word, every slot pending
     free_all(c);
     return TLR_ERR_CUDA;
   }

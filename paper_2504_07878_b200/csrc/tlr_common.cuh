@@ -52,7 +52,7 @@ __device__ __forceinline__ Partial empty_partial() {
 // V = 33000 12.31 and 11.57, one of eight shards at n = 256 18.07 and 17.34; n = 256, d = 512, V = 32000 14.5 either way.
 constexpr int kTagShift = 24;
 constexpr int kTagIdxMask = (1 << kTagShift) - 1;      // an index; all ones stand for kNoToken
-constexpr int kPendingIdx = -1;
+constexpr int kPendingIdx = 0;                         // (tag 0; a new workspace is all zeros)
 constexpr int kMaxTag = 254;
 constexpr int kTaggedPartials = 8 * 16 * 32 * 5;        // of a step: what finish_rows_kernel's lanes can own (328 KB)
 constexpr int kMaxLooks = 1 << 14;                     // about 10 ms
