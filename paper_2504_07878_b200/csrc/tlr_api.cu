@@ -388,6 +388,12 @@ void free_all(tlr_ctx* c) {
   delete c;
 }
 
+// Zeroes device memory and waits for that, on the context's own stream: a clear on the default stream is not ordered before
+// steps on streams that do not wait for the default stream, and would land whenever that stream gets to it.
+bool clear_now(const tlr_ctx* c, void* p, size_t bytes) {
+  return cudaMemsetAsync(p, 0, bytes, c->copy_stream) == cudaSuccess && cudaStreamSynchronize(c->copy_stream) == cudaSuccess;
+}
+
 // What both kinds of context share: the device check, the workspace, the staging buffers of
 // tlr_route_host and the driver's tensor-map encoder (c->encode stays null if it cannot be had).
 tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out) {
@@ -446,7 +452,7 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
       c->out_mapped[q] = nullptr;   // tlr_route_host then stages the outputs in device memory and copies them
     }
   }
-  if (cudaMemset(c->workspace, 0, 256 + tagged_bytes) != cudaSuccess) {      // the ticket, the status word, every slot pending
+  if (!clear_now(c, c->workspace, 256 + tagged_bytes)) {      // the ticket, the status word, every slot pending
     free_all(c);
     return TLR_ERR_CUDA;
   }
@@ -1175,7 +1181,7 @@ tlr_status tlr_last_device_status(tlr_ctx* ctx, uint32_t* out_host) {
   if (ctx == nullptr || out_host == nullptr) return TLR_ERR_ARG;
   if (cudaDeviceSynchronize() != cudaSuccess) return TLR_ERR_CUDA;
   if (cudaMemcpy(out_host, ctx->status, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return TLR_ERR_CUDA;
-  if (cudaMemset(ctx->status, 0, 4) != cudaSuccess) return TLR_ERR_CUDA;
+  if (!clear_now(ctx, ctx->status, 4)) return TLR_ERR_CUDA;
   return TLR_OK;
 }
 
