@@ -59,6 +59,8 @@ def _load_native_route():
         from . import _tlr_torch
     except ImportError:
         return lambda *args: None
+    if _tlr_torch.built_for != torch.__version__:
+        return lambda *args: None
     _tlr_torch.bind(ctypes.cast(load_library().tlr_route, c_void_p).value)
     return _tlr_torch.route
 

@@ -11,8 +11,7 @@
 
 namespace {
 
-using RouteFn = tlr_status (*)(tlr_ctx*, const void*, int32_t, float, int32_t*, float*, float*, uint8_t*, int32_t*, int32_t*,
-                               void*);
+using RouteFn = decltype(&tlr_route);
 RouteFn g_route = nullptr;
 
 PyObject* bind(PyObject*, PyObject* address) {
@@ -98,4 +97,8 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_tlr_torch", nullptr, -1, methods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__tlr_torch() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__tlr_torch() {
+  PyObject* m = PyModule_Create(&module);
+  if (m != nullptr && PyModule_AddStringConstant(m, "built_for", TLR_TORCH_VERSION) != 0) Py_CLEAR(m);
+  return m;
+}
