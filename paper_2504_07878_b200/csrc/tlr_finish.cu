@@ -142,28 +142,42 @@ __device__ __forceinline__ int flag_of(const uint32_t* words, int i, int log2_L)
   return (words[i >> log2_rpw] >> ((i & ((1 << log2_rpw) - 1)) << log2_L)) & 1;
 }
 
-// Block 0 of the cluster waits until every warp's word has arrived (bounded like every wait; after a time-out the status
-// word says that the index list is not to be trusted).
-__device__ __forceinline__ void wait_for_words(uint32_t bar, uint32_t* status) {
+__device__ __forceinline__ bool words_here(uint32_t bar) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\t"
+               "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+               "selp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(bar) : "memory");
+  return ok != 0u;
+}
+// Block 0 of the cluster waits until every warp's word has arrived; false if it gave up.  Bounded like every wait, and what the
+// limit covers is the cluster's own blocks: nothing the projection waits for -- a kernel in front of it may wait for seconds
+// for other GPUs -- counts.  So where the others look for their partials themselves (kTagged) this one looks for a while and
+// then waits for the projection's grid before its clock starts.
+template <bool kTagged>
+__device__ __forceinline__ bool wait_for_words(uint32_t bar, uint32_t* status) {
   unsigned long long t0 = 0;
   for (uint32_t it = 0;; ++it) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar) : "memory");
-    if (ok) return;
-    if ((it & 63u) == 63u) {
+    if (words_here(bar)) return true;
+    if ((it & 63u) == 63u && (!kTagged || it >= kMaxLooks)) {
+      if (kTagged && t0 == 0) pdl_wait();
       unsigned long long t;
       asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
       if (t0 == 0) t0 = t;
       if (t - t0 > 2000000000ull) {
         atomicOr(status, TLR_DEV_WAIT_TIMEOUT);
-        return;
+        return false;
       }
     }
   }
 }
+// After a time-out no row is listed, and block 0 stays until no other block can send to it any more (threads that have exited
+// count as arrived).  By whole warps.
+__device__ __forceinline__ void outlive_senders() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+constexpr int kNoList = -2 * kSmallRows;      // a warp's count after a time-out: the sum is below zero with it
 
 // Cluster of gridDim.x blocks, n <= 1024.  A group of L lanes (L a power of two) folds one
 // row in two passes over its partials: maximum and index first, then the sums rescaled to
@@ -295,8 +309,9 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
   }
   if (valid && gl == 0) store_row(out, out_token, out_s, out_t, a, row);
   if (blockIdx.x != 0) return;
+  bool here = true;
   if (single_block) __syncthreads();
-  else wait_for_words(bar, a.status);
+  else here = __all_sync(0xffffffffu, wait_for_words<false>(bar, a.status));
   first_routed_init(a);
   const int log2_rpw = 5 - log2_L;          // rows per warp
   int base_out = 0;
@@ -304,12 +319,12 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
     const int i = base + threadIdx.x;
     const int flag = i < a.n ? (flag_words[i >> log2_rpw] >> ((i & ((1 << log2_rpw) - 1)) << log2_L)) & 1u : 0;
     const unsigned int bal = __ballot_sync(0xffffffffu, flag != 0);
-    if (lane == 0) warp_count[warp] = __popc(bal);
+    if (lane == 0) warp_count[warp] = here ? __popc(bal) : kNoList;
     __syncthreads();
     // at most 32 warps: lane w holds warp w's count
     const int c = lane < warps ? warp_count[lane] : 0;
     const int before = __reduce_add_sync(0xffffffffu, lane < warp ? c : 0);
-    if (flag) {
+    if (flag && base_out + before >= 0) {
       a.routed_idx[base_out + before + __popc(bal & ((1u << lane) - 1u))] = i;
       first_routed_note(a, i);
     }
@@ -317,9 +332,10 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
     if (base + static_cast<int>(blockDim.x) < a.n) __syncthreads();
   }
   if (threadIdx.x == 0) {
-    *a.routed_count = base_out;
+    *a.routed_count = max(base_out, 0);
     if (a.status_copy != nullptr) *a.status_copy = atomicOr(a.status, 0u);   // every row has been scored by now
   }
+  if (base_out < 0) outlive_senders();
 }
 
 // The same for steps whose lanes own few partials (rows_shape), and then what stands between the last partial and the end of
@@ -374,10 +390,18 @@ finish_rows_kernel(const FinishLaunch a, const int log2_L) {
     if (mine) store_row(out, idx, s, t, a, row);
     if (kTagged && valid) reset_tagged(p, gl, L, a.chunks);
   } else if (blockIdx.x == 0) {
-    wait_for_words(bar, a.status);
+    const bool here = __all_sync(0xffffffffu, wait_for_words<kTagged>(bar, a.status));
     if (a.seq_len > 0) {
       for (int b = lane; b < a.n / a.seq_len; b += 32) a.first_routed[b] = a.seq_len;
       __syncwarp();
+    }
+    if (__builtin_expect(!here, 0)) {
+      if (lane == 0) {
+        *a.routed_count = 0;
+        if (a.status_copy != nullptr) *a.status_copy = atomicOr(a.status, 0u);
+      }
+      outlive_senders();
+      return;
     }
     // (A scan over the words, every lane writing the rows of its own, took a microsecond at n = 1 and more than this loop's
     // eight turns at n = 256.)

@@ -101,3 +101,40 @@ def test_a_tensor_map_that_cannot_be_encoded_is_an_error(pkg, n, d, fp8):
     torch.cuda.synchronize()
     assert np.array_equal(to_np(r.token[:n]), good)
     r.close()
+
+
+# The kernel in front of a step may be at work for longer than any limit -- here the merge of a sharded step, which looks for a
+# rank that never joins for 2.5 s -- and lets the step's kernels in early.  Their limits do not cover it.
+@pytest.mark.parametrize("n,d,fp8", [(5, 64, False), (40, 64, True), (200, 64, False)])
+def test_limits_do_not_cover_what_a_step_waits_for(pkg, n, d, fp8):
+    V = 20000
+    W, scale = S.make_W8(d, V, seed=2, std=0.2) if fp8 else (S.make_W(d, V, seed=2, std=0.2), None)
+    r = pkg.Router(W.cuda(), max_n=n, wscale=None if scale is None else scale.cuda())
+    h = S.make_h(n, d, seed=3).h.cuda()
+    first = torch.zeros(n, dtype=torch.int32, device="cuda")
+    out = (r.token, r.conf, r.entropy, r.route_mask, first, r.routed_idx, r.routed_count)
+    r.route(h, 0.01)
+    torch.cuda.synchronize()
+    tau = float(r.conf.median())                     # about half of the rows are routed
+    r.route(h, tau, seq_len=1, first_routed=first)
+    torch.cuda.synchronize()
+    want = [to_np(t).copy() for t in out]
+    count = int(want[-1][0])
+    assert 0 < count < n
+
+    slow_d, slow_V = 64, 3000
+    block = torch.zeros(pkg.tlr_shard_block_bytes(8, 2), dtype=torch.uint8, device="cuda")
+    slow = pkg.FusedVocabShardedRouter(S.make_W(slow_d, slow_V, seed=5).cuda(), 0, 8, 0, 2, [block] * 2, keep=block)
+    pkg.tlr_debug_inject(slow.ctx, 0, 2500)
+    slow.push(S.make_h(8, slow_d, seed=6).h.cuda())
+    torch.cuda.synchronize()
+    slow.finish(8, 0.5)
+    r.route(h, tau, seq_len=1, first_routed=first)
+    torch.cuda.synchronize()
+    assert pkg.tlr_last_device_status(slow.ctx) & pkg.TLR_DEV_WAIT_TIMEOUT
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    got = [to_np(t) for t in out]
+    for a, b in zip(got[:5] + [got[5][:count], got[6]], want[:5] + [want[5][:count], want[6]]):
+        assert np.array_equal(a, b)
+    slow.close()
+    r.close()
