@@ -341,7 +341,9 @@ tlr_status tlr_set_path(tlr_ctx* ctx, tlr_path path);
  * usable.  kind = 1 makes the next calls' W producer issue no copies, so the consumer's wait
  * runs out (nothing faults, traps or spins forever); wait_limit_ms shortens the limit of every
  * wait (0 = default, 2 s).  kind = 2 makes the encoding of tensor maps fail: calls that need a new one
- * return TLR_ERR_CUDA before the projection.  kind = 0 restores normal operation.  Tensor-core path only.
+ * return TLR_ERR_CUDA before the projection.  kind = 3 makes the kernel behind the projection look for partials that
+ * never come, where it looks for them while that one runs (decode batches): it gives up, raises TLR_DEV_WAIT_TIMEOUT
+ * and returns.  kind = 0 restores normal operation.  Tensor-core path only.
  */
 tlr_status tlr_debug_inject(tlr_ctx* ctx, int32_t kind, uint32_t wait_limit_ms);
 

@@ -482,6 +482,9 @@ uint32_t next_tag(tlr_ctx* c, const tlr_ctx::Step* st, int n) {
   return c->last_tag;
 }
 
+// The tag that the reader looks for (the test hook: one that nothing has).
+uint32_t reader_tag(const tlr_ctx* c, uint32_t tag) { return c->debug_kind == 3 && tag != 0 ? tlr::kMaxTag + 1 : tag; }
+
 // Enqueues the projection kernel of a call with n > 0 rows: chunk partials into ctx->partials, or with a tag into
 // ctx->tagged.  router_beside: the 8-bit head's router kernel follows (launch_mlp_beside).
 tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ctx::Step* st, cudaStream_t stream,
@@ -743,7 +746,7 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
 }
 
 tlr_status tlr_debug_inject(tlr_ctx* ctx, int32_t kind, uint32_t wait_limit_ms) {
-  if (ctx == nullptr || kind < 0 || kind > 2) return TLR_ERR_ARG;
+  if (ctx == nullptr || kind < 0 || kind > 3) return TLR_ERR_ARG;
   ctx->debug_kind = kind;
   ctx->debug_wait_ns = static_cast<unsigned long long>(wait_limit_ms) * 1000000ull;
   forget_steps(ctx);
@@ -835,7 +838,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
 
   tlr::FinishLaunch f = {};
   f.partials = tag != 0 ? ctx->tagged : ctx->partials;
-  f.tag = tag;
+  f.tag = reader_tag(ctx, tag);
   f.small_blocks = small_blocks;
   f.n = n;
   f.chunks = plan.vocab_chunks;
@@ -886,8 +889,8 @@ tlr_status tlr_shard_summary(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, in
   const uint32_t tag = ctx->classes > 1 ? 0 : next_tag(ctx, st, n);    // (settling ties waits for the grid there)
   const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, tag);
   if (ps != TLR_OK) return ps;
-  if (tlr::launch_shard_summary(st->params.partials, tag, n, plan.vocab_chunks, v_offset, ties_of(ctx, h_bf16_dev),
-                                static_cast<Partial*>(summary_dev), stream) != cudaSuccess) {
+  if (tlr::launch_shard_summary(st->params.partials, reader_tag(ctx, tag), ctx->status, n, plan.vocab_chunks, v_offset,
+                                ties_of(ctx, h_bf16_dev), static_cast<Partial*>(summary_dev), stream) != cudaSuccess) {
     if (tag != 0) ctx->tagged_ok = false;
     return TLR_ERR_CUDA;
   }
@@ -1011,7 +1014,8 @@ tlr_status tlr_shard_push(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, int32
   const int q = static_cast<int>(ctx->shard_epoch & 1u);
   tlr::ShardPush a;
   a.partials = tag != 0 ? ctx->tagged : ctx->partials;
-  a.tag = tag;
+  a.tag = reader_tag(ctx, tag);
+  a.status = ctx->status;
   a.n = n;
   a.chunks = chunks;
   a.v_offset = v_offset;

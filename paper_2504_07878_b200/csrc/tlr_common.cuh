@@ -126,6 +126,12 @@ __device__ __forceinline__ Partial warp_merge(Partial p) {
 constexpr int kPerLane = 6;            // ceil(192 / 32): the most partials a lane can own
 constexpr int kRowsPerLane = 5;        // ... in the kernels bound by latency (148 / 32): registers
 
+// A row without all of its partials is nobody's answer, whatever the projection itself has raised.
+__device__ __forceinline__ void note_missing(uint32_t* status) {
+  atomicOr(status, TLR_DEV_WAIT_TIMEOUT);
+  __threadfence();                         // before this row's flag reaches the block that copies the status word
+}
+
 // A lane's share of a row's partials -- first, first + stride, ... below `count`: maxima and sums, and the largest maximum
 // with its lowest index.
 template <int kN>
@@ -165,10 +171,12 @@ struct LaneFold {
       put(k, v, v.idx);
     }
   }
-  // Tagged partials, chunk stride 1; called by whole warps.  hint: look at nothing but the row's last one until it is there.
+  // Tagged partials, chunk stride 1; called by whole warps.  One that is not there when the projection's grid
+  // has ended counts as empty, and the status word is told.  hint: look at nothing but the row's last one until it is there.
   // A look is one trip to L2: all of a lane's loads go out before the first is examined (one after the other they took
   // 1.8 us a look).
-  __device__ __forceinline__ void take(const Partial* p, int first, int stride, int count, uint32_t tag, bool hint) {
+  __device__ __forceinline__ void take(const Partial* p, int first, int stride, int count, uint32_t tag, bool hint,
+                                       uint32_t* status) {
     const auto here = [&](int i) { return (static_cast<uint32_t>(i) >> kTagShift) == tag; };
     Partial v[kN];
     int looks = 0;
@@ -183,7 +191,11 @@ struct LaneFold {
 #pragma unroll
       for (int k = 0; k < kN; ++k)
         if (first + stride * k < count) all = all && here(v[k].idx);
-      if (__all_sync(0xffffffffu, all) || waited) break;
+      if (__all_sync(0xffffffffu, all)) break;
+      if (waited) {
+        if (!all) note_missing(status);
+        break;
+      }
       if (++looks >= kMaxLooks) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         waited = true;
@@ -193,7 +205,6 @@ struct LaneFold {
     idx = kNoToken;
 #pragma unroll
     for (int k = 0; k < kN; ++k) {
-      // (one that was never written -- the projection gave up -- counts as empty)
       const bool there = first + stride * k < count && here(v[k].idx);
       put(k, there ? v[k] : empty_partial(), there ? untagged_idx(v[k].idx) : kNoToken);
     }
@@ -246,14 +257,14 @@ __device__ __forceinline__ float group_max(float v, int L) {
   return v;
 }
 
-// Folds one row's partials (tagged ones if tag is not 0; chunk_stride is 1 then).  Every lane returns the same result.
-// `second` (optional, untagged only): the largest of the partials' maxima below the row's.
+// Folds one row's partials (tagged ones if tag is not 0; chunk_stride is 1 and `status` the context's word then).  Every lane
+// returns the same result.  `second` (optional, untagged only): the largest of the partials' maxima below the row's.
 __device__ __forceinline__ Partial fold_row(const Partial* p, int chunks, int chunk_stride, int lane,
-                                            float* second = nullptr, uint32_t tag = 0) {
+                                            float* second = nullptr, uint32_t tag = 0, uint32_t* status = nullptr) {
   Partial r;
   if (tag != 0) {
     LaneFold<kRowsPerLane> f;
-    f.take(p, lane, 32, chunks, tag, true);
+    f.take(p, lane, 32, chunks, tag, true, status);
     r.m = f.best;
     r.idx = f.idx;
     group_best(r.m, r.idx, 32);
@@ -352,7 +363,10 @@ static __device__ __forceinline__ Winner settle_ties(const Ties ties, int row, c
     int mine = kNoToken;
     if (j < chunks) {
       const Partial* q = p + static_cast<size_t>(j) * chunk_stride;
-      if (__ldcg(&q->m) >= least) mine = kTagged ? untagged_idx(__ldcg(&q->idx)) : __ldcg(&q->idx);
+      if (__ldcg(&q->m) >= least) {
+        mine = __ldcg(&q->idx);
+        if (kTagged) mine = mine != kPendingIdx ? untagged_idx(mine) : kNoToken;
+      }
     }
     unsigned int todo = __ballot_sync(group, mine < ties.V && mine != idx) & group;
     while (todo != 0u) {
@@ -457,14 +471,15 @@ bool merges_tagged(int n, int chunks, bool small_blocks);    // whether launch_f
 
 // Vocabulary-sharded decode (tlr_shard.cu): one summary per row from a shard's chunk partials,
 // and the gathered summaries [shards][n] laid out as partials [n][shards].
-// (tag not 0: tagged partials)
-cudaError_t launch_shard_summary(Partial* partials, uint32_t tag, int n, int chunks, int v_offset, const Ties& ties,
-                                 Partial* summary, cudaStream_t stream);
+// (tag not 0: tagged partials, and `status` is told if some never come)
+cudaError_t launch_shard_summary(Partial* partials, uint32_t tag, uint32_t* status, int n, int chunks, int v_offset,
+                                 const Ties& ties, Partial* summary, cudaStream_t stream);
 // Fused exchange: the summaries are stored straight into slot `rank` of every peer's exchange block and, once all
 // rows are out, this rank's flag in every peer's flag array is set to `epoch` (peer stores only).
 struct ShardPush {
   Partial* partials;         // this shard's chunk partials [n][chunks]
-  uint32_t tag;              // not 0: tagged ones
+  uint32_t tag;              // not 0: tagged ones, and
+  uint32_t* status;          // ... is told if some never come
   int n, chunks, v_offset;
   Ties ties;
   int shards;                // peers, this rank included

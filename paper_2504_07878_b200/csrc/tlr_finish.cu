@@ -371,7 +371,7 @@ finish_rows_kernel(const FinishLaunch a, const int log2_L) {
     const int count = valid ? a.chunks : 0;
     Partial* p = a.partials + static_cast<size_t>(valid ? row : 0) * a.row_stride;
     LaneFold<kRowsPerLane> f;
-    if constexpr (kTagged) f.take(p, gl, L, count, a.tag, gridDim.x > 1);
+    if constexpr (kTagged) f.take(p, gl, L, count, a.tag, gridDim.x > 1, a.status);
     else f.load(p, gl, L, count, static_cast<size_t>(a.chunk_stride));
     float m = f.best, s, t;
     int idx = f.idx;

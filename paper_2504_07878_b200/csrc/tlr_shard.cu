@@ -29,11 +29,11 @@ constexpr int kWarps = 8;
 // equal rows of W in different shards tie exactly in the merge behind -- also where one shard ran on CUDA cores and another
 // on tensor cores.
 template <bool kTies>
-__device__ __forceinline__ Partial row_summary(Partial* partials, uint32_t tag, int row, int chunks, int v_offset,
+__device__ __forceinline__ Partial row_summary(Partial* partials, uint32_t tag, uint32_t* status, int row, int chunks, int v_offset,
                                                const Ties& ties, int lane) {
   Partial* p = partials + static_cast<size_t>(row) * chunks;
   float second;
-  Partial acc = fold_row(p, chunks, 1, lane, kTies ? &second : nullptr, kTies ? 0u : tag);
+  Partial acc = fold_row(p, chunks, 1, lane, kTies ? &second : nullptr, kTies ? 0u : tag, status);
   if (!kTies && tag != 0) reset_tagged(p, lane, 32, chunks);
   if (kTies) settle_row(ties, row, p, chunks, 1, second, acc.m, acc.idx, acc.s, acc.t, lane, 32);
   if (acc.idx != kNoToken) acc.idx += v_offset;
@@ -42,7 +42,8 @@ __device__ __forceinline__ Partial row_summary(Partial* partials, uint32_t tag, 
 
 template <bool kTies>
 __global__ void __launch_bounds__(kWarps * 32)
-shard_summary_kernel(Partial* partials, uint32_t tag, int n, int chunks, int v_offset, const Ties ties, Partial* summary) {
+shard_summary_kernel(Partial* partials, uint32_t tag, uint32_t* status, int n, int chunks, int v_offset, const Ties ties,
+                     Partial* summary) {
   const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   // A programmatic dependent launch like the kernels around it: its blocks (512 small ones at most fit beside the
@@ -50,7 +51,7 @@ shard_summary_kernel(Partial* partials, uint32_t tag, int n, int chunks, int v_o
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tag == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row >= n) return;
-  const Partial acc = row_summary<kTies>(partials, tag, row, chunks, v_offset, ties, lane);
+  const Partial acc = row_summary<kTies>(partials, tag, status, row, chunks, v_offset, ties, lane);
   if (lane == 0) summary[row] = acc;
   if (tag != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -65,7 +66,7 @@ shard_push_kernel(const ShardPush a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (a.tag == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row < a.n) {
-    const Partial acc = row_summary<kTies>(a.partials, a.tag, row, a.chunks, a.v_offset, a.ties, lane);
+    const Partial acc = row_summary<kTies>(a.partials, a.tag, a.status, row, a.chunks, a.v_offset, a.ties, lane);
     for (int g = lane; g < a.shards; g += 32) a.peer_slot[g][row] = acc;     // lane g stores to peer g
   }
   if (a.tag != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -108,8 +109,8 @@ rows_merge_kernel(const int32_t* __restrict__ gathered_idx, const int32_t* __res
 
 }  // namespace
 
-cudaError_t launch_shard_summary(Partial* partials, uint32_t tag, int n, int chunks, int v_offset, const Ties& ties,
-                                 Partial* summary, cudaStream_t stream) {
+cudaError_t launch_shard_summary(Partial* partials, uint32_t tag, uint32_t* status, int n, int chunks, int v_offset,
+                                 const Ties& ties, Partial* summary, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>((n + kWarps - 1) / kWarps), 1, 1);
@@ -121,7 +122,7 @@ cudaError_t launch_shard_summary(Partial* partials, uint32_t tag, int n, int chu
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const auto kernel = ties.W != nullptr ? shard_summary_kernel<true> : shard_summary_kernel<false>;
-  return cudaLaunchKernelEx(&cfg, kernel, partials, tag, n, chunks, v_offset, ties, summary);
+  return cudaLaunchKernelEx(&cfg, kernel, partials, tag, status, n, chunks, v_offset, ties, summary);
 }
 
 cudaError_t launch_shard_push(const ShardPush& a, cudaStream_t stream) {

@@ -138,3 +138,49 @@ def test_limits_do_not_cover_what_a_step_waits_for(pkg, n, d, fp8):
         assert np.array_equal(a, b)
     slow.close()
     r.close()
+
+
+# Where the kernel behind the projection looks for the partials itself, it is the one that knows of one that never came.
+@pytest.mark.parametrize("kind", ["bf16", "8bit", "odd", "summary", "push"])
+def test_partials_that_never_come_raise_the_flag(pkg, kind):
+    n, d, V = 16, 100 if kind == "odd" else 64, 20000
+    W, scale = S.make_W8(d, V, seed=2, std=0.2) if kind == "8bit" else (S.make_W(d, V, seed=2, std=0.2), None)
+    W, scale = W.cuda(), None if scale is None else scale.cuda()
+    hid = S.make_h(n, d, seed=3)
+    h = hid.h.cuda()
+    if kind == "push":
+        block = torch.zeros(pkg.tlr_shard_block_bytes(n, 1), dtype=torch.uint8, device="cuda")
+        r = pkg.FusedVocabShardedRouter(W, 0, n, 0, 1, [block], keep=block)
+    elif kind == "summary":
+        r = pkg.VocabShardedRouter(W, 0, max_n=n, world=1)
+    else:
+        r = pkg.Router(W, max_n=n, wscale=scale)
+
+    def run():
+        if kind == "push":
+            r.push(h)
+            r.finish(n, 0.01)
+        elif kind == "summary":
+            r.finish(r.summarize(h)[None].contiguous(), n, 0.01)
+        else:
+            r.route(h, 0.01)
+        torch.cuda.synchronize()
+        return [to_np(t[:n]).copy() for t in (r.token, r.conf, r.entropy, r.route_mask)]
+
+    good = run()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    pkg.tlr_debug_inject(r.ctx, 3)
+    run()
+    assert pkg.tlr_last_device_status(r.ctx) & pkg.TLR_DEV_WAIT_TIMEOUT
+    if kind in ("bf16", "8bit", "odd"):
+        cnt = torch.zeros(1, dtype=torch.int32).pin_memory()
+        with pytest.raises(pkg.TlrError) as e:
+            pkg.tlr_route_host(r.ctx, hid.h.pin_memory(), n, 0.01, None, None, None, None, None, cnt)
+        assert e.value.code == 7
+        pkg.tlr_last_device_status(r.ctx)
+    pkg.tlr_debug_inject(r.ctx, 0)
+    again = run()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    for a, b in zip(good, again):
+        assert np.array_equal(a, b)
+    r.close()
