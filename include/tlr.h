@@ -343,7 +343,8 @@ tlr_status tlr_set_path(tlr_ctx* ctx, tlr_path path);
  * wait (0 = default, 2 s).  kind = 2 makes the encoding of tensor maps fail: calls that need a new one
  * return TLR_ERR_CUDA before the projection.  kind = 3 makes the kernel behind the projection look for partials that
  * never come, where it looks for them while that one runs (decode batches): it gives up, raises TLR_DEV_WAIT_TIMEOUT
- * and returns.  kind = 0 restores normal operation.  Tensor-core path only.
+ * and returns.  kind = 4 makes timed calls (tlr_set_kernel_timing) return TLR_ERR_CUDA right behind the projection.
+ * kind = 0 restores normal operation.  Tensor-core path only.
  */
 tlr_status tlr_debug_inject(tlr_ctx* ctx, int32_t kind, uint32_t wait_limit_ms);
 

@@ -297,7 +297,8 @@ def tlr_last_device_status(ctx) -> int:
 
 def tlr_debug_inject(ctx, kind: int, wait_limit_ms: int = 0):
     """Test hook: kind=1 drops the W copies of the next calls so a bounded wait runs out; kind=2 makes the
-    encoding of tensor maps fail; kind=3 keeps the partials from the kernel that merges them; kind=0 restores."""
+    encoding of tensor maps fail; kind=3 keeps the partials from the kernel that merges them; kind=4 lets
+    timed calls fail behind the projection; kind=0 restores."""
     _check(load_library().tlr_debug_inject(ctx, kind, wait_limit_ms), "tlr_debug_inject")
 
 

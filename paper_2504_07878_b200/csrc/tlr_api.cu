@@ -149,7 +149,8 @@ struct tlr_ctx {
                                           // buffers (ten allocations took most of the time of tlr_create)
   Partial* partials = nullptr;
   Partial* tagged = nullptr;              // partials of tagged steps (tlr_common.cuh)
-  bool tagged_ok = true;                  // false once a reader's launch has failed: its slots were not left pending
+  size_t tagged_bytes = 0;
+  bool tagged_ok = true;                  // false once slots may have been left otherwise than pending (untag)
   uint32_t last_tag = 0;
   unsigned int* ticket = nullptr;
   uint32_t* status = nullptr;
@@ -426,6 +427,7 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
     c->status = reinterpret_cast<uint32_t*>(at + 128);
     at += 256;
     c->tagged = reinterpret_cast<Partial*>(at);
+    c->tagged_bytes = tagged_bytes;
     at += tagged_bytes;
     c->partials = reinterpret_cast<Partial*>(at);
     at += partial_bytes;
@@ -480,6 +482,13 @@ uint32_t next_tag(tlr_ctx* c, const tlr_ctx::Step* st, int n) {
     return 0;
   c->last_tag = c->last_tag % tlr::kMaxTag + 1;
   return c->last_tag;
+}
+
+// After an error in a call with a tag, wherever it was: its projection may have been launched, and no reader leaves the slots
+// pending behind it.  So they are cleared there; if that cannot be had either, the context goes on without tags.
+tlr_status untag(tlr_ctx* c, uint32_t tag, cudaStream_t stream, tlr_status error) {
+  if (tag != 0 && cudaMemsetAsync(c->tagged, 0, c->tagged_bytes, stream) != cudaSuccess) c->tagged_ok = false;
+  return error;
 }
 
 // The tag that the reader looks for (the test hook: one that nothing has).
@@ -564,7 +573,7 @@ tlr_status launch_projection(tlr_ctx* ctx, const void* h_bf16_dev, int n, tlr_ct
   }
   if (e != cudaSuccess) return TLR_ERR_CUDA;
   if (ev1 != nullptr) {
-    if (cudaEventRecord(ev1, stream) != cudaSuccess) return TLR_ERR_CUDA;
+    if (ctx->debug_kind == 4 || cudaEventRecord(ev1, stream) != cudaSuccess) return TLR_ERR_CUDA;
     ctx->timed += 1;
   }
   return TLR_OK;
@@ -746,7 +755,7 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
 }
 
 tlr_status tlr_debug_inject(tlr_ctx* ctx, int32_t kind, uint32_t wait_limit_ms) {
-  if (ctx == nullptr || kind < 0 || kind > 3) return TLR_ERR_ARG;
+  if (ctx == nullptr || kind < 0 || kind > 4) return TLR_ERR_ARG;
   ctx->debug_kind = kind;
   ctx->debug_wait_ns = static_cast<unsigned long long>(wait_limit_ms) * 1000000ull;
   forget_steps(ctx);
@@ -818,7 +827,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   const uint32_t tag = !want_mlp && tlr::merges_tagged(n, plan.vocab_chunks, small_blocks) ? next_tag(ctx, st, n) : 0;
   if (n > 0) {
     const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, tag, router_beside);
-    if (ps != TLR_OK) return ps;
+    if (ps != TLR_OK) return untag(ctx, tag, stream, ps);
   }
 
   if (want_mlp && !mlp_inside && n > 0) {
@@ -864,10 +873,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   f.status = ctx->status;
   if (plan.path == TLR_PATH_TC) f.ties = ties_of(ctx, h_bf16_dev);
   f.status_copy = status_copy;
-  if (tlr::launch_finish(f, stream) != cudaSuccess) {
-    if (tag != 0) ctx->tagged_ok = false;
-    return TLR_ERR_CUDA;
-  }
+  if (tlr::launch_finish(f, stream) != cudaSuccess) return untag(ctx, tag, stream, TLR_ERR_CUDA);
   return TLR_OK;
 }
 
@@ -888,12 +894,10 @@ tlr_status tlr_shard_summary(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, in
   const tlr_plan& plan = st->plan;
   const uint32_t tag = ctx->classes > 1 ? 0 : next_tag(ctx, st, n);    // (settling ties waits for the grid there)
   const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, tag);
-  if (ps != TLR_OK) return ps;
+  if (ps != TLR_OK) return untag(ctx, tag, stream, ps);
   if (tlr::launch_shard_summary(st->params.partials, reader_tag(ctx, tag), ctx->status, n, plan.vocab_chunks, v_offset,
-                                ties_of(ctx, h_bf16_dev), static_cast<Partial*>(summary_dev), stream) != cudaSuccess) {
-    if (tag != 0) ctx->tagged_ok = false;
-    return TLR_ERR_CUDA;
-  }
+                                ties_of(ctx, h_bf16_dev), static_cast<Partial*>(summary_dev), stream) != cudaSuccess)
+    return untag(ctx, tag, stream, TLR_ERR_CUDA);
   return TLR_OK;
 }
 
@@ -1007,7 +1011,7 @@ tlr_status tlr_shard_push(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, int32
     chunks = st->plan.vocab_chunks;
     tag = ctx->classes > 1 ? 0 : next_tag(ctx, st, n);
     const tlr_status ps = launch_projection(ctx, h_bf16_dev, n, st, stream, tag);
-    if (ps != TLR_OK) return ps;
+    if (ps != TLR_OK) return untag(ctx, tag, stream, ps);
   }
   ctx->shard_epoch += 1;
   if (ctx->shard_epoch == 0) ctx->shard_epoch = 2;    // (wrapped: keep the parity sequence, never publish 0)
@@ -1025,10 +1029,7 @@ tlr_status tlr_shard_push(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, int32
   a.peer_flag = ctx->peer_flag[q];
   a.epoch = ctx->shard_epoch;
   a.ticket = ctx->ticket;
-  if (tlr::launch_shard_push(a, stream) != cudaSuccess) {
-    if (tag != 0) ctx->tagged_ok = false;
-    return TLR_ERR_CUDA;
-  }
+  if (tlr::launch_shard_push(a, stream) != cudaSuccess) return untag(ctx, tag, stream, TLR_ERR_CUDA);
   return TLR_OK;
 }
 

@@ -97,3 +97,38 @@ def test_steps_back_to_back_keep_their_partials(pkg, kind, graph):
     if graph:
         del g
     r.close()
+
+
+# A call that fails between the projection and the merge leaves partials that nobody takes.  They are nobody's either when the
+# tag comes round (after 254 steps), here in a graph captured before the failure, with other hidden states.
+@pytest.mark.parametrize("kind", ["bf16", "8bit", "odd"])
+def test_partials_of_a_failed_call_are_not_taken_by_later_ones(pkg, kind):
+    (W, scale), _, d = _head(kind)
+    n = 48
+    r = pkg.Router(W, max_n=n, wscale=scale)
+    h, other, one = (S.make_h(k, d, seed=s).h.cuda() for k, s in ((n, 1), (n, 2), (1, 3)))
+    want = _expect(kind, r, h, n)                         # tag 1
+    side = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        r.route(h, 0.5)                                   # tag 2
+    for _ in range(253):
+        r.route(one, 0.5)                                 # tags 3 .. 254 and 1
+    pkg.tlr_set_kernel_timing(r.ctx, True)
+    pkg.tlr_debug_inject(r.ctx, 4)
+    with pytest.raises(pkg.TlrError) as e:
+        r.route(other, 0.5)                               # tag 2
+    assert e.value.code == 4
+    pkg.tlr_debug_inject(r.ctx, 0)
+    pkg.tlr_set_kernel_timing(r.ctx, False)
+    outs = (r.token, r.conf, r.entropy, r.route_mask)
+    for step in (g.replay, lambda: r.route(h, 0.5)):
+        for t in outs:
+            t.zero_()
+        step()
+        torch.cuda.synchronize()
+        assert pkg.tlr_last_device_status(r.ctx) == 0
+        for a, b in zip(outs, want):
+            assert np.array_equal(to_np(a[:n]), b)
+    del g
+    r.close()
