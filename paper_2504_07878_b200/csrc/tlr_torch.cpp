@@ -57,15 +57,16 @@ PyObject* route(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
       if (!THPVariable_CheckExact(PyTuple_GET_ITEM(kept, i))) Py_RETURN_NONE;
       view[i] = THPVariable_Unpack(PyTuple_GET_ITEM(kept, i)).variable_data();
     }
+    void* rows[4];
+    for (int i = 0; i < 4; ++i) rows[i] = view[i].mutable_data_ptr();
     const void* h_ptr = h.const_data_ptr();
     int32_t* idx = data_of<int32_t>(idx_obj);
     int32_t* count = data_of<int32_t>(count_obj);
     tlr_status status;
-    Py_BEGIN_ALLOW_THREADS      // (a full launch queue waits for the GPU)
+    Py_BEGIN_ALLOW_THREADS      // (a full launch queue waits for the GPU; nothing that may throw stands in here)
     status = g_route(static_cast<tlr_ctx*>(ctx), h_ptr, static_cast<int32_t>(n), static_cast<float>(tau),
-                     static_cast<int32_t*>(view[0].mutable_data_ptr()), static_cast<float*>(view[1].mutable_data_ptr()),
-                     static_cast<float*>(view[2].mutable_data_ptr()), static_cast<uint8_t*>(view[3].mutable_data_ptr()), idx,
-                     count, stream);
+                     static_cast<int32_t*>(rows[0]), static_cast<float*>(rows[1]), static_cast<float*>(rows[2]),
+                     static_cast<uint8_t*>(rows[3]), idx, count, stream);
     Py_END_ALLOW_THREADS
     if (status != TLR_OK) return PyLong_FromLong(status);
     PyObject* out = PyTuple_New(6);

@@ -47,3 +47,21 @@ def test_native_call_refuses_what_the_other_does(pkg):
     assert e.value.code == 6
     torch.cuda.synchronize()
     r.close()
+
+
+def test_an_output_without_memory_is_an_error(pkg):
+    r = pkg.Router(S.make_W(64, 3000, seed=1, std=0.2).cuda(), max_n=5)
+    h = S.make_h(5, 64, seed=2).h.cuda()
+    conf = r.conf
+
+    def step(wrapped):
+        r.conf = wrapped
+        r._views[5] = (r.token, wrapped, r.entropy, r.route_mask)      # (were it kept)
+        r.route(h, 0.5)
+        return wrapped
+
+    with pytest.raises(RuntimeError):
+        torch.vmap(step)(torch.zeros(2, 5, device="cuda"))
+    r.conf = conf
+    assert r.route(h, 0.5)[1].shape == (5,)
+    r.close()
