@@ -1,6 +1,6 @@
 // Router.route's call without options, as one native call: the checks of h, the arguments of tlr_route and the views that are
 // handed out.  Marshalling only, like binding.py, which does the same with ctypes where this declines (anything but a plain
-// tensor; a batch size whose views are not made yet) or was not built.
+// tensor; whatever is no number for a threshold; a batch size whose views are not made yet) or was not built.
 // A step of a small batch takes the GPU less time than it took the interpreter to ask for it: n = 1, d = 256, V = 20000
 // 8.9 us per call through ctypes, 5.6 of them tlr_route and its two launches.
 #define PY_SSIZE_T_CLEAN
@@ -38,7 +38,10 @@ PyObject* route(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     const long long d = PyLong_AsLongLong(args[1]);
     const double tau = PyFloat_AsDouble(args[3]);
     void* stream = PyLong_AsVoidPtr(args[7]);
-    if (PyErr_Occurred()) return nullptr;
+    if (PyErr_Occurred()) {       // (ctypes has its own idea of what a number is, and says so)
+      PyErr_Clear();
+      Py_RETURN_NONE;
+    }
     const at::Tensor& h = THPVariable_Unpack(h_obj);
     if (!h.is_cuda() || h.scalar_type() != at::kBFloat16 || h.dim() != 2 || !h.is_contiguous() || h.size(1) != d)
       Py_RETURN_NONE;

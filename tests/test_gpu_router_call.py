@@ -65,3 +65,20 @@ def test_an_output_without_memory_is_an_error(pkg):
     r.conf = conf
     assert r.route(h, 0.5)[1].shape == (5,)
     r.close()
+
+
+def test_thresholds_are_what_ctypes_takes(pkg):
+    import ctypes
+
+    import numpy as np
+    r = pkg.Router(S.make_W(64, 3000, seed=1, std=0.2).cuda(), max_n=5)
+    h = S.make_h(5, 64, seed=2).h.cuda()
+    tau = float(r.route(h, 0.01)[1].median())
+    want = r.route(h, tau)[3].clone()
+    for same in (ctypes.c_float(tau), np.float32(tau), torch.tensor(tau)):
+        assert torch.equal(r.route(h, same)[3], want)
+    assert int(r.route(h, 2)[5]) == 5
+    for bad in (None, "0.5", 10 ** 400):
+        with pytest.raises(ctypes.ArgumentError):
+            r.route(h, bad)
+    r.close()
