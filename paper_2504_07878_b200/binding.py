@@ -391,8 +391,8 @@ class Router:
         """Enqueues one routing step; returns views of the output tensors (valid after the stream syncs)."""
         plain = tau_per_row is None and not route_above and seq_len == 0 and score_source == 0 and mlp_score is None
         if plain and stream is None and _raw_handle and self.ctx is not None:
-            done = self._native(self.ctx.value, self.d, h, tau, self._views, self.routed_idx, self.routed_count,
-                                _raw_stream(_current_device()))
+            done = self._native(self.ctx.value, self.d, h, tau, self.token, self.conf, self.entropy, self.route_mask,
+                                self.routed_idx, self.routed_count, _raw_stream(_current_device()))
             if done.__class__ is tuple:
                 return done
             if done is not None:

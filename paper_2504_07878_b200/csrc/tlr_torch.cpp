@@ -1,6 +1,6 @@
 // Router.route's call without options, as one native call: the checks of h, the arguments of tlr_route and the views that are
-// handed out.  Marshalling only, like binding.py, which does the same with ctypes where this declines (anything but a plain
-// tensor; whatever is no number for a threshold; a batch size whose views are not made yet) or was not built.
+// handed out.  Marshalling only, like binding.py, which does the same with ctypes where this declines (anything but plain
+// tensors, whatever is no number for a threshold) or was not built.
 // A step of a small batch takes the GPU less time than it took the interpreter to ask for it: n = 1, d = 256, V = 20000
 // 8.9 us per call through ctypes, 5.6 of them tlr_route and its two launches.
 #define PY_SSIZE_T_CLEAN
@@ -20,73 +20,64 @@ PyObject* bind(PyObject*, PyObject* address) {
   Py_RETURN_NONE;
 }
 
-template <class T>
-T* data_of(PyObject* tensor) {
-  return static_cast<T*>(THPVariable_Unpack(tensor).mutable_data_ptr());
+// t[:n].data for a one-dimensional contiguous tensor of at least n elements: made anew on every call (a batch size that was not
+// asked for before costs what the others do), by the tensor's own copy with another length -- a slice from Python takes four times as long.
+at::Tensor head_of(const at::Tensor& t, int64_t n) {
+  auto impl = t.unsafeGetTensorImpl()->shallow_copy_and_detach(c10::VariableVersion(0), /*allow_tensor_metadata_change=*/true);
+  impl->set_sizes_contiguous(n);
+  impl->set_allow_tensor_metadata_change(false);
+  return at::Tensor(std::move(impl));
 }
 
-// route(ctx, d, h, tau, views, routed_idx, routed_count, stream): views maps a batch size to (token, conf, entropy, route_mask).
-// The six outputs as new views; the status if tlr_route fails; None if this call is not for here.
+bool has_head(const at::Tensor& t, int64_t n) { return t.dim() == 1 && t.is_contiguous() && t.size(0) >= n; }
+
+// route(ctx, d, h, tau, token, conf, entropy, route_mask, routed_idx, routed_count, stream): the six outputs, the first four as
+// new views of n rows; the status if tlr_route fails; None if this call is not for here.
+constexpr int kFirstOut = 4, kViews = 4, kOuts = 6, kArgs = kFirstOut + kOuts + 1;
 PyObject* route(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
-  if (nargs != 8 || g_route == nullptr) Py_RETURN_NONE;
-  PyObject *h_obj = args[2], *idx_obj = args[5], *count_obj = args[6];
-  if (!THPVariable_CheckExact(h_obj) || !THPVariable_CheckExact(idx_obj) || !THPVariable_CheckExact(count_obj) ||
-      !PyDict_CheckExact(args[4]))
+  if (nargs != kArgs || g_route == nullptr || !THPVariable_CheckExact(args[2])) Py_RETURN_NONE;
+  for (int i = 0; i < kOuts; ++i)
+    if (!THPVariable_CheckExact(args[kFirstOut + i])) Py_RETURN_NONE;
+  void* ctx = PyLong_AsVoidPtr(args[0]);
+  const long long d = PyLong_AsLongLong(args[1]);
+  const double tau = PyFloat_AsDouble(args[3]);
+  void* stream = PyLong_AsVoidPtr(args[kArgs - 1]);
+  if (PyErr_Occurred()) {       // (ctypes has its own idea of what a number is, and says so)
+    PyErr_Clear();
     Py_RETURN_NONE;
+  }
   try {
-    void* ctx = PyLong_AsVoidPtr(args[0]);
-    const long long d = PyLong_AsLongLong(args[1]);
-    const double tau = PyFloat_AsDouble(args[3]);
-    void* stream = PyLong_AsVoidPtr(args[7]);
-    if (PyErr_Occurred()) {       // (ctypes has its own idea of what a number is, and says so)
-      PyErr_Clear();
-      Py_RETURN_NONE;
-    }
-    const at::Tensor& h = THPVariable_Unpack(h_obj);
+    const at::Tensor& h = THPVariable_Unpack(args[2]);
     if (!h.is_cuda() || h.scalar_type() != at::kBFloat16 || h.dim() != 2 || !h.is_contiguous() || h.size(1) != d)
       Py_RETURN_NONE;
     const int64_t n = h.size(0);
-    PyObject* key = PyLong_FromLongLong(n);
-    if (key == nullptr) return nullptr;
-    PyObject* kept = PyDict_GetItemWithError(args[4], key);      // (borrowed)
-    Py_DECREF(key);
-    if (kept == nullptr) {
-      if (PyErr_Occurred()) return nullptr;
-      Py_RETURN_NONE;
+    void* out[kOuts];
+    for (int i = 0; i < kOuts; ++i) {
+      const at::Tensor& t = THPVariable_Unpack(args[kFirstOut + i]);
+      if (i < kViews && !has_head(t, n)) Py_RETURN_NONE;
+      out[i] = t.mutable_data_ptr();
     }
-    if (!PyTuple_CheckExact(kept) || PyTuple_GET_SIZE(kept) != 4) Py_RETURN_NONE;
-    at::Tensor view[4];
-    for (int i = 0; i < 4; ++i) {
-      if (!THPVariable_CheckExact(PyTuple_GET_ITEM(kept, i))) Py_RETURN_NONE;
-      view[i] = THPVariable_Unpack(PyTuple_GET_ITEM(kept, i)).variable_data();
-    }
-    void* rows[4];
-    for (int i = 0; i < 4; ++i) rows[i] = view[i].mutable_data_ptr();
     const void* h_ptr = h.const_data_ptr();
-    int32_t* idx = data_of<int32_t>(idx_obj);
-    int32_t* count = data_of<int32_t>(count_obj);
+    at::Tensor view[kViews];
+    for (int i = 0; i < kViews; ++i) view[i] = head_of(THPVariable_Unpack(args[kFirstOut + i]), n);
     tlr_status status;
     Py_BEGIN_ALLOW_THREADS      // (a full launch queue waits for the GPU; nothing that may throw stands in here)
     status = g_route(static_cast<tlr_ctx*>(ctx), h_ptr, static_cast<int32_t>(n), static_cast<float>(tau),
-                     static_cast<int32_t*>(rows[0]), static_cast<float*>(rows[1]), static_cast<float*>(rows[2]),
-                     static_cast<uint8_t*>(rows[3]), idx, count, stream);
+                     static_cast<int32_t*>(out[0]), static_cast<float*>(out[1]), static_cast<float*>(out[2]),
+                     static_cast<uint8_t*>(out[3]), static_cast<int32_t*>(out[4]), static_cast<int32_t*>(out[5]), stream);
     Py_END_ALLOW_THREADS
     if (status != TLR_OK) return PyLong_FromLong(status);
-    PyObject* out = PyTuple_New(6);
-    if (out == nullptr) return nullptr;
-    for (int i = 0; i < 4; ++i) {
-      PyObject* o = THPVariable_Wrap(view[i]);
+    PyObject* result = PyTuple_New(kOuts);
+    if (result == nullptr) return nullptr;
+    for (int i = 0; i < kOuts; ++i) {
+      PyObject* o = i < kViews ? THPVariable_Wrap(std::move(view[i])) : Py_NewRef(args[kFirstOut + i]);
       if (o == nullptr) {
-        Py_DECREF(out);
+        Py_DECREF(result);
         return nullptr;
       }
-      PyTuple_SET_ITEM(out, i, o);
+      PyTuple_SET_ITEM(result, i, o);
     }
-    Py_INCREF(idx_obj);
-    Py_INCREF(count_obj);
-    PyTuple_SET_ITEM(out, 4, idx_obj);
-    PyTuple_SET_ITEM(out, 5, count_obj);
-    return out;
+    return result;
   } catch (const std::exception& e) {
     PyErr_SetString(PyExc_RuntimeError, e.what());
     return nullptr;

@@ -82,3 +82,39 @@ def test_thresholds_are_what_ctypes_takes(pkg):
         with pytest.raises(ctypes.ArgumentError):
             r.route(h, bad)
     r.close()
+
+
+def _unused(*args):
+    raise AssertionError("through ctypes")
+
+
+def test_native_call_takes_every_batch_size_the_first_time(pkg):
+    r = pkg.Router(S.make_W(64, 3000, seed=1, std=0.2).cuda(), max_n=64)
+    h = S.make_h(64, 64, seed=2).h.cuda()
+    through_ctypes, r._tlr_route = r._tlr_route, _unused
+    for n in list(range(65)) + [3, 64, 1]:                       # more sizes than any cache of views has
+        got = r.route(h[:n], 0.01)
+        assert all(t.shape == (n,) for t in got[:4])
+    r._tlr_route = through_ctypes
+    got[0].unsqueeze_(1)                                         # a caller's own view, changed in place
+    again = r.route(h[:1], 0.01)
+    native, r._native = r._native, lambda *args: None
+    want = r.route(h[:1], 0.01)
+    r._native = native
+    assert again[0].shape == (1,) and all(a.dtype == b.dtype and a.stride() == b.stride() and a.requires_grad == b.requires_grad
+                                          and a.is_inference() == b.is_inference() for a, b in zip(again[:4], want))
+    r.close()
+
+
+def test_native_call_writes_the_current_tensors(pkg):
+    r = pkg.Router(S.make_W(64, 3000, seed=1, std=0.2).cuda(), max_n=5)
+    h = S.make_h(5, 64, seed=2).h.cuda()
+    want = r.route(h, 0.01)[1].clone()
+    before = r.conf.detach()
+    r.conf.data = torch.zeros_like(before)                       # the same object, other memory
+    before.zero_()
+    got = r.route(h, 0.01)[1]
+    torch.cuda.synchronize()
+    assert got.data_ptr() == r.conf.data_ptr() != before.data_ptr()
+    assert torch.equal(r.conf, want) and not before.any()
+    r.close()
