@@ -31,6 +31,32 @@ at::Tensor head_of(const at::Tensor& t, int64_t n) {
 
 bool has_head(const at::Tensor& t, int64_t n) { return t.dim() == 1 && t.is_contiguous() && t.size(0) >= n; }
 
+// heads(n, t, ...): head_of every tensor, None if one has none.
+PyObject* heads(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
+  if (nargs < 1) Py_RETURN_NONE;
+  const long long n = PyLong_AsLongLong(args[0]);
+  if (PyErr_Occurred()) return nullptr;
+  for (Py_ssize_t i = 1; i < nargs; ++i)
+    if (n < 0 || !THPVariable_CheckExact(args[i]) || !has_head(THPVariable_Unpack(args[i]), n)) Py_RETURN_NONE;
+  PyObject* result = PyTuple_New(nargs - 1);
+  if (result == nullptr) return nullptr;
+  try {
+    for (Py_ssize_t i = 1; i < nargs; ++i) {
+      PyObject* o = THPVariable_Wrap(head_of(THPVariable_Unpack(args[i]), n));
+      if (o == nullptr) {
+        Py_DECREF(result);
+        return nullptr;
+      }
+      PyTuple_SET_ITEM(result, i - 1, o);
+    }
+    return result;
+  } catch (const std::exception& e) {
+    Py_DECREF(result);
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+
 // route(ctx, d, h, tau, token, conf, entropy, route_mask, routed_idx, routed_count, stream): the six outputs, the first four as
 // new views of n rows; the status if tlr_route fails; None if this call is not for here.
 constexpr int kFirstOut = 4, kViews = 4, kOuts = 6, kArgs = kFirstOut + kOuts + 1;
@@ -87,6 +113,8 @@ PyObject* route(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
 PyMethodDef methods[] = {{"bind", bind, METH_O, "the address of tlr_route"},
                          {"route", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(route)), METH_FASTCALL,
                           "one routing step"},
+                         {"heads", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(heads)), METH_FASTCALL,
+                          "views of the first n elements"},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_tlr_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

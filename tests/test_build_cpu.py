@@ -54,8 +54,11 @@ def test_the_module_is_stale_when_anything_it_is_built_from_changes(monkeypatch,
 
 def test_a_module_built_for_another_torch_is_not_used(monkeypatch):
     build.build()
-    monkeypatch.setattr(binding, "_native", None)
-    assert "built-in" in repr(binding._native_route())
-    monkeypatch.setattr(binding, "_native", None)
+    for name in ("_native", "_extension"):
+        monkeypatch.setattr(binding, name, None)
+    assert "built-in" in repr(binding._native_route()) and binding._module()
+    for name in ("_native", "_extension"):
+        monkeypatch.setattr(binding, name, None)
     monkeypatch.setattr(torch, "__version__", "0.0")
     assert binding._native_route()(1, 2) is None and "built-in" not in repr(binding._native_route())
+    assert not binding._module()

@@ -1,7 +1,9 @@
 """What Router.route hands out: views of the router's current output tensors, its own for every call (no GPU needed)."""
+import pytest
 import torch
 
 import paper_2504_07878_b200 as P
+from paper_2504_07878_b200 import binding
 
 
 def make_router(max_n):
@@ -44,3 +46,22 @@ def test_many_batch_sizes():
     for n in list(range(65)) * 2:
         assert [t.shape[0] for t in r._outputs(n)[:4]] == [n] * 4
     assert len(r._views) <= 16
+
+
+@pytest.mark.parametrize("native", [True, False])
+def test_views_are_of_the_memory_that_a_tensor_has_now(monkeypatch, native):
+    if not native:
+        monkeypatch.setattr(binding, "_extension", False)
+    r = make_router(8)
+    r._outputs(5)
+    before = r.conf.detach()
+    r.conf.data = before + 1                              # the same object, other memory
+    for n in (5, 6, 0):
+        got = r._outputs(n)
+        assert got[1].shape == (n,) and (n == 0 or got[1].data_ptr() == r.conf.data_ptr())
+        assert torch.equal(got[1], r.conf[:n]) and got[1].dtype == torch.float32 and not got[1].requires_grad
+    assert r._outputs(5)[1].data_ptr() != before.data_ptr()
+    r.token = torch.arange(4, dtype=torch.int32)          # shorter than asked for: what a slice gives
+    assert r._outputs(5)[0].shape == (4,)
+    r.token = torch.arange(32, dtype=torch.int32).view(16, 2)[:, 1]
+    assert torch.equal(r._outputs(5)[0], r.token[:5])
