@@ -987,6 +987,12 @@ tlr_status tlr_shard_attach(tlr_ctx* ctx, int32_t rank, int32_t shards, void* co
       return TLR_ERR_CUDA;
     }
   }
+  // (a copy from pageable memory may return before it has reached the device, and steps on streams that do not wait for the
+  // default stream read these tables)
+  if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
+    ctx->shard_count = 0;
+    return TLR_ERR_CUDA;
+  }
   ctx->shard_rank = rank;
   ctx->shard_count = shards;
   ctx->shard_epoch = 0;

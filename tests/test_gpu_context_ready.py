@@ -49,3 +49,29 @@ def test_a_new_context_steps_on_a_side_stream_while_the_default_stream_is_busy(p
 def _on(stream, tensors):
     with torch.cuda.stream(stream):
         return [t.cpu() for t in tensors]
+
+
+# The tables of the peers' addresses are on the device, and what came before on the default stream is complete (the block's
+# zeros), when the attaching call returns.
+def test_an_attached_context_steps_on_a_side_stream(pkg):
+    W = S.make_W(D, V, seed=3, std=0.2).cuda()
+    h = S.make_h(N, D, seed=4).h.cuda()
+    out = [torch.zeros(N, dtype=t, device="cuda") for t in (torch.int32, torch.float32, torch.float32, torch.uint8, torch.int32)]
+    out.append(torch.zeros(1, dtype=torch.int32, device="cuda"))
+    ctx = pkg.tlr_create(D, V, W, N)
+    pkg.tlr_route(ctx, h, N, 0.01, *out)
+    torch.cuda.synchronize()
+    want = to_np(out[0]).copy()
+    block = torch.empty(pkg.tlr_shard_block_bytes(N, 1), dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda._sleep(100_000_000)
+    out[0].fill_(-1)
+    block.zero_()
+    pkg.tlr_shard_attach(ctx, 0, 1, [block])
+    assert torch.cuda.default_stream().query()
+    pkg.tlr_shard_push(ctx, h, N, 0, stream=side)
+    pkg.tlr_shard_finish_fused(ctx, N, 0.01, *out, stream=side)
+    side.synchronize()
+    assert pkg.tlr_last_device_status(ctx) == 0
+    assert np.array_equal(to_np(out[0]), want)
+    pkg.tlr_destroy(ctx)
