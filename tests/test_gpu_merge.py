@@ -58,45 +58,104 @@ def _expect(kind, r, h, n):
     return [t.copy() for t in (to_np(r.token[:n]), to_np(r.conf[:n]), to_np(r.entropy[:n]), to_np(r.route_mask[:n]))]
 
 
+class _Steps:
+    """Steps of one context on the batches `h`, every one with output buffers of its own."""
+
+    def __init__(self, pkg, kind, seed, sizes):
+        self.pkg, self.kind = pkg, kind
+        (W, scale), _, d = _head(kind)
+        if seed:
+            W = W.flip(0).contiguous()
+            scale = None if scale is None else scale.flip(0).contiguous()
+        self.h = [S.make_h(n, d, seed=seed + n).h.cuda() for n in sizes]
+        top = max(sizes)
+        if kind == "push":
+            block = torch.zeros(pkg.tlr_shard_block_bytes(top, 1), dtype=torch.uint8, device="cuda")
+            self.r = pkg.FusedVocabShardedRouter(W, 0, top, 0, 1, [block], keep=block)
+        elif kind == "summary":
+            self.r = pkg.VocabShardedRouter(W, 0, max_n=top, world=1)
+        else:
+            self.r = pkg.Router(W, max_n=top, wscale=scale)
+        self.tau, self.want = [0.5] * len(sizes), []
+        for k in range(len(sizes)):
+            conf = self.alone(k)[1]
+            self.tau[k] = float(np.median(conf)) if len(conf) > 1 else 2.0        # (a row alone is routed)
+            self.want.append(self.alone(k))
+
+    def buffers(self, k):
+        n = self.h[k].shape[0]
+        out = [torch.empty(n, dtype=t, device="cuda") for t in (torch.int32, torch.float32, torch.float32, torch.uint8, torch.int32)]
+        return out + [torch.empty(1, dtype=torch.int32, device="cuda")]
+
+    def step(self, k, out):
+        pkg, ctx, h, n = self.pkg, self.r.ctx, self.h[k], self.h[k].shape[0]
+        if self.kind == "push":
+            pkg.tlr_shard_push(ctx, h, n, 0)
+            pkg.tlr_shard_finish_fused(ctx, n, self.tau[k], *out)
+        elif self.kind == "summary":
+            pkg.tlr_shard_summary(ctx, h, n, 0, self.r.summary)
+            pkg.tlr_shard_finish(ctx, self.r.summary, 1, n, self.tau[k], *out)
+        else:
+            pkg.tlr_route(ctx, h, n, self.tau[k], *out)
+
+    def alone(self, k):
+        """What a step gives when nothing else is in flight."""
+        out = self.buffers(k)
+        torch.cuda.synchronize()
+        self.step(k, out)
+        torch.cuda.synchronize()
+        return _listed(out)
+
+
+def _listed(out):
+    out = [to_np(t).copy() for t in out]
+    return out[:4] + [out[4][:int(out[5][0])], out[5]]
+
+
 # Steps that nothing waits between, of different sizes and inputs: each merge may look for its partials while the one before is
-# still at work on its own, in the same memory.  More steps than there are tags (254); and replayed, when the tags come back.
-@pytest.mark.parametrize("kind", ["bf16", "8bit", "odd"])
-@pytest.mark.parametrize("graph", [False, True])
-def test_steps_back_to_back_keep_their_partials(pkg, kind, graph):
-    (W, scale), _, d = _head(kind)
+# still at work on its own, in the same memory or, with two contexts in turn, in the other's.  More steps than there are tags
+# (254); and replayed, when the tags come back.  Every step's outputs are kept and looked at.
+@pytest.mark.parametrize("contexts", [1, 2])
+@pytest.mark.parametrize("kind,graph", [(k, g) for k in ("bf16", "8bit", "odd", "summary") for g in (False, True)] + [("push", False)])
+def test_steps_back_to_back_keep_their_partials(pkg, kind, graph, contexts):
     sizes = [1, 16, 8, 64, 17, 128] + ([] if kind == "8bit" else [256, 200, 300])
-    r = pkg.Router(W, max_n=max(sizes), wscale=scale)
-    batches = [S.make_h(n, d, seed=100 + n).h.cuda() for n in sizes]
-    want = [_expect(kind, r, h, n) for h, n in zip(batches, sizes)]
-    steps = 600
-    kept = [[torch.empty_like(t[:n]) for t in (r.token, r.conf, r.entropy, r.route_mask)] for n in sizes]
+    routers = [_Steps(pkg, kind, 100 * c, sizes) for c in range(contexts)]
+    steps = []
+    for i in range(600 * contexts):
+        s, k = routers[i % contexts], (i // contexts * 7) % len(sizes)
+        steps.append((s, k, s.buffers(k)))
 
     def loop():
-        for i in range(steps):
-            k = (i * 7) % len(sizes)
-            r.route(batches[k], 0.5)
-            if i >= steps - 2 * len(sizes):               # the last rounds are looked at
-                for dst, src in zip(kept[k], (r.token, r.conf, r.entropy, r.route_mask)):
-                    dst.copy_(src[:sizes[k]])
+        for s, k, out in steps:
+            s.step(k, out)
 
+    def check():
+        torch.cuda.synchronize()
+        for s in routers:
+            assert pkg.tlr_last_device_status(s.r.ctx) == 0
+        for i, (s, k, out) in enumerate(steps):
+            for a, b in zip(_listed(out), s.want[k]):
+                assert np.array_equal(a, b), (i, sizes[k])
+        for _, _, out in steps:
+            for t in out:
+                t.zero_()
+
+    torch.cuda.synchronize()
     if graph:
         side = torch.cuda.Stream()
-        side.wait_stream(torch.cuda.current_stream())
         g = torch.cuda.CUDAGraph()
         with torch.cuda.graph(g, stream=side):
             loop()
         for _ in range(3):
             g.replay()
-    else:
-        loop()
-    torch.cuda.synchronize()
-    assert pkg.tlr_last_device_status(r.ctx) == 0
-    for got, ref in zip(kept, want):
-        for a, b in zip(got, ref):
-            assert np.array_equal(to_np(a), b)
-    if graph:
+            check()
         del g
-    r.close()
+    else:
+        torch.cuda._sleep(20_000_000)              # the host runs ahead
+        loop()
+        check()
+    for s in routers:
+        s.r.close()
 
 
 # A call that fails between the projection and the merge leaves partials that nobody takes.  They are nobody's either when the
