@@ -81,6 +81,7 @@ constexpr int kBarrierBytes = 640;
 constexpr int kScratchBytes = kBlockM * 16;  // one Partial per row: hand-over between the epilogue groups
 constexpr int kSmemLimit = 232448;           // 227 KiB opt-in maximum per CTA
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
+constexpr unsigned long long kAheadNs = 60000000000ull;     // and a minute for the role that starts ahead of the wait for the kernel in front
 // 8-bit head: the weight scales of every epilogue warp's share of a tile, and the rows' power-of-two scales
 constexpr int kScaleBytes = kEpiWarps * (kBlockN / 2) * 4;
 constexpr int kRowScaleBytes = 64 * 4;
@@ -461,6 +462,12 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   if (warp == 0) {
     // ------------------------------------------------------------------ W producer
     if (lane == 0) {
+      // This role has not waited for the kernel in front, whose time its limit must not count.  What keeps a slab from being
+      // released the other roles notice within theirs, and it sees their flag.  (A wait for that kernel in this loop, in front
+      // of the first slab that must be released: n = 444, d = 752, V = 30000 24.8 -> 25.1 us, a bounded number of looks in
+      // front of it 25.8 and prefill at n = 8192, d = 896 4 % longer; a clock that starts again n = 600, d = 256, V = 30000
+      // 20.1 -> 20.4.  The longer limit costs nothing.)
+      const unsigned long long ahead_ns = wait_ns + kAheadNs;
       int stage = 0;
       int slab = 0;     // running slab number, the same in every role
       bool ok = true;
@@ -483,7 +490,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
           for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
             if (slab >= SB) {     // the stage is free once slab - SB has been consumed
               const int j = slab - SB;
-              if (!mbar_wait(released(j & (kRelease - 1)), (j / kRelease) & 1, abort_flag, p.status, wait_ns)) { ok = false; break; }
+              if (!mbar_wait(released(j & (kRelease - 1)), (j / kRelease) & 1, abort_flag, p.status, ahead_ns)) { ok = false; break; }
             }
             const uint32_t dst = b_ring + stage * b_stage_bytes;
             const uint32_t bar = (kCta == 2) ? map_to_cta(b_full(stage), 0) : b_full(stage);

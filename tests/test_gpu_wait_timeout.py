@@ -105,7 +105,7 @@ def test_a_tensor_map_that_cannot_be_encoded_is_an_error(pkg, n, d, fp8):
 
 # The kernel in front of a step may be at work for longer than any limit -- here the merge of a sharded step, which looks for a
 # rank that never joins for 2.5 s -- and lets the step's kernels in early.  Their limits do not cover it.
-@pytest.mark.parametrize("n,d,fp8", [(5, 64, False), (40, 64, True), (200, 64, False)])
+@pytest.mark.parametrize("n,d,fp8", [(5, 64, False), (40, 64, True), (200, 64, False), (200, 1024, False), (40, 1024, True)])
 def test_limits_do_not_cover_what_a_step_waits_for(pkg, n, d, fp8):
     V = 20000
     W, scale = S.make_W8(d, V, seed=2, std=0.2) if fp8 else (S.make_W(d, V, seed=2, std=0.2), None)
