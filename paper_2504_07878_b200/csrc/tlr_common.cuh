@@ -47,7 +47,8 @@ __device__ __forceinline__ Partial empty_partial() {
 //   * A partial that is there says that its CTA has passed its own wait: whatever came before the projection in the stream
 //     is complete, and outputs may be written.
 //   * The reader waits for the projection grid before it ends, so that who waits for the reader's grid waits for both.
-// Tagged steps have partials of their own (no other path writes there).  Per step in a stream, untagged and tagged: n = 1,
+// Tagged steps have partials of their own (no other path writes there).  Per step in a stream with the calls queued ahead (a
+// host that asks for one after the other has its own part in the smallest steps), untagged and tagged: n = 1,
 // d = 256, V = 20000 7.30 and 6.20 us, n = 16, d = 896, V = 151936 44.26 and 42.90 (8-bit head 28.4 and 27.1), n = 64, d = 300,
 // V = 33000 12.31 and 11.57, one of eight shards at n = 256 18.07 and 17.34; n = 256, d = 512, V = 32000 14.5 either way.
 constexpr int kTagShift = 24;

@@ -340,8 +340,8 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
 
 // The same for steps whose lanes own few partials (rows_shape), and then what stands between the last partial and the end of
 // the step is latency alone: the compaction has a warp of its own -- the last one of block 0 -- that waits for the words and
-// does it while the others still work out their entropies and store their rows.  Per step in a stream, with finish_small_kernel
-// and with this one (partials not tagged): n = 1, d = 256, V = 20000 8.36 and 7.30 us, n = 16, d = 896, V = 151936 45.73 and 44.26
+// does it while the others still work out their entropies and store their rows.  Per step in a stream, calls queued ahead,
+// with finish_small_kernel and with this one (partials not tagged): n = 1, d = 256, V = 20000 8.36 and 7.30 us, n = 16, d = 896, V = 151936 45.73 and 44.26
 // (8-bit head 30.0 and 28.4), n = 64, d = 512, V = 32000 12.24 and 11.03, n = 128 there 13.26 and 12.13.
 // kTagged: the partials are tagged ones (tlr_common.cuh), no peers and no learned router.
 // kRowWarps: 16, or 8 where a block of 17 warps would not stand beside a CTA of the projection.  No register may be spilled: a kernel that writes local memory ends a

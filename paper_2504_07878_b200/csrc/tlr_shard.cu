@@ -47,7 +47,8 @@ shard_summary_kernel(Partial* partials, uint32_t tag, uint32_t* status, int n, i
   const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   // A programmatic dependent launch like the kernels around it: its blocks (512 small ones at most fit beside the
-  // projection's CTAs) wait for the projection where they stand, and a merge kernel behind it may be scheduled now.
+  // projection's CTAs) wait for the projection or its tagged partials where they stand, and a merge kernel behind it may be
+  // scheduled now.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tag == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row >= n) return;
@@ -62,7 +63,8 @@ shard_push_kernel(const ShardPush a) {
   const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   // Programmatic dependent launch: scheduled while the projection kernel finishes, and the merge kernel behind
-  // this one may be scheduled now; the partials are read only after the projection has completed.
+  // this one may be scheduled now.  Untagged partials are read only after the projection has completed, tagged ones as they
+  // arrive; either way the flags below are set behind it.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (a.tag == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row < a.n) {

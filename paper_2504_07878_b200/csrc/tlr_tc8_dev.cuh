@@ -60,8 +60,8 @@ __device__ __forceinline__ float split_scale(float amax) {
 
 // x * inv as the sum of two e4m3 numbers: p1 = round(x), p2 = round(x - p1), two elements at a time and in halves: down to
 // 2^-17 a bf16 number below 256 is a half, and below that both parts are zero (e4m3's smallest step is 2^-9).
-// (In floats, with the magnitudes compared one by one: n = 16, d = 896, V = 151936 26.9 us per step, so 26.5; n = 32, d = 512,
-// V = 30000 9.36 and 9.19.)
+// (In floats, with the magnitudes compared one by one: n = 16, d = 896, V = 151936 26.9 us per step (calls queued ahead), so
+// 26.5; n = 32, d = 512, V = 30000 9.36 and 9.19.)
 __device__ __forceinline__ void split_pair(float x0, float x1, uint16_t& p1, uint16_t& p2) {
   const __half2 x = __floats2half2_rn(x0, x1);
   p1 = to_e4m3x2(*reinterpret_cast<const uint32_t*>(&x));
