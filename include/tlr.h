@@ -363,6 +363,13 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
                                 int32_t capacity, int32_t* count, tlr_plan* plan_out);
 
 /*
+ * tlr_debug_plan_two_blocks -- the same for the schedule in which a unit is two blocks of 256 token rows (n > 128; batches of
+ * more than 256 rows use it where it leaves no worker more to do): the tiles are those of both blocks.
+ */
+tlr_status tlr_debug_plan_two_blocks(int32_t n, int32_t V, int32_t sm_count, int32_t mlp_hidden, int32_t* out,
+                                 int32_t capacity, int32_t* count, tlr_plan* plan_out);
+
+/*
  * tlr_debug_shard_table -- host-only: the addresses tlr_shard_attach derives for one rank and one parity of the
  * call counter from the ranks' exchange-block addresses (no GPU needed; used by the CPU tests of the layout).
  * slot_out[g] / flag_out[g] = where rank `rank` stores its summaries / its flag on peer g.

@@ -91,6 +91,8 @@ def load_library() -> ctypes.CDLL:
     lib.tlr_route_ex.restype = c_int32
     lib.tlr_debug_plan_tiles.argtypes = [c_int32, c_int32, c_int32, c_int32, P, c_int32, POINTER(c_int32), POINTER(TlrPlan)]
     lib.tlr_debug_plan_tiles.restype = c_int32
+    lib.tlr_debug_plan_two_blocks.argtypes = lib.tlr_debug_plan_tiles.argtypes
+    lib.tlr_debug_plan_two_blocks.restype = c_int32
     lib.tlr_debug_inject.argtypes = [P, c_int32, c_uint32]
     lib.tlr_debug_inject.restype = c_int32
     lib.tlr_set_router_mlp.argtypes = [P, c_int32, P, P, P, c_float]
@@ -310,17 +312,17 @@ def tlr_debug_inject(ctx, kind: int, wait_limit_ms: int = 0):
     _check(load_library().tlr_debug_inject(ctx, kind, wait_limit_ms), "tlr_debug_inject")
 
 
-def tlr_debug_plan_tiles(n: int, V: int, sm_count: int = 148, mlp_hidden: int = 0):
+def tlr_debug_plan_tiles(n: int, V: int, sm_count: int = 148, mlp_hidden: int = 0, blocks: int = 1):
     """Host-only: the tensor-core kernel's tile schedule as an int32 array [tiles, 5] and its plan
-    (mlp_hidden > 0: with a learned router of that width inside the launch)."""
+    (mlp_hidden > 0: with a learned router of that width inside the launch; blocks = 2: units of two row blocks)."""
     import numpy as np
     lib = load_library()
     count, plan = c_int32(0), TlrPlan()
-    _check(lib.tlr_debug_plan_tiles(n, V, sm_count, mlp_hidden, c_void_p(0), 0, byref(count), byref(plan)),
-           "tlr_debug_plan_tiles")
+    call = lib.tlr_debug_plan_two_blocks if blocks == 2 else lib.tlr_debug_plan_tiles
+    _check(call(n, V, sm_count, mlp_hidden, c_void_p(0), 0, byref(count), byref(plan)), "tlr_debug_plan_tiles")
     out = np.zeros((count.value, 5), dtype=np.int32)
-    _check(lib.tlr_debug_plan_tiles(n, V, sm_count, mlp_hidden, c_void_p(out.ctypes.data), count.value, byref(count),
-                                    byref(plan)), "tlr_debug_plan_tiles")
+    _check(call(n, V, sm_count, mlp_hidden, c_void_p(out.ctypes.data), count.value, byref(count), byref(plan)),
+           "tlr_debug_plan_tiles")
     return out, plan
 
 

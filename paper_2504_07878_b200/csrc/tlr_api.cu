@@ -47,13 +47,14 @@ const Tuning& tuning() {
 // router in the launch (mlp_hidden > 0) one more unit per row unit, over the rows of its first
 // layer, follows the vocabulary units in the same round-robin order and is counted in the loads.
 // With residue classes (d no multiple of 8) every class gets the same number of chunks.
-void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan) {
+void tc_plan(int n, int V, int cta, int blocks, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan) {
   int g = (classes > 1 ? kOddBoxRows : 16) * cta;
   {
     const int e = tuning().granule;   // tuning switch
     if (e >= g && e <= 256 && e % g == 0 && 256 % e == 0) g = e;
   }
-  const int row_units = (n + 128 * cta - 1) / (128 * cta);
+  const int unit_rows = 128 * cta * blocks;
+  const int row_units = (n + unit_rows - 1) / unit_rows;
   const int granules = ((V + classes - 1) / classes + g - 1) / g;      // of the longest class
   const int mlp_rows = mlp_hidden > 0 ? ((mlp_hidden + 16 * cta - 1) / (16 * cta)) * (16 * cta) : 0;
   const long long mlp_tiles = (mlp_rows + 255) / 256;
@@ -101,6 +102,8 @@ void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden,
       best_tiles = static_cast<int>(tiles);
     }
   }
+  plan->blocks = blocks;
+  plan->passes = best_passes * blocks;
   plan->row_units = row_units;
   plan->classes = classes;
   plan->chunks = best * classes;
@@ -292,7 +295,7 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     if (c->fp8) {
       tlr::tc8_configure(n <= tlr::tc8_max_rows() ? n : tlr::tc8_max_rows(), c->d, &cfg);
       workers_max = c->sm_count;
-      tlr::tc_plan(n <= 128 ? n : 128, c->V, 1, workers_max, tlr::kMaxChunks, 0, 1, &tp);
+      tlr::tc_plan(n <= 128 ? n : 128, c->V, 1, 1, workers_max, tlr::kMaxChunks, 0, 1, &tp);
       out->launches = n > 0 ? (cfg.inline_split ? 2 : 3) : 1;
     } else {
       int rows = n;
@@ -305,7 +308,15 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
       }
       tlr::tc_configure(rows, c->d + (c->classes > 1 ? tlr::odd_max_shift(c->d) : 0), c->V, c->sm_count, &cfg);
       workers_max = c->sm_count / cfg.cta;
-      tlr::tc_plan(rows, c->V, cfg.cta, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, c->classes, &tp);
+      tlr::tc_plan(rows, c->V, cfg.cta, 1, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, c->classes, &tp);
+      if (cfg.mode == tlr::RowMode::kM128 && c->classes == 1 && tlr::tc_two_blocks(n, c->d)) {
+        tlr::TcPlan two;
+        tlr::tc_plan(n, c->V, 2, 2, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, 1, &two);
+        if (tlr::tc_two_blocks_pay(two, tp)) {
+          tp = two;
+          tlr::tc_configure_two(c->d, &cfg);
+        }
+      }
     }
     const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;
     st->workers = units < workers_max ? units : workers_max;
@@ -314,13 +325,14 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
     out->grid = st->workers * cfg.cta;
     out->block = tlr::tc_threads();
     out->smem_bytes = cfg.smem_bytes;
-    out->reserved = cfg.mode == tlr::RowMode::kM128Keep ? 1 : 0;
+    out->reserved = cfg.mode == tlr::RowMode::kM128Keep ? 1 : (cfg.mode == tlr::RowMode::kM128Two ? 2 : 0);
     p.n = n;
     p.d = c->d;
     p.V = c->V;
     tlr::tc_set_schedule(tp, &p);
     p.a_rows = cfg.a_rows;
     p.part_rows = cfg.part_rows;
+    p.lag = cfg.lag;
     p.a_stages = cfg.a_stages;
     p.b_stages = cfg.b_stages;
     p.wait_limit_ns = c->debug_wait_ns;
@@ -586,6 +598,38 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
                              int32_t* routed_idx_dev, int32_t* routed_count_dev, void* cuda_stream,
                              uint32_t* status_copy);
 
+// The schedule as tlr_debug_plan_tiles reports it, with `blocks` row blocks to a unit.
+static tlr_status plan_tiles(int blocks, int32_t n, int32_t V, int32_t sm_count, int32_t mlp_hidden, int32_t* out,
+                             int32_t capacity, int32_t* count, tlr_plan* plan_out) {
+  if (n <= 0 || V <= 0 || sm_count < 2 || mlp_hidden < 0 || count == nullptr || capacity < 0 ||
+      (capacity > 0 && out == nullptr))
+    return TLR_ERR_ARG;
+  tlr::TcConfig cfg;
+  tlr::TcPlan tp;
+  tlr::tc_configure(n, 2048, V, sm_count, &cfg);
+  const int workers_max = sm_count / cfg.cta;
+  tlr::tc_plan(n, V, cfg.cta, blocks, workers_max, tlr::kMaxChunks, mlp_hidden, 1, &tp);
+  const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;
+  const int workers = units < workers_max ? units : workers_max;
+  tlr::TcParams p = {};
+  p.n = n;
+  p.V = V;
+  tlr::tc_set_schedule(tp, &p);
+  p.mlp_hidden = tp.mlp_rows > 0 ? mlp_hidden : 0;
+  *count = tlr::tc_enumerate_tiles(p, cfg.cta, workers, out, capacity);
+  if (plan_out != nullptr) {
+    plan_out->path = TLR_PATH_TC;
+    plan_out->grid = workers * cfg.cta;
+    plan_out->block = tlr::tc_threads();
+    plan_out->row_units = tp.row_units;
+    plan_out->vocab_chunks = tp.chunks;
+    plan_out->smem_bytes = cfg.smem_bytes;
+    plan_out->launches = 2;
+    plan_out->reserved = tp.granule_rows;
+  }
+  return TLR_OK;
+}
+
 extern "C" {
 
 const char* tlr_status_string(tlr_status s) {
@@ -725,33 +769,13 @@ tlr_status tlr_set_router_mlp(tlr_ctx* ctx, int32_t d_hidden, const void* W1_bf1
 
 tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t mlp_hidden, int32_t* out,
                                 int32_t capacity, int32_t* count, tlr_plan* plan_out) {
-  if (n <= 0 || V <= 0 || sm_count < 2 || mlp_hidden < 0 || count == nullptr || capacity < 0 ||
-      (capacity > 0 && out == nullptr))
-    return TLR_ERR_ARG;
-  tlr::TcConfig cfg;
-  tlr::TcPlan tp;
-  tlr::tc_configure(n, 2048, V, sm_count, &cfg);
-  const int workers_max = sm_count / cfg.cta;
-  tlr::tc_plan(n, V, cfg.cta, workers_max, tlr::kMaxChunks, mlp_hidden, 1, &tp);
-  const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;
-  const int workers = units < workers_max ? units : workers_max;
-  tlr::TcParams p = {};
-  p.n = n;
-  p.V = V;
-  tlr::tc_set_schedule(tp, &p);
-  p.mlp_hidden = tp.mlp_rows > 0 ? mlp_hidden : 0;
-  *count = tlr::tc_enumerate_tiles(p, cfg.cta, workers, out, capacity);
-  if (plan_out != nullptr) {
-    plan_out->path = TLR_PATH_TC;
-    plan_out->grid = workers * cfg.cta;
-    plan_out->block = tlr::tc_threads();
-    plan_out->row_units = tp.row_units;
-    plan_out->vocab_chunks = tp.chunks;
-    plan_out->smem_bytes = cfg.smem_bytes;
-    plan_out->launches = 2;
-    plan_out->reserved = tp.granule_rows;
-  }
-  return TLR_OK;
+  return plan_tiles(1, n, V, sm_count, mlp_hidden, out, capacity, count, plan_out);
+}
+
+tlr_status tlr_debug_plan_two_blocks(int32_t n, int32_t V, int32_t sm_count, int32_t mlp_hidden, int32_t* out,
+                                 int32_t capacity, int32_t* count, tlr_plan* plan_out) {
+  if (n <= 128) return TLR_ERR_ARG;
+  return plan_tiles(2, n, V, sm_count, mlp_hidden, out, capacity, count, plan_out);
 }
 
 tlr_status tlr_debug_inject(tlr_ctx* ctx, int32_t kind, uint32_t wait_limit_ms) {

@@ -135,7 +135,7 @@ extern "C" tlr_status tlr_route_static(int32_t d, int32_t V, const void* W_bf16_
     if (!s->tc_ready) return TLR_ERR_CUDA;   // no silent change of kernel
     tlr::tc_configure(n, d, V, s->sm_count, &cfg);
     const int workers_max = s->sm_count / cfg.cta;
-    tlr::tc_plan(n, V, cfg.cta, workers_max, kStaticMaxChunks, 0, 1, &tp);
+    tlr::tc_plan(n, V, cfg.cta, 1, workers_max, kStaticMaxChunks, 0, 1, &tp);
     chunks = tp.chunks;
     const int units = tp.chunks * tp.row_units;
     workers = units < workers_max ? units : workers_max;

@@ -94,16 +94,33 @@ void tc_configure(int n, int d, int V, int sm_count, TcConfig* c) {
   c->a_rows = a_rows;
   c->mode = mode;
   c->part_rows = a_rows;
+  c->lag = 0;
   c->a_stages = sa;
   c->b_stages = sb;
   c->inline_split = 0;
   c->smem_bytes = 1024 + sa * a_stage + sb * b_stage + kBarrierBytes + kScratchBytes;
 }
 
+// The same with two row blocks to a unit.  The second block stays `lag` slabs of W behind the first: its MMAs of a tile's last
+// slabs run while the first accumulator is folded (about 2100 cycles, 512 a slab) and the other way round, and the W stages of
+// those slabs stay occupied meanwhile.  Lags of 3 / 4 / 5 with five stages of h and eight of W, of 5 with four and nine, and
+// single blocks, us per step: n = 8192, d = 896, V = 151936 1738 / 1691 / 1648 / 1648 and 1738, n = 4096, d = 1536 there
+// 1429 / 1405 / 1386 / 1391 and 1459, n = 512, d = 2048, V = 128256 228 / 226 / 225 / 225 and 235; 6 of eight stages leave too
+// few for loads (407 instead of 364 at n = 777, d = 1536, V = 151936; 380 with single blocks).
+void tc_configure_two(int d, TcConfig* c) {
+  const int k_slabs = (d + kRowBytes / 2 - 1) / (kRowBytes / 2);
+  c->mode = RowMode::kM128Two;
+  c->lag = c->b_stages - 3;
+  if (c->lag > 5) c->lag = 5;
+  if (c->lag > k_slabs) c->lag = k_slabs;
+  if (c->lag < 1) c->lag = 1;
+}
+
 cudaError_t tc_prepare() {
   for (const auto kernel : {tc_projection_kernel<1, RowMode::kM128, true>, tc_projection_kernel<1, RowMode::kM64, true>,
                             tc_projection_kernel<1, RowMode::kGroup8, true>, tc_projection_kernel<2, RowMode::kM128, true>,
-                            tc_projection_kernel<2, RowMode::kM128, false>, tc_projection_kernel<2, RowMode::kM128Keep, false>}) {
+                            tc_projection_kernel<2, RowMode::kM128, false>, tc_projection_kernel<2, RowMode::kM128Keep, false>,
+                            tc_projection_kernel<2, RowMode::kM128Two, false>}) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
   }
@@ -130,7 +147,8 @@ cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const Tc
   // n = 256 with 104 registers and without the limit: V = 32000, d = 512 14.25 and 14.55 us, V = 40000, d = 1024 24.1 and 24.9;
   // V = 64000, d = 512 22.9 and 22.6, d = 896 35.7 and 35.3.
   const bool beside = p.n <= 256 && p.tiles_per_unit <= 3;
-  const auto kernel = c.mode == RowMode::kM128Keep ? tc_projection_kernel<2, RowMode::kM128Keep, false>
+  const auto kernel = c.mode == RowMode::kM128Two ? tc_projection_kernel<2, RowMode::kM128Two, false>
+                      : c.mode == RowMode::kM128Keep ? tc_projection_kernel<2, RowMode::kM128Keep, false>
                       : c.cta == 2 && beside       ? tc_projection_kernel<2, RowMode::kM128, true>
                       : c.cta == 2                 ? tc_projection_kernel<2, RowMode::kM128, false>
                       : c.mode == RowMode::kGroup8 ? tc_projection_kernel<1, RowMode::kGroup8, true>

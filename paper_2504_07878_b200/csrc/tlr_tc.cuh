@@ -11,6 +11,7 @@ namespace tlr {
 enum class RowMode : int {
   kM128,      // bf16 head, more than 64 rows: MMA M = 128 (256 on a pair), one epilogue thread per row
   kM128Keep,  // the same on a pair, where all of a row unit's h fits beside the W ring: it is loaded once per unit
+  kM128Two,   // the same on a pair, two row blocks of 256 to a unit: a slab of W is read by both while it is in shared memory
   kM64,       // bf16 head, 17..64 rows: M = 64, one thread per row
   kGroup8,    // bf16 head, up to 16 rows: M = 64, eight rows in every sixteen operand rows, four threads per row
   k8Small,    // 8-bit head, up to 32 rows: both parts through one MMA with M = 64, four threads per row
@@ -24,6 +25,7 @@ struct TcConfig {
   int a_rows;       // rows of an h slab held in shared memory (16..128); on the 8-bit head both parts of h stacked
   RowMode mode;
   int part_rows;    // 8-bit head: rows of one part (a_rows / 2); otherwise a_rows
+  int lag;          // RowMode::kM128Two: how many slabs the second row block is behind the first
   int a_stages;     // depth of the h ring
   int b_stages;     // depth of the W ring
   int inline_split; // 8-bit head: 1 = n <= 16 and both parts of all of h fit in shared memory -- the kernel splits h
@@ -33,13 +35,15 @@ struct TcConfig {
 
 // Work decomposition for a given (n, V) on `workers` workers (see tc_plan).
 struct TcPlan {
-  int row_units;       // ceil(n / (128 * cta))
+  int blocks;          // row blocks of 128 * cta rows in a unit (2: RowMode::kM128Two)
+  int row_units;       // ceil(n / (128 * cta * blocks))
   int classes;         // residue classes of the vocabulary (1 unless d is odd-sized, see OddMaps)
   int chunks;          // vocabulary chunks == partials per row; a multiple of `classes`
   int granule_rows;    // a multiple of 16 * cta
   int granules;        // ceil(rows of a class / granule_rows)
   int tiles_per_unit;  // every unit is walked in this many tiles (<= 256 rows each)
   int full_tiles_first;  // 1: full 256-row tiles, then one remainder tile; 0: tiles of equal size
+  long long passes;    // of the busiest worker: tiles times row blocks (pair mode)
   int mlp_rows;        // learned-router units: hidden width rounded up to the granule (0 = none); one such unit
                        // per row unit follows the vocabulary units
 };
@@ -47,6 +51,8 @@ struct TcPlan {
 struct TcParams {
   int n, d, V;
   int row_units, chunks, tiles_per_unit, full_tiles_first, granule_rows;
+  int blocks;                         // row blocks of a unit
+  int lag;                            // two of them: how many slabs of a tile the second is behind the first
   int chunk_q, chunk_r;               // granules of a chunk: chunk_q, and one more in chunk_r of them (of a class)
   uint32_t chunk_mul;                 // ceil(2^32 / chunks of a class), 0 for one chunk
   int full_granules;                  // granules of a full tile
@@ -102,6 +108,7 @@ cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const 
 inline int tc_h_box_rows(const TcConfig& c) { return c.mode == RowMode::kGroup8 ? 8 : c.a_rows; }   // rows of h per TMA box
 // The fields of a launch's parameters that describe its work decomposition.
 inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
+  p->blocks = plan.blocks;
   p->row_units = plan.row_units;
   p->chunks = plan.chunks;
   p->tiles_per_unit = plan.tiles_per_unit;
@@ -118,7 +125,21 @@ inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
 int tc_threads();
 int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
 void tc_configure(int n, int d, int V, int sm_count, TcConfig* c);
-void tc_plan(int n, int V, int cta, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan);
+// Whether a batch of n rows may be walked in units of two row blocks (256 rows each): not where
+// h is large against L2 (126 MB, in two halves): single blocks and two, ms per step, d = 2048 and n = 8192 (34 MB), V = 60000
+// 1.549 and 1.453, n = 12000 (49 MB) 2.209 and 2.175, n = 14000 (57 MB), V = 100000 4.377 and 4.387, n = 16384 (67 MB),
+// V = 128256 6.518 and 6.573; d = 1536 and n = 16384 (50 MB), V = 60000 2.281 and 2.191.
+inline bool tc_two_blocks(int n, int d) {
+  return n > 256 && 2ll * n * d <= (50ll << 20);
+}
+// ... and whether they pay, given both plans (an odd block is a unit and counts for two, which is little among many): few units may leave the busiest worker more passes than single blocks would, of which
+// up to 4 % are given back (n = 1000, d = 896, V = 151936: 34 instead of 33, 232.5 and 229.6 us), and short walks gain nothing,
+// having their first and last slabs longer (n = 400, d = 1024, V = 30000, four passes: 29.8 and 32.0).
+inline bool tc_two_blocks_pay(const TcPlan& two, const TcPlan& one) {
+  return two.passes >= 8 && two.passes * 100 <= one.passes * 104;
+}
+void tc_configure_two(int d, TcConfig* c);
+void tc_plan(int n, int V, int cta, int blocks, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan);
 cudaError_t tc_prepare();   // opt in to the kernels' dynamic shared memory size (once per device)
 cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const TcConfig& c, int workers,
                                  cudaStream_t stream);

@@ -118,6 +118,7 @@ void tc8_configure(int n, int d, TcConfig* c) {
   c->a_rows = 2 * part_rows;
   c->mode = part_rows <= 32 ? RowMode::k8Small : (part_rows <= 64 ? RowMode::k8Half : RowMode::k8Wide);
   c->part_rows = part_rows;
+  c->lag = 0;
   c->a_stages = sa;
   c->b_stages = sb;
   c->inline_split = inl ? 1 : 0;

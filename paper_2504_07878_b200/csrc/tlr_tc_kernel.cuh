@@ -14,6 +14,8 @@
 //               covers both parts along its M, and the epilogue adds the two accumulator rows of a
 //               token before it folds them; above, two MMAs per K step (one per part) add into the
 //               same rows.
+//               Above 256 rows a unit may be two blocks of 256 rows, one accumulator each: a slab of W is then read by
+//               the MMAs of both while it is in shared memory (TwoWalk).
 //   bf16 head whose hidden size is no multiple of 8: the vocabulary is walked by residue class
 //               (see OddMaps), otherwise like the bf16 head.
 //
@@ -116,7 +118,7 @@ __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, in
   const int vocab_units = p.chunks * p.row_units;
   if (unit >= vocab_units) {          // learned-router unit: all rows of W1 for one row unit
     u.chunk = -1;
-    u.row0 = ((unit - vocab_units) * kCta + cta_rank) * kBlockM;
+    u.row0 = ((unit - vocab_units) * p.blocks * kCta + cta_rank) * kBlockM;
     u.g0 = 0;
     u.G = 0;
     u.tile_q = u.tile_r = 0;
@@ -124,7 +126,7 @@ __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, in
   }
   u.chunk = static_cast<int>(static_cast<uint32_t>(unit) / static_cast<uint32_t>(p.row_units));
   const int ru = unit - u.chunk * p.row_units;
-  u.row0 = (ru * kCta + cta_rank) * kBlockM;
+  u.row0 = (ru * p.blocks * kCta + cta_rank) * kBlockM;
   int c = u.chunk;
   if (kOdd) {                         // class by class: the chunks of a class share its rows out
     u.cls = static_cast<int>(static_cast<uint32_t>(c) / static_cast<uint32_t>(p.class_chunks));
@@ -167,6 +169,24 @@ __host__ __device__ __forceinline__ Tile tile_of(const TcParams& p, const Unit& 
   r.rows = (gb - ga) * p.granule_rows;
   return r;
 }
+
+// Two row blocks to a unit (RowMode::kM128Two): the i-th of a tile's row-block slabs is slab `slab` of block `block`.  The
+// second block is `lag` slabs behind the first, so that either accumulator is folded while the other's MMAs run: there is no
+// third and fourth one.  A unit whose second block has no rows is walked like a single one.
+struct TwoWalk {
+  int blocks, items, lag, k_slabs;
+  __device__ __forceinline__ TwoWalk(const TcParams& p, int row0, int slabs) {
+    blocks = row0 + 2 * kBlockM < p.n ? 2 : 1;       // (row0 of the unit, whichever CTA asks)
+    items = blocks * slabs;
+    lag = blocks == 2 ? min(p.lag, slabs) : slabs;
+    k_slabs = slabs;
+  }
+  __device__ __forceinline__ void at(int i, int& block, int& slab) const {
+    const int j = i - lag;
+    block = j < 0 ? 0 : (i + lag >= items ? 1 : j & 1);
+    slab = j < 0 ? i : (i + lag >= items ? i - k_slabs : (j >> 1) + (block == 0 ? lag : 0));
+  }
+};
 
 // Running online-softmax summary of one token row over the vocabulary rows a thread has seen.
 // S = sum 2^y and T = sum 2^y * y with y = (z - m) * log2(e) <= 0; both are accumulated per
@@ -348,7 +368,8 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   constexpr bool kOdd = std::is_same<Maps, OddMaps>::value;   // d no multiple of 8: vocabulary rows by residue class
   constexpr bool kFp8 = kMode >= RowMode::k8Small, kGroup8 = kMode == RowMode::kGroup8;
   constexpr bool kKeep = kMode == RowMode::kM128Keep;      // the stage of a K slab is its number, filled once per unit
-  static_assert(kCta == 1 || kMode == RowMode::kM128 || kKeep, "modes of a pair of CTAs");
+  constexpr bool kTwo = kMode == RowMode::kM128Two;
+  static_assert(kCta == 1 || kMode == RowMode::kM128 || kKeep || kTwo, "modes of a pair of CTAs");
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment: the swizzle pattern is a function of the shared-memory address.
   // (The dynamic shared memory of both CTAs of a pair starts at the same offset, so the
@@ -376,7 +397,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   auto xch_full = [&](int q) { return bar_base + 8u * (kFixed + 4 + q); };
   auto xch_empty = [&](int q) { return bar_base + 8u * (kFixed + 8 + q); };
   const uint32_t h_ready = bar_base + 8u * (kFixed + 12);   // 8-bit head: h has been split in place (inline mode)
-  // kept h: the MMAs of the unit's last tile have read K slab s
+  // kept h: the MMAs of the unit's last tile have read K slab s; two row blocks: those of both have read W stage s
   auto h_free = [&](int s) { return bar_base + 8u * (kFixed + 13 + s); };
   constexpr int kNumBarriers = kFixed + 13 + kMaxAStages;
   static_assert(kNumBarriers * 8 + 16 <= kBarrierBytes, "barrier block too small");
@@ -399,6 +420,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   if (threadIdx.x == 0) {
     if (!inl) for (int s = 0; s < SA; ++s) mbar_init(a_full(s), 1);   // (inline mode: SA = K slabs, nothing streams)
     if (kKeep) for (int s = 0; s < SA; ++s) mbar_init(h_free(s), 1);
+    if (kTwo) for (int s = 0; s < SB; ++s) mbar_init(h_free(s), 1);
     for (int s = 0; s < SB; ++s) mbar_init(b_full(s), 1);
     for (int j = 0; j < kRelease; ++j) mbar_init(released(j), 1);
     for (int b = 0; b < 2; ++b) {
@@ -490,7 +512,9 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
           for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
             if (slab >= SB) {     // the stage is free once slab - SB has been consumed
               const int j = slab - SB;
-              if (!mbar_wait(released(j & (kRelease - 1)), (j / kRelease) & 1, abort_flag, p.status, ahead_ns)) { ok = false; break; }
+              const bool got = kTwo ? mbar_wait(h_free(stage), (j / SB) & 1, abort_flag, p.status, ahead_ns)
+                                    : mbar_wait(released(j & (kRelease - 1)), (j / kRelease) & 1, abort_flag, p.status, ahead_ns);
+              if (!got) { ok = false; break; }
             }
             const uint32_t dst = b_ring + stage * b_stage_bytes;
             const uint32_t bar = (kCta == 2) ? map_to_cta(b_full(stage), 0) : b_full(stage);
@@ -523,11 +547,15 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       uint32_t ord = 0;
       for (int unit = worker; unit < units && ok; unit += workers, ++ord) {
         const Unit un = unit_of<kCta, kOdd>(p, unit, cta_rank);
-        const int h_row = kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0);
+        const int h_row0 = kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0);
+        const TwoWalk two(p, un.row0 - static_cast<int>(cta_rank) * kBlockM, k_slabs);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
-          for (int ks = 0; ks < k_slabs; ++ks, ++slab) {
+          for (int i = 0; i < (kTwo ? two.items : k_slabs); ++i, ++slab) {
+            int ks = i, block = 0;
+            if (kTwo) two.at(i, block, ks);
+            const int h_row = h_row0 + block * (kCta * kBlockM);
             if (kKeep && t > 0) continue;      // (the first tile of a unit is never empty)
             if (!h_there) {
               // here and not with the other warps above: the arithmetic of the first unit would stand between the end of the
@@ -585,11 +613,58 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       // The barrier state of the next slab is polled before the current slab's MMAs are
       // issued, so the poll's latency overlaps the issue instead of adding to it.
       bool ra = inl || mbar_test_wait(a_full(0), 0), rb = mbar_test_wait(b_full(0), 0);
+      int sb_behind = 0;           // two row blocks: the W stage of the second's next slab
       for (int unit = worker; unit < units && ok; unit += workers) {
         const Unit un = unit_of<kCta, kOdd>(p, unit, 0);
+        const TwoWalk two(p, un.row0, k_slabs);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
+          if constexpr (kTwo) {
+            const uint32_t idesc = instr_desc(mma_m, tl.rows);
+            for (int i = 0; i < two.items; ++i, ++slab) {
+              int block, ks;
+              two.at(i, block, ks);
+              const int my_acc = acc ^ block;
+              if (ks == 0) {
+                ok = __all_sync(0xffffffffu, mbar_wait(acc_empty(my_acc), acc_phase ^ 1u ^ (acc & block), abort_flag, p.status, wait_ns));
+                if (!ok) break;
+              }
+              if (!__all_sync(0xffffffffu, ra && (block != 0 || rb))) {
+                const bool got = mbar_wait(a_full(sa), pa, abort_flag, p.status, wait_ns) &&
+                                 (block != 0 || mbar_wait(b_full(sb), pb, abort_flag, p.status, wait_ns));
+                ok = __all_sync(0xffffffffu, got);
+                if (!ok) break;
+              }
+              tc_fence_after();
+              const int w_stage = block == 0 ? sb : sb_behind;
+              const uint32_t a_lo = a_lo0 + sa * a_step;
+              const uint32_t b_lo = b_lo0 + w_stage * b_step;
+              if (++sa == SA) { sa = 0; pa ^= 1u; }
+              if (block == 0) {
+                if (++sb == SB) { sb = 0; pb ^= 1u; }
+              }
+              if (block + 1 == two.blocks) {
+                if (++sb_behind == SB) sb_behind = 0;
+              }
+              ra = mbar_test_wait(a_full(sa), pa);
+              rb = mbar_test_wait(b_full(sb), pb);
+              if (elect_one()) {
+                const uint32_t d_tmem = tmem_base + my_acc * kBlockN;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  umma_bf16<kCta>(d_tmem, desc_hi | (a_lo + 2u * k), desc_hi | (b_lo + 2u * k), idesc, (ks | k) != 0 ? 1u : 0u);
+                umma_commit<kCta>(released(slab & (kRelease - 1)));
+                if (block + 1 == two.blocks) umma_commit<kCta>(h_free(w_stage));
+                if (ks + 1 == k_slabs) umma_commit<kCta>(acc_full(my_acc));
+              }
+              __syncwarp();
+            }
+            if (!ok) break;
+            if (two.blocks == 2) acc_phase ^= 1u;
+            else if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            continue;
+          }
           const bool last_tile = kKeep && (t + 1 == T || tile_of(p, un, t + 1).rows == 0);
           const uint32_t idesc = kFp8 ? instr_desc_e4m3(mma_m, tl.rows) : instr_desc(mma_m, tl.rows);
           ok = __all_sync(0xffffffffu, mbar_wait(acc_empty(acc), acc_phase ^ 1u, abort_flag, p.status, wait_ns));
@@ -669,15 +744,25 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       }
       ok = __all_sync(0xffffffffu, ok);
     }
-    for (int unit = worker; unit < units && ok; unit += workers, ++ord) {
+    for (int unit = worker; unit < units && ok; unit += workers) {
       const Unit first = unit_of<kCta, kOdd>(p, unit, cta_rank);
-      const bool warp_has_rows = first.row0 + quad_row0 < p.n;            // warp-uniform
+      const int blocks = kTwo ? TwoWalk(p, first.row0 - static_cast<int>(cta_rank) * kBlockM, k_slabs).blocks : 1;
       const bool two_tokens = kFolds == 2 && quad_row0 + 8 < p.n;   // warp-uniform
       const bool mlp_unit = !kFp8 && first.chunk < 0;
-      RowFold<kOdd> f[kFolds];
+      RowFold<kOdd> f[kFolds], f_other;          // (f_other: of the other row block)
 #pragma unroll
       for (int i = 0; i < kFolds; ++i) f[i].reset();
-      float mlp_sum = 0.f;
+      f_other.reset();
+      float mlp_sum = 0.f, mlp_other = 0.f;
+      const auto swap_blocks = [&] {
+        if (!kTwo || blocks == 1) return;
+        const RowFold<kOdd> was = f[0];
+        const float sum_was = mlp_sum;
+        f[0] = f_other;
+        f_other = was;
+        mlp_sum = mlp_other;
+        mlp_other = sum_was;
+      };
       // The walk over the unit's tiles, compiled twice: once for vocabulary units (the hot loop, free of any
       // learned-router code) and once for learned-router units.
       auto walk_tiles = [&](auto router_tag) {
@@ -691,6 +776,17 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
         const int step = frag ? 64 : 32;
         const int half = min(cols, (tl.rows / 2 + step - 1) & ~(step - 1));
         const int c_begin = grp ? half : 0, c_end = grp ? cols : half;
+        for (int block = 0; block < blocks; ++block) {
+        const auto give_back = [&] {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            if (kCta == 1) mbar_arrive(acc_empty(acc));
+            else mbar_arrive_cluster(map_to_cta(acc_empty(acc), 0));   // the leader's barrier
+          }
+        };
+        bool given = false;
+        const bool warp_has_rows = first.row0 + block * (kCta * kBlockM) + quad_row0 < p.n;      // warp-uniform
         if (kFp8 && warp_has_rows) {
           // the share's weight scales, before the accumulator is waited for
           __syncwarp();
@@ -746,6 +842,10 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
               __syncwarp();                           // the load below is warp-collective
               tmem_ld32(taddr + c0, z);
               tmem_ld_wait();
+              if (kTwo && c0 + 32 >= c_end) {     // in front of the last fold: the MMAs of the next tile wait for it
+                give_back();
+                given = true;
+              }
               if (kFp8) {
 #pragma unroll
                 for (int j = 0; j < 32; j += 4) {
@@ -769,17 +869,15 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
             }
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          if (kCta == 1) mbar_arrive(acc_empty(acc));
-          else mbar_arrive_cluster(map_to_cta(acc_empty(acc), 0));   // the leader's barrier
-        }
+        if (!given) give_back();
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        swap_blocks();
+        }
       }
       };
       if (!kOdd && mlp_unit) walk_tiles(std::integral_constant<bool, !kOdd>{});
       else walk_tiles(std::false_type{});
+      for (int block = 0; block < blocks; ++block, ++ord) {
       Partial out[kFolds];
 #pragma unroll
       for (int i = 0; i < kFolds; ++i) out[i] = f[i].result();
@@ -820,14 +918,14 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
           if (lane == 0) mbar_arrive(xch_empty(quad));
 #pragma unroll
           for (int i = 0; i < kFolds; ++i) {
-            const int row = first.row0 + my_row + 8 * i;
+            const int row = first.row0 + block * (kCta * kBlockM) + my_row + 8 * i;
             if (!writer || row >= p.n || (i == 1 && !two_tokens)) continue;
             if (mlp_unit) p.mlp_out[row] = out[i].s + other[i].s;   // lower columns first: a fixed order
             else {
               Partial* dst = p.partials + static_cast<size_t>(row) * p.chunks + first.chunk;
               Partial sum = merge(out[i], other[i]);
               if (p.tag != 0) sum.idx = tagged_idx(sum.idx, p.tag);
-              if (kCta == 2 && unit + workers >= units) {     // (stored behind the arrival at the cluster's barrier)
+              if (kCta == 2 && unit + workers >= units && block + 1 == blocks) {     // (stored behind the arrival at the cluster's barrier)
                 last = sum;
                 last_dst = dst;
               } else {
@@ -836,6 +934,8 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
             }
           }
         }
+      }
+      swap_blocks();
       }
     }
   }

@@ -1,0 +1,61 @@
+"""Batches of more than 256 rows whose work units are two blocks of 256 token rows: the schedule on the CPU, results on the GPU."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2504_07878_b200 as P
+import tlr_synth as S
+from oracle import route_oracle as O
+
+from .parity import check_against_oracle, check_self_consistency
+
+
+@pytest.mark.parametrize("n,V,hidden", [(257, 300, 0), (512, 128256, 0), (777, 151936, 256), (1000, 17, 0), (2049, 60000, 40),
+                                        (4096, 151936, 1024), (16384, 128256, 0)])
+def test_tiles_of_both_blocks_cover_every_logit_once(n, V, hidden):
+    tiles, plan = P.tlr_debug_plan_tiles(n, V, 148, hidden, blocks=2)
+    g, vocab_units = plan.reserved, plan.vocab_chunks * plan.row_units
+    assert plan.row_units == -(-n // 512) and plan.vocab_chunks <= 192 and plan.grid <= 148
+    for ru in range(plan.row_units):
+        for router in (False, True) if hidden else (False,):
+            sel = tiles[(tiles[:, 2] == 512 * ru) & ((tiles[:, 1] >= vocab_units) == router)]
+            sel = sel[np.argsort(sel[:, 3])]
+            start, end = (V, V + -(-hidden // 32) * 32) if router else (0, -(-V // g) * g)
+            assert sel[0, 3] == start and sel[-1, 3] + sel[-1, 4] == end and np.all(sel[:, 4] <= 256)
+            assert np.array_equal(sel[1:, 3], (sel[:, 3] + sel[:, 4])[:-1])
+    for unit in np.unique(tiles[:, 1]):
+        assert len(np.unique(tiles[tiles[:, 1] == unit, 0])) == 1
+
+
+# One slab of K, two, as many as the second block is behind and more; second blocks of one row, of all rows and (25 blocks) of
+# none; several units per worker, empty tiles; with a learned router, whose tiles are the same walk.
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,d,V,hidden", [(257, 64, 67000, 0), (300, 320, 68000, 0), (512, 384, 67000, 300), (769, 640, 35000, 40),
+                                          (1000, 896, 36000, 0), (1500, 712, 24000, 64), (6200, 72, 5500, 0)])
+def test_two_blocks_match_the_oracle(n, d, V, hidden):
+    W = S.make_W(d, V, seed=n, std=0.08)
+    hid = S.make_h(n, d, seed=d, W=W, planted_fraction=0.1)
+    rows = np.unique(np.concatenate([np.arange(0, n, 11), np.arange(250, 262) % n, np.arange(max(0, n - 140), n)]))
+    ref = O.route_oracle(S.bf16_bits(hid.h)[rows], S.bf16_bits(W), 0.5)
+    r = P.Router(W.cuda(), max_n=n)
+    options = {}
+    if hidden:
+        gen = torch.Generator().manual_seed(hidden)
+        W1 = (torch.randn(hidden, d, generator=gen) / d ** 0.5).to(torch.bfloat16)
+        b1, w2 = torch.randn(hidden, generator=gen) * 0.1, torch.randn(hidden, generator=gen) * 0.2
+        r.set_router_mlp(W1.cuda(), b1.cuda(), w2.cuda(), 0.2)
+        options["mlp_score"] = torch.full((n,), float("nan"), device="cuda")
+    assert P.tlr_plan_query(r.ctx, n).reserved == 2
+    for _ in range(3):
+        r.route(hid.h.cuda(), 0.5, **options)
+    torch.cuda.synchronize()
+    assert P.tlr_last_device_status(r.ctx) == 0
+    names = ("token", "conf", "entropy", "route_mask", "routed_idx", "routed_count")
+    full = {k: getattr(r, k).cpu().numpy()[:n] for k in names}
+    full["routed_count"] = int(full["routed_count"][0])
+    check_self_consistency(full, 0.5, V)
+    check_against_oracle(ref, {k: full[k][rows] for k in names[:4]})
+    if hidden:
+        want = O.mlp_router_score(S.bf16_bits(hid.h), S.bf16_bits(W1), b1.numpy(), w2.numpy(), 0.2)
+        assert np.max(np.abs(options["mlp_score"].cpu().numpy() - want)) <= 1e-5     # fp32 sums of exact products
+    r.close()
