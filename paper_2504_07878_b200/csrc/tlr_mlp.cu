@@ -144,6 +144,15 @@ mlp_mma_kernel(const MlpLaunch a) {
   const unsigned short* W1 = static_cast<const unsigned short*>(a.W1);
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
   float acc[4][4] = {};
+  // Bound by the trips to memory, one per batch, that take about 3 us each beside the stream of W where they go to HBM: with few
+  // rows this kernel then ends behind the projection.  So the block's rows of W1 are asked for at once.  n = 2, d = 1712,
+  // V = 49399, 225 units 31.4 -> 26.8 us per step, n = 10, d = 896, V = 60000 17.6 -> 16.3, n = 40, d = 1024 there 20.6 both.
+  if (blockIdx.x == 0) {
+    const char* rows = reinterpret_cast<const char*>(W1 + static_cast<size_t>(unit0) * a.d);
+    const size_t bytes = static_cast<size_t>(min(kMlpUnits, a.d_hidden - unit0)) * a.d * 2;
+    for (size_t at = threadIdx.x * 128u; at < bytes; at += 32 * kMmaWarps * 128u)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(rows + at));
+  }
   // A thread's 16 bytes are eight consecutive k values; which k an MMA calls which does not matter as long as both
   // operands agree, so words 0, 1 go to one MMA (16 k values over the four threads) and words 2, 3 to the next.
   const int steps = (a.d + 31) / 32, s0 = steps * warp / kMmaWarps, s1 = steps * (warp + 1) / kMmaWarps;
