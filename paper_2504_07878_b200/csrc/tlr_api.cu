@@ -156,6 +156,7 @@ struct tlr_ctx {
   bool tagged_ok = true;                  // false once slots may have been left otherwise than pending (untag)
   uint32_t last_tag = 0;
   unsigned int* ticket = nullptr;
+  uint8_t* flag_bits = nullptr;           // a bit per row (finish_kernel)
   uint32_t* status = nullptr;
 
   // staging for tlr_route_host
@@ -431,7 +432,8 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
   const size_t partial_bytes = padded(np * tlr::kMaxChunks * sizeof(Partial));
   const size_t tagged_bytes = padded(std::min<size_t>(np * 32 * tlr::kRowsPerLane, tlr::kTaggedPartials) * sizeof(Partial));
   const size_t h_bytes = padded(np * d * 2), out_bytes = padded(np * 17 + 8), pinned_bytes = padded(np * 17 + 8 + 8);
-  bool ok = cudaMalloc(&c->workspace, 256 + partial_bytes + tagged_bytes + 2 * (h_bytes + out_bytes)) == cudaSuccess;
+  const size_t flag_bytes = padded((np + 31) / 32 * 4);
+  bool ok = cudaMalloc(&c->workspace, 256 + partial_bytes + tagged_bytes + flag_bytes + 2 * (h_bytes + out_bytes)) == cudaSuccess;
   ok = ok && cudaHostAlloc(reinterpret_cast<void**>(&c->out_pinned[0]), 2 * pinned_bytes, cudaHostAllocMapped) == cudaSuccess;
   if (ok) {
     unsigned char* at = c->workspace;
@@ -443,6 +445,8 @@ tlr_status new_context(int d, int V, const void* W_dev, int max_n, tlr_ctx** out
     at += tagged_bytes;
     c->partials = reinterpret_cast<Partial*>(at);
     at += partial_bytes;
+    c->flag_bits = at;
+    at += flag_bytes;
     for (int q = 0; q < 2; ++q) {
       c->h_stage[q] = at;
       c->out_stage[q] = at + h_bytes;
@@ -894,6 +898,7 @@ static tlr_status route_step(tlr_ctx* ctx, const void* h_bf16_dev, int32_t n, fl
   f.routed_idx = routed_idx_dev;
   f.routed_count = routed_count_dev;
   f.ticket = ctx->ticket;
+  f.flag_bits = ctx->flag_bits;
   f.status = ctx->status;
   if (plan.path == TLR_PATH_TC) f.ties = ties_of(ctx, h_bf16_dev);
   f.status_copy = status_copy;
@@ -952,6 +957,7 @@ tlr_status tlr_shard_finish(tlr_ctx* ctx, const void* summaries_dev, int32_t sha
   f.routed_idx = routed_idx_dev;
   f.routed_count = routed_count_dev;
   f.ticket = ctx->ticket;
+  f.flag_bits = ctx->flag_bits;
   f.status = ctx->status;
   if (tlr::launch_finish(f, stream) != cudaSuccess) return TLR_ERR_CUDA;
   return TLR_OK;
@@ -1094,6 +1100,7 @@ tlr_status tlr_shard_finish_fused(tlr_ctx* ctx, int32_t n, float tau, int32_t* t
   f.routed_idx = routed_idx_dev;
   f.routed_count = routed_count_dev;
   f.ticket = ctx->ticket;
+  f.flag_bits = ctx->flag_bits;
   f.status = ctx->status;
   if (tlr::launch_finish(f, stream) != cudaSuccess) return TLR_ERR_CUDA;
   return TLR_OK;

@@ -17,8 +17,8 @@
 //              SM beside a CTA of the tensor-core projection kernel, so
 //              the blocks are resident and waiting before that kernel ends, and the next
 //              call's CTAs do not have to wait for the merge to leave their SMs.
-//   larger n   many blocks of 8 warps; the block that finishes last (fence + ticket
-//              counter, no spinning) compacts the flags of all rows.
+//   larger n   many blocks of 8 warps, which leave their rows' flags as bits; the block that
+//              finishes last (fence + ticket counter, no spinning) compacts those of all rows.
 #include "tlr_common.cuh"
 #include "tlr_tc.cuh"
 
@@ -445,20 +445,30 @@ finish_kernel(const FinishLaunch a) {
   pdl_enter();
   wait_for_peers(a);
 
+  __shared__ int warp_flag[kFinishWarps];
+  int flag = 0;
   if (row < a.n) {
     const Partial* p = a.partials + static_cast<size_t>(row) * a.row_stride;
     float second;
     Partial acc = fold_row(p, a.chunks, a.chunk_stride, lane, kTies ? &second : nullptr);
     if constexpr (kTies)
       settle_row(a.ties, row, p, a.chunks, a.chunk_stride, second, acc.m, acc.idx, acc.s, acc.t, lane, 32);
-    if (lane == 0) store_row(decide_row(acc.s, acc.t, a, row), acc.idx, acc.s, acc.t, a, row);
+    if (lane == 0) {
+      const Scored r = decide_row(acc.s, acc.t, a, row);
+      store_row(r, acc.idx, acc.s, acc.t, a, row);
+      flag = r.flag;
+    }
   }
+  if (lane == 0) warp_flag[warp] = flag;
 
   // ---- which block is last?
   __shared__ int is_last;
-  __shared__ int warp_count[kFinishWarps];
   __syncthreads();
   if (threadIdx.x == 0) {
+    unsigned int bits = 0;
+#pragma unroll
+    for (int w = 0; w < kFinishWarps; ++w) bits |= static_cast<unsigned int>(warp_flag[w] != 0) << w;
+    a.flag_bits[blockIdx.x] = static_cast<uint8_t>(bits);      // row i: bit i % 8 of byte i / 8
     __threadfence();
     const unsigned int t = atomicAdd(a.ticket, 1u);
     is_last = (t == gridDim.x - 1) ? 1 : 0;
@@ -467,25 +477,55 @@ finish_kernel(const FinishLaunch a) {
   if (!is_last) return;
   __threadfence();
 
-  // ---- ordered compaction by the last block
+  // ---- ordered compaction by the last block, which everything behind it in the stream waits for.  The flags are bits: a thread
+  // has 64 rows, a pass 16384, and the second half of a pass writes word by word, a lane to a row.  (From the flag bytes of the
+  // output, 256 rows a pass with a trip to L2 and two barriers each, over PCIe where the outputs are in host memory: n = 2000,
+  // d = 256, V = 20000 33.4 us per step, so 31.2, n = 16384 there 228.5 and 211.5; n = 4000, d = 512, V = 30000 from and to host
+  // memory 241 and 218.)
   first_routed_init(a);
+  __shared__ unsigned int word_of[2 * kFinishThreads];
+  __shared__ int before_of[2 * kFinishThreads];
+  __shared__ int warp_count[kFinishWarps];
+  const int words = (a.n + 31) >> 5;
   int base_out = 0;
-  for (int base = 0; base < a.n; base += kFinishThreads) {
-    const int i = base + threadIdx.x;
-    const int flag = (i < a.n) ? (int)__ldcg(a.route_mask + i) : 0;
-    const unsigned int bal = __ballot_sync(0xffffffffu, flag != 0);
-    if (lane == 0) warp_count[warp] = __popc(bal);
+  for (int base = 0; base < words; base += 2 * kFinishThreads) {
+    unsigned int m[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int w = base + 2 * threadIdx.x + k;
+      m[k] = w < words ? __ldcg(reinterpret_cast<const unsigned int*>(a.flag_bits) + w) : 0u;
+      if (w == words - 1 && (a.n & 31) != 0) m[k] &= (1u << (a.n & 31)) - 1u;
+    }
+    const int mine = __popc(m[0]) + __popc(m[1]);
+    int upto = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, upto, off);
+      if (lane >= off) upto += v;
+    }
+    if (lane == 31) warp_count[warp] = upto;
     __syncthreads();
-    int before = 0, total = 0;
+    int before = upto - mine, total = 0;
 #pragma unroll
     for (int w = 0; w < kFinishWarps; ++w) {
       const int c = warp_count[w];
       before += (w < warp) ? c : 0;
       total += c;
     }
-    if (flag) {
-      a.routed_idx[base_out + before + __popc(bal & ((1u << lane) - 1u))] = i;
-      first_routed_note(a, i);
+    word_of[2 * threadIdx.x] = m[0];
+    word_of[2 * threadIdx.x + 1] = m[1];
+    before_of[2 * threadIdx.x] = base_out + before;
+    before_of[2 * threadIdx.x + 1] = base_out + before + __popc(m[0]);
+    __syncthreads();
+    const int here = min(words - base, 2 * kFinishThreads);
+#pragma unroll 4
+    for (int w = warp; w < here; w += kFinishWarps) {
+      const unsigned int word = word_of[w];
+      if ((word >> lane) & 1u) {
+        const int i = 32 * (base + w) + lane;
+        a.routed_idx[before_of[w] + __popc(word & ((1u << lane) - 1u))] = i;
+        first_routed_note(a, i);
+      }
     }
     base_out += total;
     __syncthreads();
@@ -546,6 +586,7 @@ bool merges_tagged(int n, int chunks, bool small) {
 }
 
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
+  if (a.n > kSmallRows && a.flag_bits == nullptr) return cudaErrorInvalidValue;
   if (a.chunks > 32 * kPerLane || (a.tag != 0 && !merges_tagged(a.n, a.chunks, a.small_blocks))) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.dynamicSmemBytes = 0;
