@@ -313,7 +313,7 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
       if (cfg.mode == tlr::RowMode::kM128 && c->classes == 1 && tlr::tc_two_blocks(n, c->d)) {
         tlr::TcPlan two;
         tlr::tc_plan(n, c->V, 2, 2, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, 1, &two);
-        if (tlr::tc_two_blocks_pay(two, tp)) {
+        if (tlr::tc_two_blocks_pay(two, tp, c->d)) {
           tp = two;
           tlr::tc_configure_two(c->d, &cfg);
         }

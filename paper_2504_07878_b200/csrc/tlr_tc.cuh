@@ -132,11 +132,15 @@ void tc_configure(int n, int d, int V, int sm_count, TcConfig* c);
 inline bool tc_two_blocks(int n, int d) {
   return n > 256 && 2ll * n * d <= (50ll << 20);
 }
-// ... and whether they pay, given both plans (an odd block is a unit and counts for two, which is little among many): few units may leave the busiest worker more passes than single blocks would, of which
-// up to 4 % are given back (n = 1000, d = 896, V = 151936: 34 instead of 33, 232.5 and 229.6 us), and short walks gain nothing,
-// having their first and last slabs longer (n = 400, d = 1024, V = 30000, four passes: 29.8 and 32.0).
-inline bool tc_two_blocks_pay(const TcPlan& two, const TcPlan& one) {
-  return two.passes >= 8 && two.passes * 100 <= one.passes * 104;
+// ... and whether they pay, given both plans.  Few units may leave the busiest worker more passes than single blocks would, of
+// which up to 4 % are given back (n = 1000, d = 896, V = 151936: 34 instead of 33, 232.5 and 229.6 us; an odd block is a unit and
+// counts for two, which is little among many).  Short walks have their first and last slabs longer, all the more the fewer slabs a
+// pass has: single blocks and two, n = 1000, d = 256, V = 36000 (8 passes of 4 slabs) 26.2 and 28.8 us, n = 400, d = 1024,
+// V = 30000 (4 of 16) 29.8 and 32.0, n = 1000, d = 640, V = 36000 (8 of 10) 39.5 and 40.9 in a short run, 46.2 and 45.9 in a long
+// one, d = 1024 there (8 of 16) 60.9 and 59.9, n = 4096, d = 640, V = 18944 (16 of 10) 79.5 and 77.9.
+inline bool tc_two_blocks_pay(const TcPlan& two, const TcPlan& one, int d) {
+  const int k_slabs = (d + 63) / 64;
+  return k_slabs >= 8 && two.passes * k_slabs >= 128 && two.passes * 100 <= one.passes * 104;
 }
 void tc_configure_two(int d, TcConfig* c);
 void tc_plan(int n, int V, int cta, int blocks, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan);

@@ -27,11 +27,11 @@ def test_tiles_of_both_blocks_cover_every_logit_once(n, V, hidden):
         assert len(np.unique(tiles[tiles[:, 1] == unit, 0])) == 1
 
 
-# One slab of K, two, as many as the second block is behind and more; second blocks of one row, of all rows and (25 blocks) of
-# none; several units per worker, empty tiles; with a learned router, whose tiles are the same walk.
+# The fewest slabs of K and more, in part; second blocks of one row, of all rows and (25 blocks) of none; several units per worker;
+# with a learned router, whose tiles are the same walk.
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,d,V,hidden", [(257, 64, 67000, 0), (300, 320, 68000, 0), (512, 384, 67000, 300), (769, 640, 35000, 40),
-                                          (1000, 896, 36000, 0), (1500, 712, 24000, 64), (6200, 72, 5500, 0)])
+@pytest.mark.parametrize("n,d,V,hidden", [(257, 1024, 67000, 0), (300, 712, 105000, 0), (769, 584, 61000, 40), (1000, 896, 43000, 0),
+                                          (1500, 712, 35000, 300), (6200, 584, 11500, 0)])
 def test_two_blocks_match_the_oracle(n, d, V, hidden):
     W = S.make_W(d, V, seed=n, std=0.08)
     hid = S.make_h(n, d, seed=d, W=W, planted_fraction=0.1)
