@@ -463,7 +463,7 @@ struct FinishLaunch {
   int32_t* routed_idx;
   int32_t* routed_count;
   unsigned int* ticket;     // zero before the launch; the kernel leaves it zero again
-  uint8_t* flag_bits;       // n > 1024: the rows' flags, ceil(n / 32) words
+  uint8_t* flag_bits;       // the rows' flags, ceil(n / 32) words (finish_kernel)
   uint32_t* status;
   Ties ties;
   uint32_t* status_copy;    // optional: receives the status word once every row is scored (host-mapped memory)

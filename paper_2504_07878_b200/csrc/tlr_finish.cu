@@ -12,8 +12,8 @@
 //              per row, all rows at once) and sends the route flags to block 0, which compacts
 //              them.  No ticket, no second launch, one L2 round trip for the partials.
 //              finish_rows_kernel where a lane owns at most 5 partials: the compaction has a warp
-//              of its own.  Otherwise finish_small_kernel, 512 threads where a lane group still owns
-//              at most 6 partials (else 1024).  Blocks of 17 or 9 warps, and of 512 threads, fit on an
+//              of its own.  Otherwise finish_small_kernel, 512 threads where a lane still owns
+//              at most 6 partials (else 1024, and where that is not enough, the kernel for larger n).  Blocks of 17 or 9 warps, and of 512 threads, fit on an
 //              SM beside a CTA of the tensor-core projection kernel, so
 //              the blocks are resident and waiting before that kernel ends, and the next
 //              call's CTAs do not have to wait for the merge to leave their SMs.
@@ -180,9 +180,9 @@ __device__ __forceinline__ void outlive_senders() {
 constexpr int kNoList = -2 * kSmallRows;      // a warp's count after a time-out: the sum is below zero with it
 
 // Cluster of gridDim.x blocks, n <= 1024.  A group of L lanes (L a power of two) folds one
-// row in two passes over its partials: maximum and index first, then the sums rescaled to
-// that maximum.  L is chosen on the host so that every row has its group: n * L <=
-// gridDim.x * 1024.
+// row: maximum and index first, then the sums rescaled to
+// that maximum.  L is chosen on the host so that every row has its group, n * L <=
+// gridDim.x * 1024, and a lane at most kPerLane partials.
 template <bool kTies>
 __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int log2_L) {
   __shared__ int warp_count[kSmallThreads / 32];
@@ -191,7 +191,6 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
   const int L = 1 << log2_L;
   const int group = (blockIdx.x * blockDim.x + threadIdx.x) >> log2_L;
   const int gl = threadIdx.x & (L - 1);
-  const bool one_pass = ((a.chunks + L - 1) >> log2_L) <= kPerLane;
   // Every warp of the cluster sends the flags of its 32 / L rows -- bit r * L for its row r -- as one word to block 0,
   // which waits for all words on a barrier of its own.  (st.async delivers the word and its arrival in one trip: n = 64, d = 512, V = 32000 11.90 us per step; flag
   // bytes in distributed shared memory with a cluster barrier behind them 12.96; n = 256 14.61 and 15.55.)
@@ -218,8 +217,8 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
     float m = -INFINITY;
     int idx = kNoToken;
     float s = 0.f, t = 0.f, second = -INFINITY;
-    if (one_pass) {
-      // few partials per lane: one pass, the partials stay in registers
+    {
+      // one pass, the partials stay in registers
       Partial q[kPerLane];
 #pragma unroll
       for (int k = 0; k < kPerLane; ++k) {
@@ -255,38 +254,6 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
           t += e * (q[k].t + dm * q[k].s);
         }
         if constexpr (kTies) second = q[k].m < m ? fmaxf(second, q[k].m) : second;
-      }
-    } else {
-      // many partials per lane: maximum and index first, then the rescaled sums
-      if (valid) {
-        for (int j = gl; j < a.chunks; j += L) {
-          const float2 mi = __ldcg(reinterpret_cast<const float2*>(p + j * cs));
-          const int qi = __float_as_int(mi.y);
-          if (mi.x > m || (mi.x == m && qi < idx)) {
-            m = mi.x;
-            idx = qi;
-          }
-        }
-      }
-      for (int off = L >> 1; off > 0; off >>= 1) {
-        const float om = __shfl_xor_sync(0xffffffffu, m, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
-        if (om > m || (om == m && oi < idx)) {
-          m = om;
-          idx = oi;
-        }
-      }
-      if (valid) {
-        for (int j = gl; j < a.chunks; j += L) {
-          const float4 raw = __ldcg(reinterpret_cast<const float4*>(p + j * cs));
-          if (!(raw.z == 0.f)) {
-            const float dm = raw.x - m;
-            const float e = exp2f(dm * kLog2e);
-            s += raw.z * e;
-            t += e * (raw.w + dm * raw.z);
-          }
-          if constexpr (kTies) second = raw.x < m ? fmaxf(second, raw.x) : second;
-        }
       }
     }
     for (int off = L >> 1; off > 0; off >>= 1) {
@@ -481,7 +448,8 @@ finish_kernel(const FinishLaunch a) {
   // has 64 rows, a pass 16384, and the second half of a pass writes word by word, a lane to a row.  (From the flag bytes of the
   // output, 256 rows a pass with a trip to L2 and two barriers each, over PCIe where the outputs are in host memory: n = 2000,
   // d = 256, V = 20000 33.4 us per step, so 31.2, n = 16384 there 228.5 and 211.5; n = 4000, d = 512, V = 30000 from and to host
-  // memory 241 and 218.)
+  // memory 241 and 218.  Words through shuffles instead of shared memory, so that these blocks stand beside the projection's
+  // CTAs: n = 2000 31.5 and 32.8.)
   first_routed_init(a);
   __shared__ unsigned int word_of[2 * kFinishThreads];
   __shared__ int before_of[2 * kFinishThreads];
@@ -541,7 +509,7 @@ namespace {
 
 // The launch of the small merge kernel for n <= kSmallRows rows.
 struct SmallShape {
-  int blocks, threads, lanes;
+  int blocks, threads, lanes;      // lanes: 0 where a lane would own more than kPerLane partials
 };
 SmallShape small_shape(int n, int chunks) {
   SmallShape s;
@@ -560,6 +528,10 @@ SmallShape small_shape(int n, int chunks) {
   const int e = tuning().finish_threads;   // tuning switch (TLR_FINISH_THREADS)
   if (e == 256 || e == 512 || e == 1024) s.threads = e;
   s.lanes = lanes_for(s.threads);
+  // Eight blocks that walk a row's partials twice take 12 us, many blocks with a warp to a row 6: n = 640, d = 256, V = 18944
+  // (49 partials, eight lanes) 21.8 and 17.3 us per step.  With at most kPerLane to a lane the eight blocks are the faster ones:
+  // V = 60000 there (37 partials) 30.9 and 32.5.
+  if ((chunks + s.lanes - 1) / s.lanes > kPerLane) s.lanes = 0;
   return s;
 }
 
@@ -586,7 +558,6 @@ bool merges_tagged(int n, int chunks, bool small) {
 }
 
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
-  if (a.n > kSmallRows && a.flag_bits == nullptr) return cudaErrorInvalidValue;
   if (a.chunks > 32 * kPerLane || (a.tag != 0 && !merges_tagged(a.n, a.chunks, a.small_blocks))) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.dynamicSmemBytes = 0;
@@ -596,21 +567,23 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (a.n <= kSmallRows) {
-    int blocks, threads, lanes, row_warps;
-    const bool ties = a.ties.W != nullptr;
-    auto kernel = ties ? finish_small_ties_kernel : finish_small_kernel;
-    if (rows_shape(a.n, a.chunks, a.small_blocks, &row_warps, &blocks, &lanes)) {
-      threads = (row_warps + 1) * 32;
-      if (ties) kernel = a.tag != 0 ? finish_rows_kernel<true, true, 8> : finish_rows_kernel<true, false, 8>;
-      else if (row_warps == 8) kernel = a.tag != 0 ? finish_rows_kernel<false, true, 8> : finish_rows_kernel<false, false, 8>;
-      else kernel = a.tag != 0 ? finish_rows_kernel<false, true, 16> : finish_rows_kernel<false, false, 16>;
-    } else {
-      const SmallShape s = small_shape(a.n, a.chunks);
-      blocks = s.blocks;
-      threads = s.threads;
-      lanes = s.lanes;
-    }
+  int blocks = 0, threads = 0, lanes = 0, row_warps;
+  const bool ties = a.ties.W != nullptr;
+  auto kernel = ties ? finish_small_ties_kernel : finish_small_kernel;
+  if (rows_shape(a.n, a.chunks, a.small_blocks, &row_warps, &blocks, &lanes)) {
+    threads = (row_warps + 1) * 32;
+    if (ties) kernel = a.tag != 0 ? finish_rows_kernel<true, true, 8> : finish_rows_kernel<true, false, 8>;
+    else if (row_warps == 8) kernel = a.tag != 0 ? finish_rows_kernel<false, true, 8> : finish_rows_kernel<false, false, 8>;
+    else kernel = a.tag != 0 ? finish_rows_kernel<false, true, 16> : finish_rows_kernel<false, false, 16>;
+  } else if (a.n <= kSmallRows) {
+    const SmallShape s = small_shape(a.n, a.chunks);
+    blocks = s.blocks;
+    threads = s.threads;
+    lanes = s.lanes;
+  } else {
+    lanes = 0;
+  }
+  if (lanes > 0) {
     int log2_L = 0;
     while ((1 << log2_L) < lanes) ++log2_L;
     attr[1].id = cudaLaunchAttributeClusterDimension;
@@ -622,10 +595,10 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
     return cudaLaunchKernelEx(&cfg, kernel, a, log2_L);
   }
-  const int blocks = (a.n + kFinishWarps - 1) / kFinishWarps;
-  cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
+  if (a.flag_bits == nullptr) return cudaErrorInvalidValue;
+  cfg.gridDim = dim3(static_cast<unsigned>((a.n + kFinishWarps - 1) / kFinishWarps), 1, 1);
   cfg.blockDim = dim3(kFinishThreads, 1, 1);
-  return cudaLaunchKernelEx(&cfg, a.ties.W != nullptr ? finish_kernel<true> : finish_kernel<false>, a);
+  return cudaLaunchKernelEx(&cfg, ties ? finish_kernel<true> : finish_kernel<false>, a);
 }
 
 }  // namespace tlr

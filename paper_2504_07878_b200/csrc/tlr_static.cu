@@ -31,6 +31,8 @@ constexpr int kStaticMaxChunks = 192;
 constexpr size_t kPartialBytes = static_cast<size_t>(kStaticMaxRows) * kStaticMaxChunks * sizeof(tlr::Partial);
 constexpr size_t kTicketOffset = kPartialBytes;        // unsigned int
 constexpr size_t kStatusOffset = kPartialBytes + 64;   // uint32_t, used when the caller passes no status word
+constexpr size_t kFlagOffset = kPartialBytes + 128;    // a bit per row
+static_assert(kStaticMaxRows <= 8 * 128, "flag bits");
 constexpr size_t kScratchBytes = kPartialBytes + 256;
 
 // The scratch itself.  In host code this name is only a handle for the runtime's symbol
@@ -207,6 +209,7 @@ extern "C" tlr_status tlr_route_static(int32_t d, int32_t V, const void* W_bf16_
   f.routed_idx = routed_idx_dev;
   f.routed_count = routed_count_dev;
   f.ticket = ticket;
+  f.flag_bits = s->scratch + kFlagOffset;
   f.status = status;
   if (tlr::launch_finish(f, stream) != cudaSuccess) return TLR_ERR_CUDA;
   return TLR_OK;

@@ -34,3 +34,22 @@ def test_list_of_large_batches(n):
     below = (conf < np.float32(tau)).reshape(n // L, L)
     assert np.array_equal(first.cpu().numpy(), np.where(below.any(axis=1), below.argmax(axis=1), L))
     r.close()
+
+
+# More partials per row than the lanes of eight blocks can keep: many blocks, as above 1024 rows.  (d = 96, V = 18944: 49 per row.)
+@pytest.mark.parametrize("n", [600, 639, 768])
+def test_middle_batches_of_many_partials(n):
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    W = (torch.randn((18944, 96), generator=gen, device="cuda") * 0.2).to(torch.bfloat16)
+    h = torch.randn((n, 96), generator=gen, device="cuda").to(torch.bfloat16)
+    r = P.Router(W, max_n=n)
+    assert P.tlr_plan_query(r.ctx, n).vocab_chunks > 48
+    for tau in (0.02, 2.0, 0.0, 0.02):
+        _, conf, _, mask, idx, count = r.route(h, tau)
+        z = h.double() @ W.double().T
+        want = torch.softmax(z, dim=1).amax(dim=1)
+        assert torch.all((conf - want).abs() <= 2e-5 * want)      # (fp32 sums of exact products, see the parity tests)
+        flags = (conf < tau).cpu().numpy()
+        assert np.array_equal(mask.cpu().numpy() != 0, flags)
+        assert int(count.item()) == flags.sum() and np.array_equal(idx.cpu().numpy()[:flags.sum()], np.flatnonzero(flags))
+    r.close()
