@@ -103,6 +103,7 @@ void tc_plan(int n, int V, int cta, int blocks, int workers, int max_chunks, int
     }
   }
   plan->blocks = blocks;
+  plan->group_units = row_units;
   plan->passes = best_passes * blocks;
   plan->row_units = row_units;
   plan->classes = classes;
@@ -310,11 +311,12 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
       tlr::tc_configure(rows, c->d + (c->classes > 1 ? tlr::odd_max_shift(c->d) : 0), c->V, c->sm_count, &cfg);
       workers_max = c->sm_count / cfg.cta;
       tlr::tc_plan(rows, c->V, cfg.cta, 1, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, c->classes, &tp);
-      if (cfg.mode == tlr::RowMode::kM128 && c->classes == 1 && tlr::tc_two_blocks(n, c->d)) {
+      if (cfg.mode == tlr::RowMode::kM128 && c->classes == 1 && n > 256) {
         tlr::TcPlan two;
         tlr::tc_plan(n, c->V, 2, 2, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, 1, &two);
         if (tlr::tc_two_blocks_pay(two, tp, c->d)) {
           tp = two;
+          tp.group_units = tlr::tc_two_group(n, c->d, tp.row_units);
           tlr::tc_configure_two(c->d, &cfg);
         }
       }

@@ -36,6 +36,7 @@ struct TcConfig {
 // Work decomposition for a given (n, V) on `workers` workers (see tc_plan).
 struct TcPlan {
   int blocks;          // row blocks of 128 * cta rows in a unit (2: RowMode::kM128Two)
+  int group_units;     // row units of a group (blocks == 2)
   int row_units;       // ceil(n / (128 * cta * blocks))
   int classes;         // residue classes of the vocabulary (1 unless d is odd-sized, see OddMaps)
   int chunks;          // vocabulary chunks == partials per row; a multiple of `classes`
@@ -52,7 +53,8 @@ struct TcParams {
   int n, d, V;
   int row_units, chunks, tiles_per_unit, full_tiles_first, granule_rows;
   int blocks;                         // row blocks of a unit
-  int lag;                            // two of them: how many slabs of a tile the second is behind the first
+  int group_units;                    // two of them: row units of a group (all groups but the last)
+  int lag;                            // ... and how many slabs of a tile the second is behind the first
   int chunk_q, chunk_r;               // granules of a chunk: chunk_q, and one more in chunk_r of them (of a class)
   uint32_t chunk_mul;                 // ceil(2^32 / chunks of a class), 0 for one chunk
   int full_granules;                  // granules of a full tile
@@ -109,6 +111,7 @@ inline int tc_h_box_rows(const TcConfig& c) { return c.mode == RowMode::kGroup8 
 // The fields of a launch's parameters that describe its work decomposition.
 inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
   p->blocks = plan.blocks;
+  p->group_units = plan.group_units;
   p->row_units = plan.row_units;
   p->chunks = plan.chunks;
   p->tiles_per_unit = plan.tiles_per_unit;
@@ -125,14 +128,18 @@ inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
 int tc_threads();
 int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
 void tc_configure(int n, int d, int V, int sm_count, TcConfig* c);
-// Whether a batch of n rows may be walked in units of two row blocks (256 rows each): not where
-// h is large against L2 (126 MB, in two halves): single blocks and two, ms per step, d = 2048 and n = 8192 (34 MB), V = 60000
-// 1.549 and 1.453, n = 12000 (49 MB) 2.209 and 2.175, n = 14000 (57 MB), V = 100000 4.377 and 4.387, n = 16384 (67 MB),
-// V = 128256 6.518 and 6.573; d = 1536 and n = 16384 (50 MB), V = 60000 2.281 and 2.191.
-inline bool tc_two_blocks(int n, int d) {
-  return n > 256 && 2ll * n * d <= (50ll << 20);
+// Units of two row blocks are walked group by group of row units, so many to a group that their h takes up to 50 MB.  There are
+// more workers than row units then, several read the same h from either half of L2 (126 MB), which keep a copy each, and two copies
+// must fit beside W.  W comes from HBM once more per group, which is little.  ms per step at d = 2048 with single blocks (each
+// row unit's h is read by one worker there), with one group, with groups of up to 50 and of up to 34 MB: n = 16384, V = 128256
+// 6.32, 6.35, 5.99 and 5.99, n = 14000, V = 100000 4.21, 4.21, 4.05 and 4.06; at 50 MB one group is as good as two (n = 12000,
+// V = 60000 2.17, 2.11 and 2.10; d = 1536, n = 16384 there 2.24, 2.13 and 2.14).
+inline int tc_two_group(int n, int d, int row_units) {
+  constexpr long long kGroupBytes = 50ll << 20;
+  const long long groups = (2ll * n * d + kGroupBytes - 1) / kGroupBytes;
+  return static_cast<int>((row_units + groups - 1) / groups);
 }
-// ... and whether they pay, given both plans.  Few units may leave the busiest worker more passes than single blocks would, of
+// Whether units of two row blocks pay, given both plans.  Few units may leave the busiest worker more passes than single blocks would, of
 // which up to 4 % are given back (n = 1000, d = 896, V = 151936: 34 instead of 33, 232.5 and 229.6 us; an odd block is a unit and
 // counts for two, which is little among many).  Short walks have their first and last slabs longer, all the more the fewer slabs a
 // pass has: single blocks and two, n = 1000, d = 256, V = 36000 (8 passes of 4 slabs) 26.2 and 28.8 us, n = 400, d = 1024,

@@ -110,7 +110,7 @@ struct Tile {
 // cheap: no division per tile, two 32-bit ones per unit.  With 64-bit ones here and one per tile this function took 720
 // cycles of the 2020 between a unit's last slab and the next one's first (now 260 of 1340), a tile 1150 (now 1025):
 // prefill at n = 8192, d = 896 1743 -> 1713 us, n = 2000, d = 1024, V = 100000 341 -> 329, n = 1, d = 256 8.64 -> 8.45.
-template <int kCta, bool kOdd = false>
+template <int kCta, bool kOdd = false, bool kTwo = false>
 __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, int cta_rank) {
   Unit u;
   u.cls = 0;
@@ -124,8 +124,13 @@ __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, in
     u.tile_q = u.tile_r = 0;
     return u;
   }
-  u.chunk = static_cast<int>(static_cast<uint32_t>(unit) / static_cast<uint32_t>(p.row_units));
-  const int ru = unit - u.chunk * p.row_units;
+  // (two row blocks: group by group of row units, and in a group chunk by chunk, see tc_two_group)
+  const int group = kTwo ? static_cast<int>(static_cast<uint32_t>(unit) / static_cast<uint32_t>(p.chunks * p.group_units)) : 0;
+  const int ru0 = kTwo ? group * p.group_units : 0;
+  const int group_rows = kTwo ? (p.row_units - ru0 < p.group_units ? p.row_units - ru0 : p.group_units) : p.row_units;
+  const int at = unit - p.chunks * ru0;
+  u.chunk = static_cast<int>(static_cast<uint32_t>(at) / static_cast<uint32_t>(group_rows));
+  const int ru = ru0 + at - u.chunk * group_rows;
   u.row0 = (ru * p.blocks * kCta + cta_rank) * kBlockM;
   int c = u.chunk;
   if (kOdd) {                         // class by class: the chunks of a class share its rows out
@@ -494,7 +499,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       int slab = 0;     // running slab number, the same in every role
       bool ok = true;
       for (int unit = worker; unit < units && ok; unit += workers) {
-        const Unit un = unit_of<kCta, kOdd>(p, unit, cta_rank);
+        const Unit un = unit_of<kCta, kOdd, kTwo>(p, unit, cta_rank);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
           if (tl.rows == 0) continue;
@@ -546,7 +551,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       bool h_there = false;
       uint32_t ord = 0;
       for (int unit = worker; unit < units && ok; unit += workers, ++ord) {
-        const Unit un = unit_of<kCta, kOdd>(p, unit, cta_rank);
+        const Unit un = unit_of<kCta, kOdd, kTwo>(p, unit, cta_rank);
         const int h_row0 = kFp8 ? 0 : un.row0 + (kOdd ? un.cls * p.h_class_rows : 0);
         const TwoWalk two(p, un.row0 - static_cast<int>(cta_rank) * kBlockM, k_slabs);
         for (int t = 0; t < T && ok; ++t) {
@@ -615,7 +620,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       bool ra = inl || mbar_test_wait(a_full(0), 0), rb = mbar_test_wait(b_full(0), 0);
       int sb_behind = 0;           // two row blocks: the W stage of the second's next slab
       for (int unit = worker; unit < units && ok; unit += workers) {
-        const Unit un = unit_of<kCta, kOdd>(p, unit, 0);
+        const Unit un = unit_of<kCta, kOdd, kTwo>(p, unit, 0);
         const TwoWalk two(p, un.row0, k_slabs);
         for (int t = 0; t < T && ok; ++t) {
           const Tile tl = tile_of(p, un, t);
@@ -745,7 +750,7 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
       ok = __all_sync(0xffffffffu, ok);
     }
     for (int unit = worker; unit < units && ok; unit += workers) {
-      const Unit first = unit_of<kCta, kOdd>(p, unit, cta_rank);
+      const Unit first = unit_of<kCta, kOdd, kTwo>(p, unit, cta_rank);
       const int blocks = kTwo ? TwoWalk(p, first.row0 - static_cast<int>(cta_rank) * kBlockM, k_slabs).blocks : 1;
       const bool two_tokens = kFolds == 2 && quad_row0 + 8 < p.n;   // warp-uniform
       const bool mlp_unit = !kFp8 && first.chunk < 0;
