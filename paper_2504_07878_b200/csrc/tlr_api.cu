@@ -622,7 +622,7 @@ static tlr_status plan_tiles(int blocks, int32_t n, int32_t V, int32_t sm_count,
   p.V = V;
   tlr::tc_set_schedule(tp, &p);
   p.mlp_hidden = tp.mlp_rows > 0 ? mlp_hidden : 0;
-  *count = tlr::tc_enumerate_tiles(p, cfg.cta, workers, out, capacity);
+  *count = tlr::tc_enumerate_tiles(p, cfg.cta, blocks, workers, out, capacity);
   if (plan_out != nullptr) {
     plan_out->path = TLR_PATH_TC;
     plan_out->grid = workers * cfg.cta;

@@ -558,7 +558,7 @@ bool merges_tagged(int n, int chunks, bool small) {
 }
 
 cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
-  if (a.chunks > 32 * kPerLane || (a.tag != 0 && !merges_tagged(a.n, a.chunks, a.small_blocks))) return cudaErrorInvalidValue;
+  if (a.chunks > 32 * kPerLane) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.dynamicSmemBytes = 0;
   cfg.stream = stream;
@@ -575,6 +575,8 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     if (ties) kernel = a.tag != 0 ? finish_rows_kernel<true, true, 8> : finish_rows_kernel<true, false, 8>;
     else if (row_warps == 8) kernel = a.tag != 0 ? finish_rows_kernel<false, true, 8> : finish_rows_kernel<false, false, 8>;
     else kernel = a.tag != 0 ? finish_rows_kernel<false, true, 16> : finish_rows_kernel<false, false, 16>;
+  } else if (a.tag != 0) {          // (tagged partials are rows_shape's only, see merges_tagged)
+    return cudaErrorInvalidValue;
   } else if (a.n <= kSmallRows) {
     const SmallShape s = small_shape(a.n, a.chunks);
     blocks = s.blocks;

@@ -15,12 +15,12 @@ int tc_threads() { return kThreads; }
 // Host enumeration of the schedule the kernel walks (the same tile_of the device code uses):
 // one record {worker, unit, row0, v0, rows} per non-empty tile of CTA rank 0, in walking order.
 // Tiles of learned-router units are reported with v0 counted from V upwards.
-int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity) {
+int tc_enumerate_tiles(const TcParams& p, int cta, int blocks, int workers, int* out, int capacity) {
   int count = 0;
   const int units = (p.chunks + (p.mlp_hidden > 0 ? 1 : 0)) * p.row_units;
   for (int w = 0; w < workers; ++w) {
     for (int unit = w; unit < units; unit += workers) {
-      const Unit un = p.blocks == 2 ? unit_of<2, false, true>(p, unit, 0) : cta == 2 ? unit_of<2>(p, unit, 0) : unit_of<1>(p, unit, 0);
+      const Unit un = blocks == 2 ? unit_of<2, false, true>(p, unit, 0) : cta == 2 ? unit_of<2>(p, unit, 0) : unit_of<1>(p, unit, 0);
       for (int t = 0; t < p.tiles_per_unit; ++t) {
         const Tile tl = tile_of(p, un, t);
         if (tl.rows == 0) continue;

@@ -52,8 +52,7 @@ struct TcPlan {
 struct TcParams {
   int n, d, V;
   int row_units, chunks, tiles_per_unit, full_tiles_first, granule_rows;
-  int blocks;                         // row blocks of a unit
-  int group_units;                    // two of them: row units of a group (all groups but the last)
+  int group_units;                    // two row blocks to a unit: row units of a group (all groups but the last)
   int lag;                            // ... and how many slabs of a tile the second is behind the first
   int chunk_q, chunk_r;               // granules of a chunk: chunk_q, and one more in chunk_r of them (of a class)
   uint32_t chunk_mul;                 // ceil(2^32 / chunks of a class), 0 for one chunk
@@ -110,7 +109,6 @@ cudaError_t launch_odd_projection(const OddMaps& maps, const TcParams& p, const 
 inline int tc_h_box_rows(const TcConfig& c) { return c.mode == RowMode::kGroup8 ? 8 : c.a_rows; }   // rows of h per TMA box
 // The fields of a launch's parameters that describe its work decomposition.
 inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
-  p->blocks = plan.blocks;
   p->group_units = plan.group_units;
   p->row_units = plan.row_units;
   p->chunks = plan.chunks;
@@ -126,7 +124,7 @@ inline void tc_set_schedule(const TcPlan& plan, TcParams* p) {
   p->full_granules = 256 / plan.granule_rows;
 }
 int tc_threads();
-int tc_enumerate_tiles(const TcParams& p, int cta, int workers, int* out, int capacity);
+int tc_enumerate_tiles(const TcParams& p, int cta, int blocks, int workers, int* out, int capacity);
 void tc_configure(int n, int d, int V, int sm_count, TcConfig* c);
 // Units of two row blocks are walked group by group of row units, so many to a group that their h takes up to 50 MB.  There are
 // more workers than row units then, several read the same h from either half of L2 (126 MB), which keep a copy each, and two copies

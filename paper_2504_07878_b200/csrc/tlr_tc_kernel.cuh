@@ -118,7 +118,7 @@ __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, in
   const int vocab_units = p.chunks * p.row_units;
   if (unit >= vocab_units) {          // learned-router unit: all rows of W1 for one row unit
     u.chunk = -1;
-    u.row0 = ((unit - vocab_units) * p.blocks * kCta + cta_rank) * kBlockM;
+    u.row0 = ((unit - vocab_units) * (kTwo ? 2 : 1) * kCta + cta_rank) * kBlockM;
     u.g0 = 0;
     u.G = 0;
     u.tile_q = u.tile_r = 0;
@@ -131,7 +131,7 @@ __host__ __device__ __forceinline__ Unit unit_of(const TcParams& p, int unit, in
   const int at = unit - p.chunks * ru0;
   u.chunk = static_cast<int>(static_cast<uint32_t>(at) / static_cast<uint32_t>(group_rows));
   const int ru = ru0 + at - u.chunk * group_rows;
-  u.row0 = (ru * p.blocks * kCta + cta_rank) * kBlockM;
+  u.row0 = (ru * (kTwo ? 2 : 1) * kCta + cta_rank) * kBlockM;
   int c = u.chunk;
   if (kOdd) {                         // class by class: the chunks of a class share its rows out
     u.cls = static_cast<int>(static_cast<uint32_t>(c) / static_cast<uint32_t>(p.class_chunks));
