@@ -36,8 +36,8 @@ RIDGE_ROWS_HBM = 256            # at or below this many rows the step is reporte
 # hash of that source is recorded here and traffic is reported as null when the source differs.
 NCU_TRAFFIC = {
     "kernel_sources": ["paper_2504_07878_b200/csrc/tlr_tc_kernel.cuh", "paper_2504_07878_b200/csrc/tlr_tc_ptx.cuh"],
-    "sha256": "fcf89e609fd9e23d0e21baf5e0466ac0df3e3ca03c8d3b4ed7a579125d5fc6c4",
-    "bytes_per_launch": {"decode256": 274.47e6, "decode16": 274.19e6, "sweep512": 529.45e6},
+    "sha256": "fdbd77304915644e481c77d303dbe4d323662ebe984b08b06e7c5f549d3f0495",
+    "bytes_per_launch": {"decode256": 274.55e6, "decode16": 273.99e6, "sweep512": 531.59e6},
 }
 
 

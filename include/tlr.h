@@ -64,11 +64,12 @@ typedef struct {
   int32_t path;          /* tlr_path actually used */
   int32_t grid;          /* CTAs launched */
   int32_t block;         /* threads per CTA */
-  int32_t row_units;     /* ceil(n / rows per CTA tile) */
+  int32_t row_units;     /* ceil(n / rows of a work unit) */
   int32_t vocab_chunks;  /* partial results per row that the merge step folds */
   int32_t smem_bytes;    /* dynamic shared memory per CTA */
   int32_t launches;      /* kernels launched per tlr_route call */
-  int32_t reserved;      /* tlr_plan_query: 1 where a CTA pair keeps a row unit's h in shared memory for the whole unit */
+  int32_t reserved;      /* tlr_plan_query: 1 where a CTA pair keeps a row unit's h in shared memory for the whole unit,
+                          * 2 where a unit is two blocks of 256 rows that share W's slabs */
 } tlr_plan;
 
 /* Bits of the device status word (tlr_last_device_status). */
