@@ -213,25 +213,27 @@ __device__ __forceinline__ void finish_small(const FinishLaunch& a, const int lo
   float out_s, out_t;
   {
     const Partial* p = a.partials + static_cast<size_t>(valid ? row : 0) * a.row_stride;
-    const size_t cs = static_cast<size_t>(a.chunk_stride);
+    const int cs = a.chunk_stride;
     float m = -INFINITY;
     int idx = kNoToken;
     float s = 0.f, t = 0.f, second = -INFINITY;
     {
-      // one pass, the partials stay in registers
+      // one pass, the partials stay in registers: every load goes out before the first is looked at, and behind the last
+      // partial the last one is loaded again
       Partial q[kPerLane];
+      if (valid) {
 #pragma unroll
-      for (int k = 0; k < kPerLane; ++k) {
-        const int j = gl + L * k;
-        if (valid && j < a.chunks) {
-          const float4 raw = __ldcg(reinterpret_cast<const float4*>(p + j * cs));
+        for (int k = 0; k < kPerLane; ++k) {
+          const float4 raw = __ldcg(reinterpret_cast<const float4*>(p + min(gl + L * k, a.chunks - 1) * cs));
           q[k].m = raw.x;
           q[k].idx = __float_as_int(raw.y);
           q[k].s = raw.z;
           q[k].t = raw.w;
-        } else {
-          q[k] = empty_partial();
         }
+      }
+#pragma unroll
+      for (int k = 0; k < kPerLane; ++k) {
+        if (!valid || gl + L * k >= a.chunks) q[k] = empty_partial();
         if (q[k].m > m || (q[k].m == m && q[k].idx < idx)) {
           m = q[k].m;
           idx = q[k].idx;
@@ -389,9 +391,10 @@ finish_rows_kernel(const FinishLaunch a, const int log2_L) {
   }
 }
 
-// 32 registers: with 38 a shard's step of n = 444, d = 752, 6766 rows of W takes 15.8 us instead of 14.1, and a spilled one
-// costs 2 to 4 % of most small steps.
-__global__ void __launch_bounds__(kSmallThreads)
+// 32 registers, none spilled (which costs 2 to 4 % of most small steps), and a lane's loads all in flight: with 36 and a
+// condition per load n = 765, d = 976, V = 3005 13.5 instead of 13.0 us, n = 542, d = 888, V = 7195 17.1 and 16.7, n = 700, d = 400,
+// V = 20000 19.1 and 18.6 (but n = 619, d = 160, V = 19901 16.1 and 16.4).
+__global__ void __maxnreg__(32)
 finish_small_kernel(const FinishLaunch a, const int log2_L) {
   finish_small<false>(a, log2_L);
 }

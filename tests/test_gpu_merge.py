@@ -50,6 +50,25 @@ def test_edges_of_the_merge_blocks(pkg, kind, n):
     r.close()
 
 
+# A lane owns up to six partials, the last ones of its row or fewer: 21 to 24 partials for four lanes, 37 for eight; the rows end
+# inside a warp.
+@pytest.mark.parametrize("n,V,chunks", [(513, 1985, 21), (765, 2082, 22), (601, 2179, 23), (700, 1500, 24), (1023, 9260, 37)])
+def test_lanes_with_six_partials(pkg, n, V, chunks):
+    W, h = S.make_W(D, V, seed=n, std=0.2), S.make_h(n, D, seed=V).h
+    ref = O.route_oracle(S.bf16_bits(h), S.bf16_bits(W), 0.0)
+    tau = float(np.float32(np.median(ref.conf) * 1.01))
+    r = pkg.Router(W.cuda(), max_n=n)
+    assert pkg.tlr_plan_query(r.ctx, n).vocab_chunks == chunks
+    r.route(h.cuda(), tau)
+    torch.cuda.synchronize()
+    assert pkg.tlr_last_device_status(r.ctx) == 0
+    got = _outputs(r, n)
+    check_against_oracle(O.with_threshold(ref, tau), got)
+    mask = got["route_mask"]
+    assert got["routed_count"] == mask.sum() and np.array_equal(got["routed_idx"][:mask.sum()], np.flatnonzero(mask))
+    r.close()
+
+
 def _expect(kind, r, h, n):
     """What the router gives for a batch when nothing else is in flight."""
     torch.cuda.synchronize()
