@@ -13,7 +13,8 @@
 //              them.  No ticket, no second launch, one L2 round trip for the partials.
 //              finish_rows_kernel where a lane owns at most 5 partials: the compaction has a warp
 //              of its own.  Otherwise finish_small_kernel, 512 threads where a lane still owns
-//              at most 6 partials (else 1024, and where that is not enough, the kernel for larger n).  Blocks of 17 or 9 warps, and of 512 threads, fit on an
+//              at most 6 partials (else 1024, and where that is not enough, the kernel for larger n; so, too,
+//              with four lanes and ties to settle).  Blocks of 17 or 9 warps, and of 512 threads, fit on an
 //              SM beside a CTA of the tensor-core projection kernel, so
 //              the blocks are resident and waiting before that kernel ends, and the next
 //              call's CTAs do not have to wait for the merge to leave their SMs.
@@ -584,7 +585,12 @@ cudaError_t launch_finish(const FinishLaunch& a, cudaStream_t stream) {
     const SmallShape s = small_shape(a.n, a.chunks);
     blocks = s.blocks;
     threads = s.threads;
-    lanes = s.lanes;
+    // Settling a row's winner reads a row of W and of h by the row's lanes, beside the projection's shared memory with hardly any
+    // L1: with four lanes that takes longer than all the rest, and by how much changes with the order of the loads.  So a warp
+    // to a row in many blocks: n = 529, d = 522, V = 4165 36.0 and 21.1 us per step, n = 602, d = 794, V = 54687 125 and 80,
+    // n = 740, d = 204, V = 16622 24.5 and 22.8; short rows take longer there, n = 856, d = 108, V = 16628 22.3 and 23.4, and so do
+    // some with eight lanes, n = 480, d = 141, V = 40408 25.8 and 26.6.
+    lanes = ties && s.lanes < 8 && a.ties.d > 128 ? 0 : s.lanes;
   } else {
     lanes = 0;
   }

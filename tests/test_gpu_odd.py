@@ -5,7 +5,7 @@ import torch
 
 import tlr_synth as S
 from oracle import route_oracle as O
-from tests.parity import check_against_oracle, check_self_consistency, run_gpu
+from tests.parity import check_against_oracle, check_self_consistency, head_with_equal_rows, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -64,6 +64,27 @@ def test_equal_rows_of_different_classes_tie_to_the_lowest_index(pkg, n, d):
     assert sure.sum() >= n // 2
     gpu = run_gpu(pkg, W2.cuda(), hid.h, 0.5)
     assert np.array_equal(gpu["token"][sure], ref.token[sure])
+
+
+# Batches whose rows have four lanes in eight blocks or a warp in many (d > 128): winners with copies in other classes, the
+# list and the first routed positions.
+@pytest.mark.parametrize("n,d,V", [(513, 129, 2500), (640, 130, 3001), (600, 127, 2500), (1024, 300, 4000), (777, 999, 6001)])
+def test_middle_batches_settle_their_winners(pkg, n, d, V):
+    W, h, token, sure = head_with_equal_rows(n, d, V)
+    gpu = check(pkg, W, h, 0.5)
+    assert np.array_equal(gpu["token"][sure], token[sure])
+    L = 3 if n % 3 == 0 else 1
+    r = pkg.Router(W.cuda(), max_n=n)
+    first = torch.full((n // L,), -9, dtype=torch.int32, device="cuda")
+    tau = torch.from_numpy(np.where(np.arange(n) % 5 == 0, 2.0, 0.5).astype(np.float32)).cuda()
+    r.route(h.cuda(), 0.0, tau_per_row=tau, seq_len=L, first_routed=first)
+    torch.cuda.synchronize()
+    mask = gpu["conf"] < tau.cpu().numpy()
+    assert np.array_equal(r.route_mask[:n].cpu().numpy() == 1, mask) and int(r.routed_count.item()) == mask.sum()
+    assert np.array_equal(r.routed_idx[:mask.sum()].cpu().numpy(), np.flatnonzero(mask))
+    rows = mask.reshape(-1, L)[:n // L]
+    assert np.array_equal(first.cpu().numpy(), np.where(rows.any(axis=1), rows.argmax(axis=1), L))
+    r.close()
 
 
 # One row whose logits all lie below -1e30: what it gives is not specified, but nothing is read beyond W for it and the other
