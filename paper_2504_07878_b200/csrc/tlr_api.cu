@@ -314,10 +314,9 @@ void plan_step(const tlr_ctx* c, int n, bool mlp, tlr_ctx::Step* st) {
       if (cfg.mode == tlr::RowMode::kM128 && c->classes == 1 && n > 256) {
         tlr::TcPlan two;
         tlr::tc_plan(n, c->V, 2, 2, workers_max, tlr::kMaxChunks, mlp ? c->mlp_hidden : 0, 1, &two);
-        if (tlr::tc_two_blocks_pay(two, tp, c->d)) {
+        if (tlr::tc_two_blocks_pay(two, tp, c->d) && tlr::tc_configure_two(c->d, &cfg)) {
           tp = two;
           tp.group_units = tlr::tc_two_group(n, c->d, tp.row_units);
-          tlr::tc_configure_two(c->d, &cfg);
         }
       }
     }
@@ -613,6 +612,7 @@ static tlr_status plan_tiles(int blocks, int32_t n, int32_t V, int32_t sm_count,
   tlr::TcConfig cfg;
   tlr::TcPlan tp;
   tlr::tc_configure(n, 2048, V, sm_count, &cfg);
+  if (blocks == 2 && !tlr::tc_configure_two(2048, &cfg)) return TLR_ERR_UNSUPPORTED;
   const int workers_max = sm_count / cfg.cta;
   tlr::tc_plan(n, V, cfg.cta, blocks, workers_max, tlr::kMaxChunks, mlp_hidden, 1, &tp);
   const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;

@@ -106,14 +106,17 @@ void tc_configure(int n, int d, int V, int sm_count, TcConfig* c) {
 // those slabs stay occupied meanwhile.  Lags of 3 / 4 / 5 with five stages of h and eight of W, of 5 with four and nine, and
 // single blocks, us per step: n = 8192, d = 896, V = 151936 1738 / 1691 / 1648 / 1648 and 1738, n = 4096, d = 1536 there
 // 1429 / 1405 / 1386 / 1391 and 1459, n = 512, d = 2048, V = 128256 228 / 226 / 225 / 225 and 235; 6 of eight stages leave too
-// few for loads (407 instead of 364 at n = 777, d = 1536, V = 151936; 380 with single blocks).
-void tc_configure_two(int d, TcConfig* c) {
+// few for loads (407 instead of 364 at n = 777, d = 1536, V = 151936; 380 with single blocks).  False, and nothing changed, where
+// the W ring (TLR_TC_RINGS) does not hold the slabs that lie between the two: lag + 1, before the second block frees the first.
+bool tc_configure_two(int d, TcConfig* c) {
+  if (c->b_stages < 2) return false;
   const int k_slabs = (d + kRowBytes / 2 - 1) / (kRowBytes / 2);
   c->mode = RowMode::kM128Two;
   c->lag = c->b_stages - 3;
   if (c->lag > 5) c->lag = 5;
   if (c->lag > k_slabs) c->lag = k_slabs;
   if (c->lag < 1) c->lag = 1;
+  return true;
 }
 
 cudaError_t tc_prepare() {

@@ -147,7 +147,7 @@ inline bool tc_two_blocks_pay(const TcPlan& two, const TcPlan& one, int d) {
   const int k_slabs = (d + 63) / 64;
   return k_slabs >= 8 && two.passes * k_slabs >= 128 && two.passes * 100 <= one.passes * 104;
 }
-void tc_configure_two(int d, TcConfig* c);
+bool tc_configure_two(int d, TcConfig* c);
 void tc_plan(int n, int V, int cta, int blocks, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan);
 cudaError_t tc_prepare();   // opt in to the kernels' dynamic shared memory size (once per device)
 cudaError_t launch_tc_projection(const TcMaps& maps, const TcParams& p, const TcConfig& c, int workers,

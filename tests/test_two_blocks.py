@@ -1,4 +1,8 @@
 """Batches of more than 256 rows whose work units are two blocks of 256 token rows: the schedule on the CPU, results on the GPU."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -25,6 +29,18 @@ def test_tiles_of_both_blocks_cover_every_logit_once(n, V, hidden):
             assert np.array_equal(sel[1:, 3], (sel[:, 3] + sel[:, 4])[:-1])
     for unit in np.unique(tiles[:, 1]):
         assert len(np.unique(tiles[tiles[:, 1] == unit, 0])) == 1
+
+
+# With a lag of one the second block reads a slab of W behind the first block's next one: two stages, or such batches stay on
+# single blocks, which work with one.
+@pytest.mark.parametrize("rings,status", [("5,1", 3), ("5,2", 0), ("1,8", 0), ("4,9", 0)])
+def test_a_ring_that_cannot_hold_both_blocks_slabs(rings, status):
+    code = ("import ctypes, paper_2504_07878_b200 as P; c = ctypes.c_int32(0)\n"
+            "print(P.load_library().tlr_debug_plan_two_blocks(512, 128256, 148, 0, None, 0, ctypes.byref(c), None),"
+            " P.load_library().tlr_debug_plan_tiles(512, 128256, 148, 0, None, 0, ctypes.byref(c), None))")
+    run = subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                         env=dict(os.environ, TLR_TC_RINGS=rings), capture_output=True, text=True)
+    assert run.returncode == 0 and run.stdout.split() == [str(status), "0"], run.stdout + run.stderr
 
 
 # The fewest slabs of K and more, in part; second blocks of one row, of all rows and (25 blocks) of none; several units per worker;
