@@ -137,15 +137,26 @@ inline int tc_two_group(int n, int d, int row_units) {
   const long long groups = (2ll * n * d + kGroupBytes - 1) / kGroupBytes;
   return static_cast<int>((row_units + groups - 1) / groups);
 }
-// Whether units of two row blocks pay, given both plans.  Few units may leave the busiest worker more passes than single blocks would, of
-// which up to 4 % are given back (n = 1000, d = 896, V = 151936: 34 instead of 33, 232.5 and 229.6 us; an odd block is a unit and
-// counts for two, which is little among many).  Short walks have their first and last slabs longer, all the more the fewer slabs a
-// pass has: single blocks and two, n = 1000, d = 256, V = 36000 (8 passes of 4 slabs) 26.2 and 28.8 us, n = 400, d = 1024,
-// V = 30000 (4 of 16) 29.8 and 32.0, n = 1000, d = 640, V = 36000 (8 of 10) 39.5 and 40.9 in a short run, 46.2 and 45.9 in a long
-// one, d = 1024 there (8 of 16) 60.9 and 59.9, n = 4096, d = 640, V = 18944 (16 of 10) 79.5 and 77.9.
+// Whether units of two row blocks pay, given both plans.  They halve what W brings from L2 into shared memory, and how much that is
+// depends on where its rows begin: with d % 16 == 8 every other row begins off a 32-byte sector, so that a slab's 128 bytes take five
+// sectors instead of four, and loads of W bound single blocks.  Rows on sectors bring the least, and with one row unit, where every
+// worker reads the same h at the same time, nothing.  Single blocks and two, us per step at the power limit:
+//   d % 16 == 8   n = 450, d = 1032, V = 108884 125.5 and 114.0, n = 860, d = 1288, V = 54527 140.2 and 127.4, n = 392, d = 2024,
+//                 V = 37250 82.6 and 76.1 (128 slabs of row blocks per worker); below that n = 293, d = 568, V = 30010 21.1 and 23.3
+//   one row unit  n = 402, d = 880, V = 87086 72.0 and 78.3, n = 434, d = 1120, V = 104871 107.8 and 114.1, n = 512, d = 2048,
+//                 V = 128256 226 to 230 and 227 to 233
+//   two row units 128 to 260 slabs 0.92 to 1.06 times as fast, 0.97 on average (n = 900, d = 1024, V = 60000 105.9 and 109.3), from 260 on
+//                 1.01 (n = 1024, d = 2048, V = 128256 440 and 413); with a learned router's units in the launch 1.04 from 128 on
+//                 (n = 833, d = 1184, V = 54769 119.6 and 112.8)
+//   more          0.96 to 1.09, 1.00 on average up to 260 slabs, then 1.01 to 1.05 (n = 8192, d = 896, V = 151936 1697 and 1599)
+// Few units may leave the busiest worker more passes than single blocks would, of which up to 4 % are given back (n = 777, d = 1536,
+// V = 151936: 34 instead of 33, 351 to 372 and 357 to 364): a last unit of one block counts for two here, so that most batches of an
+// odd number of blocks, up to some twenty, stay on single ones.
 inline bool tc_two_blocks_pay(const TcPlan& two, const TcPlan& one, int d) {
   const int k_slabs = (d + 63) / 64;
-  return k_slabs >= 8 && two.passes * k_slabs >= 128 && two.passes * 100 <= one.passes * 104;
+  const bool off_sectors = d % 16 != 0;
+  const int least = off_sectors || two.mlp_rows > 0 || two.row_units > 2 ? 128 : 260;
+  return k_slabs >= 8 && (off_sectors || two.row_units >= 2) && two.passes * k_slabs >= least && two.passes * 100 <= one.passes * 104;
 }
 bool tc_configure_two(int d, TcConfig* c);
 void tc_plan(int n, int V, int cta, int blocks, int workers, int max_chunks, int mlp_hidden, int classes, TcPlan* plan);
