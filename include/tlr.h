@@ -364,9 +364,10 @@ tlr_status tlr_debug_plan_tiles(int32_t n, int32_t V, int32_t sm_count, int32_t 
                                 int32_t capacity, int32_t* count, tlr_plan* plan_out);
 
 /*
- * tlr_debug_plan_two_blocks -- the same for the schedule in which a unit is two blocks of 256 token rows (n > 128; batches of
- * more than 256 rows use it where it leaves no worker more to do): the tiles are those of both blocks.  TLR_ERR_UNSUPPORTED
- * where a ring that TLR_TC_RINGS asks for is too short for it.
+ * tlr_debug_plan_two_blocks -- the same for the schedule in which a unit is two blocks of 256 token rows (n > 128), at the
+ * hidden size 2048, where large batches are walked in groups of row units: the tiles are those of both blocks.  Batches of more
+ * than 256 rows take it by hidden size and length of the walk, and where it gives the busiest worker at most 4 % more tiles.
+ * TLR_ERR_UNSUPPORTED where a ring that TLR_TC_RINGS asks for is too short for it.
  */
 tlr_status tlr_debug_plan_two_blocks(int32_t n, int32_t V, int32_t sm_count, int32_t mlp_hidden, int32_t* out,
                                  int32_t capacity, int32_t* count, tlr_plan* plan_out);

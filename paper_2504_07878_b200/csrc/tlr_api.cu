@@ -615,6 +615,7 @@ static tlr_status plan_tiles(int blocks, int32_t n, int32_t V, int32_t sm_count,
   if (blocks == 2 && !tlr::tc_configure_two(2048, &cfg)) return TLR_ERR_UNSUPPORTED;
   const int workers_max = sm_count / cfg.cta;
   tlr::tc_plan(n, V, cfg.cta, blocks, workers_max, tlr::kMaxChunks, mlp_hidden, 1, &tp);
+  if (blocks == 2) tp.group_units = tlr::tc_two_group(n, 2048, tp.row_units);
   const int units = (tp.chunks + (tp.mlp_rows > 0 ? 1 : 0)) * tp.row_units;
   const int workers = units < workers_max ? units : workers_max;
   tlr::TcParams p = {};

@@ -9,20 +9,22 @@
 //               CTA stages its own 128 rows of h and HALF of the W tile, and the pair's
 //               tensor cores read both halves, so a W byte enters shared memory once
 //               per 256 token rows.                                          (n > 128)
+//               Above 256 rows a unit may be two blocks of 256 rows, one accumulator each: a slab of W is then read by
+//               the MMAs of both while it is in shared memory (TwoWalk).
 //   8-bit (e4m3) head for decode batches of at most 128 rows: h is the sum of two e4m3
 //               parts, stacked in one operand slab.  Up to 64 rows ONE kind::f8f6f4 MMA per K step
 //               covers both parts along its M, and the epilogue adds the two accumulator rows of a
 //               token before it folds them; above, two MMAs per K step (one per part) add into the
 //               same rows.
-//               Above 256 rows a unit may be two blocks of 256 rows, one accumulator each: a slab of W is then read by
-//               the MMAs of both while it is in shared memory (TwoWalk).
 //   bf16 head whose hidden size is no multiple of 8: the vocabulary is walked by residue class
 //               (see OddMaps), otherwise like the bf16 head.
 //
 // Decomposition.  The vocabulary is cut into `chunks` contiguous ranges of granules
 // (a multiple of 16 * kCta rows); the token rows into units of 128 * kCta.  A work unit is
 // (chunk, row unit); units are numbered chunk-major so that workers running at the
-// same time share W through L2, and worker w takes units w, w + workers, ...  Inside
+// same time share W through L2, and worker w takes units w, w + workers, ...  (two row
+// blocks: units of 512 rows, numbered group by group of row units and chunk-major in a
+// group).  Inside
 // a unit the chunk is walked in `tiles_per_unit` tiles of at most 256 vocabulary rows
 // (the MMA's N), each a K-loop over d in slabs of 128 bytes per row.  With a learned router
 // attached (bf16 head) one more unit per row unit follows the vocabulary units: its "vocabulary"
@@ -180,13 +182,13 @@ __host__ __device__ __forceinline__ Tile tile_of(const TcParams& p, const Unit& 
 // third and fourth one.  A unit whose second block has no rows is walked like a single one.
 struct TwoWalk {
   int blocks, items, lag, k_slabs;
-  __device__ __forceinline__ TwoWalk(const TcParams& p, int row0, int slabs) {
+  __host__ __device__ __forceinline__ TwoWalk(const TcParams& p, int row0, int slabs) {
     blocks = row0 + 2 * kBlockM < p.n ? 2 : 1;       // (row0 of the unit, whichever CTA asks)
     items = blocks * slabs;
-    lag = blocks == 2 ? min(p.lag, slabs) : slabs;
+    lag = blocks == 2 && p.lag < slabs ? p.lag : slabs;
     k_slabs = slabs;
   }
-  __device__ __forceinline__ void at(int i, int& block, int& slab) const {
+  __host__ __device__ __forceinline__ void at(int i, int& block, int& slab) const {
     const int j = i - lag;
     block = j < 0 ? 0 : (i + lag >= items ? 1 : j & 1);
     slab = j < 0 ? i : (i + lag >= items ? i - k_slabs : (j >> 1) + (block == 0 ? lag : 0));
@@ -389,7 +391,8 @@ __device__ __forceinline__ void tc_projection_body(const Maps& maps, const TcPar
   const uint32_t bar_base = b_ring + SB * b_stage_bytes;
   // Barriers: a_full / b_full per ring stage (data landed); released[j] completes when the
   // MMAs of slab number j (mod kRelease) have finished reading shared memory -- one commit
-  // per slab serves both rings: the producer of slab i waits for slab i - depth;
+  // per slab serves both rings: the producer of slab i waits for slab i - depth (two row blocks:
+  // the h ring alone, whose slabs are numbered as they are walked; the W ring has h_free);
   // acc_full / acc_empty per accumulator.
   auto a_full = [&](int s) { return bar_base + 8u * s; };
   auto b_full = [&](int s) { return bar_base + 8u * (kMaxAStages + s); };

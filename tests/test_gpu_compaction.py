@@ -53,3 +53,35 @@ def test_middle_batches_of_many_partials(n):
         assert np.array_equal(mask.cpu().numpy() != 0, flags)
         assert int(count.item()) == flags.sum() and np.array_equal(idx.cpu().numpy()[:flags.sum()], np.flatnonzero(flags))
     r.close()
+
+
+# The same kernel with the options of a call: thresholds per row, first routed positions, the learned router's scores -- and where
+# near-ties are settled (d % 8 != 0; chunks by residue class).
+@pytest.mark.parametrize("n,d,V", [(600, 96, 18944), (869, 97, 26475), (996, 101, 33000), (440, 142, 46443)])
+def test_middle_batches_with_options(n, d, V):
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    rand = lambda *size: torch.randn(size, generator=gen, device="cuda")  # noqa: E731
+    W, h = (rand(V, d) * 0.2).to(torch.bfloat16), rand(n, d).to(torch.bfloat16)
+    r = P.Router(W, max_n=n)
+    W1, b1, w2 = (rand(40, d) / d ** 0.5).to(torch.bfloat16), rand(40) * 0.1, rand(40) * 0.2
+    r.set_router_mlp(W1, b1, w2, 0.1)
+    assert P.tlr_plan_query(r.ctx, n).vocab_chunks > (96 if n <= 512 else 48)
+    z = h.double() @ W.double().T
+    want = torch.softmax(z, dim=1).amax(dim=1)
+    learned = torch.sigmoid(torch.relu(h.double() @ W1.double().T + b1) @ w2.double() + 0.1)
+    L = 4 if n % 4 == 0 else 11
+    tau = torch.where(torch.rand(n, generator=gen, device="cuda") < 0.5, 0.02, 0.2)
+    for source in (P.TLR_SCORE_CONF, P.TLR_SCORE_MLP):
+        first = torch.full((n // L,), -1, dtype=torch.int32, device="cuda")
+        score = torch.full((n,), float("nan"), device="cuda")
+        token, conf, _, mask, idx, count = r.route(h, 0.0, tau_per_row=tau if source == P.TLR_SCORE_CONF else tau + 0.4,
+                                                   seq_len=L, first_routed=first, score_source=source, mlp_score=score)
+        assert torch.all((conf - want).abs() <= 2e-5 * want) and torch.all((score - learned).abs() <= 1e-5)
+        assert torch.all(z.gather(1, token.long()[:, None])[:, 0] >= z.amax(dim=1) - 1e-4)
+        flags = (conf < tau if source == P.TLR_SCORE_CONF else score < tau + 0.4).cpu().numpy()
+        assert 0 < flags.sum() < n and np.array_equal(mask.cpu().numpy() != 0, flags)
+        assert int(count.item()) == flags.sum() and np.array_equal(idx.cpu().numpy()[:flags.sum()], np.flatnonzero(flags))
+        rows = flags.reshape(-1, L)
+        assert np.array_equal(first.cpu().numpy(), np.where(rows.any(axis=1), rows.argmax(axis=1), L))
+    assert P.tlr_last_device_status(r.ctx) == 0
+    r.close()

@@ -13,12 +13,14 @@ from tests.parity import to_np
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [48, 300])          # one CTA per worker / a pair of CTAs per worker
-def test_wait_runs_out_and_context_survives(pkg, n):
-    d, V = 128, 40000
+# one CTA per worker / a pair of CTAs per worker / two row blocks to a unit, the second of 44 and of all 256 rows
+@pytest.mark.parametrize("n,d,V,two", [(48, 128, 40000, False), (300, 128, 40000, False), (300, 712, 105000, True),
+                                       (1024, 584, 61000, True)])
+def test_wait_runs_out_and_context_survives(pkg, n, d, V, two):
     W = S.make_W(d, V, seed=2, std=0.1)
     hid = S.make_h(n, d, seed=3)
     r = pkg.Router(W.cuda(), max_n=n)
+    assert (pkg.tlr_plan_query(r.ctx, n).reserved == 2) == two
     h = hid.h.cuda()
 
     def run():

@@ -91,6 +91,21 @@ def test_static_entry_point_small_batch_and_no_status_word(pkg):
             assert got["free_after"] == got["free_before"]
 
 
+# Rows with more partials than the lanes of eight blocks keep: the merge kernel with many blocks, with its ticket and its flag
+# bits in the fixed scratch; twice, the second time with fewer rows.
+@pytest.mark.parametrize("n,d,V", [(640, 96, 18944), (1024, 72, 33000)])
+def test_static_entry_point_many_partials(pkg, n, d, V):
+    W = S.make_W(d, V, seed=n, std=0.2)
+    Wd = W.cuda()
+    h = S.make_h(n, d, seed=d, W=W, planted_fraction=0.1).h
+    for rows, tau in ((n, 0.5), (n - 31, 2.0), (n, 0.0), (n, 0.5)):
+        got, want = route_static(pkg, Wd, h[:rows], tau), run_gpu(pkg, Wd, h[:rows], tau)
+        assert want["plan"].vocab_chunks > 48 and got["status"] == 0 and want["status"] == 0
+        check_self_consistency(got, tau, V)
+        assert_same(got, want)
+        assert np.all(got["routed_idx"][got["routed_count"]:] == -3)
+
+
 def test_static_entry_point_small_hidden_size_and_limits(pkg):
     # d % 8 != 0 takes the CUDA-core kernel; more rows than the fixed scratch holds is an error
     W = S.make_W(36, 1500, seed=4, std=0.2)
