@@ -145,8 +145,12 @@ mlp_mma_kernel(const MlpLaunch a) {
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
   float acc[4][4] = {};
   // Bound by the trips to memory, one per batch, that take about 3 us each beside the stream of W where they go to HBM: with few
-  // rows this kernel then ends behind the projection.  So the block's rows of W1 are asked for at once.  n = 2, d = 1712,
-  // V = 49399, 225 units 31.4 -> 26.8 us per step, n = 10, d = 896, V = 60000 17.6 -> 16.3, n = 40, d = 1024 there 20.6 both.
+  // rows this kernel then ends behind the projection.  So the block's rows of W1 are asked for at once.  us per step without and
+  // with it, where the step finds nothing in L2: n = 2, d = 1712, V = 49399, 225 units 31.2 and 27.4, n = 4, d = 2048, V = 20000, 128 units
+  // 26.1 and 21.8, n = 33, d = 1696, V = 20698, 421 units 26.9 and 22.6, n = 16, d = 896, V = 151936, 256 units 29.0 and 28.9.  Where the step
+  // before has left all of W and W1 there, the requests stand in the way of the loads: n = 4, d = 2048, V = 32000, 512 units 16.1 and
+  // 18.6, n = 48, d = 1536, V = 30000, 300 units 17.0 and 18.5, n = 10, d = 896, V = 60000, 256 units 14.7 both; a decoder's other layers
+  // see to it that it has not.
   if (blockIdx.x == 0) {
     const char* rows = reinterpret_cast<const char*>(W1 + static_cast<size_t>(unit0) * a.d);
     const size_t bytes = static_cast<size_t>(min(kMlpUnits, a.d_hidden - unit0)) * a.d * 2;
