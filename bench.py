@@ -36,8 +36,8 @@ RIDGE_ROWS_HBM = 256            # at or below this many rows the step is reporte
 # hash of that source is recorded here and traffic is reported as null when the source differs.
 NCU_TRAFFIC = {
     "kernel_sources": ["paper_2504_07878_b200/csrc/tlr_tc_kernel.cuh", "paper_2504_07878_b200/csrc/tlr_tc_ptx.cuh"],
-    "sha256": "fdbd77304915644e481c77d303dbe4d323662ebe984b08b06e7c5f549d3f0495",
-    "bytes_per_launch": {"decode256": 274.55e6, "decode16": 273.99e6, "sweep512": 531.59e6},
+    "sha256": "d62bfbe3c65ac2b74298ddbf3d92a9a768b37a9e58fa621656d3e779caee64da",
+    "bytes_per_launch": {"decode256": 274.45e6, "decode16": 274.45e6, "sweep512": 529.37e6},
 }
 
 
